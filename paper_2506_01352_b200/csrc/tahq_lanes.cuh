@@ -1,0 +1,410 @@
+// Tile kernels in which a lane holds 64 bytes of the tensor (sm_100a): 32 elements of bfloat16 or 16 of binary32, so
+// that a tile of 32, 64 or 128 elements belongs to 1 ... 8 neighbouring lanes.  Few values to a lane mean 80 registers
+// and 24 warps on an SM (a lane that holds a whole tile needs 128 and gets 16), and the tensor moves between
+// registers and memory in whole 32-byte sectors without a stage in shared memory.
+//
+// A warp works on "rounds" of 32 / P tiles (P lanes to a tile), the CTA's rounds dealt out over its warps one by one,
+// and asks for the next round's bytes before it works on the current one.  Tiles that are transformed (Eq. 4) cost
+// twice as much as the others: they are put aside, lane by lane with what the lane has loaded of them, in a queue
+// of the warp in shared memory, and when a whole warp's worth has gathered they make up a round of their own.
+#pragma once
+
+#include "tahq_stream.cuh"
+
+namespace tahq {
+
+// one CTA per SM: the bit map in front of a CTA's tiles is counted once per SM, not once per few warps
+constexpr int kLaneThreads = 768;
+constexpr int kLaneWarps = kLaneThreads / 32;   // (a multiple of every P: a lane's bit in the bit-map words is fixed)
+
+template <class C>
+struct LaneCfg {
+  static constexpr int E = 64 / C::ESZ;        // elements of a lane
+  static constexpr int P = C::G / E;           // lanes of a tile
+  static constexpr int TPR = 32 / P;           // tiles of a round
+  static constexpr int TB = C::G * C::ESZ;     // bytes of a tile
+  static_assert(kLaneWarps % P == 0, "a warp's rounds take the same part of their bit-map word");
+};
+
+template <bool WIDE>
+__device__ __forceinline__ void store_64_bytes(uint8_t *dst, const uint32_t (&o)[16]) {
+#pragma unroll
+  for (int i = 0; i < 16; i += 8) {
+    if constexpr (WIDE) {   // (streaming: the tensor is not read again by this library)
+      asm volatile("st.global.cs.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst + 4 * i), "r"(o[i]),
+                   "r"(o[i + 1]), "r"(o[i + 2]), "r"(o[i + 3]), "r"(o[i + 4]), "r"(o[i + 5]), "r"(o[i + 6]), "r"(o[i + 7])
+                   : "memory");
+    } else {                // the tensor's base is only 16-byte aligned
+      __stcs(reinterpret_cast<uint4 *>(dst + 4 * i), make_uint4(o[i], o[i + 1], o[i + 2], o[i + 3]));
+      __stcs(reinterpret_cast<uint4 *>(dst + 4 * i) + 1, make_uint4(o[i + 4], o[i + 5], o[i + 6], o[i + 7]));
+    }
+  }
+}
+
+// Words of a lane's codes.  32 codes of W bits are W whole words; 16 codes start on a half word if W is odd and the
+// lane is, and lie in W / 2 words rounded up (`half`: 16 if they do, else 0).
+template <int E, int NWORD>
+__device__ __forceinline__ void load_codes(const uint32_t *tile, uint32_t sub, uint32_t W, uint32_t (&w)[NWORD]) {
+  const uint32_t first = E == 32 ? sub * W : (sub * W) >> 1;
+  const uint32_t n = E == 32 ? W : (W + 1) >> 1;
+#pragma unroll
+  for (int j = 0; j < NWORD; ++j) w[j] = (j < E / 16 || (uint32_t)j < n) ? __ldg(tile + first + j) : 0u;
+}
+
+// z + q*s for a lane's codes of W = 2, 3 or 4 bits (W is a lane's own value): eight codes -- W whole bytes -- are
+// brought to the bottom of a word, masked where they sit and OR-ed into the mantissa of 2^23 (giving 2^23 + q*2^p
+// exactly); one subtraction and one fused multiply-add with s*2^-p give the same bits as fma((float)q, s, z).
+template <int E, int NWORD>
+__device__ __forceinline__ void dequant_narrow_lane(const uint32_t (&w)[NWORD], uint32_t sub, uint32_t W, float s, float z,
+                                                    float2 (&p)[E / 2]) {
+  uint32_t g[E / 8];
+  if constexpr (E == 32) {
+    g[0] = w[0];
+    g[1] = __funnelshift_rc(w[0], w[1], 8u * W);          // (16, 24 or 32: the clamped form shifts by a whole word)
+    g[2] = __funnelshift_rc(w[1], w[2], 16u * W - 32u);   // (0, 16 or 32)
+    const bool two = W == 2u;
+    g[3] = __funnelshift_rc(two ? w[1] : w[2], two ? 0u : w[3], two ? 16u : 24u * W - 64u);   // (16; 8 or 32)
+  } else {
+    const uint32_t sh = (sub & W & 1u) * 16u;
+    const uint32_t v0 = __funnelshift_r(w[0], w[1], sh), v1 = w[1] >> sh;
+    g[0] = v0;
+    g[1] = __funnelshift_rc(v0, v1, 8u * W);
+  }
+  uint32_t two23;
+  asm volatile("mov.u32 %0, 0x4B000000;" : "=r"(two23));
+  const float step = __uint_as_float((127u - W) << 23);   // 2^-W
+  uint32_t mk[4];
+  float sc[4];
+  mk[0] = (1u << W) - 1u;
+  sc[0] = s;
+#pragma unroll
+  for (int i = 1; i < 4; ++i) { mk[i] = mk[i - 1] << W; sc[i] = sc[i - 1] * step; }   // s * 2^-(W i), exact
+#pragma unroll
+  for (int j = 0; j < E / 8; ++j) {
+    const uint32_t hi = g[j] >> (4u * W);
+#pragma unroll
+    for (int i = 0; i < 8; i += 2) {
+      uint32_t m0, m1;
+      asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(m0) : "r"(i < 4 ? g[j] : hi), "r"(mk[i & 3]), "r"(two23));
+      asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(m1) : "r"(i < 4 ? g[j] : hi), "r"(mk[(i + 1) & 3]), "r"(two23));
+      const float2 f = add2(f2(__uint_as_float(m0), __uint_as_float(m1)), f2(-8388608.0f));   // q * 2^p, exact
+      p[4 * j + i / 2] = fma2(f, f2(sc[i & 3], sc[(i + 1) & 3]), f2(z));
+    }
+  }
+}
+template <int W, int E, int NWORD>
+__device__ __forceinline__ void dequant_lane_w(const uint32_t (&w)[NWORD], uint32_t sub, float s, float z, float2 (&p)[E / 2]) {
+  float x[E];
+  if constexpr (E == 16 && W % 2) {
+    const uint32_t sh = (sub & 1u) * 16u;
+    uint32_t v[NWORD];
+#pragma unroll
+    for (int j = 0; j < NWORD; ++j) v[j] = __funnelshift_r(w[j], j + 1 < NWORD ? w[j + 1 < NWORD ? j + 1 : j] : 0u, sh);
+    unpack_dequant<W, E>(v, s, z, x);
+  } else {
+    unpack_dequant<W, E>(w, s, z, x);
+  }
+#pragma unroll
+  for (int i = 0; i < E / 2; ++i) p[i] = f2(x[2 * i], x[2 * i + 1]);
+}
+template <bool NARROW, int E, int NWORD>
+__device__ __forceinline__ void dequant_lane(const uint32_t (&w)[NWORD], uint32_t sub, uint32_t W, float s, float z,
+                                             float2 (&p)[E / 2]) {
+  if constexpr (NARROW) {
+    dequant_narrow_lane<E, NWORD>(w, sub, W, s, z, p);
+  } else {   // wider codes: the two widths of a call are neighbours, and most calls have one
+    switch (W) {
+      case 4: dequant_lane_w<4, E>(w, sub, s, z, p); break;
+      case 5: dequant_lane_w<5, E>(w, sub, s, z, p); break;
+      case 6: dequant_lane_w<6, E>(w, sub, s, z, p); break;
+      case 7: dequant_lane_w<7, E>(w, sub, s, z, p); break;
+      default: dequant_lane_w<8, E>(w, sub, s, z, p); break;
+    }
+    __syncwarp();
+  }
+}
+
+// Butterfly of Eq. 4 on a tile spread over P lanes, E elements each: strides below E inside the lane, the others
+// between lanes (lower half: own + other; upper half: other - own; the products by +-1 are exact).
+template <int E, int P>
+__device__ __forceinline__ void butterfly_lanes(float2 (&p)[E / 2], uint32_t sub) {
+  butterfly2<E / 2>(p);
+#pragma unroll
+  for (int h = 1; h < P; h *= 2) {
+    const float2 sg = f2((sub & h) ? -1.0f : 1.0f);
+#pragma unroll
+    for (int i = 0; i < E / 2; ++i) {
+      const float2 o = f2(__shfl_xor_sync(kFull, p[i].x, h), __shfl_xor_sync(kFull, p[i].y, h));
+      p[i] = fma2(p[i], sg, o);
+    }
+  }
+}
+
+// ------------------------------------------------------------------------------------------
+// Decode (Sec. 3.3, Algorithm 1 line 5)
+//
+// Bound by instruction issue (0.6 per scheduler and cycle at 770 instructions per 32 tiles of 64) and, from a gibibyte
+// on, half by the tensor's way to DRAM.  Against a lane per tile with the codes and rows staged in shared memory, 16
+// warps per SM: 22.3 -> 18.6 us for 8192 x 4096 bf16 at 3.8 bits, 78.5 -> 74.3 us for 16384 x 5120 fp32, 323 -> 293 us
+// for 65536 x 8192 bf16 with 1 % outlier channels, 12.5 -> 9.6 us for 8192 x 768 fp32, where a warp of the older
+// kernel had three units of 32 tiles one after the other.  With 16 elements to a bf16 lane 22.6 us, with three
+// CTAs of 8 warps per SM instead of one of 24 (each counting the bit map in front of it) 21.1 us.
+// ------------------------------------------------------------------------------------------
+template <class C, bool NARROW>
+struct DecodeLanes {
+  static constexpr int NWORD = C::BF16 ? (NARROW ? 4 : 8) : (NARROW ? 2 : 4);   // words of a lane's codes at the largest width
+  // per warp: the queue of lanes put aside (two times 32: codes; scale/zero, tile, width and pivot) and the rows of a
+  // round of them, where the pivot's coordinates change places
+  static constexpr int WARP = 64 * (NWORD * 4 + 16) + 32 * 64;
+  static constexpr int SMEM = kLaneWarps * WARP;
+};
+
+// The elements of a lane -> the tensor's type.
+template <class C>
+__device__ __forceinline__ void lane_words(const float2 (&p)[LaneCfg<C>::E / 2], uint32_t (&o)[16]) {
+#pragma unroll
+  for (int i = 0; i < LaneCfg<C>::E / 2; ++i) {
+    if constexpr (C::BF16) {
+      const __nv_bfloat162 h2 = __floats2bfloat162_rn(p[i].x, p[i].y);
+      o[i] = *reinterpret_cast<const uint32_t *>(&h2);
+    } else {
+      o[2 * i] = __float_as_uint(p[i].x);
+      o[2 * i + 1] = __float_as_uint(p[i].y);
+    }
+  }
+}
+
+// 32 lanes of the queue (the first n of them count), whole tiles with their lanes side by side: codes, the butterfly,
+// coordinates 0 and d change places again, the rows leave.
+template <class C, bool NARROW, bool WIDE_ST>
+__device__ __forceinline__ void decode_flagged_round(const uint32_t *q_codes, const uint4 *q_info, uint4 *rows, uint32_t head,
+                                                     uint32_t n, uint8_t *out_cta) {
+  using D = LaneCfg<C>;
+  constexpr int E = D::E, P = D::P, NWORD = DecodeLanes<C, NARROW>::NWORD;
+  const uint32_t lane = threadIdx.x & 31u, sub = lane % P;
+  const uint32_t at = (head + (lane < n ? lane : sub)) & 63u;
+  const uint4 info = q_info[at];
+  uint32_t w[NWORD];
+#pragma unroll
+  for (int j = 0; j < NWORD / 2; ++j) {
+    const uint2 v = reinterpret_cast<const uint2 *>(q_codes)[64 * j + at];
+    w[2 * j] = v.x; w[2 * j + 1] = v.y;
+  }
+  float s = __half2float(__ushort_as_half((unsigned short)(info.x & 0xffffu)));
+  float z = __half2float(__ushort_as_half((unsigned short)(info.x >> 16)));
+  // 1/sqrt(G) a power of two: scaling s and z beforehand scales every later value exactly, so the result has the
+  // same bits as multiplying at the end
+  constexpr bool kFold = C::G == 64 || C::G == 16;
+  if (kFold) { s *= hadamard_scale<C>(); z *= hadamard_scale<C>(); }
+  float2 p[E / 2];
+  dequant_lane<NARROW, E>(w, sub, info.z & 15u, s, z, p);
+  butterfly_lanes<E, P>(p, sub);
+  if (!kFold) {
+#pragma unroll
+    for (int i = 0; i < E / 2; ++i) p[i] = mul2(p[i], f2(hadamard_scale<C>()));   // feeds no addition
+  }
+  uint32_t o[16];
+  lane_words<C>(p, o);
+  auto piece = [&](uint32_t l, uint32_t q) -> uint4 * { return rows + l * 4u + (q ^ ((l >> 1) & 3u)); };   // XOR-swizzled
+#pragma unroll
+  for (int q = 0; q < 4; ++q) *piece(lane, q) = make_uint4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
+  __syncwarp();
+  if (sub == 0) {
+    using T = typename std::conditional<C::BF16, uint16_t, uint32_t>::type;
+    constexpr uint32_t EPP = 16 / C::ESZ;   // elements of a piece
+    const uint32_t d = (info.z >> 4) & (C::G - 1);   // masked: a foreign buffer cannot reach outside the tile
+    T *const p0 = reinterpret_cast<T *>(piece(lane, 0));
+    T *const pd = reinterpret_cast<T *>(piece(lane + d / E, d % E / EPP)) + d % EPP;
+    const T x0 = *p0, xd = *pd;
+    *p0 = xd;
+    *pd = x0;
+  }
+  __syncwarp();
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const uint4 v = *piece(lane, q);
+    o[4 * q] = v.x; o[4 * q + 1] = v.y; o[4 * q + 2] = v.z; o[4 * q + 3] = v.w;
+  }
+  if (lane < n) store_64_bytes<WIDE_ST>(out_cta + (uint64_t)info.y * D::TB, o);
+}
+
+template <class C, bool NARROW, bool WIDE_ST>
+__global__ void __launch_bounds__(kLaneThreads, 1) decode_lanes_kernel(const Args a) {
+  using D = LaneCfg<C>;
+  using S = DecodeLanes<C, NARROW>;
+  constexpr int NT = kLaneThreads, E = D::E, P = D::P, TPR = D::TPR, NWORD = S::NWORD;
+  constexpr uint32_t kTB = C::G / 8;   // bytes of a tile's codes per bit of width
+  extern __shared__ __align__(128) uint8_t smem_dl[];
+  __shared__ uint2 s_word[NT];         // the segment's bit-map words, higher-width tiles of the CTA in front of each
+  __shared__ uint32_t s_sum[2][32];    // per warp: set bits of its words of the segment, of its share of the words in front
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t sub = (uint32_t)lane % P;   // this lane's part of its tile
+  const unsigned lt = (1u << lane) - 1u;
+  uint32_t *const q_codes = reinterpret_cast<uint32_t *>(smem_dl + (size_t)warp * S::WARP);   // [NWORD / 2][64] pairs
+  uint4 *const q_info = reinterpret_cast<uint4 *>(q_codes + 64 * NWORD);
+  uint4 *const rows = q_info + 64;
+  TraceScope trace(a.trace, 5);
+  grid_dependency_wait();   // the packed buffer may be the work of the kernel in front (and so are cleared flags)
+  trace.started();
+  const uint32_t *bitmap = reinterpret_cast<const uint32_t *>(a.packed + a.off_bitmap);
+
+  // the CTA's rounds, the bit-map words that hold their tiles
+  const uint64_t n_rounds = (a.n_tiles + TPR - 1) / TPR;
+  const uint64_t r0 = n_rounds * blockIdx.x / gridDim.x, r1 = n_rounds * (blockIdx.x + 1ull) / gridDim.x;
+  const uint64_t u0 = r0 / P, u1 = (r1 + P - 1) / P;
+  const uint64_t tile_cta = u0 * 32;
+
+  // The prologue's loads -- the header, the bit-map words of the CTA's first segment, the words in front of its slice --
+  // are all requested before the first barrier: one round trip to L2.
+  const bool checks = blockIdx.x == 0 || a.own_prefix;
+  const uint32_t hdr_w = (checks && threadIdx.x < 32) ? __ldg(reinterpret_cast<const uint32_t *>(a.packed) + threadIdx.x) : 0u;
+  auto bm_word = [&](uint64_t i) -> uint32_t {   // bits beyond the last tile cleared
+    if (!a.mixed) return 0u;
+    const uint64_t left = a.n_tiles - i * 32;
+    return __ldg(bitmap + i) & (left >= 32u ? 0xffffffffu : ((1u << (uint32_t)left) - 1u));
+  };
+  uint32_t word = u0 + threadIdx.x < u1 ? bm_word(u0 + threadIdx.x) : 0u;
+  uint32_t front = 0;   // a.own_prefix: this thread's share of the higher-width tiles in front of the CTA's words
+  if (a.own_prefix && a.mixed) {   // 128-bit loads, four in flight per thread, then the last few words one by one
+    const uint4 *b4 = reinterpret_cast<const uint4 *>(bitmap);
+    const uint32_t n4 = (uint32_t)(u0 / 4);
+    for (uint32_t i = threadIdx.x; i < n4; i += 4u * NT) {
+      uint4 v[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) v[j] = i + j * NT < n4 ? __ldg(b4 + i + j * NT) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) front += __popc(v[j].x) + __popc(v[j].y) + __popc(v[j].z) + __popc(v[j].w);
+    }
+    if (threadIdx.x < (uint32_t)(u0 & 3)) front += __popc(__ldg(bitmap + (uint64_t)n4 * 4 + threadIdx.x));
+  }
+  if (r0 == r1) {   // (never the first CTA, nor the last)
+    bool stop;
+    if (!a.own_prefix) cta_exclusive_prefix<NT>(a, 0, false, stop);
+    return;
+  }
+
+  const bool wrong = checks && threadIdx.x < 32 && hdr_w != a.header[threadIdx.x];
+  const uint8_t *pay = nullptr;   // the CTA's first code
+  bool stop = false;
+  uint32_t seg_hi = 0;   // higher-width tiles of this CTA's earlier segments
+  uint32_t pay_left = 0;   // bytes of the payload from the CTA's first code (a corrupt bit map must not lead outside)
+  uint32_t qhead = 0, qn = 0;
+  const uint32_t *const sz_cta = reinterpret_cast<const uint32_t *>(a.packed + a.off_sz) + tile_cta;
+  const uint8_t *const pv_cta = a.packed + a.off_pivot + tile_cta;
+  uint8_t *const out_cta = a.out + tile_cta * (uint64_t)D::TB + sub * 64u;
+  const uint32_t n_rel = a.n_tiles - tile_cta < 0xffffffffull ? (uint32_t)(a.n_tiles - tile_cta) : 0xffffffffu;
+
+  for (uint64_t s0 = u0; s0 < u1; s0 += NT) {
+    const uint64_t s1 = s0 + NT < u1 ? s0 + NT : u1;
+    if (s0 != u0) {
+      word = s0 + threadIdx.x < u1 ? bm_word(s0 + threadIdx.x) : 0u;
+      __syncthreads();   // every warp is done with the previous segment's words
+    }
+    // running count over the segment's words, one per thread; the words in front
+    uint32_t incl = (uint32_t)__popc(word);
+#pragma unroll
+    for (int o = 1; o < 32; o *= 2) {
+      const uint32_t v = __shfl_up_sync(kFull, incl, o);
+      if (lane >= o) incl += v;
+    }
+    front = __reduce_add_sync(kFull, front);
+    if (lane == 31) { s_sum[0][warp] = incl; s_sum[1][warp] = front; }
+    const bool refuse = __syncthreads_or(wrong) != 0;
+    const uint32_t sw = lane < kLaneWarps ? s_sum[0][lane] : 0u;
+    const uint32_t before = __reduce_add_sync(kFull, lane < warp ? sw : 0u), total = __reduce_add_sync(kFull, sw);
+    s_word[threadIdx.x] = make_uint2(word, seg_hi + before + incl - (uint32_t)__popc(word));
+    if (s0 == u0) {   // Sec. 3.4: higher-width tiles in front of the CTA's words; what was found in the header
+      // CTA 0 compares the received header with the one these parameters produce; what it finds travels with the
+      // offset prefix, so a refused buffer leaves the output untouched.  (a.own_prefix: every CTA does this itself
+      // and counts the bit map in front of its slice itself: nothing has to be cleared beforehand, and the last CTA,
+      // which sees the whole count, writes the status.)
+      const bool last = blockIdx.x == gridDim.x - 1 && threadIdx.x == 0;
+      uint64_t base_hi;
+      if (a.own_prefix) {
+        base_hi = __reduce_add_sync(kFull, lane < kLaneWarps ? s_sum[1][lane] : 0u);
+        stop = refuse;
+        if (last)   // (at most 65536 words: one segment)
+          *a.status = (refuse ? 1u /* TAHQ_DEV_BAD_HEADER */ : 0u) |
+                      ((a.mixed && !refuse && base_hi + total != a.n_groups * a.k_hi) ? 2u /* TAHQ_DEV_BAD_BITMAP */ : 0u);
+      } else {
+        // a CTA publishes the count of the words that start in its range (one shared by two CTAs counts in the first)
+        if (refuse && threadIdx.x == 0) atomicOr(a.status, 1u);
+        const uint64_t uc0 = (r0 + P - 1) / P;
+        uint32_t n = 0;
+        for (uint64_t i = uc0 + threadIdx.x; i < u1; i += NT) n += __popc(bm_word(i));
+        n = block_sum<NT>(n);
+        base_hi = cta_exclusive_prefix<NT>(a, n, refuse, stop);
+        if (last && a.mixed && !stop && base_hi + n != a.n_groups * a.k_hi) atomicOr(a.status, 2u);
+        if (uc0 != u0) base_hi -= (uint32_t)__popc(bm_word(u0));
+      }
+      const uint64_t pay0 = (uint64_t)kTB * ((uint64_t)a.lo * tile_cta + base_hi);
+      if (pay0 < a.payload_bytes) {
+        pay = a.packed + a.off_payload + pay0;
+        pay_left = a.payload_bytes - pay0 < 0xffffffffull ? (uint32_t)(a.payload_bytes - pay0) : 0xffffffffu;
+      }
+    }
+    __syncthreads();
+    if (stop) return;
+
+    // the warp's rounds; their tiles take the same bits of their words
+    const uint64_t rs0 = s0 * P > r0 ? s0 * P : r0, rs1 = s1 * P < r1 ? s1 * P : r1;
+    const uint32_t k1 = (uint32_t)(rs1 - s0 * P);
+    uint32_t k = (uint32_t)(rs0 - s0 * P) + warp;
+    const uint32_t t = k % P * TPR + (uint32_t)lane / P, bit = 1u << t, below = bit - 1u;
+    const uint32_t seg_tile = (uint32_t)(s0 - u0) * 32u + t;   // from the CTA's first
+    {   // does the segment's last code lie inside the payload?  If not, the bit map is corrupt and the rest is left out.
+      const uint32_t tiles = (uint32_t)(s1 - u0) * 32u;
+      if ((uint64_t)kTB * ((uint64_t)a.lo * (tiles < n_rel ? tiles : n_rel) + seg_hi + total) > pay_left) return;
+    }
+    uint32_t w[NWORD], sz, wp;   // the next round: codes; scale and zero-point; width + 16 * pivot byte, 0: no tile
+    auto load = [&](uint32_t kk) {
+      const uint2 bw = s_word[kk / P];
+      const uint32_t tile = seg_tile + kk / P * 32u, W = a.lo + ((bw.x & bit) ? 1u : 0u);
+      const uint32_t off = kTB * (a.lo * tile + bw.y + (uint32_t)__popc(bw.x & below));
+      wp = 0;
+      if (tile < n_rel) {
+        load_codes<E, NWORD>(reinterpret_cast<const uint32_t *>(pay + off), sub, W, w);
+        sz = __ldg(sz_cta + tile);
+        wp = W | (uint32_t)__ldg(pv_cta + tile) << 4;
+      }
+    };
+    if (k < k1) load(k);
+    for (; k < k1; k += kLaneWarps) {
+      uint32_t cw[NWORD];
+#pragma unroll
+      for (int j = 0; j < NWORD; ++j) cw[j] = w[j];
+      const uint32_t csz = sz, cwp = wp, tile = seg_tile + k / P * 32u;
+      if (k + kLaneWarps < k1) load(k + kLaneWarps);
+      const bool flagged = (cwp & 0x800u) != 0;
+      const unsigned held = __ballot_sync(kFull, flagged);
+      if (flagged) {   // put aside
+        const uint32_t at = (qhead + qn + (uint32_t)__popc(held & lt)) & 63u;
+#pragma unroll
+        for (int j = 0; j < NWORD / 2; ++j) reinterpret_cast<uint2 *>(q_codes)[64 * j + at] = make_uint2(cw[2 * j], cw[2 * j + 1]);
+        q_info[at] = make_uint4(csz, tile, cwp, 0u);
+      }
+      qn += (uint32_t)__popc(held);
+      if (held != kFull) {
+        const float s = __half2float(__ushort_as_half((unsigned short)(csz & 0xffffu)));
+        const float z = __half2float(__ushort_as_half((unsigned short)(csz >> 16)));
+        float2 p[E / 2];
+        dequant_lane<NARROW, E>(cw, sub, cwp & 15u, s, z, p);
+        uint32_t o[16];
+        lane_words<C>(p, o);
+        if (cwp != 0u && !flagged) store_64_bytes<WIDE_ST>(out_cta + (uint64_t)tile * D::TB, o);
+      }
+      if (qn >= 32u) {
+        __syncwarp();
+        decode_flagged_round<C, NARROW, WIDE_ST>(q_codes, q_info, rows, qhead, 32u, out_cta);
+        qhead = (qhead + 32u) & 63u;
+        qn -= 32u;
+        __syncwarp();
+      }
+    }
+    seg_hi += total;
+  }
+  __syncwarp();
+  if (qn) decode_flagged_round<C, NARROW, WIDE_ST>(q_codes, q_info, rows, qhead, qn, out_cta);
+}
+
+}  // namespace tahq

@@ -3,7 +3,7 @@
 #pragma once
 
 #include "tahq_host.cuh"
-#include "tahq_stream.cuh"
+#include "tahq_lanes.cuh"
 
 namespace tahq {
 
@@ -111,15 +111,27 @@ template <class C>
 static tahq_status decode_t(const Plan &pl, const Args &a, cudaStream_t st) {
   DevInfo d;
   if (!dev_info(&d)) return TAHQ_ERR_CUDA;
-  static std::atomic<int> occ_dec[64];
   (void)pl;
-  const int smem = DecStreamCfg<C>::TOTAL;
-  const int occ = prepare(decode_stream_kernel<C>, kThreads, smem, d, occ_dec);
-  if (!occ) return TAHQ_ERR_CUDA;
-  const uint64_t n_units = (a.n_tiles * C::LPT + 31) / 32;   // units of 32 rows
-  TAHQ_LAUNCH("decode", st,
-              launch_dependent(decode_stream_kernel<C>, persistent_grid((n_units + kWarps - 1) / kWarps, d, occ),
-                               kThreads, smem, st, a));
+  if constexpr (C::G >= 32) {
+    // no width above 4 bits: the kernel compiled for just that; 256-bit stores where the tensor is aligned to them
+    const bool narrow = a.lo + a.mixed <= 4u, wide_st = (reinterpret_cast<uintptr_t>(a.out) & 31u) == 0;
+    void (*const kernels[4])(Args) = {decode_lanes_kernel<C, false, false>, decode_lanes_kernel<C, false, true>,
+                                      decode_lanes_kernel<C, true, false>, decode_lanes_kernel<C, true, true>};
+    static std::atomic<int> occ[4][64];
+    const int k = 2 * narrow + wide_st, smem = narrow ? DecodeLanes<C, true>::SMEM : DecodeLanes<C, false>::SMEM;
+    if (!prepare(kernels[k], kLaneThreads, smem, d, occ[k])) return TAHQ_ERR_CUDA;
+    const unsigned grid = persistent_grid((a.n_tiles + LaneCfg<C>::TPR - 1) / LaneCfg<C>::TPR, d, 1);
+    TAHQ_LAUNCH("decode", st, launch_dependent(kernels[k], grid, kLaneThreads, smem, st, a));
+  } else {
+    static std::atomic<int> occ_dec[64];
+    const int smem = DecStreamCfg<C>::TOTAL;
+    const int occ = prepare(decode_stream_kernel<C>, kThreads, smem, d, occ_dec);
+    if (!occ) return TAHQ_ERR_CUDA;
+    const uint64_t n_units = (a.n_tiles * C::LPT + 31) / 32;   // units of 32 rows
+    TAHQ_LAUNCH("decode", st,
+                launch_dependent(decode_stream_kernel<C>, persistent_grid((n_units + kWarps - 1) / kWarps, d, occ),
+                                 kThreads, smem, st, a));
+  }
   return cudaGetLastError() == cudaSuccess ? TAHQ_OK : TAHQ_ERR_CUDA;
 }
 

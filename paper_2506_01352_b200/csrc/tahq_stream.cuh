@@ -23,6 +23,8 @@
 
 #include <cuda.h>   // CUtensorMap (type only; the driver entry point is looked up at run time)
 
+#include <type_traits>
+
 #include "tahq_kernels.cuh"
 
 namespace tahq {
@@ -1062,103 +1064,22 @@ __global__ void __launch_bounds__(kThreads, 2) quant2_kernel(const Args a, const
 }
 
 // ------------------------------------------------------------------------------------------
-// Decode, warp-streaming (Sec. 3.3, Algorithm 1 line 5)
+// Decode of tiles of 8 and 16 elements, warp-streaming (Sec. 3.3, Algorithm 1 line 5); wider tiles: tahq_lanes.cuh
 // ------------------------------------------------------------------------------------------
-
-// z + q*s for a row of N codes whose width W (2, 3 or 4 bits) is a per-lane value.  The row's bytes
-// are first regrouped into groups of eight codes (W whole bytes each); a code is then masked where it
-// sits, OR-ed into the mantissa of 2^23 (giving 2^23 + q*2^p exactly), and one subtraction and one
-// fused multiply-add with s*2^-p give the same bits as fma((float)q, s, z).
-template <int N>
-__device__ __forceinline__ void dequant_narrow(const uint32_t (&wv)[N / 8], uint32_t W, float s, float z,
-                                               float (&x)[N]) {
-  constexpr int NG = N / 8;
-  uint32_t g[NG];
-  if (W == 4) {
-#pragma unroll
-    for (int j = 0; j < NG; ++j) g[j] = wv[j];
-  } else if (W == 3) {
-#pragma unroll
-    for (int j = 0; j < NG / 4; ++j) {
-      g[4 * j] = wv[3 * j];
-      g[4 * j + 1] = __funnelshift_r(wv[3 * j], wv[3 * j + 1], 24);
-      g[4 * j + 2] = __funnelshift_r(wv[3 * j + 1], wv[3 * j + 2], 16);
-      g[4 * j + 3] = wv[3 * j + 2] >> 8;
-    }
-  } else {
-#pragma unroll
-    for (int j = 0; j < NG / 2; ++j) {
-      g[2 * j] = wv[j];
-      g[2 * j + 1] = wv[j] >> 16;
-    }
-  }
-  uint32_t two23;
-  asm volatile("mov.u32 %0, 0x4B000000;" : "=r"(two23));
-  const uint32_t M = (1u << W) - 1u, half = 4u * W;
-  uint32_t mk[4];
-  float sc[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    mk[i] = M << (W * i);
-    sc[i] = s * __uint_as_float((127u - W * i) << 23);   // s * 2^-(W i), exact
-  }
-#pragma unroll
-  for (int j = 0; j < NG; ++j) {
-    const uint32_t lo = g[j], hi = g[j] >> half;
-#pragma unroll
-    for (int i = 0; i < 8; i += 2) {   // two codes per packed instruction (same bits as the scalar operations)
-      uint32_t m0, m1;
-      asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(m0) : "r"(i < 4 ? lo : hi), "r"(mk[i & 3]), "r"(two23));
-      asm("lop3.b32 %0, %1, %2, %3, 0xEA;" : "=r"(m1) : "r"(i < 4 ? lo : hi), "r"(mk[(i + 1) & 3]), "r"(two23));
-      const float2 f = add2(f2(__uint_as_float(m0), __uint_as_float(m1)), f2(-8388608.0f));   // q * 2^p, exact
-      const float2 r = fma2(f, f2(sc[i & 3], sc[(i + 1) & 3]), f2(z));
-      x[8 * j + i] = r.x;
-      x[8 * j + i + 1] = r.y;
-    }
-  }
-}
-
-// The row's codes (shared or global memory, 8-byte aligned for 64-wide rows) -> z + q*s.
-template <class C>
-__device__ __forceinline__ void dequant_row(const uint8_t *src, uint32_t bits, bool narrow, float s, float z,
-                                            float (&x)[C::EPT]) {
-  if constexpr (C::EPT < 32) {
-    dequant_small<C::EPT>(src, bits, s, z, x);
-  } else if (narrow) {
-    uint32_t wv[C::EPT / 8];
-    if constexpr (C::EPT == 64) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        if (j < 2 || (uint32_t)j < bits) {   // never past the row's own bytes
-          const uint2 v = reinterpret_cast<const uint2 *>(src)[j];
-          wv[2 * j] = v.x; wv[2 * j + 1] = v.y;
-        } else {
-          wv[2 * j] = 0; wv[2 * j + 1] = 0;
-        }
-      }
-    } else {
-#pragma unroll
-      for (int j = 0; j < C::EPT / 8; ++j) wv[j] = (uint32_t)j < bits ? reinterpret_cast<const uint32_t *>(src)[j] : 0u;
-    }
-    dequant_narrow<C::EPT>(wv, bits, s, z, x);
-  } else {
-    load_dequant<C::EPT>(src, bits, s, z, x);
-  }
-}
 
 // Transformed tiles (Eq. 4 inverted): codes from the packed buffer, z + q*s, the butterfly, the
 // scale, the row into the warp's output stage, coordinates 0 and d swapped back there.
 template <class C>
-__device__ __noinline__ void decode_flagged_row(const uint8_t *codes, uint32_t bits, bool narrow, uint32_t szw,
-                                                uint32_t pvb, uint8_t *ostage, int row) {
+__device__ __noinline__ void decode_flagged_row(const uint8_t *codes, uint32_t bits, uint32_t szw, uint32_t pvb,
+                                                uint8_t *ostage, int row) {
   float s = __half2float(__ushort_as_half((unsigned short)(szw & 0xffffu)));
   float z = __half2float(__ushort_as_half((unsigned short)(szw >> 16)));
-  // 1/sqrt(G) is a power of two for G = 64: scaling s and z by it beforehand scales every later value
+  // 1/sqrt(G) is a power of two for G = 16: scaling s and z by it beforehand scales every later value
   // by it exactly, so the result has the same bits as multiplying at the end
-  constexpr bool kFold = C::G == 64 || C::G == 16;
+  constexpr bool kFold = C::G == 16;
   if (kFold) { s *= hadamard_scale<C>(); z *= hadamard_scale<C>(); }
   float x[C::EPT];
-  dequant_row<C>(codes, bits, narrow, s, z, x);
+  dequant_small<C::EPT>(codes, bits, s, z, x);
   float2 p[C::EPT / 2];
 #pragma unroll
   for (int i = 0; i < C::EPT / 2; ++i) p[i] = f2(x[2 * i], x[2 * i + 1]);
@@ -1176,59 +1097,9 @@ __device__ __noinline__ void decode_flagged_row(const uint8_t *codes, uint32_t b
   row_swap_0_d<C, !C::BF16>(ostage, row, pvb & (C::G - 1));   // masked: a foreign buffer cannot reach outside the row
 }
 
-// The same for a 128-wide tile whose halves are decoded by lanes 2j and 2j+1 (all 32 lanes call; `live`: the
-// row is a held-back one): the butterfly's last stage crosses the two lanes, and coordinate d, which is swapped
-// back with coordinate 0 of the lower half, may sit in either row of the stage.
-template <class C>
-__device__ __noinline__ void decode_flagged_pair(const uint8_t *codes, bool live, uint32_t bits, bool narrow,
-                                                 uint32_t szw, uint32_t pvb, uint8_t *ostage, int row) {
-  const int half = row & 1;
-  const float s = __half2float(__ushort_as_half((unsigned short)(szw & 0xffffu)));
-  const float z = __half2float(__ushort_as_half((unsigned short)(szw >> 16)));
-  float x[C::EPT];
-  if (live) {
-    dequant_row<C>(codes, bits, narrow, s, z, x);
-  } else {
-#pragma unroll
-    for (int k = 0; k < C::EPT; ++k) x[k] = 0.0f;
-  }
-  float2 p[C::EPT / 2];
-#pragma unroll
-  for (int i = 0; i < C::EPT / 2; ++i) p[i] = f2(x[2 * i], x[2 * i + 1]);
-  butterfly2<C::EPT / 2>(p);
-  const float2 sg = f2(half ? -1.0f : 1.0f);
-#pragma unroll
-  for (int i = 0; i < C::EPT / 2; ++i) {   // lower half: own + other; upper half: other - own (products by +-1 are exact)
-    const float2 o = f2(__shfl_xor_sync(kFull, p[i].x, 1), __shfl_xor_sync(kFull, p[i].y, 1));
-    p[i] = fma2(p[i], sg, o);
-  }
-#pragma unroll
-  for (int i = 0; i < C::EPT / 2; ++i) p[i] = mul2(p[i], f2(hadamard_scale<C>()));   // feeds no addition
-#pragma unroll
-  for (int i = 0; i < C::EPT / 2; ++i) { x[2 * i] = p[i].x; x[2 * i + 1] = p[i].y; }
-#pragma unroll
-  for (int q = 0; q < C::CPR; ++q)
-    *reinterpret_cast<uint4 *>(ostage + (size_t)phys_chunk<C>(row, q) * 16) = row_piece<C>(x, q);
-  __syncwarp();
-  if (live && half == 0) {   // un-swap coordinates 0 and d (masked: a foreign buffer cannot reach outside the tile)
-    const int d = pvb & (C::G - 1), owner = d / C::EPT, dl = d % C::EPT;
-    constexpr int EPC = 16 / C::ESZ;
-    uint8_t *p0 = ostage + (size_t)phys_chunk<C>(row, 0) * 16;
-    uint8_t *pd = ostage + (size_t)phys_chunk<C>(row + owner, dl / EPC) * 16 + (size_t)(dl % EPC) * C::ESZ;
-    if constexpr (C::BF16) {
-      const uint16_t x0 = *reinterpret_cast<uint16_t *>(p0), xd = *reinterpret_cast<uint16_t *>(pd);
-      *reinterpret_cast<uint16_t *>(p0) = xd;
-      *reinterpret_cast<uint16_t *>(pd) = x0;
-    } else {
-      const uint32_t x0 = *reinterpret_cast<uint32_t *>(p0), xd = *reinterpret_cast<uint32_t *>(pd);
-      *reinterpret_cast<uint32_t *>(p0) = xd;
-      *reinterpret_cast<uint32_t *>(pd) = x0;
-    }
-  }
-}
-
 template <class C>
 struct DecStreamCfg {
+  static_assert(C::G <= 16, "wider tiles: decode_lanes_kernel");
   static constexpr int NST = C::BF16 ? 3 : 2;
   static constexpr int PAY = 32 * C::EPT + 16;          // a unit's codes at 8 bits, from the 16-byte boundary below
   static constexpr int SLOT = PAY + 32 * 4 + 32;        // + scale/zero words + pivot bytes
@@ -1248,10 +1119,8 @@ __global__ void __launch_bounds__(kThreads, 2) decode_stream_kernel(const Args a
   __shared__ uint32_t s_q[kWarps][4][kQueueCap];   // held-back tiles: tile - first tile of the CTA, higher-width tiles
                                                    // before it (and the width bit), scale/zero word, pivot byte
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  constexpr int R = C::LPT;        // lanes (rows) per tile
-  constexpr int TPU = 32 / R;      // tiles per unit of 32 rows; s_bm / s_pre hold one entry per unit (R = 2: half a word)
-  const int half = lane & (R - 1), tl = lane / R;   // this lane's half and tile inside the unit
-  const unsigned lt = (1u << tl) - 1u;
+  constexpr int TPU = 32;          // tiles per unit
+  const unsigned lt = (1u << lane) - 1u;
   TraceScope trace(a.trace, 5);
   grid_dependency_wait();   // the look-back flags are cleared by the kernel in front
   trace.started();
@@ -1262,20 +1131,17 @@ __global__ void __launch_bounds__(kThreads, 2) decode_stream_kernel(const Args a
 
   const uint64_t n_units = (a.n_tiles + TPU - 1) / TPU;
   const uint64_t u0 = n_units * blockIdx.x / gridDim.x, u1 = n_units * (blockIdx.x + 1ull) / gridDim.x;
-  const uint64_t tile_cta = u0 * TPU, row_cta = u0 * 32;
-  const bool narrow = a.lo + a.mixed <= 4u;
+  const uint64_t tile_cta = u0 * TPU;
 
   // The prologue's loads from global memory -- the header, the bit-map bits of the CTA's first units, the words in
   // front of its slice -- are all requested before the first barrier: one round trip to L2 instead of three.
   const bool checks = blockIdx.x == 0 || a.own_prefix;
   const uint32_t hdr_w = (checks && threadIdx.x < 32) ? __ldg(reinterpret_cast<const uint32_t *>(a.packed) + threadIdx.x) : 0u;
-  // the bit-map bits of unit i of the tensor (a word, or half of one), bits beyond the last tile cleared
+  // the bit-map word of unit i of the tensor, bits beyond the last tile cleared
   auto bm_raw = [&](uint64_t i) -> uint32_t {
     if (!a.mixed) return 0u;
     const uint64_t left = a.n_tiles - i * TPU;
-    uint32_t w = __ldg(bitmap + i / R);
-    if constexpr (R == 2) w = (w >> (16 * (uint32_t)(i & 1))) & 0xffffu;
-    return w & (left >= (uint64_t)TPU ? 0xffffffffu : ((1u << (uint32_t)left) - 1u));
+    return __ldg(bitmap + i) & (left >= (uint64_t)TPU ? 0xffffffffu : ((1u << (uint32_t)left) - 1u));
   };
   static_assert(kSegWords == 2 * kThreads, "two units of the first segment per thread");
   uint32_t first_bits[2];
@@ -1287,7 +1153,7 @@ __global__ void __launch_bounds__(kThreads, 2) decode_stream_kernel(const Args a
   uint32_t own_before = 0;   // a.own_prefix: this thread's share of the higher-width tiles before the CTA's slice
   if (a.own_prefix && a.mixed) {   // words before u0 are whole: 128-bit loads, then the last few one by one
     const uint4 *b4 = reinterpret_cast<const uint4 *>(bitmap);
-    const uint64_t nwb = u0 / R;                 // whole words before the slice (at most 65536 here)
+    const uint64_t nwb = u0;                     // words before the slice (at most 65536 here)
     const uint32_t n4 = (uint32_t)(nwb / 4);
     // eight loads in flight per thread: the words sit in L2, and the CTAs at the end of the tensor, which count
     // the most, set the kernel's end (one load at a time cost the last CTA 3.5 us on the LLaMA-7B shape)
@@ -1302,7 +1168,6 @@ __global__ void __launch_bounds__(kThreads, 2) decode_stream_kernel(const Args a
       for (int j = 0; j < 8; ++j) own_before += __popc(v[j].x) + __popc(v[j].y) + __popc(v[j].z) + __popc(v[j].w);
     }
     if (threadIdx.x < (uint32_t)(nwb - (uint64_t)n4 * 4)) own_before += __popc(__ldg(bitmap + (uint64_t)n4 * 4 + threadIdx.x));
-    if (R == 2 && (u0 & 1) && threadIdx.x == 0) own_before += __popc(__ldg(bitmap + nwb) & 0xffffu);
   }
   // CTA 0 compares the received header with the one these parameters produce; what it finds travels
   // with the offset prefix, so a refused buffer leaves the output untouched.
@@ -1398,21 +1263,12 @@ __global__ void __launch_bounds__(kThreads, 2) decode_stream_kernel(const Args a
   // the first n (<= 32) held-back tiles, lane j on the j-th
   auto run_flagged = [&](uint32_t n) {
     const uint32_t e = (qhead + lane) & (kQueueCap - 1);
-    const uint32_t ft = s_q[warp][0][e], fh = s_q[warp][1][e];   // row - first row of the CTA; count * 2 + width bit
-    if constexpr (R == 1) {
-      if ((uint32_t)lane < n) {
-        const uint32_t off = (uint32_t)(C::G / 8) * (a.lo * ft + (fh >> 1));
-        decode_flagged_row<C>(payload + pay_off0 + off, a.lo + (fh & 1u), narrow, s_q[warp][2][e], s_q[warp][3][e],
-                              ostage, lane);
-      }
-    } else {
-      const bool live = (uint32_t)lane < n;
-      const uint32_t bits = a.lo + (fh & 1u);
-      const uint32_t off = (uint32_t)(C::G / 8) * (a.lo * (ft >> 1) + (fh >> 1)) + (uint32_t)half * (C::EPT / 8) * bits;
-      decode_flagged_pair<C>(payload + pay_off0 + (live ? off : 0u), live, bits, narrow, s_q[warp][2][e], s_q[warp][3][e],
-                             ostage, lane);
+    const uint32_t ft = s_q[warp][0][e], fh = s_q[warp][1][e];   // tile - first tile of the CTA; count * 2 + width bit
+    if ((uint32_t)lane < n) {
+      const uint32_t off = (uint32_t)(C::G / 8) * (a.lo * ft + (fh >> 1));
+      decode_flagged_row<C>(payload + pay_off0 + off, a.lo + (fh & 1u), s_q[warp][2][e], s_q[warp][3][e], ostage, lane);
     }
-    copy_out(n >= 32u ? 0xffffffffu : ((1u << n) - 1u), [&](int r) { return row_cta + __shfl_sync(kFull, ft, r); });
+    copy_out(n >= 32u ? 0xffffffffu : ((1u << n) - 1u), [&](int r) { return tile_cta + __shfl_sync(kFull, ft, r); });
     qhead = (qhead + n) & (kQueueCap - 1);
     qn -= n;
   };
@@ -1458,19 +1314,19 @@ __global__ void __launch_bounds__(kThreads, 2) decode_stream_kernel(const Args a
 
       uint8_t *slot = ring + (size_t)slot_i * S::SLOT;
       const uint32_t word = s_bm[su], pre = s_pre[su];
-      const uint32_t hi = (word >> tl) & 1u;
+      const uint32_t hi = (word >> lane) & 1u;
       const uint32_t hib = pre + (uint32_t)__popc(word & lt);
-      const uint32_t trel0 = seg_rel + su * TPU, trel = trel0 + tl;   // relative to the CTA's first tile
+      const uint32_t trel0 = seg_rel + su * TPU, trel = trel0 + lane;   // relative to the CTA's first tile
       uint32_t off, len;
       const bool fits = unit_range(trel0, pre, word, off, len);
       const bool live = trel < n_rel && fits;
-      const uint32_t szw = reinterpret_cast<const uint32_t *>(slot + S::PAY)[tl];
-      const uint32_t pvb = live ? slot[S::PAY + 128 + tl] : 0u;
+      const uint32_t szw = reinterpret_cast<const uint32_t *>(slot + S::PAY)[lane];
+      const uint32_t pvb = live ? slot[S::PAY + 128 + lane] : 0u;
       const bool flagged = (pvb & 0x80u) != 0;
       const unsigned held = __ballot_sync(kFull, flagged);
       if (flagged) {   // Eq. 4 inverted costs three times the plain path: held back until 32 have gathered
-        const uint32_t e = (qhead + qn + (uint32_t)__popc(held & ((1u << lane) - 1u))) & (kQueueCap - 1);
-        s_q[warp][0][e] = trel * R + half;
+        const uint32_t e = (qhead + qn + (uint32_t)__popc(held & lt)) & (kQueueCap - 1);
+        s_q[warp][0][e] = trel;
         s_q[warp][1][e] = (hib << 1) | hi;
         s_q[warp][2][e] = szw;
         s_q[warp][3][e] = pvb;
@@ -1479,10 +1335,9 @@ __global__ void __launch_bounds__(kThreads, 2) decode_stream_kernel(const Args a
       if (live && !flagged) {
         const float s = __half2float(__ushort_as_half((unsigned short)(szw & 0xffffu)));
         const float z = __half2float(__ushort_as_half((unsigned short)(szw >> 16)));
-        const uint8_t *codes = slot + (uint32_t)((pay_off0 + off) & 15ull) + (uint32_t)(C::G / 8) * (a.lo * tl + (hib - pre)) +
-                               (uint32_t)half * (C::EPT / 8) * (a.lo + hi);
+        const uint8_t *codes = slot + (uint32_t)((pay_off0 + off) & 15ull) + (uint32_t)(C::G / 8) * (a.lo * lane + (hib - pre));
         float x[C::EPT];
-        dequant_row<C>(codes, a.lo + hi, narrow, s, z, x);
+        dequant_small<C::EPT>(codes, a.lo + hi, s, z, x);
 #pragma unroll
         for (int q = 0; q < C::CPR; ++q)
           *reinterpret_cast<uint4 *>(ostage + (size_t)phys_chunk<C>(lane, q) * 16) = row_piece<C>(x, q);
@@ -1495,7 +1350,7 @@ __global__ void __launch_bounds__(kThreads, 2) decode_stream_kernel(const Args a
       }
       slot_i = (slot_i + 1 == NST) ? 0 : slot_i + 1;
       copy_out_unit(__ballot_sync(kFull, live && !flagged),
-                    a.out + (tile_cta + trel0) * (uint64_t)(C::ROWB * R) + (size_t)lane * 16);
+                    a.out + (tile_cta + trel0) * (uint64_t)C::ROWB + (size_t)lane * 16);
     }
     cp_async_wait<0>();
     __syncwarp();
