@@ -1,4 +1,5 @@
-"""ctypes binding of the C ABI in include/tahq.h (argument marshalling only).
+"""Binding of the C ABI in include/tahq.h (argument marshalling only): the codec calls themselves through the
+extension module ``_call``, everything else through ctypes.
 
 Every step of encode and decode runs in the CUDA kernels of ``libtahq.so``; PyTorch is used here
 for device memory and streams.  There is no CPU fallback: importing this module without the built
@@ -37,8 +38,24 @@ class _Layout(C.Structure):
     ]
 
 
+class _Kept:
+    """Parameters whose C structure is laid out once, not on every call: any change of a field drops it."""
+
+    def __setattr__(self, name, value):
+        object.__setattr__(self, name, value)
+        object.__setattr__(self, "_bytes", None)
+
+    def raw(self) -> bytes:
+        """The bytes of the C structure."""
+        b = self._bytes
+        if b is None:
+            b = bytes(self.c())
+            object.__setattr__(self, "_bytes", b)
+        return b
+
+
 @dataclass
-class Params:
+class Params(_Kept):
     """tahq_params: one boundary tensor [tokens x hidden]; G = tile, S = group_tokens (paper notation)."""
 
     tokens: int
@@ -73,7 +90,7 @@ class _QParams(C.Structure):
 
 
 @dataclass
-class QNaiveParams:
+class QNaiveParams(_Kept):
     """Fixed-point gradient compressor (Algorithm 1 line 6): b bits, per-token or per-tensor scale, pre-scale c."""
 
     tokens: int
@@ -142,6 +159,21 @@ def lib() -> C.CDLL:
     return _lib
 
 
+_call = None
+
+
+def call():
+    """The extension module with the codec calls.  Raises if it or the library is missing."""
+    global _call
+    if _call is None:
+        lib()
+        if not os.path.exists(_build.CALL):
+            raise ImportError(f"{_build.CALL} is not built; run `python -c 'import __graft_entry__ as g; g.build()'`")
+        from . import _call as m
+        _call = m
+    return _call
+
+
 def status_string(code: int) -> str:
     return lib().tahq_status_string(int(code)).decode()
 
@@ -194,14 +226,15 @@ def trace_reset(buf: torch.Tensor) -> None:
 
 
 def _stream_handle(stream) -> int:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return int(s.cuda_stream)
+    if stream is not None:
+        return int(stream.cuda_stream)
+    # (torch.cuda.current_stream() builds an object around this number, in three microseconds)
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def tahq_encode(p: Params, d_in: int, d_packed: int, packed_cap: int, d_ws: int, ws_cap: int, stream: int) -> int:
     """Raw call: device addresses as integers, returns the tahq_status."""
-    pc = p.c()
-    return int(lib().tahq_encode(C.byref(pc), d_in, d_packed, packed_cap, d_ws, ws_cap, stream))
+    return (_call or call()).encode(p.raw(), d_in, d_packed, packed_cap, d_ws, ws_cap, stream)
 
 
 NOALLOC_SCRATCH_BYTES = 8 << 20
@@ -221,8 +254,7 @@ def tahq_encode_noalloc(p: Params, d_in: int, d_packed: int, packed_cap: int, st
 
 
 def tahq_decode(p: Params, d_packed: int, packed_bytes: int, d_out: int, d_ws: int, ws_cap: int, stream: int) -> int:
-    pc = p.c()
-    return int(lib().tahq_decode(C.byref(pc), d_packed, packed_bytes, d_out, d_ws, ws_cap, stream))
+    return (_call or call()).decode(p.raw(), d_packed, packed_bytes, d_out, d_ws, ws_cap, stream)
 
 
 def params_for(x: torch.Tensor, **kw) -> Params:
@@ -245,7 +277,7 @@ def encode(p: Params, x: torch.Tensor, packed: torch.Tensor | None = None, ws: t
     """Encode a contiguous CUDA tensor; returns the packed uint8 buffer (asynchronous on the stream)."""
     if not (x.is_cuda and x.is_contiguous()):
         raise ValueError("x must be a contiguous CUDA tensor")
-    made = [t for t in (packed, ws) if t is None]
+    made = packed is None or ws is None
     packed = alloc_packed(p, x.device) if packed is None else packed
     ws = alloc_workspace(p, x.device) if ws is None else ws
     if stream is not None and made:   # buffers made here belong to torch's current stream: tell the allocator who uses them
@@ -291,11 +323,11 @@ def qnaive_workspace_bound(p: QNaiveParams) -> int:
 
 
 def tahq_qnaive_encode(p: QNaiveParams, d_in: int, d_packed: int, cap: int, d_ws: int, ws_cap: int, stream: int) -> int:
-    return int(lib().tahq_qnaive_encode(C.byref(p.c()), d_in, d_packed, cap, d_ws, ws_cap, stream))
+    return (_call or call()).qnaive_encode(p.raw(), d_in, d_packed, cap, d_ws, ws_cap, stream)
 
 
 def tahq_qnaive_decode(p: QNaiveParams, d_packed: int, nbytes: int, d_out: int, d_ws: int, ws_cap: int, stream: int) -> int:
-    return int(lib().tahq_qnaive_decode(C.byref(p.c()), d_packed, nbytes, d_out, d_ws, ws_cap, stream))
+    return (_call or call()).qnaive_decode(p.raw(), d_packed, nbytes, d_out, d_ws, ws_cap, stream)
 
 
 def qnaive_encode(p: QNaiveParams, x: torch.Tensor, packed: torch.Tensor | None = None, ws: torch.Tensor | None = None):
@@ -304,7 +336,7 @@ def qnaive_encode(p: QNaiveParams, x: torch.Tensor, packed: torch.Tensor | None 
     if ws is None:
         ws = torch.empty(qnaive_workspace_bound(p), dtype=torch.uint8, device=x.device)
     rc = tahq_qnaive_encode(p, x.data_ptr(), packed.data_ptr(), packed.numel(), ws.data_ptr(), ws.numel(),
-                            int(torch.cuda.current_stream(x.device).cuda_stream))
+                            torch._C._cuda_getCurrentRawStream(x.device.index))
     if rc:
         raise TahqError(rc)
     return packed, ws
@@ -317,7 +349,7 @@ def qnaive_decode(p: QNaiveParams, packed: torch.Tensor, out: torch.Tensor | Non
     if ws is None:
         ws = torch.empty(qnaive_workspace_bound(p), dtype=torch.uint8, device=packed.device)
     rc = tahq_qnaive_decode(p, packed.data_ptr(), packed.numel(), out.data_ptr(), ws.data_ptr(), ws.numel(),
-                            int(torch.cuda.current_stream(packed.device).cuda_stream))
+                            torch._C._cuda_getCurrentRawStream(packed.device.index))
     if rc:
         raise TahqError(rc)
     return out, ws

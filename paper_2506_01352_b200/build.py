@@ -2,18 +2,21 @@
 
 The sources are compiled as separate translation units, in parallel, into objects under ``csrc/build``;
 only units whose sources (or any header) changed are recompiled, then everything is linked into
-``libtahq.so`` beside this file."""
+``libtahq.so`` beside this file.  ``_call.so``, the CPython face of the codec calls, is built next to it."""
 from __future__ import annotations
 
 import concurrent.futures as cf
 import glob
 import os
 import subprocess
+import sysconfig
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 _CSRC = os.path.join(_PKG, "csrc")
 _OBJ = os.path.join(_CSRC, "build")
 LIB = os.path.join(_PKG, "libtahq.so")
+CALL = os.path.join(_PKG, "_call.so")
+_CALL_SRC = os.path.join(_CSRC, "call.cpp")
 _INCLUDE = os.path.join(os.path.dirname(_PKG), "include")
 
 NVCC_FLAGS = [
@@ -43,15 +46,36 @@ def _obj_stale(src: str) -> bool:
     return any(os.path.getmtime(d) > t for d in [src, *_headers()])
 
 
-def stale() -> bool:
+def _lib_stale() -> bool:
     if not os.path.exists(LIB):
         return True
     t = os.path.getmtime(LIB)
     return any(os.path.getmtime(d) > t for d in [*sources(), *_headers()])
 
 
+def _call_stale() -> bool:
+    if not os.path.exists(CALL):
+        return True
+    t = os.path.getmtime(CALL)
+    return any(os.path.getmtime(d) > t for d in [_CALL_SRC, os.path.join(_INCLUDE, "tahq.h")])
+
+
+def stale() -> bool:
+    return _lib_stale() or _call_stale()
+
+
+def _build_call() -> None:
+    """The extension module finds libtahq.so beside itself."""
+    tmp = CALL + f".tmp{os.getpid()}"
+    subprocess.run(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"],
+                    "-o", tmp, _CALL_SRC, "-L", _PKG, "-ltahq", "-Wl,-rpath,$ORIGIN"], check=True, cwd=_CSRC)
+    os.replace(tmp, CALL)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    if not (force or stale()):
+    if not (force or _lib_stale()):
+        if _call_stale():
+            _build_call()
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
     os.makedirs(_OBJ, exist_ok=True)
@@ -74,6 +98,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
     subprocess.run([nvcc, "-shared", "-gencode", "arch=compute_100a,code=sm_100a", "-o", tmp,
                     *[_obj(s) for s in sources()]], check=True, cwd=_CSRC)
     os.replace(tmp, LIB)
+    if force or _call_stale():
+        _build_call()
     return LIB
 
 
