@@ -1,9 +1,14 @@
 // Fixed-point gradient compressor Q_Naive (Algorithm 1 lines 6-7; pre-scale g_hat = Q(c g) / c of
-// the appendix) for sm_100a.  One warp owns one token (row) at a time: a first pass finds the row's
-// largest |c g| (per-tensor scale: a small kernel finds the tensor's beforehand), a second pass --
-// the row is still in L1/L2 -- turns eight consecutive elements per lane into b bytes of codes.
-//   y = c * g;  s = max|y| / (2^(b-1) - 1);  q = clamp(round(y * (1/s)), -L, L);  code = q + L
+// the appendix) for sm_100a.
+//   y = c * g;  s = max|y| / (2^(b-1) - 1);  q = clamp(round(y * (1/s)));  code = q + L
 // with the product y * (1/s) rounded once (fused multiply-add with 1.5 * 2^23 as the addend).
+//
+// A lane owns 32 consecutive elements of a row, whose codes are b whole words (decoding binary32: 16 elements, so that
+// a lane's 64 bytes leave by two 256-bit stores).  Encode: a row belongs to as many warps as it has stretches of 1024
+// elements (short rows share a warp), so that a lane holds 32 elements however long the row is, the next row's
+// elements are asked for before the current row is worked on, and the row's largest magnitude crosses the warps
+// through shared memory.  Decode: pieces are independent and are dealt out to the lanes one by one.  Every width
+// 2 ... 16 has code of its own (all shifts static).
 #pragma once
 
 #include <cuda_bf16.h>
@@ -12,557 +17,385 @@
 
 #include <type_traits>
 
+#include "tahq_device.cuh"
+#include "tahq_host.cuh"
+
 namespace tahq {
 
-struct QArgs {
-  const uint8_t *in;      // encode: tensor
-  uint8_t *packed;
-  uint8_t *out;           // decode: tensor
-  uint64_t tokens;
-  uint32_t hidden, bits, per_tensor;
-  float prescale;
-  uint64_t off_scales, off_payload, row_bytes, total_bytes;
-  uint32_t *gmax;         // per-tensor mode: bits of max |c g| (zeroed per call)
-  uint32_t *status;
-  uint32_t header[16];
+constexpr int kQThreads = 256;
+constexpr float kQMagic = 12582912.0f;     // 1.5 * 2^23
+constexpr uint32_t kQMagicBits = 0x4B400000u;
+
+// A lane's 32 elements as loaded.
+template <bool BF16>
+struct QRaw {
+  static constexpr int NW = BF16 ? 16 : 32;
+  uint32_t w[NW];
+  // n elements (a multiple of 8, at most 32) from src, zeros behind them; `wide`: src is 32-byte aligned
+  __device__ __forceinline__ void load(const uint8_t *src, int n, bool wide) {
+    if constexpr (!BF16) {
+      if (wide) {   // (a lane's 128 bytes by 128-bit loads would take twice the passes over the L1 tags)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          if (8 * i < n) {
+            asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                         : "=r"(w[8 * i]), "=r"(w[8 * i + 1]), "=r"(w[8 * i + 2]), "=r"(w[8 * i + 3]), "=r"(w[8 * i + 4]),
+                           "=r"(w[8 * i + 5]), "=r"(w[8 * i + 6]), "=r"(w[8 * i + 7])
+                         : "l"(src + 32 * i));
+          } else {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) w[8 * i + j] = 0u;
+          }
+        }
+        return;
+      }
+    }
+    constexpr int PER = BF16 ? 8 : 4;   // elements of a 128-bit load
+#pragma unroll
+    for (int i = 0; i < 32 / PER; ++i) {
+      const uint4 v = PER * i < n ? __ldg(reinterpret_cast<const uint4 *>(src) + i) : make_uint4(0, 0, 0, 0);
+      w[4 * i] = v.x; w[4 * i + 1] = v.y; w[4 * i + 2] = v.z; w[4 * i + 3] = v.w;
+    }
+  }
+  // largest magnitude
+  __device__ __forceinline__ float max_abs() const {
+    if constexpr (BF16) {
+      uint32_t m0 = w[0], m1 = w[1];
+#pragma unroll
+      for (int i = 2; i < NW; i += 2) { m0 = bf2_max_abs(m0, w[i]); m1 = bf2_max_abs(m1, w[i + 1]); }
+      m0 = bf2_max_abs(m0, m1) & 0x7fff7fffu;
+      return __uint_as_float(max(m0 & 0xffffu, m0 >> 16) << 16);
+    } else {
+      float m0 = fabsf(__uint_as_float(w[0])), m1 = fabsf(__uint_as_float(w[1]));
+#pragma unroll
+      for (int i = 2; i < NW; i += 2) {
+        m0 = fmaxf(m0, fabsf(__uint_as_float(w[i])));
+        m1 = fmaxf(m1, fabsf(__uint_as_float(w[i + 1])));
+      }
+      return fmaxf(m0, m1);
+    }
+  }
+  // elements 2i and 2i + 1
+  __device__ __forceinline__ float2 pair(int i) const {
+    if constexpr (BF16) return f2(__uint_as_float(w[i] << 16), __uint_as_float(w[i] & 0xffff0000u));
+    else return f2(__uint_as_float(w[2 * i]), __uint_as_float(w[2 * i + 1]));
+  }
 };
 
-constexpr int kQThreads = 256;
-constexpr float kQMagic = 12582912.0f;   // 1.5 * 2^23
+// Row scale and the reciprocal the codes are formed with, from the row's largest |g|: the largest |c g| is c times
+// that, rounded (rounding keeps the order).
+template <int B>
+__device__ __forceinline__ float q_scale(float mg, float prescale, float &inv) {
+  float s = __fdiv_rn(prescale * mg, (float)((1 << (B - 1)) - 1));
+  s = s < 1.17549435e-38f ? 0.0f : s;   // below the normal range (its reciprocal may overflow): counts as zero
+  inv = s > 0.0f ? __frcp_rn(s) : 0.0f;
+  return s;
+}
 
-// eight consecutive elements, widened to binary32
-template <bool BF16>
-__device__ __forceinline__ void q_load8(const uint8_t *row, uint32_t k0, float (&v)[8]) {
-  if constexpr (BF16) {
-    const uint4 w = __ldg(reinterpret_cast<const uint4 *>(row + (size_t)k0 * 2));
-    const uint32_t u[4] = {w.x, w.y, w.z, w.w};
+// 32 codes -> B words of the row's bit stream.  Four (b <= 8) or two codes are glued by a multiply-add chain on the
+// raw bits of fma(y, 1/s, 1.5 * 2^23); the constant part of those bits, less L per code, is taken off once per chain.
+// The clamp is left out: |y| <= m and s = m / L rounded give |y * (1/s)| < L + 1/2, so it never acts on finite
+// input.  n = elements of the row among the 32: codes behind them are zero bits.
+template <bool BF16, int B>
+__device__ __forceinline__ void q_codes(const QRaw<BF16> &raw, float prescale, float inv, int n, uint32_t (&w)[B]) {
+  constexpr int GS = B <= 8 ? 4 : 2, GB = GS * B;   // codes and bits of a chain
+  constexpr uint32_t Lq = (1u << (B - 1)) - 1u;
+  constexpr uint32_t kOff = (uint32_t)(((unsigned long long)(kQMagicBits - Lq) * group_ones(B, GS)) & 0xffffffffull);
+  uint32_t M = 1u << B;
+  asm volatile("mov.u32 %0, %0;" : "+r"(M));   // opaque: the chain stays one multiply-add per code
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      v[2 * j] = __uint_as_float(u[j] << 16);
-      v[2 * j + 1] = __uint_as_float(u[j] & 0xffff0000u);
+  for (int j = 0; j < B; ++j) w[j] = 0;
+#pragma unroll
+  for (int j = 0; j < 32 / GS; ++j) {
+    uint32_t acc = 0;
+#pragma unroll
+    for (int k = GS / 2 - 1; k >= 0; --k) {
+      const float2 y = mul2(raw.pair(j * (GS / 2) + k), f2(prescale));
+      const float2 t = fma2(y, f2(inv), f2(kQMagic));   // one rounding, ties to even
+      acc = k == GS / 2 - 1 ? __float_as_uint(t.y) : acc * M + __float_as_uint(t.y);
+      acc = acc * M + __float_as_uint(t.x);
     }
-  } else {
-    const float4 a = __ldg(reinterpret_cast<const float4 *>(row + (size_t)k0 * 4));
-    const float4 b = __ldg(reinterpret_cast<const float4 *>(row + (size_t)k0 * 4) + 1);
-    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
-    v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+    uint32_t g = acc - kOff;
+    if (n < 32 && GS * j >= n) g = 0;   // (n is a multiple of 8)
+    const int bit = j * GB, wi = bit >> 5, sh = bit & 31;
+    w[wi] |= g << sh;
+    if (sh + GB > 32) w[wi + 1] |= g >> (32 - sh);
   }
 }
 
-__device__ __forceinline__ float warp_max(float m) {
+template <int B>
+__device__ __forceinline__ void q_store(uint32_t *row, uint32_t first, uint32_t row_words, const uint32_t (&w)[B]) {
+  constexpr int V = B % 4 == 0 ? 4 : B % 2 == 0 ? 2 : 1;   // words of a store; row_words is a multiple of 4
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  return m;
+  for (int j = 0; j < B; j += V) {
+    if (first + j < row_words) {
+      if constexpr (V == 4) *reinterpret_cast<uint4 *>(row + first + j) = make_uint4(w[j], w[j + 1], w[j + 2], w[j + 3]);
+      else if constexpr (V == 2) *reinterpret_cast<uint2 *>(row + first + j) = make_uint2(w[j], w[j + 1]);
+      else row[first + j] = w[j];
+    }
+  }
 }
 
-// per-tensor mode: max |c g| over the whole tensor (non-negative floats order like their bit patterns)
+// header and section padding (one CTA)
+__device__ __forceinline__ void q_frame(const QArgs &a) {
+  if (threadIdx.x == 0 && !a.per_tensor) *a.status = 0;   // (per tensor: cleared with the maximum in front)
+  if (threadIdx.x < 32) reinterpret_cast<uint32_t *>(a.packed)[threadIdx.x] = threadIdx.x < 16 ? a.header[threadIdx.x] : 0u;
+  const uint64_t n_s = a.per_tensor ? 1 : a.tokens;
+  for (uint64_t o = a.off_scales + 4 * n_s + threadIdx.x; o < a.off_payload; o += blockDim.x) a.packed[o] = 0;
+  for (uint64_t o = a.off_payload + a.tokens * a.row_bytes + threadIdx.x; o < a.total_bytes; o += blockDim.x) a.packed[o] = 0;
+}
+
+// per-tensor mode: max |g| over the whole tensor (non-negative floats order like their bit patterns)
 template <bool BF16>
 __global__ void __launch_bounds__(kQThreads) qnaive_max_kernel(const QArgs a) {
   grid_dependency_wait();   // launched as a programmatic dependent of the kernel in front
-  const uint64_t n8 = a.tokens * (uint64_t)(a.hidden / 8);
+  constexpr int ESZ = BF16 ? 2 : 4;
+  const uint64_t n = a.tokens * (uint64_t)a.hidden;
+  const bool wide = (reinterpret_cast<uintptr_t>(a.in) & 31u) == 0;
   float m = 0.0f;
-  for (uint64_t i = (uint64_t)blockIdx.x * kQThreads + threadIdx.x; i < n8; i += (uint64_t)gridDim.x * kQThreads) {
-    float v[8];
-    q_load8<BF16>(a.in + i * (uint64_t)(BF16 ? 16 : 32), 0, v);
-#pragma unroll
-    for (int k = 0; k < 8; ++k) m = fmaxf(m, fabsf(a.prescale * v[k]));
+  for (uint64_t i = ((uint64_t)blockIdx.x * kQThreads + threadIdx.x) * 32; i < n; i += (uint64_t)gridDim.x * kQThreads * 32) {
+    QRaw<BF16> raw;
+    raw.load(a.in + i * ESZ, n - i < 32 ? (int)(n - i) : 32, wide);
+    m = fmaxf(m, raw.max_abs());
   }
-  m = warp_max(m);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(kFull, m, o));
   if ((threadIdx.x & 31) == 0 && m > 0.0f) atomicMax(a.gmax, __float_as_uint(m));
 }
 
-// ---- rows of whole kilo-elements at 6 or 8 bits (the widths the paper runs the backward half at) -------------
-// A lane owns 32 consecutive elements of every 1024: they arrive by 128-bit loads and stay in registers as
-// loaded; four codes are glued by a multiply-add chain on the raw bits of fma(y, 1/s, 1.5 * 2^23) (the
-// constant part of those bits, less L per code, is taken off once per chain), and the lane's 24 or 32 bytes
-// leave by 64- or 128-bit stores.  The clamp of the general path is left out: |y| <= m and s = m / L rounded
-// give |y * (1/s)| < L + 1/2 for every scale in the normal range (a smaller one counts as zero: all codes L), so
-// it never acts on finite input.  Same bytes as the general path.
-template <bool BF16>
-struct QFast {
-  static constexpr int V = BF16 ? 4 : 8;        // 128-bit pieces holding a lane's 32 elements of one kilo-element
-  static constexpr int NCH = BF16 ? 4 : 2;      // kilo-elements a row may have (64 registers of raw data)
-  __device__ static __forceinline__ float elem(const uint4 (&raw)[V], int e) {
-    if constexpr (BF16) {
-      const uint4 &q = raw[e / 8];
-      const int wsel = (e % 8) / 2;
-      const uint32_t w = wsel == 0 ? q.x : wsel == 1 ? q.y : wsel == 2 ? q.z : q.w;
-      return (e & 1) ? __uint_as_float(w & 0xffff0000u) : __uint_as_float(w << 16);
-    } else {
-      const uint4 &q = raw[e / 4];
-      const int wsel = e % 4;
-      return __uint_as_float(wsel == 0 ? q.x : wsel == 1 ? q.y : wsel == 2 ? q.z : q.w);
-    }
-  }
-};
-
 template <bool BF16, int B>
-__device__ __forceinline__ void qnaive_encode_rows_fast(const QArgs &a, int lane, uint64_t warp, uint64_t n_warps) {
-  using F = QFast<BF16>;
+__global__ void __launch_bounds__(kQThreads, BF16 ? 3 : 2) qnaive_encode_kernel(const QArgs a) {
   constexpr int ESZ = BF16 ? 2 : 4;
-  constexpr int Lq = (1 << (B - 1)) - 1;
-  constexpr uint32_t kMb = 0x4B400000u;   // bits of 1.5 * 2^23
-  constexpr uint32_t kOnes = B == 6 ? (1u + (1u << 6) + (1u << 12) + (1u << 18)) : (1u + (1u << 8) + (1u << 16) + (1u << 24));
-  constexpr uint32_t kOff = (uint32_t)(((unsigned long long)(kMb - (uint32_t)Lq) * kOnes) & 0xffffffffull);
-  uint32_t M = 1u << B;
-  asm volatile("mov.u32 %0, %0;" : "+r"(M));   // opaque: the chain stays one multiply-add per code
-  const uint32_t C = a.hidden, nch = C / 1024u;
+  __shared__ float s_max[2][8];
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, C = a.hidden;
+  const uint32_t n_warps = blockDim.x >> 5, row_words = (uint32_t)(a.row_bytes / 4), lanes_all = (C + 31u) / 32u;
   float *scales = reinterpret_cast<float *>(a.packed + a.off_scales);
-  for (uint64_t r = warp; r < a.tokens; r += n_warps) {
-    const uint8_t *row = a.in + (r * (uint64_t)C + (uint64_t)lane * 32u) * ESZ;
-    uint8_t *orow = a.packed + a.off_payload + r * a.row_bytes;
-    uint4 raw[F::NCH][F::V];
-#pragma unroll
-    for (int ch = 0; ch < F::NCH; ++ch)
-#pragma unroll
-      for (int v = 0; v < F::V; ++v)
-        raw[ch][v] = (uint32_t)ch < nch ? __ldg(reinterpret_cast<const uint4 *>(row + (size_t)ch * 1024 * ESZ) + v)
-                                        : make_uint4(0, 0, 0, 0);
-    float m = 0.0f;
-    if (a.per_tensor) {
-      m = __uint_as_float(*a.gmax);
-    } else {
-#pragma unroll
-      for (int ch = 0; ch < F::NCH; ++ch)
-#pragma unroll
-        for (int e = 0; e < 32; ++e) m = fmaxf(m, fabsf(a.prescale * F::elem(raw[ch], e)));   // (zeros beyond the row)
-      m = warp_max(m);
-    }
-    float s = __fdiv_rn(m, (float)Lq);
-    s = s < 1.17549435e-38f ? 0.0f : s;   // below the normal range (its reciprocal may overflow): counts as zero
-    const float inv = s > 0.0f ? __frcp_rn(s) : 0.0f;
-    if (lane == 0 && (!a.per_tensor || r == 0)) scales[a.per_tensor ? 0 : r] = s;
-#pragma unroll
-    for (int ch = 0; ch < F::NCH; ++ch) {
-      if ((uint32_t)ch < nch) {
-        uint32_t g[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          uint32_t acc = 0;
-#pragma unroll
-          for (int k = 3; k >= 0; --k) {
-            const float y = a.prescale * F::elem(raw[ch], 4 * j + k);
-            const uint32_t bits = __float_as_uint(__fmaf_rn(y, inv, kQMagic));   // one rounding, ties to even
-            acc = k == 3 ? bits : acc * M + bits;
-          }
-          g[j] = acc - kOff;
-        }
-        if constexpr (B == 8) {
-          uint4 *dst = reinterpret_cast<uint4 *>(orow + (size_t)ch * 1024 + (size_t)lane * 32);
-          dst[0] = make_uint4(g[0], g[1], g[2], g[3]);
-          dst[1] = make_uint4(g[4], g[5], g[6], g[7]);
-        } else {
-          uint32_t w[6];
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            w[3 * h] = __byte_perm(g[4 * h], g[4 * h + 1], 0x4210);
-            w[3 * h + 1] = __byte_perm(g[4 * h + 1], g[4 * h + 2], 0x5421);
-            w[3 * h + 2] = __byte_perm(g[4 * h + 2], g[4 * h + 3], 0x6542);
-          }
-          uint2 *dst = reinterpret_cast<uint2 *>(orow + (size_t)ch * 768 + (size_t)lane * 24);
-#pragma unroll
-          for (int j = 0; j < 3; ++j) dst[j] = make_uint2(w[2 * j], w[2 * j + 1]);
-        }
+  const bool wide = (reinterpret_cast<uintptr_t>(a.in) & 31u) == 0;
+  grid_dependency_wait();   // launched as a programmatic dependent of the kernel in front
+  if (blockIdx.x == 0) q_frame(a);
+  float mg = a.per_tensor ? __uint_as_float(*a.gmax) : 0.0f;
+
+  // rows of the CTA at a time, and this lane's place in one of them
+  const uint32_t rows_at_once = a.row_warps > 1 ? n_warps / a.row_warps : n_warps * (32u / a.row_lanes);
+  const uint32_t slot = a.row_warps > 1 ? warp / a.row_warps : warp * (32u / a.row_lanes) + lane / a.row_lanes;
+  const uint32_t part = a.row_warps > 1 ? warp % a.row_warps * 32u + lane : lane % a.row_lanes;   // 32 elements each
+  const uint64_t step = (uint64_t)gridDim.x * rows_at_once;
+  const uint32_t parts_at_once = a.row_warps > 1 ? a.row_warps * 32u : a.row_lanes;
+  auto elements = [&](uint32_t p) { return p < lanes_all ? (C - 32u * p < 32u ? (int)(C - 32u * p) : 32) : 0; };
+  auto load = [&](QRaw<BF16> &raw, uint64_t r, uint32_t p) {
+    raw.load(a.in + (r * (uint64_t)C + 32u * p) * ESZ, r < a.tokens ? elements(p) : 0, wide);
+  };
+  auto emit = [&](const QRaw<BF16> &raw, uint64_t r, uint32_t p, float inv) {
+    uint32_t w[B];
+    q_codes<BF16, B>(raw, a.prescale, inv, elements(p), w);
+    uint32_t *row = reinterpret_cast<uint32_t *>(a.packed + a.off_payload + r * a.row_bytes);
+    if (p < lanes_all) q_store<B>(row, p * (uint32_t)B, row_words, w);
+  };
+  const uint64_t r_cta = (uint64_t)blockIdx.x * rows_at_once;
+  uint64_t r = r_cta + slot;
+  QRaw<BF16> next;
+  load(next, r, part);
+  uint32_t parity = 0;
+  for (uint64_t rc = r_cta; rc < a.tokens; rc += step, r += step) {   // (the same number of turns for every lane of the CTA)
+    const QRaw<BF16> cur = next;
+    const bool live = r < a.tokens;
+    load(next, r + step, part);
+    if (!a.per_tensor) {
+      float m = cur.max_abs();
+      for (uint32_t p = part + parts_at_once; live && p < lanes_all; p += parts_at_once) {   // (rows beyond 8192 elements)
+        QRaw<BF16> more;
+        load(more, r, p);
+        m = fmaxf(m, more.max_abs());
       }
+      __syncwarp();
+      for (uint32_t o = a.row_lanes / 2; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(kFull, m, o));
+      if (a.row_warps > 1) {
+        if (lane == 0) s_max[parity][warp] = m;
+        asm volatile("bar.sync %0, %1;" ::"r"(slot + 1u), "r"(a.row_warps * 32u) : "memory");
+        const uint32_t w0 = slot * a.row_warps;
+        m = s_max[parity][w0];
+        for (uint32_t i = 1; i < a.row_warps; ++i) m = fmaxf(m, s_max[parity][w0 + i]);
+        parity ^= 1u;   // (a warp writes this half again only after the next barrier, when all have read it)
+      }
+      mg = m;
+    }
+    float inv;
+    const float s = q_scale<B>(mg, a.prescale, inv);
+    if (live) {
+      if (part == 0 && (!a.per_tensor || r == 0)) scales[a.per_tensor ? 0 : r] = s;
+      emit(cur, r, part, inv);
+      for (uint32_t p = part + parts_at_once; p < lanes_all; p += parts_at_once) {
+        QRaw<BF16> more;
+        load(more, r, p);
+        emit(more, r, p, inv);
+      }
+      // the row's last words, behind its last lane's
+      const uint32_t from = lanes_all * (uint32_t)B;
+      if (part == 0 && from < row_words)
+        for (uint32_t o = from; o < row_words; ++o)
+          reinterpret_cast<uint32_t *>(a.packed + a.off_payload + r * a.row_bytes)[o] = 0;
     }
   }
 }
 
-template <bool BF16, int B, bool POW2>
-__device__ __forceinline__ void qnaive_decode_rows_fast(const QArgs &a, int lane, uint64_t warp, uint64_t n_warps,
-                                                        float rc) {
-  constexpr int ESZ = BF16 ? 2 : 4;
-  constexpr int Lq = (1 << (B - 1)) - 1;
-  constexpr uint32_t kMb = 0x4B400000u;
-  const float off = kQMagic + (float)Lq;   // exact
-  const uint32_t C = a.hidden, nch = C / 1024u;
+// Codes of a lane -> g_hat = (q * s) / c.  Dividing by a power of two is the same rounding as multiplying by its
+// (exact) reciprocal.
+template <bool BF16, int B, bool WIDE>
+__global__ void __launch_bounds__(kQThreads, 4) qnaive_decode_kernel(const QArgs a) {
+  constexpr int ESZ = BF16 ? 2 : 4, E = 64 / ESZ;
+  constexpr int NW = (E * B + (E == 16 && B % 2 ? 16 : 0) + 31) / 32;   // words a lane's codes lie in
+  constexpr int V = (E * B) % 128 == 0 ? 4 : (E * B) % 64 == 0 ? 2 : 1;  // words of a load
+  constexpr float kOff = kQMagic + (float)((1 << (B - 1)) - 1);         // exact
+  const uint32_t lane = threadIdx.x & 31u, C = a.hidden, row_words = (uint32_t)(a.row_bytes / 4);
+  const uint32_t total = (uint32_t)a.tokens * a.pieces, step = gridDim.x * kQThreads;
+  grid_dependency_wait();   // launched as a programmatic dependent of the kernel in front
   const float *scales = reinterpret_cast<const float *>(a.packed + a.off_scales);
-  for (uint64_t r = warp; r < a.tokens; r += n_warps) {
-    const float s = __ldg(scales + (a.per_tensor ? 0 : r));
-    const uint8_t *irow = a.packed + a.off_payload + r * a.row_bytes;
-    for (uint32_t ch = 0; ch < nch; ++ch) {
-      uint32_t g[8];   // four codes each
-      if constexpr (B == 8) {
-        const uint4 *src = reinterpret_cast<const uint4 *>(irow + (size_t)ch * 1024 + (size_t)lane * 32);
-        const uint4 v0 = __ldg(src), v1 = __ldg(src + 1);
-        g[0] = v0.x; g[1] = v0.y; g[2] = v0.z; g[3] = v0.w;
-        g[4] = v1.x; g[5] = v1.y; g[6] = v1.z; g[7] = v1.w;
-      } else {
-        const uint2 *src = reinterpret_cast<const uint2 *>(irow + (size_t)ch * 768 + (size_t)lane * 24);
-        uint32_t w[6];
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-          const uint2 v = __ldg(src + j);
-          w[2 * j] = v.x;
-          w[2 * j + 1] = v.y;
-        }
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {   // 24 bits per group, in its low three bytes
-          g[4 * h] = w[3 * h];
-          g[4 * h + 1] = __byte_perm(w[3 * h], w[3 * h + 1], 0x5543);
-          g[4 * h + 2] = __byte_perm(w[3 * h + 1], w[3 * h + 2], 0x4432);
-          g[4 * h + 3] = w[3 * h + 2] >> 8;
-        }
-      }
-      float x[32];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          uint32_t mbits;   // the code in the mantissa of 1.5 * 2^23
-          if constexpr (B == 8) mbits = __byte_perm(g[j], kMb, 0x7640 + k);
-          else mbits = ((g[j] >> (6 * k)) & 63u) | kMb;
-          const float q = __uint_as_float(mbits) - off;   // code - L, exact
-          const float t = __fmul_rn(q, s);
-          x[4 * j + k] = POW2 ? __fmul_rn(t, rc) : __fdiv_rn(t, a.prescale);
-        }
-      }
-      // The lane's 32 values as 128-bit pieces.  Neighbouring lanes swap half of them (the even lane's odd pieces
-      // against the odd lane's even ones), so that the two lanes of a pair write 32 adjacent bytes in every store
-      // instruction: stored as they are, each instruction would write half of every 32-byte sector it touches.
-      constexpr int V = BF16 ? 4 : 8;
-      uint4 pc[V];
-      if constexpr (BF16) {
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-          uint32_t u[4];
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const __nv_bfloat162 h2 = __floats2bfloat162_rn(x[8 * v + 2 * j], x[8 * v + 2 * j + 1]);
-            u[j] = *reinterpret_cast<const uint32_t *>(&h2);
-          }
-          pc[v] = make_uint4(u[0], u[1], u[2], u[3]);
-        }
-      } else {
-#pragma unroll
-        for (int v = 0; v < V; ++v)
-          pc[v] = make_uint4(__float_as_uint(x[4 * v]), __float_as_uint(x[4 * v + 1]), __float_as_uint(x[4 * v + 2]),
-                             __float_as_uint(x[4 * v + 3]));
-      }
-      const bool odd = lane & 1;
-#pragma unroll
-      for (int h = 0; h < V / 2; ++h) {   // even lane: gives piece 2h+1, gets the neighbour's piece 2h; odd lane: the reverse
-        const uint4 give = odd ? pc[2 * h] : pc[2 * h + 1];
-        uint4 got;
-        got.x = __shfl_xor_sync(0xffffffffu, give.x, 1);
-        got.y = __shfl_xor_sync(0xffffffffu, give.y, 1);
-        got.z = __shfl_xor_sync(0xffffffffu, give.z, 1);
-        got.w = __shfl_xor_sync(0xffffffffu, give.w, 1);
-        if (odd) pc[2 * h] = got; else pc[2 * h + 1] = got;
-      }
-      // now: even lane holds its own even pieces and the neighbour's even pieces (at the odd slots); the odd lane
-      // its own odd pieces (odd slots) and the neighbour's odd pieces (even slots)
-      uint8_t *pair0 = a.out + (r * (uint64_t)C + (uint64_t)(lane & ~1) * 32u + (uint64_t)ch * 1024u) * ESZ;
-#pragma unroll
-      for (int h = 0; h < V / 2; ++h) {
-        // pieces 2h and 2h+1 of the even lane's region, then of the odd lane's region
-        uint4 *even_region = reinterpret_cast<uint4 *>(pair0) + 2 * h;
-        uint4 *odd_region = reinterpret_cast<uint4 *>(pair0 + 32 * ESZ) + 2 * h;
-        // even lane: its own piece 2h, then the neighbour's piece 2h; odd lane: the neighbour's piece 2h+1, then
-        // its own piece 2h+1 (one instruction for both lanes, so each writes half of the same sector)
-        even_region[odd ? 1 : 0] = pc[2 * h];
-        odd_region[odd ? 1 : 0] = pc[2 * h + 1];
-      }
-    }
-  }
-}
-
-template <bool BF16>
-__global__ void __launch_bounds__(kQThreads, 2) qnaive_encode_kernel(const QArgs a) {
-  grid_dependency_wait();   // launched as a programmatic dependent of the kernel in front
-  constexpr int ESZ = BF16 ? 2 : 4;
-  const int lane = threadIdx.x & 31;
-  const uint64_t warp = ((uint64_t)blockIdx.x * kQThreads + threadIdx.x) >> 5;
-  const uint64_t n_warps = ((uint64_t)gridDim.x * kQThreads) >> 5;
-  const uint32_t b = a.bits, C = a.hidden;
-  const int Lq = (int)((1u << (b - 1)) - 1u);
-  const float Lf = (float)Lq;
-  float *scales = reinterpret_cast<float *>(a.packed + a.off_scales);
-
-  if (blockIdx.x == 0) {   // header and section padding
-    if (threadIdx.x < 32) reinterpret_cast<uint32_t *>(a.packed)[threadIdx.x] = threadIdx.x < 16 ? a.header[threadIdx.x] : 0u;
-    const uint64_t n_s = a.per_tensor ? 1 : a.tokens;
-    for (uint64_t o = a.off_scales + 4 * n_s + threadIdx.x; o < a.off_payload; o += kQThreads) a.packed[o] = 0;
-    for (uint64_t o = a.off_payload + a.tokens * a.row_bytes + threadIdx.x; o < a.total_bytes; o += kQThreads) a.packed[o] = 0;
-  }
-  if ((b == 6u || b == 8u) && C % 1024u == 0u && C <= (uint32_t)QFast<BF16>::NCH * 1024u) {
-    if (b == 6u) qnaive_encode_rows_fast<BF16, 6>(a, lane, warp, n_warps);
-    else qnaive_encode_rows_fast<BF16, 8>(a, lane, warp, n_warps);
-    return;
-  }
-  const uint32_t data_bytes = (uint32_t)(((uint64_t)C * b) >> 3);   // hidden is a multiple of 8
-  // pieces a lane's b bytes are stored in: the largest power of two dividing b, at most 16
-  const uint32_t gsz = (b & (0u - b)) > 16u ? 16u : (b & (0u - b));
-
-  // one group of eight elements -> the lane's b bytes of codes at dst.  B > 0: the width as a compile-time
-  // constant (all shifts static, 32-bit words); B == 0: any width, 128-bit value built with run-time shifts.
-  auto emit_w = [&](auto Bc, const float (&v)[8], float inv, uint8_t *dst) {
-    constexpr int B = decltype(Bc)::value;
-    int q[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const float y = a.prescale * v[k];
-      const float t = __fmaf_rn(y, inv, kQMagic);   // one rounding, ties to even
-      q[k] = min(max((int)(__float_as_uint(t) - 0x4B400000u), -Lq), Lq) + Lq;
-    }
-    if constexpr (B > 0) {
-      uint32_t w[B / 4 + 1];
-#pragma unroll
-      for (int j = 0; j < B / 4 + 1; ++j) w[j] = 0;
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        constexpr int dummy = 0; (void)dummy;
-        const int pos = k * B, wi = pos >> 5, sh = pos & 31;
-        w[wi] |= (uint32_t)q[k] << sh;
-        if (sh + B > 32) w[wi + 1] |= (uint32_t)q[k] >> (32 - sh);
-      }
-      if constexpr (B == 16) *reinterpret_cast<uint4 *>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
-      else if constexpr (B == 8) *reinterpret_cast<uint2 *>(dst) = make_uint2(w[0], w[1]);
-      else if constexpr (B % 4 == 0) {
-#pragma unroll
-        for (int j = 0; j < B / 4; ++j) reinterpret_cast<uint32_t *>(dst)[j] = w[j];
-      } else {   // even widths: 16-bit pieces
-#pragma unroll
-        for (int j = 0; j < B / 2; ++j) reinterpret_cast<uint16_t *>(dst)[j] = (uint16_t)(w[j >> 1] >> (16 * (j & 1)));
-      }
-    } else {
-      unsigned long long lo = 0, hi = 0;
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const unsigned long long code = (unsigned long long)(uint32_t)q[k];
-        const uint32_t pos = (uint32_t)k * b;
-        if (pos < 64) {
-          lo |= code << pos;
-          if (pos + b > 64) hi |= code >> (64 - pos);
-        } else {
-          hi |= code << (pos - 64);
-        }
-      }
-      if (gsz == 4) {
-#pragma unroll
-        for (int j = 0; j < 3; ++j)
-          if ((uint32_t)(4 * j) < b) reinterpret_cast<uint32_t *>(dst)[j] = (uint32_t)(j < 2 ? lo >> (32 * j) : hi);
-      } else if (gsz == 2) {
-#pragma unroll
-        for (int j = 0; j < 7; ++j)
-          if ((uint32_t)(2 * j) < b)
-            reinterpret_cast<uint16_t *>(dst)[j] = (uint16_t)(j < 4 ? lo >> (16 * j) : hi >> (16 * (j - 4)));
-      } else {
-#pragma unroll
-        for (int j = 0; j < 15; ++j)
-          if ((uint32_t)j < b) dst[j] = (uint8_t)(j < 8 ? lo >> (8 * j) : hi >> (8 * (j - 8)));
-      }
-    }
-  };
-  auto emit = [&](const float (&v)[8], float inv, uint8_t *dst) {
-    switch (b) {   // uniform: the widths the paper uses (6, 8, 10) and their neighbours get static code
-      case 4: emit_w(std::integral_constant<int, 4>{}, v, inv, dst); break;
-      case 6: emit_w(std::integral_constant<int, 6>{}, v, inv, dst); break;
-      case 8: emit_w(std::integral_constant<int, 8>{}, v, inv, dst); break;
-      case 10: emit_w(std::integral_constant<int, 10>{}, v, inv, dst); break;
-      case 12: emit_w(std::integral_constant<int, 12>{}, v, inv, dst); break;
-      case 16: emit_w(std::integral_constant<int, 16>{}, v, inv, dst); break;
-      default: emit_w(std::integral_constant<int, 0>{}, v, inv, dst); break;
-    }
-  };
-  constexpr int kHeld = BF16 ? 16 : 8;   // groups of eight elements a lane keeps in registers (64 registers)
-  const bool held = C <= (uint32_t)kHeld * 256u;
-
-  for (uint64_t r = warp; r < a.tokens; r += n_warps) {
-    const uint8_t *row = a.in + r * (uint64_t)C * ESZ;
-    uint8_t *orow = a.packed + a.off_payload + r * a.row_bytes;
-    float m = 0.0f;
-    if (held) {   // the row is read once: all loads in flight together, then the range, then the codes
-      uint4 raw[kHeld][BF16 ? 1 : 2];   // as loaded; widened where used
-#pragma unroll
-      for (int i = 0; i < kHeld; ++i) {
-        const uint32_t k0 = (uint32_t)i * 256u + lane * 8;
-#pragma unroll
-        for (int h = 0; h < (BF16 ? 1 : 2); ++h)
-          raw[i][h] = k0 < C ? __ldg(reinterpret_cast<const uint4 *>(row + (size_t)k0 * ESZ) + h) : make_uint4(0, 0, 0, 0);
-      }
-      auto widen = [&](int i, float (&v)[8]) {
-        if constexpr (BF16) {
-          const uint32_t u[4] = {raw[i][0].x, raw[i][0].y, raw[i][0].z, raw[i][0].w};
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            v[2 * j] = __uint_as_float(u[j] << 16);
-            v[2 * j + 1] = __uint_as_float(u[j] & 0xffff0000u);
-          }
-        } else {
-          const uint32_t u[8] = {raw[i][0].x, raw[i][0].y, raw[i][0].z, raw[i][0].w,
-                                 raw[i][BF16 ? 0 : 1].x, raw[i][BF16 ? 0 : 1].y, raw[i][BF16 ? 0 : 1].z, raw[i][BF16 ? 0 : 1].w};
-#pragma unroll
-          for (int j = 0; j < 8; ++j) v[j] = __uint_as_float(u[j]);
-        }
-      };
-      if (a.per_tensor) {
-        m = __uint_as_float(*a.gmax);
-      } else {
-#pragma unroll
-        for (int i = 0; i < kHeld; ++i) {
-          float v[8];
-          widen(i, v);
-#pragma unroll
-          for (int k = 0; k < 8; ++k) m = fmaxf(m, fabsf(a.prescale * v[k]));
-        }
-        m = warp_max(m);
-      }
-      float s = __fdiv_rn(m, Lf);
-      s = s < 1.17549435e-38f ? 0.0f : s;   // below the normal range: counts as zero
-      const float inv = s > 0.0f ? __frcp_rn(s) : 0.0f;
-      if (lane == 0 && (!a.per_tensor || r == 0)) scales[a.per_tensor ? 0 : r] = s;
-#pragma unroll
-      for (int i = 0; i < kHeld; ++i) {
-        const uint32_t k0 = (uint32_t)i * 256u + lane * 8;
-        if (k0 < C) {
-          float v[8];
-          widen(i, v);
-          emit(v, inv, orow + (size_t)(k0 >> 3) * b);
-        }
-      }
-    } else {      // long rows: a pass for the range, a second one (from L1/L2) for the codes
-      if (a.per_tensor) {
-        m = __uint_as_float(*a.gmax);
-      } else {
-#pragma unroll 4
-        for (uint32_t k0 = lane * 8; k0 < C; k0 += 256) {
-          float v[8];
-          q_load8<BF16>(row, k0, v);
-#pragma unroll
-          for (int k = 0; k < 8; ++k) m = fmaxf(m, fabsf(a.prescale * v[k]));
-        }
-        m = warp_max(m);
-      }
-      float s = __fdiv_rn(m, Lf);
-      s = s < 1.17549435e-38f ? 0.0f : s;   // below the normal range: counts as zero
-      const float inv = s > 0.0f ? __frcp_rn(s) : 0.0f;
-      if (lane == 0 && (!a.per_tensor || r == 0)) scales[a.per_tensor ? 0 : r] = s;
-#pragma unroll 2
-      for (uint32_t k0 = lane * 8; k0 < C; k0 += 256) {
-        float v[8];
-        q_load8<BF16>(row, k0, v);
-        emit(v, inv, orow + (size_t)(k0 >> 3) * b);
-      }
-    }
-    for (uint32_t o = data_bytes + lane; o < (uint32_t)a.row_bytes; o += 32) orow[o] = 0;   // the row's padding
-  }
-}
-
-template <bool BF16>
-__global__ void __launch_bounds__(kQThreads) qnaive_decode_kernel(const QArgs a) {
-  grid_dependency_wait();   // launched as a programmatic dependent of the kernel in front
-  constexpr int ESZ = BF16 ? 2 : 4;
-  const int lane = threadIdx.x & 31;
-  const uint64_t warp = ((uint64_t)blockIdx.x * kQThreads + threadIdx.x) >> 5;
-  const uint64_t n_warps = ((uint64_t)gridDim.x * kQThreads) >> 5;
-  const uint32_t b = a.bits, C = a.hidden;
-  const int Lq = (int)((1u << (b - 1)) - 1u);
+  const uint8_t *payload = a.packed + a.off_payload;
   // the received header must describe these parameters; otherwise nothing is written
-  {
-    const uint32_t w = lane < 16 ? __ldg(reinterpret_cast<const uint32_t *>(a.packed) + lane) : 0u;
-    const bool bad = lane < 16 && w != a.header[lane];
-    if (__any_sync(0xffffffffu, bad)) {
-      if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(a.status, 1u /* TAHQ_DEV_BAD_HEADER */);
-      return;
+  const uint32_t hdr = lane < 16 ? __ldg(reinterpret_cast<const uint32_t *>(a.packed) + lane) : 0u;
+
+  // piece i of the tensor: piece `pc` of row `row`; advanced without a division
+  const uint32_t d_row = step / a.pieces, d_pc = step - d_row * a.pieces;
+  uint32_t i = blockIdx.x * kQThreads + threadIdx.x;
+  uint32_t row = i / a.pieces, pc = i - row * a.pieces;
+  uint32_t w[NW];
+  float s = 0.0f;
+  auto load = [&](uint32_t rw, uint32_t p) {
+    const uint32_t first = E == 32 ? p * (uint32_t)B : (p * (uint32_t)B) >> 1;
+    const uint32_t *src = reinterpret_cast<const uint32_t *>(payload + rw * a.row_bytes);
+#pragma unroll
+    for (int j = 0; j < NW; j += V) {
+      if constexpr (V == 4) {
+        const uint4 v = first + j < row_words ? __ldg(reinterpret_cast<const uint4 *>(src + first + j)) : make_uint4(0, 0, 0, 0);
+        w[j] = v.x; w[j + 1] = v.y; w[j + 2] = v.z; w[j + 3] = v.w;
+      } else if constexpr (V == 2) {
+        const uint2 v = first + j < row_words ? __ldg(reinterpret_cast<const uint2 *>(src + first + j)) : make_uint2(0, 0);
+        w[j] = v.x; w[j + 1] = v.y;
+      } else {
+        w[j] = first + j < row_words ? __ldg(src + first + j) : 0u;
+      }
     }
-  }
-  const float *scales = reinterpret_cast<const float *>(a.packed + a.off_scales);
-  const unsigned long long mask = (1ull << b) - 1ull;
-  // dividing by a power of two is the same rounding as multiplying by its (exact) reciprocal
+    s = __ldg(scales + (a.per_tensor ? 0u : rw));
+  };
+  if (i < total) load(row, pc);
+  const bool bad = __any_sync(kFull, lane < 16 && hdr != a.header[lane & 15u]);
+  if (blockIdx.x == 0 && threadIdx.x == 0) *a.status = bad ? 1u /* TAHQ_DEV_BAD_HEADER */ : 0u;
+  if (bad) return;
   const bool pow2 = (__float_as_uint(a.prescale) & 0x007fffffu) == 0u && (__float_as_uint(a.prescale) >> 23) - 2u < 250u;
   const float rc = pow2 ? __frcp_rn(a.prescale) : 0.0f;
-  if ((b == 6u || b == 8u) && C % 1024u == 0u) {
-    if (b == 6u) {
-      if (pow2) qnaive_decode_rows_fast<BF16, 6, true>(a, lane, warp, n_warps, rc);
-      else qnaive_decode_rows_fast<BF16, 6, false>(a, lane, warp, n_warps, rc);
-    } else {
-      if (pow2) qnaive_decode_rows_fast<BF16, 8, true>(a, lane, warp, n_warps, rc);
-      else qnaive_decode_rows_fast<BF16, 8, false>(a, lane, warp, n_warps, rc);
+
+  for (; i < total; i += step) {
+    uint32_t v[NW + 1];
+#pragma unroll
+    for (int j = 0; j < NW; ++j) v[j] = w[j];
+    v[NW] = 0;
+    const float sc = s;
+    const uint32_t r0 = row, p0 = pc;
+    row += d_row;
+    pc += d_pc;
+    if (pc >= a.pieces) { pc -= a.pieces; ++row; }
+    if (i + step < total && i + step > i) load(row, pc);
+    if constexpr (E == 16 && B % 2 == 1) {   // an odd piece starts in the middle of a word
+      const uint32_t sh = (p0 & 1u) * 16u;
+#pragma unroll
+      for (int j = 0; j < NW; ++j) v[j] = __funnelshift_r(v[j], v[j + 1], sh);
     }
-    return;
-  }
-  for (uint64_t r = warp; r < a.tokens; r += n_warps) {
-    const float s = __ldg(scales + (a.per_tensor ? 0 : r));
-    const uint8_t *irow = a.packed + a.off_payload + r * a.row_bytes;
-    uint8_t *orow = a.out + r * (uint64_t)C * ESZ;
-#pragma unroll 4
-    for (uint32_t k0 = lane * 8; k0 < C; k0 += 256) {
-      // the lane's b bytes start at byte o of the row
-      const uint32_t o = (k0 >> 3) * b;
-      unsigned long long lo, hi = 0;
-      if (b == 8) {
-        lo = __ldg(reinterpret_cast<const unsigned long long *>(irow + o));
-      } else if (b == 16) {
-        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(irow + o));
-        lo = (unsigned long long)v.x | ((unsigned long long)v.y << 32);
-        hi = (unsigned long long)v.z | ((unsigned long long)v.w << 32);
-      } else {   // the aligned words that cover them (four do unless the bytes start off a word boundary)
-        const uint32_t o4 = o & ~3u, sh = (o & 3u) * 8u;
-        uint32_t w[5];
+    float2 x[E / 2];
 #pragma unroll
-        for (int j = 0; j < 5; ++j)
-          w[j] = (o4 + 4u * j < (uint32_t)a.row_bytes && (j < 4 || sh)) ? __ldg(reinterpret_cast<const uint32_t *>(irow + o4) + j) : 0u;
-        uint32_t x[4];
+    for (int k = 0; k < E / 2; ++k) {
+      uint32_t m[2];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) x[j] = __funnelshift_r(w[j], w[j + 1], sh);
-        lo = (unsigned long long)x[0] | ((unsigned long long)x[1] << 32);
-        hi = (unsigned long long)x[2] | ((unsigned long long)x[3] << 32);
+      for (int h = 0; h < 2; ++h) {   // the code in the mantissa of 1.5 * 2^23
+        const int bit = (2 * k + h) * B, wi = bit >> 5, sh = bit & 31;
+        const uint32_t c = sh == 0 ? v[wi] : sh + B <= 32 ? v[wi] >> sh : __funnelshift_r(v[wi], v[wi + 1], sh);
+        m[h] = (c & ((1u << B) - 1u)) | kQMagicBits;
       }
-      float g[8];
-      auto codes = [&](auto Bc) {
-        constexpr int B = decltype(Bc)::value;
+      const float2 q = add2(f2(__uint_as_float(m[0]), __uint_as_float(m[1])), f2(-kOff));   // code - L, exact
+      x[k] = mul2(q, f2(sc));
+    }
+    if (pow2) {
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          unsigned long long c;
-          if constexpr (B > 0) {
-            constexpr int pos = 0; (void)pos;
-            const int p0 = k * B;
-            if (p0 < 64) {
-              c = lo >> p0;
-              if (p0 + B > 64) c |= hi << (64 - p0);
-            } else {
-              c = hi >> (p0 - 64);
-            }
-            c &= (1ull << B) - 1ull;
-          } else {
-            const uint32_t p0 = (uint32_t)k * b;
-            if (p0 < 64) {
-              c = lo >> p0;
-              if (p0 + b > 64) c |= hi << (64 - p0);
-            } else {
-              c = hi >> (p0 - 64);
-            }
-            c &= mask;
-          }
-          const int q = (int)(uint32_t)c - Lq;
-          const float t = __fmul_rn((float)q, s);
-          g[k] = pow2 ? __fmul_rn(t, rc) : __fdiv_rn(t, a.prescale);
-        }
-      };
-      switch (b) {
-        case 4: codes(std::integral_constant<int, 4>{}); break;
-        case 6: codes(std::integral_constant<int, 6>{}); break;
-        case 8: codes(std::integral_constant<int, 8>{}); break;
-        case 10: codes(std::integral_constant<int, 10>{}); break;
-        case 12: codes(std::integral_constant<int, 12>{}); break;
-        case 16: codes(std::integral_constant<int, 16>{}); break;
-        default: codes(std::integral_constant<int, 0>{}); break;
-      }
+      for (int k = 0; k < E / 2; ++k) x[k] = mul2(x[k], f2(rc));
+    } else {
+#pragma unroll
+      for (int k = 0; k < E / 2; ++k) x[k] = f2(__fdiv_rn(x[k].x, a.prescale), __fdiv_rn(x[k].y, a.prescale));
+    }
+    uint32_t o[16];
+#pragma unroll
+    for (int k = 0; k < E / 2; ++k) {
       if constexpr (BF16) {
-        uint32_t u[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const __nv_bfloat162 h2 = __floats2bfloat162_rn(g[2 * j], g[2 * j + 1]);
-          u[j] = *reinterpret_cast<const uint32_t *>(&h2);
-        }
-        *reinterpret_cast<uint4 *>(orow + (size_t)k0 * 2) = make_uint4(u[0], u[1], u[2], u[3]);
+        const __nv_bfloat162 h2 = __floats2bfloat162_rn(x[k].x, x[k].y);
+        o[k] = *reinterpret_cast<const uint32_t *>(&h2);
       } else {
-        reinterpret_cast<float4 *>(orow + (size_t)k0 * 4)[0] = make_float4(g[0], g[1], g[2], g[3]);
-        reinterpret_cast<float4 *>(orow + (size_t)k0 * 4)[1] = make_float4(g[4], g[5], g[6], g[7]);
+        o[2 * k] = __float_as_uint(x[k].x);
+        o[2 * k + 1] = __float_as_uint(x[k].y);
+      }
+    }
+    const uint32_t left = (C - p0 * (uint32_t)E) * ESZ;   // bytes of the row from this piece on: a multiple of 16
+    uint8_t *dst = a.out + ((uint64_t)r0 * C + p0 * (uint32_t)E) * ESZ;
+#pragma unroll
+    for (int j = 0; j < 16; j += WIDE ? 8 : 4) {
+      if (4u * j < left) {
+        if constexpr (WIDE)   // (rows of whole 32-byte pieces)
+          asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst + 4 * j), "r"(o[j]), "r"(o[j + 1]),
+                       "r"(o[j + 2]), "r"(o[j + 3]), "r"(o[j + 4]), "r"(o[j + 5]), "r"(o[j + 6]), "r"(o[j + 7])
+                       : "memory");
+        else
+          *reinterpret_cast<uint4 *>(dst + 4 * j) = make_uint4(o[j], o[j + 1], o[j + 2], o[j + 3]);
       }
     }
   }
 }
+
+// ---- launches (one translation unit per element type: qnaive_*.cu) --------------------------------------
+template <bool BF16, int B>
+tahq_status qnaive_encode_b(QArgs a, const DevInfo &d, cudaStream_t st) {
+  static std::atomic<int> occ[64];
+  const int n = prepare(qnaive_encode_kernel<BF16, B>, kQThreads, 0, d, occ);
+  if (!n) return TAHQ_ERR_CUDA;
+  const uint32_t parts = (a.hidden + 31) / 32, stretches = (parts + 31) / 32;
+  a.row_warps = stretches < 8 ? stretches : 8;
+  a.row_lanes = 32;
+  while (a.row_warps == 1 && a.row_lanes / 2 >= parts) a.row_lanes /= 2;
+  const uint32_t threads = a.row_warps > 1 ? 32 * a.row_warps * (8 / a.row_warps) : kQThreads;   // whole rows
+  const uint32_t rows = a.row_warps > 1 ? 8 / a.row_warps : 8 * (32 / a.row_lanes);
+  const uint64_t want = (a.tokens + rows - 1) / rows, cap = (uint64_t)d.sms * n;
+  TAHQ_LAUNCH("qnaive_encode", st, launch_dependent(qnaive_encode_kernel<BF16, B>, (unsigned)(want < cap ? want : cap), threads, 0, st, a));
+  return cudaGetLastError() == cudaSuccess ? TAHQ_OK : TAHQ_ERR_CUDA;
+}
+template <bool BF16, int B>
+tahq_status qnaive_decode_b(QArgs a, const DevInfo &d, cudaStream_t st) {
+  constexpr uint32_t E = BF16 ? 32 : 16;
+  static std::atomic<int> occ[2][64];
+  const bool wide = (reinterpret_cast<uintptr_t>(a.out) & 31u) == 0 && a.hidden % (E / 2) == 0;
+  void (*const kernel)(QArgs) = wide ? qnaive_decode_kernel<BF16, B, true> : qnaive_decode_kernel<BF16, B, false>;
+  const int n = prepare(kernel, kQThreads, 0, d, occ[wide]);
+  if (!n) return TAHQ_ERR_CUDA;
+  a.pieces = (a.hidden + E - 1) / E;
+  const uint64_t want = (a.tokens * a.pieces + kQThreads - 1) / kQThreads, cap = (uint64_t)d.sms * n;
+  if (want > (1ull << 32) / kQThreads - cap) return TAHQ_ERR_UNSUPPORTED;   // (a tensor beyond 250 GB)
+  TAHQ_LAUNCH("qnaive_decode", st, launch_dependent(kernel, (unsigned)(want < cap ? want : cap), kQThreads, 0, st, a));
+  return cudaGetLastError() == cudaSuccess ? TAHQ_OK : TAHQ_ERR_CUDA;
+}
+template <bool BF16, bool ENC, int B = 2>
+tahq_status qnaive_width(const QArgs &a, const DevInfo &d, cudaStream_t st) {
+  if constexpr (B > 16) return TAHQ_ERR_INVALID_ARG;
+  else if (a.bits != (uint32_t)B) return qnaive_width<BF16, ENC, B + 1>(a, d, st);
+  else if constexpr (ENC) return qnaive_encode_b<BF16, B>(a, d, st);
+  else return qnaive_decode_b<BF16, B>(a, d, st);
+}
+template <bool BF16>
+tahq_status qnaive_encode_cfg(const QArgs &a, const DevInfo &d, cudaStream_t st) {
+  if (a.per_tensor)
+    TAHQ_LAUNCH("qnaive_max", st, launch_dependent(qnaive_max_kernel<BF16>, d.sms * 4, kQThreads, 0, st, a));
+  return qnaive_width<BF16, true>(a, d, st);
+}
+template <bool BF16>
+tahq_status qnaive_decode_cfg(const QArgs &a, const DevInfo &d, cudaStream_t st) {
+  return qnaive_width<BF16, false>(a, d, st);
+}
+#define TAHQ_INSTANTIATE_QNAIVE(BF16)                                                          \
+  template tahq_status qnaive_encode_cfg<BF16>(const QArgs &, const DevInfo &, cudaStream_t);  \
+  template tahq_status qnaive_decode_cfg<BF16>(const QArgs &, const DevInfo &, cudaStream_t);
 
 }  // namespace tahq

@@ -6,7 +6,6 @@
 
 #include "tahq_host.cuh"
 #include "tahq_kernels.cuh"
-#include "qnaive.cuh"
 
 namespace tahq {
 
@@ -314,10 +313,6 @@ void q_args(const tahq_qnaive_params *p, const QPlan &q, QArgs *a, void *ws) {
   h[10] = (uint32_t)q.row_bytes; h[11] = (uint32_t)(q.row_bytes >> 32);
   h[12] = (uint32_t)q.total_bytes; h[13] = (uint32_t)(q.total_bytes >> 32);
 }
-unsigned q_grid(uint64_t tokens, const DevInfo &d) {
-  const uint64_t want = (tokens + 7) / 8, cap = (uint64_t)d.sms * 8;
-  return (unsigned)(want < cap ? want : cap);
-}
 }  // namespace
 
 size_t tahq_qnaive_packed_bound(const tahq_qnaive_params *p) {
@@ -345,15 +340,8 @@ tahq_status tahq_qnaive_encode(const tahq_qnaive_params *p, const void *d_in, vo
   q_args(p, q, &a, d_ws);
   a.in = static_cast<const uint8_t *>(d_in);
   a.packed = static_cast<uint8_t *>(d_packed);
-  if (launch_clear(d_ws, 256, st) != TAHQ_OK) return TAHQ_ERR_CUDA;
-  const bool bf = p->dtype == TAHQ_BF16;
-  if (p->per_tensor) {
-    if (bf) TAHQ_LAUNCH("qnaive_max", st, launch_dependent(qnaive_max_kernel<true>, d.sms * 4, kQThreads, 0, st, a));
-    else TAHQ_LAUNCH("qnaive_max", st, launch_dependent(qnaive_max_kernel<false>, d.sms * 4, kQThreads, 0, st, a));
-  }
-  if (bf) TAHQ_LAUNCH("qnaive_encode", st, launch_dependent(qnaive_encode_kernel<true>, q_grid(p->tokens, d), kQThreads, 0, st, a));
-  else TAHQ_LAUNCH("qnaive_encode", st, launch_dependent(qnaive_encode_kernel<false>, q_grid(p->tokens, d), kQThreads, 0, st, a));
-  return cudaGetLastError() == cudaSuccess ? TAHQ_OK : TAHQ_ERR_CUDA;
+  if (p->per_tensor && launch_clear(d_ws, 256, st) != TAHQ_OK) return TAHQ_ERR_CUDA;   // the maximum is formed there
+  return p->dtype == TAHQ_BF16 ? qnaive_encode_cfg<true>(a, d, st) : qnaive_encode_cfg<false>(a, d, st);
 }
 
 tahq_status tahq_qnaive_decode(const tahq_qnaive_params *p, const void *d_packed, size_t packed_bytes, void *d_out,
@@ -371,12 +359,7 @@ tahq_status tahq_qnaive_decode(const tahq_qnaive_params *p, const void *d_packed
   q_args(p, q, &a, d_ws);
   a.packed = const_cast<uint8_t *>(static_cast<const uint8_t *>(d_packed));
   a.out = static_cast<uint8_t *>(d_out);
-  if (launch_clear(d_ws, 256, st) != TAHQ_OK) return TAHQ_ERR_CUDA;
-  if (p->dtype == TAHQ_BF16)
-    TAHQ_LAUNCH("qnaive_decode", st, launch_dependent(qnaive_decode_kernel<true>, q_grid(p->tokens, d), kQThreads, 0, st, a));
-  else
-    TAHQ_LAUNCH("qnaive_decode", st, launch_dependent(qnaive_decode_kernel<false>, q_grid(p->tokens, d), kQThreads, 0, st, a));
-  return cudaGetLastError() == cudaSuccess ? TAHQ_OK : TAHQ_ERR_CUDA;
+  return p->dtype == TAHQ_BF16 ? qnaive_decode_cfg<true>(a, d, st) : qnaive_decode_cfg<false>(a, d, st);
 }
 
 tahq_status tahq_selftest_wait_timeout(void *d_ws, size_t ws_cap, tahq_stream stream) {

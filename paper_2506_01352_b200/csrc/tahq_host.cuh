@@ -104,4 +104,26 @@ tahq_status encode_cfg(const Plan &pl, const Args &a, bool stochastic, cudaStrea
 template <int G, bool BF16>
 tahq_status decode_cfg(const Plan &pl, const Args &a, cudaStream_t st);
 
+// ---- fixed-point gradient compressor (qnaive.cuh; instantiated in qnaive_*.cu) -------------------------
+struct QArgs {
+  const uint8_t *in;      // encode: tensor
+  uint8_t *packed;
+  uint8_t *out;           // decode: tensor
+  uint64_t tokens;
+  uint32_t hidden, bits, per_tensor;
+  float prescale;
+  uint64_t off_scales, off_payload, row_bytes, total_bytes;
+  uint32_t *gmax;         // per-tensor mode: bits of max |g| (zeroed per call)
+  uint32_t *status;
+  uint32_t pieces;        // decode: pieces of a row
+  uint32_t row_warps;     // encode: warps that share a row (1: a warp takes one or more whole rows)
+  uint32_t row_lanes;     // encode, row_warps = 1: lanes of a row, a power of two
+  uint32_t header[16];
+};
+
+template <bool BF16>
+tahq_status qnaive_encode_cfg(const QArgs &a, const DevInfo &d, cudaStream_t st);
+template <bool BF16>
+tahq_status qnaive_decode_cfg(const QArgs &a, const DevInfo &d, cudaStream_t st);
+
 }  // namespace tahq

@@ -1,0 +1,46 @@
+"""Every width of the fixed-point compressor at rows that end inside a lane's 32 elements, inside a warp's 1024 and past
+a CTA's 8192, with few and many rows, and on tensors that start 16 bytes off a 32-byte boundary."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+from paper_2506_01352_b200 import binding as T
+from paper_2506_01352_b200 import synth
+from tests.guards import Guarded
+from tests.test_gpu_qnaive import _check
+
+pytestmark = pytest.mark.gpu
+
+
+def rows(tokens, hidden, dtype, seed):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    x = torch.randn(tokens, hidden, generator=g, device="cuda") * torch.randn(tokens, 1, generator=g, device="cuda").exp()
+    return (x * 1e-3).to(dtype)
+
+
+@pytest.mark.parametrize("bits", range(2, 17))
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("shape", [(700, 8), (261, 72), (37, 520), (19, 1024), (5, 1048), (3, 5160), (2, 16408)])
+def test_every_width_at_ragged_rows(shape, dtype, bits):
+    _check(rows(*shape, dtype, bits), bits, bits % 2, 1000.0 if bits % 3 else 1024.0)
+
+
+@pytest.mark.parametrize("bits", [6, 7, 8])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_tensors_off_a_32_byte_boundary(dtype, bits):
+    x = rows(33, 1056, dtype, bits)
+    dt = T.F32 if dtype == torch.float32 else T.BF16
+    p = T.QNaiveParams(tokens=33, hidden=1056, dtype=dt, bits=bits)
+    po = O.QNaiveParams(tokens=33, hidden=1056, dtype=dt, bits=bits)
+    nb = x.numel() * x.element_size()
+    gin, gout = Guarded(nb + 16, "cuda"), Guarded(nb + 16, "cuda")
+    src, dst = gin.view[16:].view(dtype).view(33, 1056), gout.view[16:].view(dtype).view(33, 1056)
+    src.copy_(x)
+    packed, _ = T.qnaive_encode(p, src)
+    T.qnaive_decode(p, packed, out=dst)
+    torch.cuda.synchronize()
+    gout.check("output tensor")
+    want = O.qnaive_encode(po, synth.to_host_array(x))
+    assert np.array_equal(packed.cpu().numpy(), want)
+    assert np.array_equal(synth.to_host_array(dst), O.qnaive_decode(po, want))
