@@ -31,29 +31,30 @@ template <bool BF16>
 struct QRaw {
   static constexpr int NW = BF16 ? 16 : 32;
   uint32_t w[NW];
-  // n elements (a multiple of 8, at most 32) from src, zeros behind them; `wide`: src is 32-byte aligned
-  __device__ __forceinline__ void load(const uint8_t *src, int n, bool wide) {
+  // `wide`: src is 32-byte aligned
+  __device__ __forceinline__ void load(const uint8_t *src, bool wide) {
     if constexpr (!BF16) {
       if (wide) {   // (a lane's 128 bytes by 128-bit loads would take twice the passes over the L1 tags)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          if (8 * i < n) {
-            asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                         : "=r"(w[8 * i]), "=r"(w[8 * i + 1]), "=r"(w[8 * i + 2]), "=r"(w[8 * i + 3]), "=r"(w[8 * i + 4]),
-                           "=r"(w[8 * i + 5]), "=r"(w[8 * i + 6]), "=r"(w[8 * i + 7])
-                         : "l"(src + 32 * i));
-          } else {
-#pragma unroll
-            for (int j = 0; j < 8; ++j) w[8 * i + j] = 0u;
-          }
-        }
+        for (int i = 0; i < 4; ++i)
+          asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                       : "=r"(w[8 * i]), "=r"(w[8 * i + 1]), "=r"(w[8 * i + 2]), "=r"(w[8 * i + 3]), "=r"(w[8 * i + 4]),
+                         "=r"(w[8 * i + 5]), "=r"(w[8 * i + 6]), "=r"(w[8 * i + 7])
+                       : "l"(src + 32 * i));
         return;
       }
     }
-    constexpr int PER = BF16 ? 8 : 4;   // elements of a 128-bit load
 #pragma unroll
-    for (int i = 0; i < 32 / PER; ++i) {
-      const uint4 v = PER * i < n ? __ldg(reinterpret_cast<const uint4 *>(src) + i) : make_uint4(0, 0, 0, 0);
+    for (int i = 0; i < NW / 4; ++i) {
+      const uint4 v = __ldg(reinterpret_cast<const uint4 *>(src) + i);
+      w[4 * i] = v.x; w[4 * i + 1] = v.y; w[4 * i + 2] = v.z; w[4 * i + 3] = v.w;
+    }
+  }
+  // the first n elements only (a multiple of 8), zeros behind them
+  __device__ __forceinline__ void load_some(const uint8_t *src, uint32_t n) {
+#pragma unroll
+    for (int i = 0; i < NW / 4; ++i) {
+      const uint4 v = (BF16 ? 8u : 4u) * i < n ? __ldg(reinterpret_cast<const uint4 *>(src) + i) : make_uint4(0, 0, 0, 0);
       w[4 * i] = v.x; w[4 * i + 1] = v.y; w[4 * i + 2] = v.z; w[4 * i + 3] = v.w;
     }
   }
@@ -95,9 +96,9 @@ __device__ __forceinline__ float q_scale(float mg, float prescale, float &inv) {
 // 32 codes -> B words of the row's bit stream.  Four (b <= 8) or two codes are glued by a multiply-add chain on the
 // raw bits of fma(y, 1/s, 1.5 * 2^23); the constant part of those bits, less L per code, is taken off once per chain.
 // The clamp is left out: |y| <= m and s = m / L rounded give |y * (1/s)| < L + 1/2, so it never acts on finite
-// input.  n = elements of the row among the 32: codes behind them are zero bits.
+// input.
 template <bool BF16, int B>
-__device__ __forceinline__ void q_codes(const QRaw<BF16> &raw, float prescale, float inv, int n, uint32_t (&w)[B]) {
+__device__ __forceinline__ void q_codes(const QRaw<BF16> &raw, float prescale, float inv, uint32_t (&w)[B]) {
   constexpr int GS = B <= 8 ? 4 : 2, GB = GS * B;   // codes and bits of a chain
   constexpr uint32_t Lq = (1u << (B - 1)) - 1u;
   constexpr uint32_t kOff = (uint32_t)(((unsigned long long)(kQMagicBits - Lq) * group_ones(B, GS)) & 0xffffffffull);
@@ -115,24 +116,32 @@ __device__ __forceinline__ void q_codes(const QRaw<BF16> &raw, float prescale, f
       acc = k == GS / 2 - 1 ? __float_as_uint(t.y) : acc * M + __float_as_uint(t.y);
       acc = acc * M + __float_as_uint(t.x);
     }
-    uint32_t g = acc - kOff;
-    if (n < 32 && GS * j >= n) g = 0;   // (n is a multiple of 8)
+    const uint32_t g = acc - kOff;
     const int bit = j * GB, wi = bit >> 5, sh = bit & 31;
     w[wi] |= g << sh;
     if (sh + GB > 32) w[wi + 1] |= g >> (32 - sh);
   }
 }
 
+// The words of a lane's 32 codes, of which n belong to the row (the others are zero bits), to the lane's place `dst`;
+// `room` = words of the row from there on (a multiple of the words of a store).
 template <int B>
-__device__ __forceinline__ void q_store(uint32_t *row, uint32_t first, uint32_t row_words, const uint32_t (&w)[B]) {
-  constexpr int V = B % 4 == 0 ? 4 : B % 2 == 0 ? 2 : 1;   // words of a store; row_words is a multiple of 4
+__device__ __forceinline__ void q_store(uint32_t *dst, uint32_t n, uint32_t room, uint32_t (&w)[B]) {
+  constexpr int V = B % 4 == 0 ? 4 : B % 2 == 0 ? 2 : 1;   // words of a store
+  if (n < 32u) {
+    const int bits = (int)n * B;
+#pragma unroll
+    for (int j = 0; j < B; ++j) w[j] &= bits >= 32 * (j + 1) ? 0xffffffffu : bits <= 32 * j ? 0u : (1u << (bits - 32 * j)) - 1u;
+#pragma unroll
+    for (int j = 0; j < B; ++j)
+      if ((uint32_t)j < room) dst[j] = w[j];
+    return;
+  }
 #pragma unroll
   for (int j = 0; j < B; j += V) {
-    if (first + j < row_words) {
-      if constexpr (V == 4) *reinterpret_cast<uint4 *>(row + first + j) = make_uint4(w[j], w[j + 1], w[j + 2], w[j + 3]);
-      else if constexpr (V == 2) *reinterpret_cast<uint2 *>(row + first + j) = make_uint2(w[j], w[j + 1]);
-      else row[first + j] = w[j];
-    }
+    if constexpr (V == 4) *reinterpret_cast<uint4 *>(dst + j) = make_uint4(w[j], w[j + 1], w[j + 2], w[j + 3]);
+    else if constexpr (V == 2) *reinterpret_cast<uint2 *>(dst + j) = make_uint2(w[j], w[j + 1]);
+    else dst[j] = w[j];
   }
 }
 
@@ -155,7 +164,8 @@ __global__ void __launch_bounds__(kQThreads) qnaive_max_kernel(const QArgs a) {
   float m = 0.0f;
   for (uint64_t i = ((uint64_t)blockIdx.x * kQThreads + threadIdx.x) * 32; i < n; i += (uint64_t)gridDim.x * kQThreads * 32) {
     QRaw<BF16> raw;
-    raw.load(a.in + i * ESZ, n - i < 32 ? (int)(n - i) : 32, wide);
+    if (n - i >= 32) raw.load(a.in + i * ESZ, wide);
+    else raw.load_some(a.in + i * ESZ, (uint32_t)(n - i));
     m = fmaxf(m, raw.max_abs());
   }
 #pragma unroll
@@ -163,77 +173,104 @@ __global__ void __launch_bounds__(kQThreads) qnaive_max_kernel(const QArgs a) {
   if ((threadIdx.x & 31) == 0 && m > 0.0f) atomicMax(a.gmax, __float_as_uint(m));
 }
 
-template <bool BF16, int B>
+// LONG: rows beyond 8192 elements, which a CTA's eight warps take in several stretches (the later ones read twice).
+template <bool BF16, int B, bool LONG>
 __global__ void __launch_bounds__(kQThreads, BF16 ? 3 : 2) qnaive_encode_kernel(const QArgs a) {
   constexpr int ESZ = BF16 ? 2 : 4;
-  __shared__ float s_max[2][8];
+  __shared__ uint32_t s_max[2][8];
   const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, C = a.hidden;
   const uint32_t n_warps = blockDim.x >> 5, row_words = (uint32_t)(a.row_bytes / 4), lanes_all = (C + 31u) / 32u;
   float *scales = reinterpret_cast<float *>(a.packed + a.off_scales);
   const bool wide = (reinterpret_cast<uintptr_t>(a.in) & 31u) == 0;
   grid_dependency_wait();   // launched as a programmatic dependent of the kernel in front
   if (blockIdx.x == 0) q_frame(a);
-  float mg = a.per_tensor ? __uint_as_float(*a.gmax) : 0.0f;
+  uint32_t mg = a.per_tensor ? *a.gmax : 0u;   // largest magnitude, as bits
 
   // rows of the CTA at a time, and this lane's place in one of them
-  const uint32_t rows_at_once = a.row_warps > 1 ? n_warps / a.row_warps : n_warps * (32u / a.row_lanes);
-  const uint32_t slot = a.row_warps > 1 ? warp / a.row_warps : warp * (32u / a.row_lanes) + lane / a.row_lanes;
-  const uint32_t part = a.row_warps > 1 ? warp % a.row_warps * 32u + lane : lane % a.row_lanes;   // 32 elements each
+  const bool shared_row = a.row_warps > 1;
+  const uint32_t rows_at_once = shared_row ? n_warps / a.row_warps : n_warps * (32u / a.row_lanes);
+  const uint32_t slot = shared_row ? warp / a.row_warps : warp * (32u / a.row_lanes) + lane / a.row_lanes;
+  const uint32_t part = shared_row ? warp % a.row_warps * 32u + lane : lane % a.row_lanes;   // 32 elements each
+  const uint32_t parts_at_once = shared_row ? a.row_warps * 32u : a.row_lanes;
   const uint64_t step = (uint64_t)gridDim.x * rows_at_once;
-  const uint32_t parts_at_once = a.row_warps > 1 ? a.row_warps * 32u : a.row_lanes;
-  auto elements = [&](uint32_t p) { return p < lanes_all ? (C - 32u * p < 32u ? (int)(C - 32u * p) : 32) : 0; };
-  auto load = [&](QRaw<BF16> &raw, uint64_t r, uint32_t p) {
-    raw.load(a.in + (r * (uint64_t)C + 32u * p) * ESZ, r < a.tokens ? elements(p) : 0, wide);
+  auto elements = [&](uint32_t p) { return p >= lanes_all ? 0u : C - 32u * p < 32u ? C - 32u * p : 32u; };
+  auto load_at = [&](QRaw<BF16> &raw, const uint8_t *src, uint32_t n) {
+    if (n == 32u) raw.load(src, wide);
+    else if (n) raw.load_some(src, n);
   };
-  auto emit = [&](const QRaw<BF16> &raw, uint64_t r, uint32_t p, float inv) {
+  auto emit = [&](const QRaw<BF16> &raw, uint32_t *dst, uint32_t n, uint32_t room, float inv) {
     uint32_t w[B];
-    q_codes<BF16, B>(raw, a.prescale, inv, elements(p), w);
-    uint32_t *row = reinterpret_cast<uint32_t *>(a.packed + a.off_payload + r * a.row_bytes);
-    if (p < lanes_all) q_store<B>(row, p * (uint32_t)B, row_words, w);
+    q_codes<BF16, B>(raw, a.prescale, inv, w);
+    if (n) q_store<B>(dst, n, room, w);
   };
   const uint64_t r_cta = (uint64_t)blockIdx.x * rows_at_once;
   uint64_t r = r_cta + slot;
-  QRaw<BF16> next;
-  load(next, r, part);
+  const uint32_t n_mine = elements(part);
+  const uint8_t *src = a.in + (r * (uint64_t)C + 32u * part) * ESZ;
+  uint32_t *dst = reinterpret_cast<uint32_t *>(a.packed + a.off_payload + r * a.row_bytes) + part * (uint32_t)B;
+  const uint64_t d_src = step * C * ESZ, d_dst = step * row_words;
   uint32_t parity = 0;
-  for (uint64_t rc = r_cta; rc < a.tokens; rc += step, r += step) {   // (the same number of turns for every lane of the CTA)
-    const QRaw<BF16> cur = next;
+
+  // one row: its elements are here; those of the lane's row after it are asked for
+  auto turn = [&](const QRaw<BF16> &cur, QRaw<BF16> &next) {
     const bool live = r < a.tokens;
-    load(next, r + step, part);
+    src += d_src;
+    if (!LONG && r + step < a.tokens) load_at(next, src, n_mine);
     if (!a.per_tensor) {
-      float m = cur.max_abs();
-      for (uint32_t p = part + parts_at_once; live && p < lanes_all; p += parts_at_once) {   // (rows beyond 8192 elements)
-        QRaw<BF16> more;
-        load(more, r, p);
-        m = fmaxf(m, more.max_abs());
-      }
+      uint32_t m = __float_as_uint(cur.max_abs());   // (non-negative floats order like their bit patterns)
+      if (LONG && live)
+#pragma unroll 1
+        for (uint32_t p = part + parts_at_once; p < lanes_all; p += parts_at_once) {
+          QRaw<BF16> more;
+          load_at(more, a.in + (r * (uint64_t)C + 32u * p) * ESZ, elements(p));
+          m = max(m, __float_as_uint(more.max_abs()));
+        }
       __syncwarp();
-      for (uint32_t o = a.row_lanes / 2; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(kFull, m, o));
-      if (a.row_warps > 1) {
-        if (lane == 0) s_max[parity][warp] = m;
-        asm volatile("bar.sync %0, %1;" ::"r"(slot + 1u), "r"(a.row_warps * 32u) : "memory");
-        const uint32_t w0 = slot * a.row_warps;
-        m = s_max[parity][w0];
-        for (uint32_t i = 1; i < a.row_warps; ++i) m = fmaxf(m, s_max[parity][w0 + i]);
-        parity ^= 1u;   // (a warp writes this half again only after the next barrier, when all have read it)
+      if (a.row_lanes == 32u) {
+        m = __reduce_max_sync(kFull, m);
+        if (shared_row) {
+          if (lane == 0) s_max[parity][warp] = m;
+          asm volatile("bar.sync %0, %1;" ::"r"(slot + 1u), "r"(a.row_warps * 32u) : "memory");
+          m = __reduce_max_sync(kFull, lane < a.row_warps ? s_max[parity][slot * a.row_warps + lane] : 0u);
+          parity ^= 1u;   // (a warp writes this half again only after the next barrier, when all have read it)
+        }
+      } else {
+        for (uint32_t o = a.row_lanes / 2; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(kFull, m, o));
       }
       mg = m;
     }
     float inv;
-    const float s = q_scale<B>(mg, a.prescale, inv);
+    const float s = q_scale<B>(__uint_as_float(mg), a.prescale, inv);
     if (live) {
-      if (part == 0 && (!a.per_tensor || r == 0)) scales[a.per_tensor ? 0 : r] = s;
-      emit(cur, r, part, inv);
-      for (uint32_t p = part + parts_at_once; p < lanes_all; p += parts_at_once) {
-        QRaw<BF16> more;
-        load(more, r, p);
-        emit(more, r, p, inv);
+      if (part == 0) {
+        if (!a.per_tensor || r == 0) scales[a.per_tensor ? 0 : r] = s;
+        for (uint32_t o = lanes_all * (uint32_t)B; o < row_words; ++o) dst[o] = 0;   // the row's last words, behind its last lane's
       }
-      // the row's last words, behind its last lane's
-      const uint32_t from = lanes_all * (uint32_t)B;
-      if (part == 0 && from < row_words)
-        for (uint32_t o = from; o < row_words; ++o)
-          reinterpret_cast<uint32_t *>(a.packed + a.off_payload + r * a.row_bytes)[o] = 0;
+      emit(cur, dst, n_mine, row_words - part * (uint32_t)B, inv);
+      if (LONG)
+#pragma unroll 1
+        for (uint32_t p = part + parts_at_once; p < lanes_all; p += parts_at_once) {
+          QRaw<BF16> more;
+          load_at(more, a.in + (r * (uint64_t)C + 32u * p) * ESZ, elements(p));
+          emit(more, dst + (p - part) * (uint32_t)B, elements(p), row_words - p * (uint32_t)B, inv);
+        }
+    }
+    dst += d_dst;
+    r += step;
+  };
+  QRaw<BF16> ra, rb;
+#pragma unroll
+  for (int i = 0; i < QRaw<BF16>::NW; ++i) ra.w[i] = rb.w[i] = 0u;   // (lanes behind the row's end stay at zero)
+  if (LONG) {
+    for (uint64_t rc = r_cta; rc < a.tokens; rc += step) {   // (a row to the CTA)
+      load_at(ra, src, n_mine);
+      turn(ra, rb);
+    }
+  } else {
+    if (r < a.tokens) load_at(ra, src, n_mine);
+    for (uint64_t rc = r_cta; rc < a.tokens; rc += 2 * step) {   // (the same number of turns for every lane of the CTA)
+      turn(ra, rb);
+      if (rc + step < a.tokens) turn(rb, ra);
     }
   }
 }
@@ -350,17 +387,19 @@ __global__ void __launch_bounds__(kQThreads, 4) qnaive_decode_kernel(const QArgs
 // ---- launches (one translation unit per element type: qnaive_*.cu) --------------------------------------
 template <bool BF16, int B>
 tahq_status qnaive_encode_b(QArgs a, const DevInfo &d, cudaStream_t st) {
-  static std::atomic<int> occ[64];
-  const int n = prepare(qnaive_encode_kernel<BF16, B>, kQThreads, 0, d, occ);
-  if (!n) return TAHQ_ERR_CUDA;
+  static std::atomic<int> occ[2][64];
   const uint32_t parts = (a.hidden + 31) / 32, stretches = (parts + 31) / 32;
+  const bool lng = stretches > 8;
+  void (*const kernel)(QArgs) = lng ? qnaive_encode_kernel<BF16, B, true> : qnaive_encode_kernel<BF16, B, false>;
+  const int n = prepare(kernel, kQThreads, 0, d, occ[lng]);
+  if (!n) return TAHQ_ERR_CUDA;
   a.row_warps = stretches < 8 ? stretches : 8;
   a.row_lanes = 32;
   while (a.row_warps == 1 && a.row_lanes / 2 >= parts) a.row_lanes /= 2;
   const uint32_t threads = a.row_warps > 1 ? 32 * a.row_warps * (8 / a.row_warps) : kQThreads;   // whole rows
   const uint32_t rows = a.row_warps > 1 ? 8 / a.row_warps : 8 * (32 / a.row_lanes);
   const uint64_t want = (a.tokens + rows - 1) / rows, cap = (uint64_t)d.sms * n;
-  TAHQ_LAUNCH("qnaive_encode", st, launch_dependent(qnaive_encode_kernel<BF16, B>, (unsigned)(want < cap ? want : cap), threads, 0, st, a));
+  TAHQ_LAUNCH("qnaive_encode", st, launch_dependent(kernel, (unsigned)(want < cap ? want : cap), threads, 0, st, a));
   return cudaGetLastError() == cudaSuccess ? TAHQ_OK : TAHQ_ERR_CUDA;
 }
 template <bool BF16, int B>
