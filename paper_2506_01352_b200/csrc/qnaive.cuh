@@ -173,6 +173,9 @@ __global__ void __launch_bounds__(kQThreads) qnaive_max_kernel(const QArgs a) {
   if ((threadIdx.x & 31) == 0 && m > 0.0f) atomicMax(a.gmax, __float_as_uint(m));
 }
 
+// 19 us for 8192 x 4096 bf16 at 6 bits (92 MB; with the decoder 43.0 -> 32.9 us per round trip, of which the launches that
+// cleared 256 bytes took 4): bound half by memory, half by issue.  A warp to a row held 64 registers of raw data, which left 16
+// warps on an SM and 3.5 waves of CTAs.
 // LONG: rows beyond 8192 elements, which a CTA's eight warps take in several stretches (the later ones read twice).
 template <bool BF16, int B, bool LONG>
 __global__ void __launch_bounds__(kQThreads, BF16 ? 3 : 2) qnaive_encode_kernel(const QArgs a) {
@@ -275,6 +278,21 @@ __global__ void __launch_bounds__(kQThreads, BF16 ? 3 : 2) qnaive_encode_kernel(
   }
 }
 
+// t / c in binary32, correctly rounded, for several t by one c (rc = 1/c rounded): a quotient estimate is improved twice
+// by its remainder, which a fused multiply-add gives exactly; the second step rounds correctly because the first one's
+// result is within one unit in the last place (Markstein, IA-64 and Elementary Functions, ch. 8; Brisebarre, Muller and
+// Raina, IEEE Trans. Computers 53(8), 2004).  No step may leave the normal range: see div_safe.  Half the instructions of
+// __fdiv_rn, which cannot know that the divisor stays: 8192 x 4928 bf16 at 8 bits, c = 1000, encode + decode 74.8 -> 48.6 us.
+__device__ __forceinline__ float2 div_by(float2 t, float2 nc, float2 rc) {
+  const float2 q0 = f2(__fmul_rn(t.x, rc.x), __fmul_rn(t.y, rc.y));   // (scalar: they are addends below)
+  const float2 q1 = fma2(fma2(q0, nc, t), rc, q0);
+  return fma2(fma2(q1, nc, t), rc, q1);
+}
+// Every non-zero t = q * s of a row has s <= |t| < 2^16 s: t, its quotient and remainders (above 2^-50 |t|) stay normal.
+__device__ __forceinline__ bool div_safe(float s, float c) {
+  return (s == 0.0f || (s >= 0x1p-40f && s <= 0x1p60f)) && c >= 0x1p-30f && c <= 0x1p30f;
+}
+
 // Codes of a lane -> g_hat = (q * s) / c.  Dividing by a power of two is the same rounding as multiplying by its
 // (exact) reciprocal.
 template <bool BF16, int B, bool WIDE>
@@ -319,7 +337,7 @@ __global__ void __launch_bounds__(kQThreads, 4) qnaive_decode_kernel(const QArgs
   if (blockIdx.x == 0 && threadIdx.x == 0) *a.status = bad ? 1u /* TAHQ_DEV_BAD_HEADER */ : 0u;
   if (bad) return;
   const bool pow2 = (__float_as_uint(a.prescale) & 0x007fffffu) == 0u && (__float_as_uint(a.prescale) >> 23) - 2u < 250u;
-  const float rc = pow2 ? __frcp_rn(a.prescale) : 0.0f;
+  const float rc = __frcp_rn(a.prescale);
 
   for (; i < total; i += step) {
     uint32_t v[NW + 1];
@@ -353,6 +371,9 @@ __global__ void __launch_bounds__(kQThreads, 4) qnaive_decode_kernel(const QArgs
     if (pow2) {
 #pragma unroll
       for (int k = 0; k < E / 2; ++k) x[k] = mul2(x[k], f2(rc));
+    } else if (__all_sync(__activemask(), div_safe(sc, a.prescale))) {
+#pragma unroll
+      for (int k = 0; k < E / 2; ++k) x[k] = div_by(x[k], f2(-a.prescale), f2(rc));
     } else {
 #pragma unroll
       for (int k = 0; k < E / 2; ++k) x[k] = f2(__fdiv_rn(x[k].x, a.prescale), __fdiv_rn(x[k].y, a.prescale));

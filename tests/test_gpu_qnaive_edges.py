@@ -44,3 +44,12 @@ def test_tensors_off_a_32_byte_boundary(dtype, bits):
     want = O.qnaive_encode(po, synth.to_host_array(x))
     assert np.array_equal(packed.cpu().numpy(), want)
     assert np.array_equal(synth.to_host_array(dst), O.qnaive_decode(po, want))
+
+
+@pytest.mark.parametrize("c", [3.0, 1000.0, 0.1, 8191.0, 1.0000001, 1.9999999, 3e-12, 7e13])
+@pytest.mark.parametrize("bits", [8, 13, 16])
+def test_division_by_pre_scales_that_are_no_power_of_two(bits, c):
+    """Scales from far below to far above the range in which the quotient is formed from the reciprocal."""
+    x = rows(64, 2048, torch.float32, bits) * torch.logspace(-18, 18, 64, device="cuda")[:, None]
+    x[5] = 0
+    _check(x.contiguous(), bits, 0, c)
