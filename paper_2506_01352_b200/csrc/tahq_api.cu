@@ -2,6 +2,7 @@
 // buffer and of the workspace, kernel selection and launches on the caller's stream.
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <cstring>
 
 #include "tahq_host.cuh"
@@ -53,52 +54,15 @@ static tahq_status make_plan(const tahq_params *p, Plan *pl) {
   if (pl->alloc_m > 1 && A > 8192) return TAHQ_ERR_UNSUPPORTED;
 
   pl->mixed = L.k_hi > 0;
-  pl->direct = pl->rank_per_group <= (uint64_t)kSortCap;
-  pl->cpg = 1;
-  pl->sel_m = 1;
-  pl->cand_cap = 0;
-  if (pl->mixed && !pl->direct) {
-    // one CTA per slice of the group's scores, or several slices per CTA so that the grid stays near one wave
-    const uint64_t slices = (pl->rank_per_group + kSelSlice - 1) / kSelSlice;
-    uint64_t m = (slices * L.n_groups + 255) / 256;
-    m = m < 1 ? 1 : m > 64 ? 64 : m;
-    pl->sel_m = (uint32_t)m;
-    pl->cpg = (uint32_t)((slices + m - 1) / m);
-    const uint64_t cap = 32768ull;   // select_kernel copes with more candidates than the list holds
-    pl->cand_cap = (uint32_t)(pl->rank_per_group < cap ? pl->rank_per_group : cap);
-  }
-  const bool hist = pl->mixed && !pl->direct;
-  uint64_t o = 256;                                         // status word and friends
+  pl->whole_words = pl->alloc_m == 1 && L.tiles_per_group % 32 == 0;
+  uint64_t o = 256;                                         // status word
   pl->ws_flags = o;  o += 8ull * kMaxGrid;
-  pl->ws_ncand = o;  o = up(o + (hist ? 4 * L.n_groups : 0), 256);
-  pl->ws_done = o;   o = up(o + (hist ? 4 * L.n_groups : 0), 256);
-  pl->ws_nabove = o; o = up(o + (hist ? 4 * L.n_groups : 0), 256);
-  pl->ws_hist = o;   o += hist ? 4ull * kBins * L.n_groups : 0;
-  pl->ws_zero_end = o;                                      // [0, ws_zero_end) is cleared by every encode
+  pl->ws_zero_end = o;                                      // [0, ws_zero_end) is cleared by a decode with a look-back
   pl->ws_scores = o; o = up(o + (pl->mixed ? 4 * (L.n_tiles / pl->alloc_m) : 0), 256);
-  pl->ws_theta = o;  o = up(o + (pl->mixed ? 8 * L.n_groups : 0), 256);
-  pl->ws_cand = o;   o = up(o + 8ull * pl->cand_cap * L.n_groups, 256);
-  pl->fast = pl->alloc_m == 1 && L.tiles_per_group % 32 == 0;
-  // The selection on thread-block clusters: one cluster of up to 16 CTAs per ranking group.  The largest cluster
-  // whose CTAs hold at most 16384 scores each (32768 in smaller clusters) and of which the device holds one per
-  // group at the same time: groups that wait for a free cluster pay the whole chain of dependent steps again
-  // (measured: 8 groups of 163840 tiles in clusters of 16 took 38 us, of which 22 us was the second wave).  Beyond
-  // that the multi-CTA selection with its global histograms is the faster one (52 against 77 us on groups of 524288
-  // tiles: it spreads a group over more than 16 CTAs).
-  pl->csel = 0;
-  pl->csel_per_cta = 0;
-  if (pl->fast && pl->mixed) {
-    for (uint32_t cs = 16; cs >= 1; cs /= 2) {
-      if (cs > 1 && L.tiles_per_group <= (uint64_t)(cs / 2) * 8192) continue;   // a smaller cluster does at 8192 per CTA
-      const uint64_t per = ((L.tiles_per_group + cs - 1) / cs + 31) / 32 * 32;
-      if (per > (cs == 16 ? 16384u : 32768u)) break;                             // smaller clusters only hold more per CTA
-      const uint32_t cap = select_cluster_capacity(cs, (uint32_t)per);
-      if (cap == 0 || L.n_groups <= cap || cs == 1) { pl->csel = cs; pl->csel_per_cta = (uint32_t)per; break; }
-    }
-  }
-  // (128-wide tiles have no streaming score kernel with global histograms: such groups take the CTA-synchronous kernels)
-  if (G == 128 && pl->mixed && !pl->csel) pl->fast = false;
-  pl->ws_pre = o;    o = up(o + ((pl->alloc_m == 1 && L.tiles_per_group % 32 == 0 && pl->mixed) ? 4 * (L.n_tiles / 32) : 0), 256);
+  pl->ws_pre = o;    o = up(o + (pl->mixed ? 4 * ((L.n_tiles + 31) / 32) : 0), 256);
+  // words of the selection's slices, where a group's may not fit into shared memory
+  const bool long_groups = pl->mixed && pl->rank_per_group > 32ull * kWordsShared;
+  pl->ws_words = o;  o = up(o + (long_groups ? 8 * L.n_groups * ((pl->rank_per_group + 31) / 32 + 16) : 0), 256);
   pl->ws_total = o;
   return TAHQ_OK;
 }
@@ -151,28 +115,21 @@ static void fill_args(const tahq_params *p, const Plan &pl, uint8_t *ws, Args *a
   a->eps_ratio = p->eps_ratio;
   a->status = reinterpret_cast<uint32_t *>(ws);
   a->trace = g_trace;
-  a->fast = pl.fast;
-  a->epoch = reinterpret_cast<unsigned long long *>(ws + 64);
-  a->zero_begin = ws + pl.ws_ncand;
-  a->zero_n16 = (pl.ws_zero_end - pl.ws_ncand) / 16;
+  a->whole_words = pl.whole_words;
   a->pre = reinterpret_cast<uint32_t *>(ws + pl.ws_pre);
-  a->no_hist = pl.csel != 0;
-  a->ncand = reinterpret_cast<uint32_t *>(ws + pl.ws_ncand);
-  a->hist = reinterpret_cast<uint32_t *>(ws + pl.ws_hist);
+  a->words = reinterpret_cast<uint32_t *>(ws + pl.ws_words);
   a->scores = reinterpret_cast<float *>(ws + pl.ws_scores);
-  a->done = reinterpret_cast<uint32_t *>(ws + pl.ws_done);
-  a->nabove = reinterpret_cast<uint32_t *>(ws + pl.ws_nabove);
   a->bf16 = p->dtype == TAHQ_BF16;
   a->tile = p->tile;
   a->flags = reinterpret_cast<unsigned long long *>(ws + pl.ws_flags);
-  a->theta = reinterpret_cast<unsigned long long *>(ws + pl.ws_theta);
-  a->cand = reinterpret_cast<unsigned long long *>(ws + pl.ws_cand);
-  a->cand_cap = pl.cand_cap;
-  a->cpg = pl.cpg;
-  a->sel_m = pl.sel_m;
-  a->direct = pl.direct;
   // the screening score leaves varsigma out; its share of the score is below G * varsigma / ln 2
-  a->exact_scores = pl.direct || pl.alloc_m > 1 || (double)p->tile * (double)p->eps_log > 1e-5;
+  a->exact_scores = pl.alloc_m > 1 || (double)p->tile * (double)p->eps_log > 1e-5;
+  {   // 1024 bins for the scores up to two below the largest possible, 3072 above
+    const float knee = std::log2((float)(pl.alloc_m * p->tile)) - 2.0f;
+    a->step_lo = 16.0f * 1024.0f / knee;
+    a->step_hi = 8.0f * 3064.0f;   // (a few bins are left for rounding above the largest)
+    a->step_off = a->step_hi * knee - 16.0f * 1024.0f;
+  }
   fill_header(p, pl, a->header);
 }
 
@@ -223,7 +180,10 @@ tahq_status tahq_encode(const tahq_params *p, const void *d_in, void *d_packed, 
   fill_args(p, pl, static_cast<uint8_t *>(d_ws), &a);
   a.in = static_cast<const uint8_t *>(d_in);
   a.packed = static_cast<uint8_t *>(d_packed);
-  if (!pl.fast && launch_clear(d_ws, pl.ws_zero_end, st) != TAHQ_OK) return TAHQ_ERR_CUDA;
+  // groups that share words of the bit map: the selection puts those together on zeroes
+  if (pl.mixed && !pl.whole_words && pl.alloc_m == 1 &&
+      launch_clear(a.packed + a.off_bitmap, up((pl.L.n_tiles + 7) / 8, 128), st) != TAHQ_OK)
+    return TAHQ_ERR_CUDA;
   const bool bf = p->dtype == TAHQ_BF16, sr = p->rounding == 1;
   switch (p->tile) {
     case 8: return bf ? encode_cfg<8, true>(pl, a, sr, st) : encode_cfg<8, false>(pl, a, sr, st);
@@ -250,7 +210,7 @@ tahq_status tahq_decode(const tahq_params *p, const void *d_packed, size_t packe
   a.out = static_cast<uint8_t *>(d_out);
   // Up to 65536 bit-map words (256 KiB) the streaming kernel needs no look-back and nothing cleared: one launch.
   a.own_prefix = (pl.L.n_tiles + 31) / 32 <= 65536;
-  if (!a.own_prefix && launch_clear(d_ws, pl.ws_ncand, st) != TAHQ_OK) return TAHQ_ERR_CUDA;   // status + flags
+  if (!a.own_prefix && launch_clear(d_ws, pl.ws_zero_end, st) != TAHQ_OK) return TAHQ_ERR_CUDA;   // status + flags
   const bool bf = p->dtype == TAHQ_BF16;
   switch (p->tile) {
     case 8: return bf ? decode_cfg<8, true>(pl, a, st) : decode_cfg<8, false>(pl, a, st);
@@ -277,7 +237,6 @@ tahq_status tahq_encode_noalloc(const tahq_params *p, const void *d_in, void *d_
     g_noalloc_addr[dev] = ptr;
     g_noalloc_ready[dev].store(1, std::memory_order_release);
   }
-  // tahq_encode clears the head of the workspace (status, flags, histograms, counters) on the stream
   return tahq_encode(p, d_in, d_packed, packed_cap, g_noalloc_addr[dev], TAHQ_NOALLOC_SCRATCH_BYTES, stream);
 }
 

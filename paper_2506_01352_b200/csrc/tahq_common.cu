@@ -5,7 +5,7 @@
 #include <vector>
 
 #include "tahq_host.cuh"
-#include "tahq_select_cluster.cuh"
+#include "tahq_select.cuh"
 
 namespace tahq {
 
@@ -84,101 +84,79 @@ bool make_row_map(const void *base, uint64_t n_rows, bool bf16, CUtensorMap *tm)
 
 // ---- kernels that do not depend on the tile configuration ---------------------------------------------
 
-// Zero the first `bytes` (a multiple of 16) of the workspace with a kernel, so that the call's next kernel can
-// be its programmatic dependent.
-tahq_status launch_clear(void *d_ws, uint64_t bytes, cudaStream_t st) {
+// Zero `bytes` (a multiple of 16) with a kernel, so that the call's next kernel can be its programmatic dependent.
+tahq_status launch_clear(void *p, uint64_t bytes, cudaStream_t st) {
   const uint64_t n16 = bytes / 16;
   uint64_t grid = (n16 + kThreads - 1) / kThreads;
   grid = grid < 1 ? 1 : grid > 592 ? 592 : grid;
-  TAHQ_LAUNCH("clear", st, clear_kernel<<<(unsigned)grid, kThreads, 0, st>>>(static_cast<uint4 *>(d_ws), n16, g_trace));
+  TAHQ_LAUNCH("clear", st, launch_dependent(clear_kernel, (unsigned)grid, kThreads, 0, st, static_cast<uint4 *>(p), n16, g_trace));
   return cudaGetLastError() == cudaSuccess ? TAHQ_OK : TAHQ_ERR_CUDA;
 }
 
-tahq_status launch_select(const Args &a, cudaStream_t st) {
-  static std::atomic<int> ready[64];
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return TAHQ_ERR_CUDA;
-  const int sel_smem = kSortCap * 8;
-  if (!ready[dev & 63].load(std::memory_order_acquire)) {
-    if (cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, sel_smem) != cudaSuccess)
-      return TAHQ_ERR_CUDA;
-    ready[dev & 63].store(1, std::memory_order_release);
-  }
-  cudaError_t e;
-  TAHQ_LAUNCH("select", st,
-              e = launch_dependent(select_kernel, (unsigned)(a.n_groups * a.cpg), kSelThreads, sel_smem, st, a));
-  return e == cudaSuccess ? TAHQ_OK : TAHQ_ERR_CUDA;
-}
-
 // ---- selection on thread-block clusters ----------------------------------------------------------------
-static size_t select_cluster_smem(uint32_t per_cta) {
-  return (size_t)per_cta * 4 + (size_t)kBins * 4 + (size_t)(kClKeys + kSelThreads) * 8 + 2 * ((size_t)kClMaxPerCta / 32 * 4) +
-         (size_t)kClLocal * 2;
-}
-static bool select_cluster_ready(int dev) {
+constexpr size_t kSelSmem = (size_t)(kClKeys + kSelThreads) * 8 + (size_t)kBins * 4 + (size_t)kClKeys * 4 + (size_t)kWordsShared * 4;
+
+static bool select_ready(int dev) {
   static std::atomic<int> ready[64];
   if (ready[dev & 63].load(std::memory_order_acquire)) return true;
-  if (cudaFuncSetAttribute(select_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 204 * 1024) != cudaSuccess ||
-      cudaFuncSetAttribute(select_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-    (void)cudaGetLastError();
-    return false;
-  }
+  for (auto kernel : {select_kernel<true>, select_kernel<false>})
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSelSmem) != cudaSuccess ||
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+      (void)cudaGetLastError();
+      return false;
+    }
   ready[dev & 63].store(1, std::memory_order_release);
   return true;
 }
 
-// Clusters of `cs` CTAs of the selection kernel, each CTA with `per_cta` scores, that the device holds at the same
-// time (asked once per device and shape).  More ranking groups than that would run in waves, each wave the whole
-// chain of dependent steps.  0: the device cannot be asked (no GPU in this process).
-uint32_t select_cluster_capacity(uint32_t cs, uint32_t per_cta) {
-  static std::atomic<int> cache[64][5][17];   // device, log2(cs), per_cta / 2048: capacity + 1
-  int dev = 0, lg = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) { (void)cudaGetLastError(); return 0; }
-  while ((1u << lg) < cs) ++lg;
-  if (lg > 4 || per_cta > (uint32_t)kClMaxPerCta) return 0;
-  std::atomic<int> &slot = cache[dev & 63][lg][per_cta / 2048];
-  const int v = slot.load(std::memory_order_acquire);
-  if (v > 0) return (uint32_t)(v - 1);
-  if (!select_cluster_ready(dev)) return 0;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(cs);
-  cfg.blockDim = dim3(kSelThreads);
-  cfg.dynamicSmemBytes = select_cluster_smem((per_cta / 2048 + 1) * 2048 > (uint32_t)kClMaxPerCta ? (uint32_t)kClMaxPerCta
-                                                                                                 : (per_cta / 2048 + 1) * 2048);
-  cudaLaunchAttribute attr[1];
+static void cluster_config(cudaLaunchConfig_t *cfg, cudaLaunchAttribute *attr, unsigned grid, uint32_t cs, cudaStream_t st) {
+  *cfg = {};
+  cfg->gridDim = dim3(grid);
+  cfg->blockDim = dim3(kSelThreads);
+  cfg->dynamicSmemBytes = kSelSmem;
+  cfg->stream = st;
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = cs;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg->attrs = attr;
+  cfg->numAttrs = 1;
+}
+
+// Clusters of 2^lg CTAs of the selection kernel that the device holds at the same time (asked once per device and size).
+// More ranking groups than that run in waves, each wave the whole chain of dependent steps.  0: cannot be asked.
+static uint32_t select_capacity(int dev, int lg) {
+  static std::atomic<int> cache[64][5];   // capacity + 1
+  std::atomic<int> &slot = cache[dev & 63][lg];
+  const int v = slot.load(std::memory_order_acquire);
+  if (v > 0) return (uint32_t)(v - 1);
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr[1];
+  cluster_config(&cfg, attr, 1u << lg, 1u << lg, nullptr);
   int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, select_cluster_kernel, &cfg) != cudaSuccess) { (void)cudaGetLastError(); return 0; }
+  if (cudaOccupancyMaxActiveClusters(&n, select_kernel<true>, &cfg) != cudaSuccess) { (void)cudaGetLastError(); return 0; }
   slot.store(n + 1, std::memory_order_release);
   return (uint32_t)n;
 }
 
-// One cluster of `cs` CTAs per ranking group, launched as a programmatic dependent of the score kernel.
-tahq_status launch_select_cluster(const Args &a, uint32_t cs, uint32_t per_cta, cudaStream_t st) {
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || !select_cluster_ready(dev)) return TAHQ_ERR_CUDA;
-  const size_t smem = select_cluster_smem(per_cta);
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(a.n_groups * cs));
-  cfg.blockDim = dim3(kSelThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
+// One cluster per ranking group, launched as a programmatic dependent of the score kernel.
+tahq_status launch_select(const Args &a, const DevInfo &d, cudaStream_t st) {
+  if (!select_ready(d.dev)) return TAHQ_ERR_CUDA;
+  // The smallest cluster whose threads can hold their scores in registers (8192 x 768 in 8 groups of 12288: 5.9 us in
+  // clusters of 4, 8 us in clusters of 16), at most 16 CTAs, and one of which the device holds one per group at once.
+  int lg = 4;
+  constexpr uint64_t kSlice = (uint64_t)kHeld * kSelThreads;
+  while (lg > 0 && (a.rank_per_group <= kSlice << (lg - 1) || a.n_groups > select_capacity(d.dev, lg))) --lg;
+  const uint32_t cs = 1u << lg, per_cta = (uint32_t)(((a.rank_per_group + cs - 1) / cs + 31) / 32 * 32);
+  cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = cs;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
+  cluster_config(&cfg, attr, (unsigned)(a.n_groups * cs), cs, st);
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
   cfg.numAttrs = 2;
   cudaError_t e;
-  TAHQ_LAUNCH("select", st, e = cudaLaunchKernelEx(&cfg, select_cluster_kernel, a, per_cta));
+  TAHQ_LAUNCH("select", st, e = cudaLaunchKernelEx(&cfg, per_cta <= (uint32_t)(kHeld * kSelThreads) ? select_kernel<true> : select_kernel<false>,
+                                                  a, per_cta));
   return e == cudaSuccess ? TAHQ_OK : TAHQ_ERR_CUDA;
 }
 

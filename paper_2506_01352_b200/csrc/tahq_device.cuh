@@ -6,7 +6,7 @@
 // thread through shared memory: rows are copied (16-byte cp.async, or tiled TMA with the 128-byte
 // swizzle) into an XOR-swizzled stage from which every thread reads its own row with conflict-free
 // 128-bit loads.  tahq_stream.cuh builds per-warp stages of 32 rows from these blocks,
-// tahq_kernels.cuh per-CTA stages of 256 thread-rows (128-wide tiles, two lanes per tile).
+// 
 #pragma once
 
 #include <cuda_bf16.h>
@@ -17,8 +17,7 @@
 namespace tahq {
 
 constexpr int kThreads = 256;          // threads per CTA of the tile kernels
-constexpr int kBins = 4096;            // first-level histogram of the top-p% selection
-constexpr float kBinScale = 512.0f;    // bins per unit of score (scores lie in [0, log2 128]; beyond 8: the last bin)
+constexpr int kBins = 4096;            // histogram of the top-p% selection
 constexpr unsigned kFull = 0xffffffffu;
 
 // ------------------------------------------------------------------------------------------
@@ -135,33 +134,6 @@ __device__ __forceinline__ void tma_load_rows(void *dst, const void *tmap, int r
       "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
       ::"r"(smem_u32(dst)), "l"(tmap), "r"(0), "r"(row0), "r"(smem_u32(bar))
       : "memory");
-}
-
-// Copy the rows of chunk `c` (tiles [c*TPC, (c+1)*TPC), clipped to n_tiles) into a swizzled stage.
-// Rows past the end of the tensor are zero-filled.
-template <class C>
-__device__ __forceinline__ void issue_chunk(const uint8_t *in, uint64_t n_tiles, uint64_t c, uint8_t *stage,
-                                            const float *scores = nullptr) {
-  const uint64_t tile0 = c * C::TPC;
-  if (scores && threadIdx.x < C::TPC / 4) {   // the chunk's scores ride along behind the rows
-    const uint64_t first = tile0 + (uint64_t)threadIdx.x * 4;
-    const int left = first < n_tiles ? (int)(n_tiles - first < 4 ? n_tiles - first : 4) : 0;
-    cp_async16(stage + C::STAGE_BYTES + (size_t)threadIdx.x * 16, left ? scores + first : scores, left * 4);
-  }
-  const uint8_t *src = in + tile0 * (uint64_t)(C::G * C::ESZ) + (size_t)threadIdx.x * 16;
-  // chunk index ci = i*kThreads + tid lies in row ci / CPR, whose swizzle depends on tid only
-  uint8_t *dst = stage + (size_t)((int)threadIdx.x ^ swz<C>((int)threadIdx.x / C::CPR)) * 16;
-  if (tile0 + C::TPC <= n_tiles) {
-#pragma unroll
-    for (int i = 0; i < C::CPR; ++i) cp_async16(dst + (size_t)i * kThreads * 16, src + (size_t)i * kThreads * 16, 16);
-  } else {
-    const uint32_t valid_bytes = (uint32_t)(n_tiles - tile0) * C::G * C::ESZ;
-#pragma unroll
-    for (int i = 0; i < C::CPR; ++i) {
-      const bool ok = (uint32_t)(i * kThreads + (int)threadIdx.x) * 16u < valid_bytes;
-      cp_async16(dst + (size_t)i * kThreads * 16, ok ? src + (size_t)i * kThreads * 16 : in, ok ? 16 : 0);
-    }
-  }
 }
 
 // Eight consecutive elements (oct `o`) of this thread's row, widened to binary32.
@@ -437,18 +409,6 @@ __device__ __forceinline__ uint32_t score_key32(float s) {
 __device__ __forceinline__ uint64_t rank_key(float s, uint32_t idx_in_group) {
   return ((uint64_t)score_key32(s) << 32) | (uint64_t)(0xffffffffu - idx_in_group);
 }
-__device__ __forceinline__ uint32_t score_bin(float s) {
-  float t = fmaxf(s, 0.0f) * kBinScale;
-  t = fminf(t, (float)(kBins - 1));
-  return (uint32_t)t;   // truncation: monotone non-decreasing in s
-}
-// The position of a score on the axis of the bins, for comparisons with the band around a bin: scores beyond the
-// last bin (allocation tiles wider than 256 channels reach log2 A > 8) all count into that bin, so they must not
-// look as if they lay above it.
-__device__ __forceinline__ float score_bin_pos(float s) {
-  return fminf(fmaxf(s, 0.0f) * kBinScale, (float)(kBins - 1) + 0.5f);
-}
-
 // ------------------------------------------------------------------------------------------
 // Eq. 3-4 and the quantiser on a register-resident row
 // ------------------------------------------------------------------------------------------
@@ -555,15 +515,6 @@ __device__ __forceinline__ void row_swap_0_d(uint8_t *stage, int row, int d) {
   }
 }
 
-// ------------------------------------------------------------------------------------------
-// Stable counting sort of the 256 threads of a CTA by a 2-bit class, so that the warps that go
-// on are (nearly) uniform in (transformed?, higher width?) and neither the Hadamard butterfly nor
-// the width-specific packing runs divergent.  Two __syncthreads inside.
-// ------------------------------------------------------------------------------------------
-struct ClassSort {
-  int src;   // which thread's tile this thread processes from now on
-  int cls;   // class of that tile
-};
 // Largest and second-largest magnitude of a row (Eq. 3), no index.
 template <class C>
 __device__ __forceinline__ void row_top2(const uint8_t *stage, int row, float &a1, float &a2) {

@@ -20,15 +20,11 @@ struct Plan {
   tahq_layout L;
   uint32_t f;             // budget % 1000
   bool mixed;             // two widths in use (k_hi > 0)
-  bool direct;            // small ranking groups: select straight from the scores
-  bool fast;              // ranking groups are whole units of 32 tiles and A = G: no clearing
-                          // launch, widths and offsets come ready from select_kernel
-  uint32_t cpg, cand_cap, sel_m;
-  uint32_t csel, csel_per_cta;   // selection on thread-block clusters: CTAs per ranking group (0: not used), scores per CTA
+  bool whole_words;       // ranking groups are whole words of the bit map and A = G
   uint32_t alloc_m;            // quantisation tiles per allocation tile (Sec. 3.2; 1 by default)
   uint64_t rank_per_group, rank_k;   // allocation tiles per ranking group, and how many of them get the higher width
   // workspace offsets
-  uint64_t ws_flags, ws_ncand, ws_done, ws_nabove, ws_hist, ws_zero_end, ws_scores, ws_theta, ws_cand, ws_pre, ws_total;
+  uint64_t ws_flags, ws_zero_end, ws_scores, ws_pre, ws_words, ws_total;
 };
 
 // ---- launch bookkeeping --------------------------------------------------------------------------------
@@ -91,10 +87,8 @@ cudaError_t launch_dependent(void (*kernel)(P...), unsigned grid, unsigned block
 }
 
 // ---- kernels that do not depend on the tile configuration (tahq_common.cu) ------------------------------
-tahq_status launch_clear(void *d_ws, uint64_t bytes, cudaStream_t st);
-tahq_status launch_select(const Args &a, cudaStream_t st);
-tahq_status launch_select_cluster(const Args &a, uint32_t ctas_per_group, uint32_t per_cta, cudaStream_t st);
-uint32_t select_cluster_capacity(uint32_t ctas_per_group, uint32_t per_cta);   // clusters resident at once (0: unknown)
+tahq_status launch_clear(void *p, uint64_t bytes, cudaStream_t st);
+tahq_status launch_select(const Args &a, const DevInfo &d, cudaStream_t st);
 tahq_status launch_alloc_score(const Args &a, const DevInfo &d, cudaStream_t st);
 tahq_status launch_wait_selftest(const Args &a, cudaStream_t st);
 

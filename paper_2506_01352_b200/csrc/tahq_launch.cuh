@@ -7,11 +7,6 @@
 
 namespace tahq {
 
-template <class C> struct Stages {
-  static constexpr int STATS = 2;
-  static constexpr int QUANT = (C::ROWB == 256) ? 2 : (C::ROWB == 128 ? 2 : 3);
-};
-
 template <class C, bool SR>
 static tahq_status encode_t(const Plan &pl, const Args &a_in, cudaStream_t st) {
   DevInfo d;
@@ -19,15 +14,10 @@ static tahq_status encode_t(const Plan &pl, const Args &a_in, cudaStream_t st) {
   Args a = a_in;
   CUtensorMap tmap;
   a.use_tma = (C::ROWB == 128 && make_row_map(a.in, a.n_tiles * C::LPT, C::BF16, &tmap)) ? 1u : 0u;   // rows of 128 bytes
-  const uint64_t n_chunks = (a.n_tiles + C::TPC - 1) / C::TPC;
-  static std::atomic<int> occ_stats[64], occ_quant[64];
-  if (pl.mixed && pl.alloc_m > 1) {   // Sec. 3.2 with A = m * G: one warp per allocation tile, exact scores
-    if (launch_alloc_score(a, d, st) != TAHQ_OK) return TAHQ_ERR_CUDA;
-  }
   if (pl.mixed) {
-    if (pl.alloc_m > 1) {
-      // scores are in place
-    } else if (a.no_hist) {   // the selection bins the scores itself: scores only
+    if (pl.alloc_m > 1) {   // Sec. 3.2 with A = m * G: one warp per allocation tile, exact scores
+      if (launch_alloc_score(a, d, st) != TAHQ_OK) return TAHQ_ERR_CUDA;
+    } else {
       constexpr int NS = C::ROWB <= 128 ? 3 : 2;
       const int smem = kWarps * NS * StreamCfg<C>::UNIT_BYTES + 256;   // ring slots, then the warps' mbarriers
       static std::atomic<int> occ_sc[64], occ_sc_exact[64];
@@ -42,68 +32,22 @@ static tahq_status encode_t(const Plan &pl, const Args &a_in, cudaStream_t st) {
         TAHQ_LAUNCH("stats", st, launch_dependent(score_kernel<C, NS, true>, grid, kThreads, smem, st, a, tmap));
       else
         TAHQ_LAUNCH("stats", st, launch_dependent(score_kernel<C, NS, false>, grid, kThreads, smem, st, a, tmap));
-    } else if constexpr (C::LPT == 1) {
-      constexpr int NS = C::ROWB <= 128 ? 3 : 2;
-      const int smem = kWarps * NS * StreamCfg<C>::UNIT_BYTES + 256;   // ring slots, then the warps' mbarriers
-      static std::atomic<int> occ_exact[64];
-      const int occ = a.exact_scores ? prepare(stats_stream_kernel<C, NS, true>, kThreads, smem, d, occ_exact)
-                                     : prepare(stats_stream_kernel<C, NS, false>, kThreads, smem, d, occ_stats);
-      if (!occ) return TAHQ_ERR_CUDA;
-      const uint64_t n_units = (a.n_tiles + 31) / 32;
-      const unsigned grid = persistent_grid((n_units + kWarps - 1) / kWarps, d, occ);
-      if (a.exact_scores)
-        TAHQ_LAUNCH("stats", st, launch_dependent(stats_stream_kernel<C, NS, true>, grid, kThreads, smem, st, a, tmap));
-      else
-        TAHQ_LAUNCH("stats", st, launch_dependent(stats_stream_kernel<C, NS, false>, grid, kThreads, smem, st, a, tmap));
-    } else {
-      constexpr int NS = Stages<C>::STATS;
-      const int smem = NS * C::STAGE_BYTES;
-      const int occ = prepare(stats_kernel<C, NS>, kThreads, smem, d, occ_stats);
-      if (!occ) return TAHQ_ERR_CUDA;
-      TAHQ_LAUNCH("stats", st,
-                  launch_dependent(stats_kernel<C, NS>, persistent_grid(n_chunks, d, occ), kThreads, smem, st, a));
     }
-    if ((pl.csel ? launch_select_cluster(a, pl.csel, pl.csel_per_cta, st) : launch_select(a, st)) != TAHQ_OK) return TAHQ_ERR_CUDA;
+    if (launch_select(a, d, st) != TAHQ_OK) return TAHQ_ERR_CUDA;
   }
   const bool narrow = a.lo + a.mixed <= 4u;   // no width above 4 bits: the kernel compiled for just that
-  if (pl.fast) {   // widths and offsets come ready from the selection: warps stream units of 32 rows independently
-    constexpr int NQ = 2;
-    const int smem = StreamCfg<C>::smem_bytes(NQ);
-    static std::atomic<int> occ_fast[64], occ_fast_wide[64];
-    const uint64_t n_units = (a.n_tiles * C::LPT + 31) / 32;
-    const int occ = narrow ? prepare(quant2_kernel<C, NQ, SR, true>, kThreads, smem, d, occ_fast)
-                           : prepare(quant2_kernel<C, NQ, SR, false>, kThreads, smem, d, occ_fast_wide);
-    if (!occ) return TAHQ_ERR_CUDA;
-    const unsigned grid = persistent_grid((n_units + kWarps - 1) / kWarps, d, occ);
-    if (narrow)
-      TAHQ_LAUNCH("quant_pack", st, launch_dependent(quant2_kernel<C, NQ, SR, true>, grid, kThreads, smem, st, a, tmap));
-    else
-      TAHQ_LAUNCH("quant_pack", st, launch_dependent(quant2_kernel<C, NQ, SR, false>, grid, kThreads, smem, st, a, tmap));
-    return cudaGetLastError() == cudaSuccess ? TAHQ_OK : TAHQ_ERR_CUDA;
-  }
-  if constexpr (C::LPT == 1) {   // one lane per tile, widths from the scores: prologue with a look-back over the CTAs
-    constexpr int NQ = 2;
-    const int smem = StreamCfg<C>::smem_bytes(NQ);
-    static std::atomic<int> occ_wide[64];
-    const uint64_t n_units = (a.n_tiles + 31) / 32;
-    const int occ = narrow ? prepare(quant_pack_stream_kernel<C, NQ, SR, true>, kThreads, smem, d, occ_quant)
-                           : prepare(quant_pack_stream_kernel<C, NQ, SR, false>, kThreads, smem, d, occ_wide);
-    if (!occ) return TAHQ_ERR_CUDA;
-    const unsigned grid = persistent_grid((n_units + kWarps - 1) / kWarps, d, occ);
-    if (narrow)
-      TAHQ_LAUNCH("quant_pack", st,
-                  launch_dependent(quant_pack_stream_kernel<C, NQ, SR, true>, grid, kThreads, smem, st, a, tmap));
-    else
-      TAHQ_LAUNCH("quant_pack", st,
-                  launch_dependent(quant_pack_stream_kernel<C, NQ, SR, false>, grid, kThreads, smem, st, a, tmap));
-  } else {
-    constexpr int NQ = Stages<C>::QUANT;
-    const int smem = NQ * (C::STAGE_BYTES + C::TPC * 4);
-    const int occ = prepare(quant_pack_kernel<C, NQ, SR>, kThreads, smem, d, occ_quant);
-    if (!occ) return TAHQ_ERR_CUDA;
-    TAHQ_LAUNCH("quant_pack", st,
-                launch_dependent(quant_pack_kernel<C, NQ, SR>, persistent_grid(n_chunks, d, occ), kThreads, smem, st, a));
-  }
+  constexpr int NQ = 2;
+  const int smem = StreamCfg<C>::smem_bytes(NQ);
+  static std::atomic<int> occ_narrow[64], occ_wide[64];
+  const uint64_t n_units = (a.n_tiles * C::LPT + 31) / 32;
+  const int occ = narrow ? prepare(quant2_kernel<C, NQ, SR, true>, kThreads, smem, d, occ_narrow)
+                         : prepare(quant2_kernel<C, NQ, SR, false>, kThreads, smem, d, occ_wide);
+  if (!occ) return TAHQ_ERR_CUDA;
+  const unsigned grid = persistent_grid((n_units + kWarps - 1) / kWarps, d, occ);
+  if (narrow)
+    TAHQ_LAUNCH("quant_pack", st, launch_dependent(quant2_kernel<C, NQ, SR, true>, grid, kThreads, smem, st, a, tmap));
+  else
+    TAHQ_LAUNCH("quant_pack", st, launch_dependent(quant2_kernel<C, NQ, SR, false>, grid, kThreads, smem, st, a, tmap));
   return cudaGetLastError() == cudaSuccess ? TAHQ_OK : TAHQ_ERR_CUDA;
 }
 

@@ -1,29 +1,38 @@
-// Kernels of the TAH-Quant boundary codec (sm_100a) that do not depend on the tile configuration: the
-// exact top-k_hi selection of Sec. 3.2 (select_kernel), the scores of allocation tiles wider than the
-// quantisation tile (alloc_score_kernel), the workspace clear and the self-test of the bounded waits.
-// Compiled once (tahq_common.cu).
+// Sec. 3.2 and 3.4 between scoring and quantise + pack (sm_100a): the exact top-k_hi selection of every ranking group,
+// the bit map and the running count of higher-width tiles; the scores of allocation tiles wider than the quantisation
+// tile; the workspace clear and the self-test of the bounded waits.  Compiled once (tahq_common.cu).
 #pragma once
+
+#include <cooperative_groups.h>
 
 #include "tahq_kernels.cuh"
 
 namespace tahq {
 
-// Self-test of the bounded waits: CTA 1 waits for a count that CTA 0 never publishes.  The wait gives
-// up after kSpinLimit polls, the status word gets TAHQ_DEV_TIMEOUT, and the kernel returns.
-// Clears the part of the workspace that a call needs zeroed (status word, look-back flags, counters,
-// histograms); the call's first tile kernel is launched as its programmatic dependent.
+namespace cg = cooperative_groups;
+
+constexpr int kSelThreads = 512;       // threads per CTA of select_kernel: two CTAs fit on an SM
+constexpr int kClKeys = 4096;          // candidate keys that are ranked in shared memory
+constexpr int kClMaxCtas = 16;
+constexpr int kHeld = 8;               // scores a thread keeps in registers
+constexpr int kCoarse = 64, kFine = kBins / kCoarse;
+
+
+// Zeroes 16-byte pieces; the call's first tile kernel is launched as its programmatic dependent.
 __global__ void __launch_bounds__(kThreads) clear_kernel(uint4 *p, uint64_t n16, unsigned long long *trace_buf) {
   TraceScope trace(trace_buf, 0);
+  grid_dependency_wait();
   for (uint64_t i = blockIdx.x * (uint64_t)kThreads + threadIdx.x; i < n16; i += (uint64_t)gridDim.x * kThreads)
     p[i] = make_uint4(0, 0, 0, 0);
 }
 
+// Self-test of the bounded waits: CTA 1 waits for a count that CTA 0 never publishes.  The wait gives
+// up after kSpinLimit polls, the status word gets TAHQ_DEV_TIMEOUT, and the kernel returns.
 __global__ void __launch_bounds__(kThreads) wait_selftest_kernel(const Args a) {
   if (blockIdx.x == 0) return;
   bool unused;
   cta_exclusive_prefix(a, 1, false, unused);
 }
-
 
 // ------------------------------------------------------------------------------------------
 // Eq. 1-2 over allocation tiles wider than the quantisation tile (Sec. 3.2, A = m * G, up to 8192
@@ -79,7 +88,10 @@ __global__ void __launch_bounds__(kThreads) alloc_score_kernel(const Args a) {
   const uint64_t n_warps = ((uint64_t)gridDim.x * kThreads) >> 5;
   const uint32_t A = a.alloc_m * a.tile, n_oct = A / 8;
   const uint64_t n_alloc = a.n_tiles / a.alloc_m;
+  TraceScope trace(a.trace, 1);
   grid_dependency_wait();
+  trace.started();
+  clear_bitmap(a);
   for (uint64_t t = warp; t < n_alloc; t += n_warps) {
     const uint8_t *base = a.in + t * (uint64_t)A * (BF16 ? 2 : 4);
     const float L1 = alloc_tree<BF16>(base, n_oct, lane, [](float m) { return m; });
@@ -89,15 +101,31 @@ __global__ void __launch_bounds__(kThreads) alloc_score_kernel(const Args a) {
       return p * lg2_fma(p + a.eps_log);
     });
     if (lane == 0) {
-      const float sc = 0.0f - S;
-      a.scores[t] = sc;
-      if (!a.direct) atomicAdd(a.hist + (t / a.rank_per_group) * kBins + score_bin(sc), 1u);
+      a.scores[t] = 0.0f - S;
     }
   }
 }
 
 // ------------------------------------------------------------------------------------------
-// Sec. 3.2: exact top-k_hi per ranking group -> theta[g], the ranking key of the k_hi-th tile
+// Sec. 3.2: exact top-k_hi per ranking group.  One thread-block cluster of up to 16 CTAs per group, a slice of the
+// group's scores to each CTA; what the CTAs have to tell each other -- histogram columns, candidate keys, counts --
+// travels through distributed shared memory between two cluster barriers.
+//
+//   1  every CTA bins its scores, fine (4096 bins) and coarse (64)
+//   2  after the first barrier every CTA reads the cluster's coarse counts, finds the coarse bin of the k_hi-th ranked
+//      tile, reads the 64 fine counts inside it and has the threshold bin B
+//   3  tiles well above / below bin B are decided: the bits of those above are the first version of the slice's
+//      words.  The few inside the band are listed and get their exact score (8 lanes per tile of 64, straight from the
+//      tensor, all in flight together); their ranking keys are stored into every CTA's copy of the key list (slots
+//      handed out by the first CTA's counter)
+//   4  after the second barrier every CTA ranks its copy of the list for itself, counts the band tiles of earlier
+//      slices that made it and sets the bits of its own
+//   5  the words of the slice leave as words of the bit map with their running counts.  A ranking group may start
+//      anywhere in a word and a ranked tile may stand for several quantisation tiles (A > G): words that two slices
+//      share are put together by atomicOr on zeroed memory.
+//
+// If there are more candidates than the list holds (thousands of near-equal scores) the cluster runs a radix selection
+// over the slices instead (selection_by_radix).
 // ------------------------------------------------------------------------------------------
 
 // r-th largest (1-based) key of a sequence, radix select with 8 bits a pass.  get(i, key) returns
@@ -166,362 +194,511 @@ __device__ __forceinline__ unsigned long long radix_select(uint64_t count, uint3
   return prefix;
 }
 
-// Screening scores differ from exact ones by less than kScreenErr = 1e-4 (see tile_score_screen); the
-// band around the threshold bin reaches 0.25 bin = 4.9e-4 beyond it on each side (kBinScale bins per unit
-// of score), more than twice that error.
-constexpr float kScreenBand = 0.25f;
-
-// Higher-width tiles before every unit of 32 tiles of one ranking group (Sec. 3.4: the offsets of the codes):
-// pre[u] = base + set bits in the words before word u.  The words are in global memory, written by other CTAs
-// or patched by atomics just before: they are read through L2.  Called by one whole CTA of kSelThreads threads.
-__device__ __forceinline__ void scan_group_words(const uint32_t *words, uint32_t n_words, uint32_t base, uint32_t *pre) {
-  __shared__ uint32_t s_ws[kSelThreads / 32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint32_t carry = base;
-  for (uint32_t w0 = 0; w0 < n_words; w0 += 4 * kSelThreads) {
-    const uint32_t i = w0 + 4 * threadIdx.x;
-    uint32_t c[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) c[j] = i + j < n_words ? (uint32_t)__popc(__ldcg(words + i + j)) : 0u;
-    const uint32_t mine = c[0] + c[1] + c[2] + c[3];
-    uint32_t incl = mine;
-#pragma unroll
-    for (int o = 1; o < 32; o *= 2) {
-      const uint32_t v = __shfl_up_sync(kFull, incl, o);
-      if (lane >= o) incl += v;
-    }
-    if (lane == 31) s_ws[warp] = incl;
-    __syncthreads();
-    uint32_t before = carry + incl - mine, total = 0;
-#pragma unroll
-    for (int w = 0; w < kSelThreads / 32; ++w) {
-      const uint32_t v = s_ws[w];
-      before += w < warp ? v : 0u;
-      total += v;
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      if (i + j < n_words) pre[i + j] = before;
-      before += c[j];
-    }
-    carry += total;
-    __syncthreads();
-  }
+// exact score of tile `tp` by the NOCT lanes that share it (all 32 lanes of the warp call this)
+__device__ __forceinline__ float exact_score_any(const uint8_t *tp, uint32_t noct, bool bf16, uint32_t sub, float eps_l1,
+                                                 float eps_log) {
+  if (bf16)
+    return noct == 1   ? exact_score_coop<1, true>(tp, sub, eps_l1, eps_log)
+           : noct == 2 ? exact_score_coop<2, true>(tp, sub, eps_l1, eps_log)
+           : noct == 4 ? exact_score_coop<4, true>(tp, sub, eps_l1, eps_log)
+           : noct == 8 ? exact_score_coop<8, true>(tp, sub, eps_l1, eps_log)
+                       : exact_score_coop<16, true>(tp, sub, eps_l1, eps_log);
+  return noct == 1   ? exact_score_coop<1, false>(tp, sub, eps_l1, eps_log)
+         : noct == 2 ? exact_score_coop<2, false>(tp, sub, eps_l1, eps_log)
+         : noct == 4 ? exact_score_coop<4, false>(tp, sub, eps_l1, eps_log)
+         : noct == 8 ? exact_score_coop<8, false>(tp, sub, eps_l1, eps_log)
+                     : exact_score_coop<16, false>(tp, sub, eps_l1, eps_log);
 }
 
-__global__ void __launch_bounds__(kSelThreads) select_kernel(const Args a) {
-  extern __shared__ __align__(16) unsigned long long s_keys[];   // kSortCap keys
-  __shared__ uint32_t s_warp[kSelThreads / 32];
-  __shared__ uint32_t s_sel[2];
-  __shared__ uint32_t s_last;
-  const uint64_t g = blockIdx.x / a.cpg;
-  const uint64_t ng = a.rank_per_group;
-  const float *sc = a.scores + g * ng;
+// r-th largest of n distinct keys in shared memory (n <= kClKeys), the same value returned to every thread: they go
+// into kSelThreads buckets by score first and only the bucket that holds rank r is counted; thousands of equal scores
+// fall through to the radix selection.
+__device__ __noinline__ unsigned long long rank_keys_shared(unsigned long long *s_keys, uint32_t n, uint32_t r,
+                                                               unsigned long long *s_few /* kSelThreads */) {
+  __shared__ unsigned long long s_ans;
+  __shared__ uint32_t s_cnt[kSelThreads];
+  __shared__ uint32_t s_sub[kSelThreads];
+  __shared__ uint32_t s_wsum[kSelThreads / 32];
+  __shared__ uint32_t s_lo, s_hi, s_nsub, s_pick[2];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  auto from_smem = [&](uint64_t i, unsigned long long &key) { key = s_keys[i]; return true; };
-  TraceScope trace(a.trace, 2);
-  grid_dependency_wait();   // scores and histograms are the score kernel's
-  trace.started();
-
-  if (a.direct) {   // small group: rank all of its tiles here (one CTA per group)
-    for (uint32_t i = threadIdx.x; i < (uint32_t)ng; i += kSelThreads) s_keys[i] = rank_key(sc[i], i);
-    __syncthreads();
-    const unsigned long long t = radix_select(ng, (uint32_t)a.rank_k, from_smem);
-    if (threadIdx.x == 0) a.theta[g] = t;
-    if (a.fast) {   // the group's bit-map words (Sec. 3.2) and the offsets' running count (Sec. 3.4), ready for the encoder
-      if (blockIdx.x == 0 && threadIdx.x == 0) *a.epoch = *a.epoch + 1ull;   // this call's tag is used up
-      uint32_t *words = reinterpret_cast<uint32_t *>(a.packed + a.off_bitmap) + g * (ng / 32);
-      for (uint32_t i = threadIdx.x; i < (uint32_t)ng; i += kSelThreads) {
-        const unsigned m = __ballot_sync(kFull, s_keys[i] >= t);
-        if (lane == 0) words[i >> 5] = m;
-      }
-      __threadfence();
-      __syncthreads();
-      scan_group_words(words, (uint32_t)(ng / 32), (uint32_t)(g * a.k_hi), a.pre + g * (ng / 32));
+  if (threadIdx.x == 0) { s_ans = ~0ull; s_lo = 0xffffffffu; s_hi = 0; s_nsub = 0; s_pick[0] = 0; s_pick[1] = 0; }
+  s_cnt[threadIdx.x] = 0;
+  __syncthreads();
+  {   // the scores, mapped to unsigned integers of the same order: smallest and largest
+    uint32_t mn = 0xffffffffu, mx = 0;
+    for (uint32_t i = threadIdx.x; i < n; i += kSelThreads) {
+      const uint32_t m = (uint32_t)(s_keys[i] >> 32);
+      mn = m < mn ? m : mn;
+      mx = m > mx ? m : mx;
     }
-    return;
-  }
-  if (a.fast && blockIdx.x == 0 && threadIdx.x == 0) *a.epoch = *a.epoch + 1ull;   // this call's tag is used up
-  uint32_t *const words = reinterpret_cast<uint32_t *>(a.packed + a.off_bitmap) + g * (ng / 32);   // (a.fast)
-
-  // this CTA's first slice of the group's scores, in flight while the threshold bin is being found
-  const uint64_t lo0 = (blockIdx.x % a.cpg) * (uint64_t)a.sel_m * kSelSlice;
-  float sv[4];
 #pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const uint64_t i = lo0 + (uint64_t)u * kSelThreads + threadIdx.x;
-    sv[u] = i < ng ? __ldg(sc + i) : 0.0f;
+    for (int o = 16; o > 0; o >>= 1) {
+      const uint32_t v = __shfl_xor_sync(kFull, mn, o), w = __shfl_xor_sync(kFull, mx, o);
+      mn = v < mn ? v : mn;
+      mx = w > mx ? w : mx;
+    }
+    if (lane == 0) { atomicMin(&s_lo, mn); atomicMax(&s_hi, mx); }
   }
-
-  // ---- A: the bin that holds the k_hi-th ranked tile (every CTA of the group finds it for itself)
-  const uint32_t *gh = a.hist + g * kBins;
-  constexpr int BPT = kBins / kSelThreads;
-  uint32_t hb[BPT], mine = 0;
+  __syncthreads();
+  const uint32_t lo_m = s_lo, span = s_hi - s_lo;
+  // (a multiplication in binary32 instead of a 64-bit division per key: rounding keeps the map non-decreasing,
+  // which is all the buckets need)
+  const float per_bucket = span ? (float)(kSelThreads - 1) / (float)span : 0.0f;
+  auto bucket_of = [&](unsigned long long key) {
+    const uint32_t b = (uint32_t)((float)((uint32_t)(key >> 32) - lo_m) * per_bucket);
+    return b < (uint32_t)kSelThreads - 1u ? b : (uint32_t)kSelThreads - 1u;
+  };
+  for (uint32_t i = threadIdx.x; i < n; i += kSelThreads) atomicAdd(&s_cnt[bucket_of(s_keys[i])], 1u);
+  __syncthreads();
+  {   // keys in the buckets above this thread's bucket (one bucket per thread)
+    const uint32_t c = s_cnt[threadIdx.x];
+    uint32_t incl = c;
 #pragma unroll
-  for (int j = 0; j < BPT; ++j) { hb[j] = gh[threadIdx.x * BPT + j]; mine += hb[j]; }
-  uint32_t incl = mine;   // suffix sums: tiles in bins above this thread's bins
+    for (int o = 1; o < 32; o *= 2) {
+      const uint32_t v = __shfl_down_sync(kFull, incl, o);
+      if (lane + o < 32) incl += v;
+    }
+    if (lane == 0) s_wsum[warp] = incl;
+    __syncthreads();
+    uint32_t above = incl - c;
+    for (int w = warp + 1; w < kSelThreads / 32; ++w) above += s_wsum[w];
+    if (above < r && above + c >= r) { s_pick[0] = threadIdx.x; s_pick[1] = r - above; }
+  }
+  __syncthreads();
+  const uint32_t bsel = s_pick[0], rsel = s_pick[1];
+  if (rsel != 0 && s_cnt[bsel] <= (uint32_t)kSelThreads) {
+    for (uint32_t i = threadIdx.x; i < n; i += kSelThreads)
+      if (bucket_of(s_keys[i]) == bsel) s_sub[atomicAdd(&s_nsub, 1u)] = i;
+    __syncthreads();
+    const uint32_t ns = s_nsub;
+    const unsigned long long mine = threadIdx.x < ns ? s_keys[s_sub[threadIdx.x]] : 0ull;
+    if (threadIdx.x < ns) s_few[threadIdx.x] = mine;
+    __syncthreads();
+    if (threadIdx.x < ns) {
+      uint32_t larger = 0;
+      for (uint32_t i = 0; i < ns; ++i) larger += s_few[i] > mine ? 1u : 0u;
+      if (larger == rsel - 1) s_ans = mine;
+    }
+    __syncthreads();
+    return s_ans;
+  }
+  // thousands of equal scores: digit by digit
+  return radix_select(n, r, [&](uint64_t i, unsigned long long &key) { key = s_keys[i]; return true; });
+}
+
+struct SelShared {
+  uint32_t part[kClMaxCtas];     // tiles above the band in each CTA's slice
+  uint32_t tot[kClMaxCtas];      // (radix) set bits in each CTA's words
+  uint32_t n_keys;               // (first CTA) list slots handed out so far
+  uint32_t n_total;              // candidates of the whole cluster (every CTA is told)
+  uint32_t digit_pick[2];        // radix selection: chosen digit, remaining rank
+};
+
+// A score on the axis of the bins, in steps, 16 to a bin (non-decreasing in the score; not yet cut to whole steps).  Scores
+// lie in [0, log2 A]; three quarters of the bins are given to the top two units, where most tiles and the threshold are:
+// with bins of one width a threshold in the dense part had 2.6 times as many candidates.
+struct StepMap { float lo, hi, off; };   // max(s * lo, s * hi - off)
+__device__ __forceinline__ float score_pos(float s, const StepMap &m) { return fmaxf(s * m.lo, __fmaf_rn(s, m.hi, -m.off)); }
+__device__ __forceinline__ int score_step(float s, const StepMap &m) {
+  return (int)fminf(fmaxf(score_pos(s, m), 0.0f), (float)(16 * kBins - 1));
+}
+// Screening scores differ from exact ones by less than 1e-4 (see tile_score_screen), 2.5 steps at most.  With k_hi-th largest
+// screening score in bin B, a tile whose screening score lies more than twice that outside bin B is certainly inside or
+// outside the top k_hi; six steps also cover the cut to whole steps.
+constexpr int kScreenBand = 6;
+
+// More candidates than the key list holds: the band's tiles get their exact score in place (decided ones +-infinity), and
+// a radix selection over the finite scores of all slices, 8 bits a pass, gives the threshold key; every CTA sums the
+// cluster's digit counts for itself.  Sets the slice's words and returns the higher-width tiles of the slices before
+// it.  (Out of line: the usual path runs once per launch from a cold instruction cache and stays compact.)
+__device__ __noinline__ uint32_t selection_by_radix(const Args &a, float *sc, const uint8_t *tiles, uint32_t tile_bytes, uint32_t n_loc,
+                                                    uint32_t i0, int lo_v, int hi_v, uint32_t rr, uint32_t *words,
+                                                    uint32_t *s_digit, uint32_t *s_red, SelShared &sh) {
+  cg::cluster_group cl = cg::this_cluster();
+  const uint32_t CS = cl.num_blocks(), rank = cl.block_rank();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t noct = a.tile / 8, per = 32u / noct, sub = (uint32_t)lane % noct, grp = (uint32_t)lane / noct;
+  for (uint32_t c0 = (uint32_t)warp * 32u; c0 < n_loc; c0 += kSelThreads) {
+    const uint32_t i = c0 + lane;
+    const float s = i < n_loc ? sc[i] : 0.0f;
+    const int v = score_step(s, {a.step_lo, a.step_hi, a.step_off});
+    const bool cand = i < n_loc && v >= lo_v && v < hi_v;
+    if (i < n_loc && !cand) sc[i] = __int_as_float(v >= hi_v ? 0x7f800000 : (int)0xff800000);
+    unsigned m = __ballot_sync(kFull, cand);
+    if (a.exact_scores) continue;
+    const uint32_t n = (uint32_t)__popc(m);
+    for (uint32_t q = 0; q < n; q += per) {
+      const bool live = q + grp < n;
+      const uint32_t b = __fns(m, 0, (int)(live ? q + grp : 0u) + 1);
+      const float ex = exact_score_any(tiles + (uint64_t)(c0 + b) * tile_bytes, noct, a.bf16 != 0, sub, a.eps_l1, a.eps_log);
+      if (live && sub == 0) sc[c0 + b] = ex;
+    }
+  }
+  __threadfence_block();
+  unsigned long long prefix = 0, mask = 0;
+  uint32_t r = rr;
+  for (int shift = 56; shift >= 0; shift -= 8) {
+    if (threadIdx.x < 256) s_digit[threadIdx.x] = 0;
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < n_loc; i += kSelThreads) {
+      const float s = __ldcg(sc + i);
+      if ((__float_as_uint(s) & 0x7f800000u) != 0x7f800000u) {
+        const unsigned long long key = rank_key(s, i0 + i);
+        if ((key & mask) == prefix) atomicAdd(&s_digit[(unsigned)(key >> shift) & 255u], 1u);
+      }
+    }
+    cl.sync();
+    uint32_t cnt = 0;   // thread d < 256: keys of the cluster with digit d
+    if (threadIdx.x < 256)
+      for (uint32_t q = 0; q < CS; ++q) cnt += cl.map_shared_rank(s_digit, q)[threadIdx.x];
+    uint32_t incl = cnt;   // keys with a larger digit: suffix scan over the 256 counts (warps 0..7)
+#pragma unroll
+    for (int o = 1; o < 32; o *= 2) {
+      const uint32_t v = __shfl_down_sync(kFull, incl, o);
+      if (lane + o < 32) incl += v;
+    }
+    if (lane == 0 && warp < 8) s_red[warp] = incl;
+    __syncthreads();
+    if (threadIdx.x < 256) {
+      uint32_t above = incl - cnt;
+      for (int w = warp + 1; w < 8; ++w) above += s_red[w];
+      if (above < r && above + cnt >= r) { sh.digit_pick[0] = threadIdx.x; sh.digit_pick[1] = r - above; }
+    }
+    cl.sync();   // everybody has read everybody's counts (they are cleared next pass) and made the pick
+    prefix |= (unsigned long long)sh.digit_pick[0] << shift;
+    mask |= 0xffull << shift;
+    r = sh.digit_pick[1];
+  }
+  // every tile against the threshold; the slices' counts have to be exchanged
+  uint32_t bits_here = 0;
+  for (uint32_t c0 = (uint32_t)warp * 32u; c0 < n_loc; c0 += kSelThreads) {
+    const uint32_t i = c0 + lane;
+    const unsigned m = __ballot_sync(kFull, i < n_loc && rank_key(__ldcg(sc + i), i0 + i) >= prefix);   // +inf is above every threshold
+    if (lane == 0) { words[c0 >> 5] = m; bits_here += (uint32_t)__popc(m); }
+  }
+  __syncthreads();
+  if (lane == 0) s_red[warp] = bits_here;
+  __syncthreads();
+  if (threadIdx.x < CS) {
+    uint32_t T = 0;
+    for (int w = 0; w < kSelThreads / 32; ++w) T += s_red[w];
+    cl.map_shared_rank(&sh, threadIdx.x)->tot[rank] = T;
+  }
+  cl.sync();
+  uint32_t before = 0;
+  for (uint32_t q = 0; q < rank; ++q) before += sh.tot[q];
+  cl.sync();   // nobody leaves while its memory may still be written
+  return before;
+}
+
+// The bin among n ascending counts, held `per` to a lane by one warp, that holds the k-th largest, and the rank inside it.
+template <int PER>
+__device__ __forceinline__ void find_bin(const uint32_t (&c)[PER], uint32_t k, uint32_t &bin, uint32_t &rank_in) {
+  const int lane = threadIdx.x & 31;
+  uint32_t mine = 0;
+#pragma unroll
+  for (int j = 0; j < PER; ++j) mine += c[j];
+  uint32_t incl = mine;   // counts in this lane's bins and higher
 #pragma unroll
   for (int o = 1; o < 32; o *= 2) {
     const uint32_t v = __shfl_down_sync(kFull, incl, o);
     if (lane + o < 32) incl += v;
   }
-  if (lane == 0) s_warp[warp] = incl;
-  __syncthreads();
-  uint32_t above = incl - mine;
-  for (int w = warp + 1; w < kSelThreads / 32; ++w) above += s_warp[w];
-  const uint32_t k = (uint32_t)a.rank_k;
-  if (above < k && above + mine >= k) {
+  uint32_t above = incl - mine, b = 0, r = 0;
+  const bool here = above < k && incl >= k;
 #pragma unroll
-    for (int j = BPT - 1; j >= 0; --j) {
-      if (above < k && above + hb[j] >= k) { s_sel[0] = threadIdx.x * BPT + j; s_sel[1] = k - above; }
-      above += hb[j];
+  for (int j = PER - 1; j >= 0; --j) {
+    if (above < k && above + c[j] >= k) { b = (uint32_t)(lane * PER + j); r = k - above; }
+    above += c[j];
+  }
+  const unsigned m = __ballot_sync(kFull, here);
+  const int src = m ? __ffs(m) - 1 : 0;   // (always found: k_hi is at most the number of tiles)
+  bin = __shfl_sync(kFull, b, src);
+  rank_in = __shfl_sync(kFull, r, src);
+}
+
+// HELD: a thread's scores stay in registers between binning and deciding (slices of up to kHeld * kSelThreads);
+// longer slices are read again, from L2.
+template <bool HELD>
+__global__ void __launch_bounds__(kSelThreads, 2) select_kernel(const __grid_constant__ Args a, const uint32_t per_cta) {
+  constexpr int NW = kSelThreads / 32;
+  cg::cluster_group cl = cg::this_cluster();
+  const uint32_t CS = cl.num_blocks(), rank = cl.block_rank();
+  const uint64_t g = blockIdx.x / CS;
+  const uint32_t ng = (uint32_t)a.rank_per_group, k = (uint32_t)a.rank_k;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const StepMap map = {a.step_lo, a.step_hi, a.step_off};
+  extern __shared__ __align__(16) uint8_t smem_sel[];
+  unsigned long long *s_keys = reinterpret_cast<unsigned long long *>(smem_sel);        // [kClKeys + kSelThreads]
+  uint32_t *s_hist = reinterpret_cast<uint32_t *>(s_keys + kClKeys + kSelThreads);      // [kBins]; later the words' running counts
+  uint32_t *s_cand = s_hist + kBins;                                                    // [kClKeys] band tiles of the slice
+  uint32_t *s_words = s_cand + kClKeys;                                                 // [kWordsShared]
+  __shared__ SelShared sh;
+  __shared__ uint32_t s_coarse[256];          // the CTA's coarse counts [kCoarse]; (radix) digit counts
+  __shared__ __align__(8) uint32_t s_sum[2][kCoarse];   // the cluster's coarse counts; its fine counts in the chosen coarse bin
+  __shared__ uint32_t s_red[32];
+  __shared__ uint32_t s_ncand, s_nabove, s_base, s_made;
+  TraceScope trace(a.trace, 2);
+
+  const uint32_t i0 = rank * per_cta;                                   // first tile of the slice, inside the group
+  const uint32_t n_loc = i0 < ng ? (ng - i0 < per_cta ? ng - i0 : per_cta) : 0u;
+  const uint32_t n_words = (n_loc + 31u) / 32u, n_it = (n_loc + 4 * kSelThreads - 1) / (4 * kSelThreads);
+  // the slice's words (and running counts): in shared memory, or in the workspace when the slice is very long
+  const bool in_smem = per_cta <= 32u * kWordsShared;
+  uint32_t *words = s_words, *wpre = s_hist;
+  if (!in_smem) {
+    words = a.words + g * 2ull * ((ng + 31u) / 32u + kClMaxCtas) + 2ull * (i0 / 32u);
+    wpre = words + n_words;
+  }
+  for (uint32_t b = threadIdx.x; b < (uint32_t)kBins; b += kSelThreads) s_hist[b] = 0;
+  if (threadIdx.x < 2 * kCoarse) s_sum[0][threadIdx.x] = 0;
+  if (threadIdx.x == 0) { sh.n_keys = 0; sh.n_total = 0; s_ncand = 0; s_nabove = 0; s_made = 0; }
+  grid_dependency_wait();   // the scores are the score kernel's
+  trace.started();
+  float *sc = a.scores + g * (uint64_t)ng + i0;
+  // ---- 1: the slice's histogram.  In turn `it` warp w takes 128 tiles from 128 * (it * NW + w) on, a lane four of them.
+  const bool vec = ((reinterpret_cast<uintptr_t>(sc)) & 15u) == 0;
+  auto first_of = [&](uint32_t it) { return (it * NW + (uint32_t)warp) * 128u + (uint32_t)lane * 4u; };
+  auto load4 = [&](uint32_t it) -> float4 {   // -2 behind the slice's end (a score is above -1e-4)
+    const uint32_t i = first_of(it);
+    if (vec && i + 4u <= n_loc) return __ldg(reinterpret_cast<const float4 *>(sc + i));
+    return make_float4(i < n_loc ? __ldg(sc + i) : -2.0f, i + 1u < n_loc ? __ldg(sc + i + 1) : -2.0f,
+                       i + 2u < n_loc ? __ldg(sc + i + 2) : -2.0f, i + 3u < n_loc ? __ldg(sc + i + 3) : -2.0f);
+  };
+  auto bin4 = [&](const float4 &v) {
+    if (v.x > -1.0f) atomicAdd(&s_hist[score_step(v.x, map) >> 4], 1u);
+    if (v.y > -1.0f) atomicAdd(&s_hist[score_step(v.y, map) >> 4], 1u);
+    if (v.z > -1.0f) atomicAdd(&s_hist[score_step(v.z, map) >> 4], 1u);
+    if (v.w > -1.0f) atomicAdd(&s_hist[score_step(v.w, map) >> 4], 1u);
+  };
+  float4 held[kHeld / 4];   // the scores, or (long slices) the first ones
+#pragma unroll
+  for (int it = 0; it < kHeld / 4; ++it) held[it] = load4(it);
+  __syncthreads();
+  if constexpr (HELD) {
+#pragma unroll
+    for (int it = 0; it < kHeld / 4; ++it) bin4(held[it]);
+  } else {
+    for (uint32_t it0 = 0; it0 < n_it; it0 += kHeld / 4) {
+      float4 cur[kHeld / 4];
+#pragma unroll
+      for (int j = 0; j < kHeld / 4; ++j) { cur[j] = held[j]; held[j] = load4(it0 + kHeld / 4 + j); }
+#pragma unroll
+      for (int j = 0; j < kHeld / 4; ++j) bin4(cur[j]);
     }
   }
   __syncthreads();
-  const uint32_t B = s_sel[0], r = s_sel[1];
-
-  // ---- B: the scores so far are screening scores s~ (approximate log2), within kScreenErr of the
-  // exact ones, so the exact k_hi-th largest score lies within kScreenErr of bin B.  Tiles whose s~
-  // is more than 2*kScreenErr above (below) the bin are certainly inside (outside) the top k_hi: their
-  // score is replaced by +inf (-inf).  The rest are candidates: their exact score is recomputed from
-  // the tensor, stored, and ranked exactly in step C.
-  // A CTA takes sel_m consecutive slices (a large tensor still fills the GPU only once, so the chain of
-  // dependent steps above and below is paid once, not once per wave of CTAs).  Candidates collect in the
-  // shared memory that step C uses for its keys; they are re-scored when the next slice might not fit,
-  // and at the end.
-  uint32_t *s_list = reinterpret_cast<uint32_t *>(s_keys);   // index inside the group
-  constexpr uint32_t kListCap = 2 * kSortCap;
-  __shared__ uint32_t s_nlist, s_nabove, s_slot0;
-  if (threadIdx.x == 0) { s_nlist = 0; s_nabove = 0; }
-  __syncthreads();
-  float *scw = a.scores + g * ng;
-  const float band_lo = (float)B - kScreenBand, band_hi = (float)(B + 1) + kScreenBand;
-  const uint32_t tile_bytes = a.tile * (a.bf16 ? 2u : 4u);
-  const uint32_t noct = a.tile / 8, per_round = kSelThreads / noct;
-  const uint32_t sub = threadIdx.x % noct;
-  auto rescore = [&]() {   // called by the whole CTA, after a barrier: s_nlist is settled
-    const uint32_t nl = s_nlist;
-    if (threadIdx.x == 0) s_slot0 = atomicAdd(&a.ncand[g], nl);
-    __syncthreads();
-    const uint32_t slot0 = s_slot0;
-    // candidates, densely over the threads: NOCT = tile/8 neighbouring lanes share one candidate
-    for (uint32_t j0 = 0; j0 < nl; j0 += per_round) {   // uniform trip count: whole warps take part
-      const uint32_t j = j0 + threadIdx.x / noct;
-      const bool live = j < nl;
-      const uint64_t i = s_list[live ? j : 0];
-      const uint8_t *tp = a.in + (g * ng + i) * (uint64_t)tile_bytes;
-      float ex;
-      if (a.exact_scores) {   // nothing to recompute (and with wider allocation tiles tp is not the tile)
-        ex = scw[i];
-      } else if (a.bf16) {
-        ex = noct == 1   ? exact_score_coop<1, true>(tp, sub, a.eps_l1, a.eps_log)
-             : noct == 2 ? exact_score_coop<2, true>(tp, sub, a.eps_l1, a.eps_log)
-             : noct == 4 ? exact_score_coop<4, true>(tp, sub, a.eps_l1, a.eps_log)
-             : noct == 8 ? exact_score_coop<8, true>(tp, sub, a.eps_l1, a.eps_log)
-                         : exact_score_coop<16, true>(tp, sub, a.eps_l1, a.eps_log);
-      } else {
-        ex = noct == 1   ? exact_score_coop<1, false>(tp, sub, a.eps_l1, a.eps_log)
-             : noct == 2 ? exact_score_coop<2, false>(tp, sub, a.eps_l1, a.eps_log)
-             : noct == 4 ? exact_score_coop<4, false>(tp, sub, a.eps_l1, a.eps_log)
-             : noct == 8 ? exact_score_coop<8, false>(tp, sub, a.eps_l1, a.eps_log)
-                         : exact_score_coop<16, false>(tp, sub, a.eps_l1, a.eps_log);
-      }
-      if (live && sub == 0) {
-        scw[i] = ex;
-        if (slot0 + j < a.cand_cap) a.cand[g * a.cand_cap + slot0 + j] = rank_key(ex, (uint32_t)i);
-      }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) s_nlist = 0;
+  {   // eight threads to a coarse bin (turned, so that few lanes meet in a bank)
+    const uint32_t c = threadIdx.x >> 3, j = threadIdx.x & 7u;
+    uint32_t sum = 0;
+#pragma unroll
+    for (uint32_t i = 0; i < 8; ++i) sum += s_hist[c * kFine + j * 8u + ((i + j + 2u * c) & 7u)];
+#pragma unroll
+    for (int o = 1; o < 8; o *= 2) sum += __shfl_xor_sync(kFull, sum, o);
+    if (j == 0) s_coarse[c] = sum;
+  }
+  cl.sync();
+  // ---- 2: the bin of the k_hi-th ranked tile.  Reads of another CTA's shared memory take a few hundred cycles each and
+  // share a narrow path: two per thread here and two below.  What follows them is done by every warp for itself.
+  uint32_t Bc, kin, Bf, unused;
+  auto cluster_sum = [&](const uint32_t *counts, uint32_t *sum) {   // kCoarse counts of every CTA
+    static_assert(kCoarse == 64 && kFine == 64 && kSelThreads == 512 && kClMaxCtas <= 16, "two CTAs to a thread");
+    const uint32_t c = threadIdx.x & 63u, r = threadIdx.x >> 6;
+    uint32_t p = r < CS ? cl.map_shared_rank(counts, r)[c] : 0u;
+    if (r + 8u < CS) p += cl.map_shared_rank(counts, r + 8u)[c];
+    if (p) atomicAdd(&sum[c], p);
     __syncthreads();
   };
-  uint32_t nl_seen = 0;
-  for (uint32_t m = 0; m < a.sel_m; ++m) {
-    const uint64_t lo = lo0 + (uint64_t)m * kSelSlice;
-    if (lo >= ng) break;
-    float nx[4];   // the next slice's scores, in flight while this one is classified
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const uint64_t i = lo + kSelSlice + (uint64_t)u * kSelThreads + threadIdx.x;
-      nx[u] = (m + 1 < a.sel_m && i < ng) ? __ldg(sc + i) : 0.0f;
-    }
-    if (nl_seen + (uint32_t)kSelSlice > kListCap) {   // (the same value in every thread)
-      rescore();
-      nl_seen = 0;
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const uint64_t i = lo + (uint64_t)u * kSelThreads + threadIdx.x;
-      const float t = score_bin_pos(sv[u]);
-      const bool in = i < ng;
-      const bool above = in && t > band_hi, below = in && t < band_lo;
-      if (above) scw[i] = __int_as_float(0x7f800000);
-      if (below) scw[i] = __int_as_float(0xff800000);
-      const unsigned ma = __ballot_sync(kFull, above);
-      if (ma && lane == 0) atomicAdd(&s_nabove, (uint32_t)__popc(ma));
-      if (a.fast && in && lane == 0) words[i >> 5] = ma;   // the bits that are certain; candidates are added below
-      const bool take = in && !above && !below;
-      const unsigned mk = __ballot_sync(kFull, take);
-      if (mk) {
-        uint32_t base = 0;
-        if (lane == 0) base = atomicAdd(&s_nlist, (uint32_t)__popc(mk));
-        base = __shfl_sync(kFull, base, 0);
-        if (take) s_list[base + __popc(mk & ((1u << lane) - 1u))] = (uint32_t)i;
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) sv[u] = nx[u];
-    __syncthreads();       // the slice's candidates are all listed ...
-    nl_seen = s_nlist;
-    __syncthreads();       // ... and counted by everyone before the next slice adds to them
+  cluster_sum(s_coarse, s_sum[0]);
+  {
+    const uint32_t c[2] = {s_sum[0][lane * 2], s_sum[0][lane * 2 + 1]};
+    find_bin<2>(c, k, Bc, kin);
   }
-  if (threadIdx.x == 0 && s_nabove) atomicAdd(&a.nabove[g], s_nabove);
-  rescore();
-
-  // ---- C: the CTA that finishes the group last ranks the candidates exactly
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(&a.done[g], 1u) == a.cpg - 1;
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  const uint32_t n = *reinterpret_cast<volatile uint32_t *>(a.ncand + g);
-  const uint32_t nab = *reinterpret_cast<volatile uint32_t *>(a.nabove + g);
-  uint32_t rr = (uint32_t)a.rank_k - nab;   // rank of the threshold tile among the candidates
-  __shared__ unsigned long long s_theta;
-  if (threadIdx.x == 0) s_theta = ~0ull;
-  __syncthreads();
-  bool listed = n <= a.cand_cap;   // the candidates are all in the list (the usual case)
-  if (nab >= (uint32_t)a.rank_k || rr > n) {   // only possible if the screening error exceeded its bound
-    if (threadIdx.x == 0) atomicOr(a.status, 8u /* TAHQ_DEV_INTERNAL */);
-    rr = rr > n ? n : 1u;
+  cluster_sum(s_hist + Bc * kFine, s_sum[1]);
+  {
+    const uint32_t c[2] = {s_sum[1][lane * 2], s_sum[1][lane * 2 + 1]};
+    find_bin<2>(c, kin, Bf, unused);
   }
-  (void)r;
-  const unsigned long long *cand = a.cand + g * a.cand_cap;
-  if (n == 0) {
-    // nothing to rank (only after a violated bound): the threshold stays above every key
-  } else if (listed) {
-    // Up to kSortCap - kSelThreads candidates are copied to shared memory.  A handful are ranked by counting, for
-    // every key, the larger ones.  More (a threshold in the dense part of the scores: hundreds to thousands per
-    // group) first go into kSelThreads buckets by score, spread evenly between the smallest and the largest; the
-    // bucket that holds rank rr is found by a suffix sum and only its few keys are counted against each other.
-    const bool in_smem = n <= (uint32_t)(kSortCap - kSelThreads);
-    if (in_smem) {
-      for (uint32_t i = threadIdx.x; i < n; i += kSelThreads) s_keys[i] = __ldcg(cand + i);
-      __syncthreads();
-    }
-    auto key_at = [&](uint32_t i) { return in_smem ? s_keys[i] : __ldcg(cand + i); };
-    if (n <= 64u) {
-      if (threadIdx.x < n) {
-        const unsigned long long mine = s_keys[threadIdx.x];
-        uint32_t larger = 0;
-        for (uint32_t i = 0; i < n; ++i) larger += s_keys[i] > mine ? 1u : 0u;
-        if (larger == rr - 1) s_theta = mine;   // keys are distinct: exactly one thread
-      }
-    } else {
-      __shared__ uint32_t s_cnt[kSelThreads];   // keys per bucket
-      __shared__ uint32_t s_sub[kSelThreads];   // the keys (their indices) of the bucket that holds rank rr
-      __shared__ uint32_t s_lo, s_hi, s_nsub;
-      if (threadIdx.x == 0) { s_lo = 0xffffffffu; s_hi = 0; s_nsub = 0; s_sel[0] = 0; s_sel[1] = 0; }
-      s_cnt[threadIdx.x] = 0;
-      __syncthreads();
-      {   // the scores, mapped to unsigned integers of the same order: smallest and largest
-        uint32_t mn = 0xffffffffu, mx = 0;
-        for (uint32_t i = threadIdx.x; i < n; i += kSelThreads) {
-          const uint32_t m = (uint32_t)(key_at(i) >> 32);
-          mn = m < mn ? m : mn;
-          mx = m > mx ? m : mx;
-        }
+  // ---- 3: decide what is certain; list the band's tiles
+  const int B = (int)(Bc * kFine + Bf), band = a.exact_scores ? 0 : kScreenBand;
+  const int lo_v = B * 16 - band, hi_v = (B + 1) * 16 + band;
+  {
+    // step(s) >= v for a whole v is score_pos(s) >= v; the last bin has nothing above it
+    const float lo_f = (float)lo_v, hi_f = hi_v > 16 * kBins - 1 ? __int_as_float(0x7f800000) : (float)hi_v;
+    uint32_t n_above = 0;
+    auto decide = [&](uint32_t it, const float4 &v) {
+      const float t[4] = {score_pos(v.x, map), score_pos(v.y, map), score_pos(v.z, map), score_pos(v.w, map)};
+      const float e[4] = {v.x, v.y, v.z, v.w};
+      uint32_t above = 0, cand = 0;   // of the lane's four tiles
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          const uint32_t v = __shfl_xor_sync(kFull, mn, o), w = __shfl_xor_sync(kFull, mx, o);
-          mn = v < mn ? v : mn;
-          mx = w > mx ? w : mx;
-        }
-        if (lane == 0) { atomicMin(&s_lo, mn); atomicMax(&s_hi, mx); }
+      for (int j = 0; j < 4; ++j) {
+        above |= t[j] >= hi_f ? 1u << j : 0u;
+        cand |= (e[j] > -1.0f && !(t[j] >= hi_f) && !(t[j] < lo_f)) ? 1u << j : 0u;
       }
-      __syncthreads();
-      const uint32_t lo_m = s_lo, span = s_hi - s_lo;
-      // (a multiplication in binary32 instead of a 64-bit division per key: rounding keeps the map non-decreasing,
-      // which is all the buckets need)
-      const float per_bucket = span ? (float)(kSelThreads - 1) / (float)span : 0.0f;
-      auto bucket_of = [&](unsigned long long key) {
-        const uint32_t b = (uint32_t)((float)((uint32_t)(key >> 32) - lo_m) * per_bucket);
-        return b < (uint32_t)kSelThreads - 1u ? b : (uint32_t)kSelThreads - 1u;
-      };
-      for (uint32_t i = threadIdx.x; i < n; i += kSelThreads) atomicAdd(&s_cnt[bucket_of(key_at(i))], 1u);
-      __syncthreads();
-      {   // keys in the buckets above this thread's bucket (one bucket per thread)
-        const uint32_t c = s_cnt[threadIdx.x];
-        uint32_t incl = c;
+      // eight lanes hold a word
+      uint32_t word = above << (4 * (lane & 7));
+#pragma unroll
+      for (int o = 1; o < 8; o *= 2) word |= __shfl_xor_sync(kFull, word, o);
+      const uint32_t w = (it * NW + (uint32_t)warp) * 4u + (uint32_t)(lane >> 3);
+      if ((lane & 7) == 0 && w < n_words) words[w] = word;   // the bits that are certain; the band's winners are added in step 4
+      n_above += (uint32_t)__popc(above);
+      if (__any_sync(kFull, cand != 0u)) {
+        const uint32_t mine = (uint32_t)__popc(cand);
+        uint32_t incl = mine;
 #pragma unroll
         for (int o = 1; o < 32; o *= 2) {
-          const uint32_t v = __shfl_down_sync(kFull, incl, o);
-          if (lane + o < 32) incl += v;
+          const uint32_t x = __shfl_up_sync(kFull, incl, o);
+          if (lane >= o) incl += x;
         }
-        if (lane == 0) s_warp[warp] = incl;
-        __syncthreads();
-        uint32_t above = incl - c;
-        for (int w = warp + 1; w < kSelThreads / 32; ++w) above += s_warp[w];
-        if (above < rr && above + c >= rr) { s_sel[0] = threadIdx.x; s_sel[1] = rr - above; }
+        uint32_t base = 0;
+        if (lane == 31) base = atomicAdd(&s_ncand, incl);
+        uint32_t slot = __shfl_sync(kFull, base, 31) + incl - mine;
+        const uint32_t i = first_of(it);
+        for (uint32_t m = cand; m; m &= m - 1u, ++slot)
+          if (slot < (uint32_t)kClKeys) s_cand[slot] = i + (uint32_t)__ffs(m) - 1u;
       }
-      __syncthreads();
-      const uint32_t bsel = s_sel[0], rsel = s_sel[1];
-      if (rsel != 0 && s_cnt[bsel] <= (uint32_t)kSelThreads) {
-        for (uint32_t i = threadIdx.x; i < n; i += kSelThreads)
-          if (bucket_of(key_at(i)) == bsel) s_sub[atomicAdd(&s_nsub, 1u)] = i;
-        __syncthreads();
-        const uint32_t ns = s_nsub;
-        unsigned long long *s_few = s_keys + kSortCap - kSelThreads;   // the bucket's keys, behind the copied ones
-        const unsigned long long mine = threadIdx.x < ns ? key_at(s_sub[threadIdx.x]) : 0ull;
-        if (threadIdx.x < ns) s_few[threadIdx.x] = mine;
-        __syncthreads();
-        if (threadIdx.x < ns) {
-          uint32_t larger = 0;
-          for (uint32_t i = 0; i < ns; ++i) larger += s_few[i] > mine ? 1u : 0u;
-          if (larger == rsel - 1) s_theta = mine;   // keys are distinct: exactly one thread
-        }
-      } else {   // thousands of equal scores: bit by bit
-        unsigned long long t;
-        if (in_smem) t = radix_select(n, rr, from_smem);
-        else t = radix_select(n, rr, [&](uint64_t i, unsigned long long &key) {
-          key = __ldcg(cand + i);
-          return true;
-        });
-        if (threadIdx.x == 0) s_theta = t;
+    };
+    if constexpr (HELD) {
+#pragma unroll
+      for (int it = 0; it < kHeld / 4; ++it)
+        if ((uint32_t)it < n_it) decide(it, held[it]);
+    } else {
+#pragma unroll
+      for (int it = 0; it < kHeld / 4; ++it) held[it] = load4(it);
+      for (uint32_t it0 = 0; it0 < n_it; it0 += kHeld / 4) {
+        float4 cur[kHeld / 4];
+#pragma unroll
+        for (int j = 0; j < kHeld / 4; ++j) { cur[j] = held[j]; held[j] = load4(it0 + kHeld / 4 + j); }
+#pragma unroll
+        for (int j = 0; j < kHeld / 4; ++j)
+          if (it0 + j < n_it) decide(it0 + j, cur[j]);
       }
     }
-  } else {   // more candidates than the list holds: they are exactly the tiles whose stored score is finite
-    const unsigned long long t = radix_select(ng, rr, [&](uint64_t i, unsigned long long &key) {
-      const float s = __ldcg(scw + i);
-      key = rank_key(s, (uint32_t)i);
-      return (__float_as_uint(s) & 0x7f800000u) != 0x7f800000u;
-    });
-    if (threadIdx.x == 0) s_theta = t;
+    n_above = __reduce_add_sync(kFull, n_above);
+    if (lane == 0 && n_above) atomicAdd(&s_nabove, n_above);
   }
   __syncthreads();
-  const unsigned long long theta = s_theta;
-  if (threadIdx.x == 0) a.theta[g] = theta;
-  if (!a.fast) return;
-  // ---- D: the candidates at or above the threshold get their bit; then the running count of set bits over
-  // the group's words gives every unit of 32 tiles the offset of its codes (Sec. 3.4)
-  if (listed) {
-    for (uint32_t i = threadIdx.x; i < n; i += kSelThreads) {
-      const unsigned long long key = __ldcg(cand + i);
-      if (key >= theta) {
-        const uint32_t idx = 0xffffffffu - (uint32_t)key;   // the tile's index inside the group
-        atomicOr(words + (idx >> 5), 1u << (idx & 31u));
+  const uint32_t nc = s_ncand, n_listed = nc <= (uint32_t)kClKeys ? nc : 0u;   // (too many: the cluster's total says so to all)
+  if (threadIdx.x == 0) s_base = nc ? atomicAdd(&cl.map_shared_rank(&sh, 0)->n_keys, nc) : 0u;
+  if (threadIdx.x < CS) {
+    SelShared *o = cl.map_shared_rank(&sh, threadIdx.x);
+    o->part[rank] = s_nabove;
+    if (nc) atomicAdd(&o->n_total, nc);
+  }
+  const uint32_t tile_bytes = a.tile * (a.bf16 ? 2u : 4u);
+  const uint8_t *tiles = a.in + (g * (uint64_t)ng + i0) * tile_bytes;   // (not used with wider allocation tiles: their scores are exact)
+  {
+    const uint32_t noct = a.exact_scores ? 1u : a.tile / 8, sub = (uint32_t)threadIdx.x % noct, per_round = (uint32_t)kSelThreads / noct;
+    for (uint32_t j0 = 0; j0 < n_listed; j0 += per_round) {   // uniform trip count: whole warps take part
+      const uint32_t j = j0 + threadIdx.x / noct;
+      const bool live = j < n_listed;
+      const uint32_t i = s_cand[live ? j : 0];
+      const float ex = a.exact_scores ? sc[i] : exact_score_any(tiles + (uint64_t)i * tile_bytes, noct, a.bf16 != 0, sub, a.eps_l1, a.eps_log);
+      if (j0 == 0) __syncthreads();   // s_base
+      // the keys go into every CTA's copy of the list: nobody has to fetch them from one CTA afterwards
+      const uint32_t at = s_base + j;
+      if (live && at < (uint32_t)kClKeys) {
+        const unsigned long long key = rank_key(ex, i0 + i);
+        for (uint32_t r = sub; r < CS; r += noct) cl.map_shared_rank(s_keys, r)[at] = key;
       }
     }
-  } else {   // every word anew, from the stored scores (certain ones are +-infinity by now)
-    for (uint64_t i = threadIdx.x; i < ng; i += kSelThreads) {
-      const unsigned m = __ballot_sync(kFull, rank_key(__ldcg(scw + i), (uint32_t)i) >= theta);
-      if (lane == 0) words[i >> 5] = m;
+  }
+  cl.sync();
+  // ---- 4: who of the band made it, found by every CTA for itself from its copy of the list (from here on nobody touches
+  // another CTA's shared memory, unless the list overflowed)
+  const uint32_t n = sh.n_total, p_lane = lane < (int)CS ? sh.part[lane] : 0u;
+  const uint32_t nab = __reduce_add_sync(kFull, p_lane);   // tiles above the band
+  uint32_t before = __reduce_add_sync(kFull, lane < (int)rank ? p_lane : 0u);   // ... in the slices before this one
+  uint32_t rr = k - nab;   // candidates that get the higher width
+  if (nab >= k || rr > n) {   // only possible if the screening error exceeded its bound
+    if (rank == 0 && threadIdx.x == 0) atomicOr(a.status, 8u /* TAHQ_DEV_INTERNAL */);
+    rr = rr > n ? n : 1u;
+  }
+  if (n > (uint32_t)kClKeys) {
+    before = selection_by_radix(a, sc, tiles, tile_bytes, n_loc, i0, lo_v, hi_v, rr, words, s_coarse, s_red, sh);
+  } else {
+    // band tiles that made it: those of the slices before this one are counted, those of this slice get their bit
+    auto won = [&](unsigned long long key) {
+      const uint32_t idx = 0xffffffffu - (uint32_t)key;   // tile inside the group
+      if (idx < i0) atomicAdd(&s_made, 1u);
+      else if (idx - i0 < n_loc) atomicOr(&words[(idx - i0) >> 5], 1u << ((idx - i0) & 31u));
+    };
+    if (n <= 128u) {   // a warp to a key: it counts the larger ones (keys are distinct)
+      for (uint32_t q = (uint32_t)warp; q < n; q += NW) {
+        const unsigned long long mine = s_keys[q];
+        uint32_t larger = 0;
+        for (uint32_t i = 0; i < n; i += 32) larger += (uint32_t)__popc(__ballot_sync(kFull, i + lane < n && s_keys[i + lane] > mine));
+        if (lane == 0 && larger < rr) won(mine);
+      }
+    } else {
+      const unsigned long long theta = rank_keys_shared(s_keys, n, rr, s_keys + kClKeys);
+      for (uint32_t i = threadIdx.x; i < n; i += kSelThreads)
+        if (s_keys[i] >= theta) won(s_keys[i]);
+    }
+    __syncthreads();
+    before += s_made;
+  }
+  before += (uint32_t)(g * a.rank_k);   // ranked tiles of the higher width in front of the slice, over the whole tensor
+
+  // ---- 5: running counts, words, and out.  512 words at a time.
+  uint32_t *const bitmap = reinterpret_cast<uint32_t *>(a.packed + a.off_bitmap);
+  const uint64_t t0 = (g * (uint64_t)ng + i0) * a.alloc_m;   // first quantisation tile of the slice
+  auto word_at = [&](uint32_t w) { return *(volatile const uint32_t *)(words + w); };   // (in the workspace: changed by atomics)
+  uint32_t carry = before;
+  for (uint32_t w0 = 0; w0 < n_words; w0 += kSelThreads) {
+    const uint32_t w = w0 + threadIdx.x, wv = w < n_words ? word_at(w) : 0u, c = (uint32_t)__popc(wv);
+    uint32_t incl = c;
+#pragma unroll
+    for (int o = 1; o < 32; o *= 2) {
+      const uint32_t v = __shfl_up_sync(kFull, incl, o);
+      if (lane >= o) incl += v;
+    }
+    if (w0) __syncthreads();
+    if (lane == 31) s_red[warp] = incl;
+    __syncthreads();
+    const uint32_t sum = lane < NW ? s_red[lane] : 0u;
+    const uint32_t ex = carry + incl - c + __reduce_add_sync(kFull, lane < warp ? sum : 0u);
+    carry += __reduce_add_sync(kFull, sum);
+    if (w < n_words) {
+      if (a.whole_words) {   // groups of whole words, A = G: the words are the bit map's
+        bitmap[t0 / 32 + w] = wv;
+        a.pre[t0 / 32 + w] = ex;
+      } else {
+        wpre[w] = ex;
+      }
     }
   }
-  __threadfence();
+  if (a.whole_words) return;
   __syncthreads();
-  scan_group_words(words, (uint32_t)(ng / 32), (uint32_t)(g * a.k_hi), a.pre + g * (ng / 32));
+  const uint32_t m = a.alloc_m, off = (uint32_t)(t0 & 31u);   // the slice starts at bit `off` of its first word
+  const uint64_t n_out = (uint64_t)n_loc * m + off;           // bits from the start of that word
+  if (n_loc == 0) return;
+  for (uint32_t j = threadIdx.x; (uint64_t)j * 32u < n_out; j += kSelThreads) {
+    const uint64_t word = t0 / 32 + j;
+    const int64_t q0 = (int64_t)j * 32 - off;                 // the word's first tile, from the slice's first (negative: not ours)
+    uint32_t bits = 0;
+    if (m == 1u) {
+      if (q0 < 0) {
+        bits = word_at(0) << off;
+      } else {
+        const uint32_t w = (uint32_t)q0 >> 5;
+        bits = __funnelshift_r(word_at(w), w + 1u < n_words ? word_at(w + 1u) : 0u, (uint32_t)q0 & 31u);
+      }
+    } else {
+      const uint32_t q_end = n_out < (uint64_t)(j + 1) * 32u ? (uint32_t)(n_out - off) : (uint32_t)(q0 + 32);
+      for (uint32_t q = q0 < 0 ? 0u : (uint32_t)q0; q < q_end;) {   // a ranked tile's run of quantisation tiles at a time
+        const uint32_t r = q / m, e = (r + 1u) * m < q_end ? (r + 1u) * m : q_end, len = e - q;
+        if ((word_at(r >> 5) >> (r & 31u)) & 1u) bits |= (len >= 32u ? 0xffffffffu : (1u << len) - 1u) << (uint32_t)((int64_t)q - q0);
+        q = e;
+      }
+    }
+    if (q0 >= 0 && (uint64_t)(j + 1) * 32u <= n_out) bitmap[word] = bits;
+    else atomicOr(bitmap + word, bits);   // shared with a neighbouring slice or group
+    if (q0 >= 0) {
+      const uint32_t r = (uint32_t)q0 / m, in = (uint32_t)q0 - r * m;
+      a.pre[word] = m * (wpre[r >> 5] + (uint32_t)__popc(word_at(r >> 5) & ((1u << (r & 31u)) - 1u))) + (((word_at(r >> 5) >> (r & 31u)) & 1u) ? in : 0u);
+    }
+  }
 }
 
 }  // namespace tahq

@@ -8,9 +8,7 @@
 // in its loop.  Rows of 128 bytes arrive by one tiled TMA copy per unit on the warp's own mbarriers,
 // other row sizes by 16-byte cp.async.  Two things make the independence possible.
 //   * Sec. 3.2 / 3.4: the widths are known before quantise + pack starts: the selection has written the
-//     bit map and, per bit-map word, the number of higher-width tiles in front of it (quant2_kernel), or
-//     the scores and thresholds are in memory and a prologue turns the CTA's slice of them into bit-map
-//     words and (one look-back over the CTAs) byte offsets (quant_pack_stream_kernel).
+//     bit map and, per bit-map word, the number of higher-width tiles in front of it.
 //   * Eq. 3-4: tiles that pass the pivot test cost about three times as much as the others.  A lane
 //     handles an unflagged tile on the spot; tiles that may be flagged are only noted in a queue of
 //     row indices private to the warp.  When 32 are queued, their rows are fetched again (from L2,
@@ -163,101 +161,7 @@ __device__ __forceinline__ void words_minmax(const uint32_t (&w)[C::ROWB / 4], f
 }
 
 // ------------------------------------------------------------------------------------------
-// Eq. 1-2, warp-streaming: entropy score per tile, per-group histogram of binned scores (Sec. 3.2)
-// ------------------------------------------------------------------------------------------
-template <class C, int NST, bool EXACT>
-__device__ __forceinline__ void stats_phase(const Args &a, const void *tmap, uint8_t *smem, unsigned long long *bars,
-                                            uint32_t *s_hist, unsigned long long tag) {
-  using S = StreamCfg<C>;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  bool cleared = false;   // a.fast: the wait for the cleared histograms is behind this CTA
-  UnitRing<C, NST> ring;   // TMA needs 1024-byte aligned slots; otherwise the cp.async path does the same job
-  ring.init(smem + (size_t)warp * NST * S::UNIT_BYTES, bars + warp * NST,
-            (a.use_tma && (smem_u32(smem) & 1023u) == 0) ? tmap : nullptr, lane);
-  const bool use_hist = !a.direct && !a.no_hist;
-  const uint64_t n_units = (a.n_tiles + 31) / 32;
-  const uint64_t u0 = n_units * blockIdx.x / gridDim.x, u1 = n_units * (blockIdx.x + 1ull) / gridDim.x;
-  if (use_hist)
-    for (int b = threadIdx.x; b < kBins; b += kThreads) s_hist[b] = 0;
-
-  // the CTA's units, one stretch per ranking group: a unit belongs to the group of its first tile
-  uint64_t us = u0;
-  while (us < u1) {
-    const uint64_t g = (us * 32) / a.tiles_per_group;
-    const uint64_t g_end = (g + 1) * a.tiles_per_group;            // first tile of the next group
-    uint64_t ue = (g_end + 31) / 32;
-    if (ue > u1 || !use_hist) ue = u1;
-    // The stretch is read back to front: the units read last are the ones the encoder, which walks the same
-    // stretch front to back right afterwards, asks for first, while they are still in L2.
-    const uint64_t nu = ue - us;
-#pragma unroll
-    for (int s = 0; s < NST; ++s) {
-      const uint64_t k = warp + (uint64_t)s * kWarps;
-      if (k < nu) ring.issue(a, ue - 1 - k, s);
-      ring.commit();
-    }
-    __syncthreads();   // the histogram is clear
-    int slot = 0;
-    for (uint64_t k = warp; k < nu; k += kWarps) {
-      const uint64_t u = ue - 1 - k;
-      ring.wait(a, slot);
-      const uint8_t *stage = ring.slot(slot);
-      // small groups are ranked on exact scores; large ones are screened first (see select_kernel)
-      const float s = EXACT ? tile_score<C>(stage, lane, a.eps_l1, a.eps_log)
-                            : tile_score_screen<C>(stage, lane, a.eps_l1);
-      __syncwarp();
-      {
-        const uint64_t kn = k + (uint64_t)NST * kWarps;
-        if (kn < nu) ring.issue(a, ue - 1 - kn, slot);
-        ring.commit();
-      }
-      slot = (slot + 1 == NST) ? 0 : slot + 1;
-      const uint64_t tile = u * 32 + lane;
-      if (tile < a.n_tiles) {
-        a.scores[tile] = s;
-        if (use_hist) {
-          if (tile < g_end) atomicAdd(&s_hist[score_bin(s)], 1u);
-          else atomicAdd(a.hist + (g + 1) * kBins + score_bin(s), 1u);   // the unit straddles two groups
-        }
-      }
-    }
-    cp_async_wait<0>();
-    __syncthreads();
-    if (use_hist) {   // add this stretch's counts to the group's histogram
-      if (a.fast && !cleared) {   // ... which the call's first CTAs have cleared (long ago, as a rule)
-        ws_clear_wait(a, tag);
-        cleared = true;
-      }
-      uint32_t *gh = a.hist + g * kBins;
-      for (int b = threadIdx.x; b < kBins; b += kThreads) {
-        const uint32_t v = s_hist[b];
-        if (v) { atomicAdd(gh + b, v); s_hist[b] = 0; }
-      }
-    }
-    us = ue;
-  }
-}
-
-template <class C, int NST, bool EXACT>
-__global__ void __launch_bounds__(kThreads, 2) stats_stream_kernel(const Args a, const __grid_constant__ CUtensorMap tmap) {
-  extern __shared__ __align__(1024) uint8_t smem_1k[];
-  uint8_t *smem = smem_1k;
-  __shared__ uint32_t s_hist[kBins];   // this CTA's counts for the ranking group it is in
-  TraceScope trace(a.trace, 1);
-  grid_dependency_wait();   // the histograms are cleared by the kernel in front, or by this kernel's first CTAs
-  trace.started();
-  unsigned long long tag = 0ull;
-  if (a.fast) {
-    if (!a.no_hist) tag = ws_clear_begin(a);
-    else if (blockIdx.x == 0 && threadIdx.x == 0) *a.status = 0;   // nothing else of the workspace has to start at zero
-  }
-  stats_phase<C, NST, EXACT>(a, &tmap, smem, reinterpret_cast<unsigned long long *>(smem + (size_t)kWarps * NST * StreamCfg<C>::UNIT_BYTES),
-                      s_hist, tag);
-}
-
-// ------------------------------------------------------------------------------------------
-// Eq. 1-2 for calls whose selection bins the scores itself (a.no_hist): scores only, no histogram,
-// no group boundaries -- a warp streams units of 32 tiles and stores 32 scores per unit.
+// Eq. 1-2: scores only, no group boundaries -- a warp streams units of 32 rows and stores their scores.
 // ------------------------------------------------------------------------------------------
 
 // Screening score (see tile_score_screen for the formula and its error) of a row of bfloat16 held as raw
@@ -596,279 +500,12 @@ __device__ __forceinline__ uint32_t scan_segment(const uint32_t *s_bm, uint32_t 
 
 constexpr int kQueueCap = 64;   // tile indices a warp can hold back (32 left over + 32 of one unit)
 
-// NARROW: no width above 4 bits in this call (compiling the unit loop for the one case it meets makes it
-// 1.5 us faster on the LLaMA-7B shape than finding out at run time)
-template <class C, int NST, bool SR, bool NARROW>
-__device__ __forceinline__ void quant_phase(const Args &a, const void *tmap, uint8_t *smem) {
-  using S = StreamCfg<C>;
-  unsigned long long *bars = reinterpret_cast<unsigned long long *>(smem + (size_t)kWarps * (NST + 1) * S::UNIT_BYTES);
-  __shared__ uint32_t s_bm[kSegWords];    // bit-map words of the segment
-  __shared__ uint32_t s_pre[kSegWords];   // higher-width tiles of the segment before each word
-  __shared__ uint32_t s_wsum[kWarps];
-  __shared__ uint32_t s_qtile[kWarps][kQueueCap];   // held-back tile: (tile - first tile of the CTA) * 2 + higher width
-  __shared__ uint32_t s_qhib[kWarps][kQueueCap];    // held-back tile: higher-width tiles before it, from the CTA's first
-  __shared__ uint32_t s_pool[2][kWarps * 32];        // the warps' last, partly filled batches, pooled at the end
-  __shared__ uint32_t s_pool_n;
-  if (threadIdx.x == 0) s_pool_n = 0;   // (read only after barriers further down)
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const unsigned lt = (1u << lane) - 1u;
-  UnitRing<C, NST> ring;
-  ring.init(smem + (size_t)warp * (NST + 1) * S::UNIT_BYTES, bars + warp * NST,
-            (a.use_tma && (smem_u32(smem) & 1023u) == 0) ? tmap : nullptr, lane);
-  uint8_t *fstage = ring.slot(NST);   // rows fetched again for the flagged path (always by cp.async)
-  uint32_t *sz32 = reinterpret_cast<uint32_t *>(a.packed + a.off_sz);
-  uint8_t *pivot = a.packed + a.off_pivot;
-  uint32_t *bitmap = reinterpret_cast<uint32_t *>(a.packed + a.off_bitmap);
-  uint8_t *payload = a.packed + a.off_payload;
-
-  const uint64_t n_units = (a.n_tiles + 31) / 32;
-  const uint64_t u0 = n_units * blockIdx.x / gridDim.x, u1 = n_units * (blockIdx.x + 1ull) / gridDim.x;
-  const uint64_t tile_cta = u0 * 32;
-
-  // the first units of a segment start moving before anything else
-  auto prime = [&](uint64_t s0, uint64_t s1) {
-#pragma unroll
-    for (int s = 0; s < NST; ++s) {
-      const uint64_t u = s0 + warp + (uint64_t)s * kWarps;
-      if (u < s1) ring.issue(a, u, s);
-      ring.commit();
-    }
-  };
-
-  // The scores that the first rounds of the bit-map pass need are asked for first, into the slot that holds
-  // re-fetched rows later: left to that pass they are one load per thread and round, each waiting for the one
-  // before (0.45 us per round; the scores were written on the far side of the L2).
-  constexpr uint32_t kStagedRounds = S::UNIT_BYTES / 128;   // 32 scores per warp and round
-  const bool staged = a.mixed && a.alloc_m == 1;
-  float *const sc_stage = reinterpret_cast<float *>(fstage);
-  if (staged) {
-    const uint64_t t1 = (u0 + kSegWords < u1 ? u0 + kSegWords : u1) * 32;
-    uint32_t r = 0;
-    for (uint64_t t = u0 * 32 + threadIdx.x; t < t1 && t < a.n_tiles && r < kStagedRounds; t += kThreads, ++r)
-      cp_async4(sc_stage + r * 32 + lane, a.scores + t);
-    cp_async_commit();
-  }
-  prime(u0, u0 + kSegWords < u1 ? u0 + kSegWords : u1);
-
-  if (blockIdx.x == 0) {   // header and the zero padding behind every section
-    if (threadIdx.x < 32) reinterpret_cast<uint32_t *>(a.packed)[threadIdx.x] = a.header[threadIdx.x];
-    for (int s = 0; s < 4; ++s) {
-      const uint64_t from = s == 0 ? a.off_bitmap + 4 * n_units : s == 1 ? a.off_sz + 4 * a.n_tiles
-                          : s == 2 ? a.off_pivot + a.n_tiles : a.off_payload + a.payload_bytes;
-      const uint64_t to = s == 0 ? a.off_sz : s == 1 ? a.off_pivot : s == 2 ? a.off_payload : a.total_bytes;
-      for (uint64_t o = from + threadIdx.x; o < to; o += kThreads) a.packed[o] = 0;
-    }
-  }
-
-  if (u0 == u1) {   // more CTAs than units: still take part in the look-back
-    bool unused;
-    if (a.mixed) cta_exclusive_prefix(a, 0, false, unused);
-    cp_async_wait<0>();
-    return;
-  }
-  const bool single = u1 - u0 <= (uint64_t)kSegWords;
-  uint64_t counted = 0;
-  if (a.mixed && !single) {   // long slices: count first, the look-back needs the CTA's total
-    GroupCursor pc;
-    pc.init(a, u0 * 32);
-    const uint64_t t1 = u1 * 32 < a.n_tiles ? u1 * 32 : a.n_tiles;
-    uint32_t n = 0;
-    for (uint64_t tb = u0 * 32; tb < t1; tb += kThreads) {
-      const uint64_t t = tb + threadIdx.x;
-      if (t < t1) n += pc.is_hi(a, t, threadIdx.x) ? 1u : 0u;
-      pc.advance(a, kThreads);
-    }
-    counted = block_sum(n);
-  }
-
-  uint64_t base_hi = 0;    // higher-width tiles before this CTA, over the whole tensor
-  uint32_t seg_hi = 0;     // higher-width tiles of this CTA's earlier segments
-  uint32_t qhead = 0, qn = 0;   // this warp's queue of held-back tiles (circular)
-  uint32_t f_n = 0;             // rows on their way into (or waiting in) fstage
-  uint32_t f_tile = 0, f_hib = 0;   // lane j's row of fstage
-  const uint64_t row_bytes = (uint64_t)C::ROWB;
-  const bool narrow = NARROW;
-
-  // fetch the rows of the first n (<= 32) queued tiles again; lane j keeps the j-th tile's particulars
-  auto gather = [&](uint32_t n) {
-    f_tile = s_qtile[warp][(qhead + lane) & (kQueueCap - 1)];
-    f_hib = s_qhib[warp][(qhead + lane) & (kQueueCap - 1)];
-#pragma unroll
-    for (int i = 0; i < C::CPR; ++i) {
-      const int piece = i * 32 + lane, r = piece / C::CPR, q = piece % C::CPR;
-      const uint32_t tr = __shfl_sync(kFull, f_tile, r) >> 1;
-      const bool ok = (uint32_t)r < n;
-      cp_async16(fstage + (size_t)phys_chunk<C>(r, q) * 16,
-                 ok ? a.in + (tile_cta + tr) * row_bytes + (size_t)q * 16 : a.in, ok ? 16 : 0);
-    }
-    cp_async_commit();
-    f_n = n;
-    qhead = (qhead + n) & (kQueueCap - 1);
-    qn -= n;
-  };
-  // Eq. 3-4 on the rows of fstage, lane j on row j
-  auto run_flagged = [&]() {
-    if ((uint32_t)lane < f_n) {
-      const uint64_t tile = tile_cta + (f_tile >> 1);
-      const uint64_t off = (uint64_t)(C::G / 8) * ((uint64_t)a.lo * tile + base_hi + f_hib);
-      encode_queued_row<C, SR>(a.tau, a.eps_ratio, fstage, lane, a.lo + (f_tile & 1u), narrow,
-                               reinterpret_cast<uint32_t *>(payload + off), sz32 + tile, pivot + tile, a.seed,
-                               tile * (unsigned long long)C::G);
-    }
-    f_n = 0;
-    __syncwarp();
-  };
-
-  for (uint64_t s0 = u0; s0 < u1; s0 += kSegWords) {
-    const uint64_t s1 = s0 + kSegWords < u1 ? s0 + kSegWords : u1;
-    const uint32_t nw = (uint32_t)(s1 - s0);
-    if (s0 != u0) {
-      __syncthreads();   // every warp is done with the previous segment's words
-      prime(s0, s1);
-    }
-    // ---- bit-map words of the segment (Sec. 3.2), written to the packed buffer as they are formed
-    if (a.mixed) {
-      GroupCursor pc;
-      pc.init(a, s0 * 32);
-      const bool use_stage = staged && s0 == u0;
-      if (use_stage) {   // the scores asked for at the start (older than every group of the ring)
-        if (ring.tmap) cp_async_wait<0>();
-        else cp_async_wait<NST>();
-      }
-      uint32_t r = 0;
-      for (uint64_t tb = s0 * 32; tb < s1 * 32; tb += kThreads, ++r) {
-        const uint64_t t = tb + threadIdx.x;
-        const bool hi = t < a.n_tiles && ((use_stage && r < kStagedRounds)
-                                              ? pc.is_hi_score(a, sc_stage[r * 32 + lane], threadIdx.x)
-                                              : pc.is_hi(a, t, threadIdx.x));
-        const unsigned word = __ballot_sync(kFull, hi);
-        if (lane == 0 && (t >> 5) < s1) {
-          s_bm[(t >> 5) - s0] = word;
-          bitmap[t >> 5] = word;
-        }
-        pc.advance(a, kThreads);
-      }
-    } else {
-      for (uint32_t i = threadIdx.x; i < nw; i += kThreads) {
-        s_bm[i] = 0;
-        bitmap[s0 + i] = 0;
-      }
-    }
-    __syncthreads();
-    const uint32_t seg_total = scan_segment(s_bm, nw, seg_hi, s_pre, s_wsum);
-    if (s0 == u0 && a.mixed) {   // Sec. 3.4: higher-width tiles of all CTAs before this one
-      bool unused;
-      base_hi = cta_exclusive_prefix(a, single ? (uint64_t)seg_total : counted, false, unused);
-    }
-    __syncthreads();
-
-    // ---- the warp's units of this segment; inside the loop everything is relative to the CTA's first
-    // tile and first payload byte, in 32-bit arithmetic
-    int slot = 0;
-    uint8_t *const pay_cta = payload + (uint64_t)(C::G / 8) * ((uint64_t)a.lo * tile_cta + base_hi);
-    uint32_t *const sz_cta = sz32 + tile_cta;
-    uint8_t *const pv_cta = pivot + tile_cta;
-    const uint32_t n_rel = a.n_tiles - tile_cta < 0xffffffffull ? (uint32_t)(a.n_tiles - tile_cta) : 0xffffffffu;
-    const uint32_t su1 = (uint32_t)(s1 - s0), seg_rel = (uint32_t)(s0 - u0) * 32u;
-    for (uint32_t su = warp; su < su1; su += kWarps) {   // su = unit index inside the segment
-      if (f_n && ring.tmap) cp_async_wait<0>();   // the rows fetched again one round ago (their own group here)
-      ring.wait(a, slot);                         // this unit has landed (cp.async: and so have those rows)
-      if (f_n) run_flagged();
-      if (qn >= 32u) gather(32u);
-
-      uint8_t *stage = ring.slot(slot);
-      uint32_t w[S::WORDS];
-      row_load_words<C>(stage, lane, w);
-      __syncwarp();
-      {   // the slot is free again: fetch the unit that comes NST rounds later
-        const uint32_t sn = su + (uint32_t)NST * kWarps;
-        if (sn < su1) ring.issue(a, s0 + sn, slot);
-        ring.commit();
-      }
-      slot = (slot + 1 == NST) ? 0 : slot + 1;
-
-      const uint32_t word = s_bm[su];
-      const uint32_t hi = (word >> lane) & 1u;
-      const uint32_t trel = seg_rel + su * 32u + lane;   // tile - first tile of the CTA
-      const bool live = trel < n_rel;
-      const uint32_t hib = s_pre[su] + (uint32_t)__popc(word & lt);
-
-      // Eq. 3, first look: the second-largest magnitude is at least the smaller of |min| and |max| (they
-      // sit at different positions, or every element is equal), so a tile whose largest magnitude does
-      // not exceed tau * (that + varrho) cannot be flagged.  The others are held back for the exact test.
-      float mn, mx;
-      words_minmax<C>(w, mn, mx);
-      const float m_big = fmaxf(fabsf(mn), fabsf(mx)), m_small = fminf(fabsf(mn), fabsf(mx));
-      const bool maybe = live && m_big > a.tau * (m_small + a.eps_ratio);
-      const unsigned held = __ballot_sync(kFull, maybe);
-      if (maybe) {
-        const uint32_t e = (qhead + qn + (uint32_t)__popc(held & lt)) & (kQueueCap - 1);
-        s_qtile[warp][e] = (trel << 1) | hi;
-        s_qhib[warp][e] = hib;
-      }
-      qn += (uint32_t)__popc(held);
-      if (live && !maybe) {
-        const uint32_t off = (uint32_t)(C::G / 8) * (a.lo * trel + hib);
-        sz_cta[trel] = encode_plain_words<C, SR>(w, mn, mx, a.lo + hi, narrow, reinterpret_cast<uint32_t *>(pay_cta + off),
-                                                 a.seed, (tile_cta + trel) * (unsigned long long)C::G);
-        pv_cta[trel] = 0;
-      }
-      __syncwarp();
-    }
-    cp_async_wait<0>();
-    __syncwarp();
-    seg_hi += seg_total;
-  }
-  // ---- what is still held back: full batches first, then the warps pool their remainders so that the
-  // CTA runs as few partly filled batches as possible (on a small tensor these are half of all batches)
-  if (f_n) run_flagged();
-  while (qn >= 32u) {
-    gather(32u);
-    cp_async_wait<0>();
-    __syncwarp();
-    run_flagged();
-  }
-  {
-    uint32_t base = 0;
-    if (lane == 0 && qn) base = atomicAdd(&s_pool_n, qn);
-    base = __shfl_sync(kFull, base, 0);
-    if ((uint32_t)lane < qn) {
-      s_pool[0][base + lane] = s_qtile[warp][(qhead + lane) & (kQueueCap - 1)];
-      s_pool[1][base + lane] = s_qhib[warp][(qhead + lane) & (kQueueCap - 1)];
-    }
-    __syncthreads();
-    const uint32_t n = s_pool_n;
-    for (uint32_t t0 = (uint32_t)warp * 32u; t0 < n; t0 += kWarps * 32u) {
-      const uint32_t cnt = n - t0 < 32u ? n - t0 : 32u;
-      s_qtile[warp][lane] = (uint32_t)lane < cnt ? s_pool[0][t0 + lane] : 0u;   // through the warp's own queue
-      s_qhib[warp][lane] = (uint32_t)lane < cnt ? s_pool[1][t0 + lane] : 0u;
-      __syncwarp();
-      qhead = 0;
-      qn = cnt;
-      gather(cnt);
-      cp_async_wait<0>();
-      __syncwarp();
-      run_flagged();
-    }
-  }
-}
-
-template <class C, int NST, bool SR, bool NARROW>
-__global__ void __launch_bounds__(kThreads, 2) quant_pack_stream_kernel(const Args a, const __grid_constant__ CUtensorMap tmap) {
-  extern __shared__ __align__(1024) uint8_t smem_1k[];
-  uint8_t *smem = smem_1k;
-  TraceScope trace(a.trace, 3);
-  grid_dependency_wait();   // scores and thresholds are the selection kernel's
-  trace.started();
-  quant_phase<C, NST, SR, NARROW>(a, &tmap, smem);
-}
-
 // ------------------------------------------------------------------------------------------
-// Quantise + pack for calls whose widths and offsets come ready from select_kernel (a.fast): the bit-map
-// word of a unit of 32 tiles is in the packed buffer already and a.pre[unit] is the number of higher-width
-// tiles before it, so a warp needs nothing from the rest of its CTA -- no pass over the scores, no scan, no
-// look-back over the CTAs -- and starts on its first unit at once.  Tiles that may be transformed are handled
-// as in quant_phase (queue of 32, rows fetched again, one lane per row).
+// Quantise + pack.  The bit-map word of a unit of 32 tiles is in the packed buffer already and a.pre[unit] is the
+// number of higher-width tiles before it, so a warp needs nothing from the rest of its CTA -- no pass over the
+// scores, no scan, no look-back over the CTAs -- and starts on its first unit at once.  NARROW: no width above 4 bits
+// in this call (compiling the unit loop for the one case it meets makes it 1.5 us faster on the LLaMA-7B shape than
+// finding out at run time).
 // ------------------------------------------------------------------------------------------
 template <class C, int NST, bool SR, bool NARROW>
 __global__ void __launch_bounds__(kThreads, 2) quant2_kernel(const Args a, const __grid_constant__ CUtensorMap tmap) {
