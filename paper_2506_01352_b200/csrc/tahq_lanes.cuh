@@ -407,4 +407,472 @@ __global__ void __launch_bounds__(kLaneThreads, 1) decode_lanes_kernel(const Arg
   if (qn) decode_flagged_round<C, NARROW, WIDE_ST>(q_codes, q_info, rows, qhead, qn, out_cta);
 }
 
+// ------------------------------------------------------------------------------------------
+// Quantise + pack (Eq. 3-4, Sec. 3.3-3.4)
+//
+// The quantiser of a tile and everything about its place are worked out by each of its lanes, and the butterfly crosses
+// lanes by shuffles, so this kernel issues more instructions per tile than quant2_kernel, where a lane owns a tile (1190
+// against 850 per 32 tiles of 64 bf16).  What it gains: 20 or 24 warps on an SM, no ring of slots to fill, and a warp's
+// work comes in pieces of half a unit and less.  Binary32, where a tile fills 256 bytes and quant2_kernel has 8 warps on an
+// SM: 12.2 -> 9.3 us for 8192 x 768, 28.2 -> 23.1 us for 10240 x 2240, 82 -> 78 us for 16384 x 6720.  For bf16 see
+// quant_lanes_pays.
+// ------------------------------------------------------------------------------------------
+template <class C>
+struct QuantLanes {
+  static constexpr int NT = C::BF16 ? 640 : 768, WARPS = NT / 32;   // (32 elements to a lane need more registers than 16)
+  static_assert(WARPS % LaneCfg<C>::P == 0, "a warp's rounds take the same part of their bit-map word");
+  // per warp: the queue of lanes put aside, two times 32: their 64 bytes in four pieces; where the tile's codes go, tile
+  // and width
+  static constexpr int WARP = 64 * (64 + 8);
+  static constexpr int SMEM = WARPS * WARP;
+};
+
+// A lane's 64 bytes of the tensor, aligned to 16 or (WIDE) 32 bytes.
+template <bool WIDE>
+__device__ __forceinline__ void load_64_bytes(const uint8_t *src, uint32_t (&w)[16]) {
+  if constexpr (WIDE) {
+#pragma unroll
+    for (int i = 0; i < 16; i += 8)
+      asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                   : "=r"(w[i]), "=r"(w[i + 1]), "=r"(w[i + 2]), "=r"(w[i + 3]), "=r"(w[i + 4]), "=r"(w[i + 5]), "=r"(w[i + 6]),
+                     "=r"(w[i + 7])
+                   : "l"(src + 4 * i));
+  } else {
+#pragma unroll
+    for (int i = 0; i < 16; i += 4) {
+      const uint4 v = __ldg(reinterpret_cast<const uint4 *>(src + 4 * i));
+      w[i] = v.x; w[i + 1] = v.y; w[i + 2] = v.z; w[i + 3] = v.w;
+    }
+  }
+}
+
+// Codes of a lane -> the tile's bit stream.  t(k) = q_k + 1.5*2^23 for a compile-time k; `dst` = the tile's first word.
+// 16 codes of an odd width end in the middle of a word, which the lane shares with its neighbour: the even lane of the
+// pair stores it.  All lanes of a warp call this; `mine`: the lane stores.
+template <int E, bool NARROW, class F>
+__device__ __forceinline__ void pack_lane(F &&t, uint32_t W, uint32_t sub, uint32_t *dst, bool mine) {
+  if constexpr (NARROW) {   // the width is a lane's own value of 2, 3 or 4: see pack_store_narrow
+    constexpr int NG = E / 8;
+    constexpr uint32_t K2 = (uint32_t)((0x4B400000ull * group_ones(2, 8)) & 0xffffffffull);
+    constexpr uint32_t K3 = (uint32_t)((0x4B400000ull * group_ones(3, 8)) & 0xffffffffull);
+    constexpr uint32_t K4 = (uint32_t)((0x4B400000ull * group_ones(4, 8)) & 0xffffffffull);
+    const bool four = W == 4u, three = W == 3u;
+    uint32_t M = four ? 16u : three ? 8u : 4u;
+    asm volatile("mov.u32 %0, %0;" : "+r"(M));   // opaque to the optimiser: keeps the multiply
+    const uint32_t KW = four ? K4 : three ? K3 : K2;
+    uint32_t g[NG];
+#pragma unroll
+    for (int j = 0; j < NG; ++j) {   // eight codes, W whole bytes
+      uint32_t acc = __float_as_uint(t(8 * j + 7));
+#pragma unroll
+      for (int i = 6; i >= 0; --i) acc = acc * M + __float_as_uint(t(8 * j + i));
+      g[j] = acc - KW;
+    }
+    const uint32_t s0 = four ? 0x3210u : three ? 0x4210u : 0x5410u;   // the first group, then bytes of the second
+    if constexpr (E == 32) {
+      const bool two = W == 2u;
+      const uint32_t w0 = __byte_perm(g[0], g[1], s0);
+      const uint32_t w1 = __byte_perm(two ? g[2] : g[1], two ? g[3] : g[2], four ? 0x3210u : three ? 0x5421u : 0x5410u);
+      const uint32_t w2 = __byte_perm(g[2], g[3], four ? 0x3210u : 0x6542u);
+      dst += sub * W;
+      const uint32_t n = mine ? W : 0u;   // (four stores under conditions of their own: no branches)
+      if (n > 0u) dst[0] = w0;
+      if (n > 1u) dst[1] = w1;
+      if (n > 2u) dst[2] = w2;
+      if (n > 3u) dst[3] = g[3];
+    } else {
+      uint32_t v0 = __byte_perm(g[0], g[1], s0), v1 = three ? g[1] >> 8 : g[1];
+      const uint32_t o = __shfl_xor_sync(kFull, v0, 1);
+      const bool odd = sub & 1u;
+      if (three) {
+        if (odd) v0 = __funnelshift_r(v0, v1, 16);
+        else v1 |= o << 16;
+      }
+      dst += (sub * W + 1u) >> 1;
+      if (mine) dst[0] = v0;
+      if (mine && (four || (three && !odd))) dst[1] = v1;
+    }
+  } else {
+    auto width = [&](auto wc) {
+      constexpr int CW = decltype(wc)::value, NW = (E * CW + 31) / 32;
+      uint32_t w[NW + 1];
+      w[NW] = 0;
+      {
+        uint32_t v[E * CW % 32 ? 2 * NW : NW];   // (pack_magic writes whole words)
+        if constexpr (E * CW % 32) {
+          float z[32];
+#pragma unroll
+          for (int k = 0; k < 32; ++k) z[k] = k < E ? t(k < E ? k : 0) : kMagic;
+          pack_magic<CW, 32>([&](int k) { return z[k]; }, v);
+        } else {
+          pack_magic<CW, E>(t, v);
+        }
+#pragma unroll
+        for (int j = 0; j < NW; ++j) w[j] = v[j];
+      }
+      const uint32_t first = E == 32 ? sub * (uint32_t)CW : (sub * (uint32_t)CW + 1u) >> 1;
+      uint32_t n = NW;
+      if constexpr (E * CW % 32) {
+        const uint32_t o = __shfl_xor_sync(__activemask(), w[0], 1);   // (the neighbour has the same width)
+        if (sub & 1u) {
+#pragma unroll
+          for (int j = 0; j < NW; ++j) w[j] = __funnelshift_r(w[j], w[j + 1], 16);
+          n = NW - 1;
+        } else {
+          w[NW - 1] |= o << 16;
+        }
+      }
+      if (mine)
+#pragma unroll
+        for (int j = 0; j < NW; ++j)
+          if ((uint32_t)j < n) dst[first + j] = w[j];
+    };
+    switch (W) {   // (the lower width is at least 4 here)
+      case 4: width(std::integral_constant<int, 4>{}); break;
+      case 5: width(std::integral_constant<int, 5>{}); break;
+      case 6: width(std::integral_constant<int, 6>{}); break;
+      case 7: width(std::integral_constant<int, 7>{}); break;
+      default: width(std::integral_constant<int, 8>{}); break;
+    }
+    __syncwarp();
+  }
+}
+
+// Where things of one tile go; the lower width, and what depends on it, for it and the next width.
+struct QuantOut {
+  uint32_t *payload, *sz;
+  uint8_t *pivot;
+  uint32_t lo;
+  WidthConst wc;
+};
+
+// Codes from the differences to the zero-point: pair(i) = (x[2i] - z, x[2i+1] - z) for a compile-time i.  mn, mx: the
+// range of the tile.  All lanes of a warp call this; `mine`: the lane has a tile to store.
+template <class C, bool SR, bool NARROW, class F>
+__device__ __forceinline__ void quantise_pack_lane(F &&pair, float mn, float mx, const Quantiser &q, uint32_t W, uint32_t sub,
+                                                   uint32_t *dst, bool mine, unsigned long long seed, unsigned long long first) {
+  constexpr int E = LaneCfg<C>::E;
+  if constexpr (SR) {
+    float d[E];
+#pragma unroll
+    for (int i = 0; i < E / 2; ++i) { const float2 p = pair(i); d[2 * i] = p.x; d[2 * i + 1] = p.y; }
+    stochastic_codes<E>(d, q.inv_s, q.qmax, seed, first);
+    pack_lane<E, NARROW>([&](int k) { return d[k]; }, W, sub, dst, mine);
+  } else {
+    // the clamp is left out when the whole warp's tiles provably stay inside: see quantise_pairs
+    const float ymin = (mn - q.z) * q.inv_s, ymax = (mx - q.z) * q.inv_s;
+    const bool safe = !mine || (ymin >= -0.4999f && ymax < q.qmax + 0.4999f);
+    const float2 is = f2(q.inv_s), mg = f2(kMagic);
+    if (__all_sync(kFull, safe)) {   // (the codes are formed where the packing asks for them)
+      pack_lane<E, NARROW>([&](int k) { const float2 t = fma2(pair(k >> 1), is, mg); return (k & 1) ? t.y : t.x; }, W, sub, dst, mine);
+    } else {
+      const float top = kMagic + q.qmax;
+      pack_lane<E, NARROW>([&](int k) {
+        const float2 t = fma2(pair(k >> 1), is, mg);
+        return fminf(fmaxf((k & 1) ? t.y : t.x, kMagic), top);
+      }, W, sub, dst, mine);
+    }
+  }
+}
+
+// Smallest and largest element of the lane's 64 bytes.
+template <class C>
+__device__ __forceinline__ void lane_minmax(const uint32_t (&w)[16], float &mn, float &mx) {
+  if constexpr (C::BF16) {
+    uint32_t lo = bf2_min(bf2_min(w[0], w[1]), w[2]), hi = bf2_max(bf2_max(w[0], w[1]), w[2]);
+    uint32_t lo2 = bf2_min(bf2_min(w[3], w[4]), w[5]), hi2 = bf2_max(bf2_max(w[3], w[4]), w[5]);
+#pragma unroll
+    for (int j = 6; j < 14; j += 4) {
+      lo = bf2_min(bf2_min(lo, w[j]), w[j + 1]); hi = bf2_max(bf2_max(hi, w[j]), w[j + 1]);
+      lo2 = bf2_min(bf2_min(lo2, w[j + 2]), w[j + 3]); hi2 = bf2_max(bf2_max(hi2, w[j + 2]), w[j + 3]);
+    }
+    lo = bf2_min(bf2_min(lo, w[14]), w[15]); hi = bf2_max(bf2_max(hi, w[14]), w[15]);
+    lo = bf2_min(lo, lo2); hi = bf2_max(hi, hi2);
+    mn = fminf(__uint_as_float(lo << 16), __uint_as_float(lo & 0xffff0000u));
+    mx = fmaxf(__uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u));
+  } else {
+    mn = __uint_as_float(w[0]);
+    mx = mn;
+    float mn2 = __uint_as_float(w[1]), mx2 = mn2;
+#pragma unroll
+    for (int j = 2; j < 16; j += 2) {
+      mn = fminf(mn, __uint_as_float(w[j])); mx = fmaxf(mx, __uint_as_float(w[j]));
+      mn2 = fminf(mn2, __uint_as_float(w[j + 1])); mx2 = fmaxf(mx2, __uint_as_float(w[j + 1]));
+    }
+    mn = fminf(mn, mn2);
+    mx = fmaxf(mx, mx2);
+  }
+}
+
+// Largest and second-largest magnitude of the lane's 64 bytes.
+template <class C>
+__device__ __forceinline__ void lane_top2(const uint32_t (&w)[16], float &a1, float &a2) {
+  if constexpr (C::BF16) {
+    uint32_t p1 = 0, p2 = 0, q1 = 0, q2 = 0;   // two independent (largest, second) pairs per 16-bit half
+#pragma unroll
+    for (int j = 0; j < 16; j += 2) {
+      p2 = bf2_max_abs(p2, bf2_min_abs(p1, w[j])); p1 = bf2_max_abs(p1, w[j]);
+      q2 = bf2_max_abs(q2, bf2_min_abs(q1, w[j + 1])); q1 = bf2_max_abs(q1, w[j + 1]);
+    }
+    const uint32_t m1 = bf2_max_abs(p1, q1) & 0x7fff7fffu;
+    const uint32_t m2 = bf2_max_abs(bf2_min_abs(p1, q1), bf2_max_abs(p2, q2)) & 0x7fff7fffu;
+    const uint32_t e1 = m1 & 0xffffu, o1 = m1 >> 16, e2 = m2 & 0xffffu, o2 = m2 >> 16;
+    a1 = __uint_as_float(max(e1, o1) << 16);
+    a2 = __uint_as_float(max(min(e1, o1), max(e2, o2)) << 16);
+  } else {
+    float p1 = 0.0f, p2 = 0.0f, q1 = 0.0f, q2 = 0.0f;
+#pragma unroll
+    for (int j = 0; j < 16; j += 2) {
+      const float t0 = fabsf(__uint_as_float(w[j])), t1 = fabsf(__uint_as_float(w[j + 1]));
+      p2 = fmaxf(p2, fminf(p1, t0)); p1 = fmaxf(p1, t0);
+      q2 = fmaxf(q2, fminf(q1, t1)); q1 = fmaxf(q1, t1);
+    }
+    a1 = fmaxf(p1, q1);
+    a2 = fmaxf(fminf(p1, q1), fmaxf(p2, q2));
+  }
+}
+
+// Elements 2i and 2i+1 of the lane's 64 bytes, plus c.
+template <class C>
+__device__ __forceinline__ float2 lane_pair_plus(const uint32_t (&w)[16], int i, float c) {
+  float2 d;
+  if constexpr (C::BF16) bf2_add_f32(w[i], c, d.x, d.y);
+  else d = add2(f2(__uint_as_float(w[2 * i]), __uint_as_float(w[2 * i + 1])), f2(c));
+  return d;
+}
+
+// 32 lanes of the queue (the first n of them count), whole tiles with their lanes side by side: the exact pivot test
+// (Eq. 3), the pivot swap in shared memory, the butterfly (Eq. 4), range, codes, bit stream.
+template <class C, bool SR, bool NARROW>
+__device__ __forceinline__ void encode_queued_round(float tau, float eps_ratio, uint4 *q_raw, const uint2 *q_info, uint32_t head,
+                                                    uint32_t n, const QuantOut &out, unsigned long long seed) {
+  using D = LaneCfg<C>;
+  constexpr int E = D::E, P = D::P, EPC = 16 / C::ESZ;   // EPC: elements of a 16-byte piece
+  const uint32_t lane = threadIdx.x & 31u, sub = lane % P;
+  const uint32_t slot = (head + (lane < n ? lane : sub)) & 63u;
+  const uint2 info = q_info[slot];
+  uint32_t w[16];
+  auto fetch = [&]() {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const uint4 v = q_raw[64 * q + slot];
+      w[4 * q] = v.x; w[4 * q + 1] = v.y; w[4 * q + 2] = v.z; w[4 * q + 3] = v.w;
+    }
+  };
+  fetch();
+  float a1, a2;
+  lane_top2<C>(w, a1, a2);
+#pragma unroll
+  for (int h = 1; h < P; h *= 2) {
+    const float o1 = __shfl_xor_sync(kFull, a1, h), o2 = __shfl_xor_sync(kFull, a2, h);
+    a2 = fmaxf(fminf(a1, o1), fmaxf(a2, o2));
+    a1 = fmaxf(a1, o1);
+  }
+  const float t1 = a2 + eps_ratio;
+  const float t2 = tau * t1;
+  const bool flag = a1 > t2;   // Eq. 3
+  // the first position of the largest magnitude: the lane's first piece that holds it, its first element in there
+  uint32_t d = 0xffu;
+  {
+    int hit = -1;
+#pragma unroll
+    for (int q = 3; q >= 0; --q) {
+      bool here;
+      if constexpr (C::BF16) {
+        const uint32_t t = bf2_max_abs(bf2_max_abs(w[4 * q], w[4 * q + 1]), bf2_max_abs(w[4 * q + 2], w[4 * q + 3])) & 0x7fff7fffu;
+        here = max(t & 0xffffu, t >> 16) == __float_as_uint(a1) >> 16;
+      } else {
+        here = fmaxf(fmaxf(fabsf(__uint_as_float(w[4 * q])), fabsf(__uint_as_float(w[4 * q + 1]))),
+                     fmaxf(fabsf(__uint_as_float(w[4 * q + 2])), fabsf(__uint_as_float(w[4 * q + 3])))) == a1;
+      }
+      hit = here ? q : hit;
+    }
+    if (hit >= 0) {
+      const uint4 v = q_raw[64 * hit + slot];
+      const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+      uint32_t kk = EPC - 1;
+#pragma unroll
+      for (int j = 3; j >= 0; --j) {
+        if constexpr (C::BF16) {
+          kk = ((u[j] >> 16) & 0x7fffu) == __float_as_uint(a1) >> 16 ? 2 * j + 1 : kk;
+          kk = (u[j] & 0x7fffu) == __float_as_uint(a1) >> 16 ? 2 * j : kk;
+        } else {
+          kk = fabsf(__uint_as_float(u[j])) == a1 ? j : kk;
+        }
+      }
+      d = sub * E + hit * EPC + kk;
+    }
+#pragma unroll
+    for (int h = 1; h < P; h *= 2) d = min(d, __shfl_xor_sync(kFull, d, h));
+  }
+  __syncwarp();
+  if (flag && sub == 0 && lane < n) {   // Eq. 4: the pivot swap P_d
+    using T = typename std::conditional<C::BF16, uint16_t, uint32_t>::type;
+    T *const p0 = reinterpret_cast<T *>(q_raw + slot);
+    T *const pd = reinterpret_cast<T *>(q_raw + 64 * (d % E / EPC) + ((slot + d / E) & 63u)) + d % EPC;
+    const T x0 = *p0, xd = *pd;
+    *p0 = xd;
+    *pd = x0;
+  }
+  __syncwarp();
+  fetch();
+  float2 p[E / 2];
+  auto widen = [&]() {
+#pragma unroll
+    for (int i = 0; i < E / 2; ++i) {
+      if constexpr (C::BF16) p[i] = lane_pair_plus<C>(w, i, -0.0f);
+      else p[i] = f2(__uint_as_float(w[2 * i]), __uint_as_float(w[2 * i + 1]));
+    }
+  };
+  widen();
+  // Eq. 4: (1/sqrt G) H_G.  For G = 64 the factor is a power of two: the products are exact, so the
+  // factor is applied to the range and inside the quantiser's subtraction instead of element by element.
+  constexpr bool kFold = C::G == 64;
+  butterfly_lanes<E, P>(p, sub);   // (nearly every tile of the queue is flagged: all lanes go through it)
+  if (!kFold) {
+#pragma unroll
+    for (int i = 0; i < E / 2; ++i)   // scalar products: they are added to right after
+      p[i] = f2(p[i].x * hadamard_scale<C>(), p[i].y * hadamard_scale<C>());
+  }
+  if (!flag) {
+    fetch();
+    widen();
+  }
+  float mn = fminf(p[0].x, p[0].y), mx = fmaxf(p[0].x, p[0].y);
+#pragma unroll
+  for (int i = 1; i < E / 2; ++i) {
+    mn = fminf(mn, fminf(p[i].x, p[i].y));
+    mx = fmaxf(mx, fmaxf(p[i].x, p[i].y));
+  }
+#pragma unroll
+  for (int h = 1; h < P; h *= 2) {
+    mn = fminf(mn, __shfl_xor_sync(kFull, mn, h));
+    mx = fmaxf(mx, __shfl_xor_sync(kFull, mx, h));
+  }
+  const float pre = (kFold && flag) ? hadamard_scale<C>() : 1.0f;
+  mn *= pre;
+  mx *= pre;
+  const bool hi = (info.y & 1u) != 0u;
+  const uint64_t tile = info.y >> 1;
+  const Quantiser q = make_quantiser(mn, mx, 0u, hi, out.wc);
+  const float2 nz = f2(-q.z), pr = f2(pre);
+  // (pre * x) - z as one fused multiply-add: the product is exact
+  quantise_pack_lane<C, SR, NARROW>([&](int i) { return fma2(p[i], pr, nz); }, mn, mx, q, out.lo + (hi ? 1u : 0u), sub,
+                                    out.payload + (uint64_t)(C::G / 32) * info.x, lane < n, seed,
+                                    tile * (unsigned long long)C::G + sub * E);
+  if (lane < n && sub == 0) {
+    out.sz[tile] = q.sz;
+    out.pivot[tile] = flag ? (uint8_t)(0x80u | d) : (uint8_t)0;
+  }
+}
+
+template <class C, bool SR, bool NARROW, bool WIDE>
+__global__ void __launch_bounds__(QuantLanes<C>::NT, 1) quant_lanes_kernel(const Args a) {
+  using D = LaneCfg<C>;
+  constexpr int E = D::E, P = D::P, TPR = D::TPR, WARPS = QuantLanes<C>::WARPS;
+  extern __shared__ __align__(128) uint8_t smem_ql[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t sub = (uint32_t)lane % P;   // this lane's part of its tile
+  const unsigned lt = (1u << lane) - 1u;
+  uint4 *const q_raw = reinterpret_cast<uint4 *>(smem_ql + (size_t)warp * QuantLanes<C>::WARP);   // [4][64]
+  uint2 *const q_info = reinterpret_cast<uint2 *>(q_raw + 4 * 64);
+  TraceScope trace(a.trace, 3);
+  grid_dependency_wait();   // bit map and running counts are the selection kernel's; the tensor may be a kernel's too
+  trace.started();
+  uint32_t *const bitmap = reinterpret_cast<uint32_t *>(a.packed + a.off_bitmap);
+  const uint32_t n_tiles = (uint32_t)a.n_tiles, lo = a.lo;   // (at most 2^26)
+  const QuantOut out = {reinterpret_cast<uint32_t *>(a.packed + a.off_payload), reinterpret_cast<uint32_t *>(a.packed + a.off_sz),
+                        a.packed + a.off_pivot, lo, WidthConst(lo)};
+
+  // the CTA's rounds, dealt out over its warps; a lane's tile always has the same bit in its bit-map word
+  const uint32_t n_rounds = (n_tiles + TPR - 1) / TPR;
+  const uint32_t r1 = (uint32_t)((uint64_t)n_rounds * (blockIdx.x + 1u) / gridDim.x);
+  uint32_t r = (uint32_t)((uint64_t)n_rounds * blockIdx.x / gridDim.x) + warp;
+  const uint32_t bit = r % P * TPR + (uint32_t)lane / P, below = (1u << bit) - 1u;
+  uint32_t raw[16], word = 0, before = 0;   // the next round: 64 bytes of the tile; its bit-map word, higher-width tiles in front
+  auto load = [&](uint32_t k) {
+    const uint32_t tile = k / P * 32u + bit;
+    if (tile < n_tiles) load_64_bytes<WIDE>(a.in + (uint64_t)tile * D::TB + sub * 64u, raw);
+    if (a.mixed) { word = __ldg(bitmap + k / P); before = __ldg(a.pre + k / P); }
+  };
+#pragma unroll
+  for (int i = 0; i < 16; ++i) raw[i] = 0;
+  if (r < r1) load(r);
+
+  if (blockIdx.x == 0) {   // header and the zero padding behind every section
+    if (threadIdx.x == 0 && !a.mixed) *a.status = 0;   // (with two widths in use the score kernel has done it)
+    if (threadIdx.x < 32) reinterpret_cast<uint32_t *>(a.packed)[threadIdx.x] = a.header[threadIdx.x];
+    for (int s = 0; s < 4; ++s) {
+      const uint64_t from = s == 0 ? a.off_bitmap + 4 * ((a.n_tiles + 31) / 32) : s == 1 ? a.off_sz + 4 * a.n_tiles
+                          : s == 2 ? a.off_pivot + a.n_tiles : a.off_payload + a.payload_bytes;
+      const uint64_t to = s == 0 ? a.off_sz : s == 1 ? a.off_pivot : s == 2 ? a.off_payload : a.total_bytes;
+      for (uint64_t o = from + threadIdx.x; o < to; o += QuantLanes<C>::NT) a.packed[o] = 0;
+    }
+  }
+
+  uint32_t qhead = 0, qn = 0;
+  while (r < r1 || qn) {   // (one place for the queue's rounds: the last, partly filled one is run behind the others)
+    if (r < r1) {
+      uint32_t w[16];
+#pragma unroll
+      for (int i = 0; i < 16; ++i) w[i] = raw[i];
+      const uint32_t hi = (word >> bit) & 1u, tile = r / P * 32u + bit;
+      const uint32_t n8 = lo * tile + before + (uint32_t)__popc(word & below);   // the tile's codes start G/8 times this many bytes in
+      if (r + WARPS < r1) load(r + WARPS);
+      if (!a.mixed && lane == 0 && r % P == 0) bitmap[r / P] = 0;
+      const bool live = tile < n_tiles;
+
+      // Eq. 3, first look: the second-largest magnitude is at least the smaller of |min| and |max| (they
+      // sit at different positions, or every element is equal), so a tile whose largest magnitude does
+      // not exceed tau * (that + varrho) cannot be flagged.  The others are put aside for the exact test.
+      float mn, mx;
+      lane_minmax<C>(w, mn, mx);
+#pragma unroll
+      for (int h = 1; h < P; h *= 2) {
+        mn = fminf(mn, __shfl_xor_sync(kFull, mn, h));
+        mx = fmaxf(mx, __shfl_xor_sync(kFull, mx, h));
+      }
+      const float m_big = fmaxf(fabsf(mn), fabsf(mx)), m_small = fminf(fabsf(mn), fabsf(mx));
+      const bool maybe = live && m_big > a.tau * (m_small + a.eps_ratio);
+      const unsigned held = __ballot_sync(kFull, maybe);
+      if (maybe) {
+        const uint32_t at = (qhead + qn + (uint32_t)__popc(held & lt)) & 63u;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) q_raw[64 * q + at] = make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
+        q_info[at] = make_uint2(n8, (tile << 1) | hi);
+      }
+      qn += (uint32_t)__popc(held);
+      if (held != kFull) {
+        const bool mine = live && !maybe;
+        const Quantiser q = make_quantiser(mn, mx, 0u, hi != 0u, out.wc);
+        const float nz = -q.z;   // x + (-z) is x - z
+        quantise_pack_lane<C, SR, NARROW>([&](int i) { return lane_pair_plus<C>(w, i, nz); }, mn, mx, q, lo + hi, sub,
+                                          out.payload + (uint64_t)(C::G / 32) * n8, mine, a.seed,
+                                          tile * (unsigned long long)C::G + sub * E);
+        if (mine && sub == 0) {
+          out.sz[tile] = q.sz;
+          out.pivot[tile] = 0;
+        }
+      }
+      r += WARPS;
+    }
+    if (qn >= 32u || (r >= r1 && qn)) {
+      const uint32_t n = qn < 32u ? qn : 32u;
+      __syncwarp();
+      encode_queued_round<C, SR, NARROW>(a.tau, a.eps_ratio, q_raw, q_info, qhead, n, out, a.seed);
+      qhead = (qhead + n) & 63u;
+      qn -= n;
+      __syncwarp();
+    }
+  }
+}
+
+// Binary32 always; bfloat16 while a warp has at most two rounds, that is while the time is that of a warp's chain and not of
+// the instructions (both sides measured, 64-wide tiles, quant2_kernel against this: 1500 tiles 7.2 / 3.9 us, 59 thousand
+// 5.6 / 5.3, 95 thousand -- two rounds -- 6.8 / 6.3, 127 thousand 7.7 / 8.9, 524 thousand 22.5 / 27.8).
+template <class C>
+bool quant_lanes_pays(uint64_t n_rounds, int sms) {
+  return C::G >= 32 && (!C::BF16 || n_rounds <= 2ull * QuantLanes<C>::WARPS * (unsigned)sms);
+}
+
 }  // namespace tahq

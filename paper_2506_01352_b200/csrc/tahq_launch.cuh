@@ -36,18 +36,34 @@ static tahq_status encode_t(const Plan &pl, const Args &a_in, cudaStream_t st) {
     if (launch_select(a, d, st) != TAHQ_OK) return TAHQ_ERR_CUDA;
   }
   const bool narrow = a.lo + a.mixed <= 4u;   // no width above 4 bits: the kernel compiled for just that
-  constexpr int NQ = 2;
-  const int smem = StreamCfg<C>::smem_bytes(NQ);
-  static std::atomic<int> occ_narrow[64], occ_wide[64];
-  const uint64_t n_units = (a.n_tiles * C::LPT + 31) / 32;
-  const int occ = narrow ? prepare(quant2_kernel<C, NQ, SR, true>, kThreads, smem, d, occ_narrow)
-                         : prepare(quant2_kernel<C, NQ, SR, false>, kThreads, smem, d, occ_wide);
-  if (!occ) return TAHQ_ERR_CUDA;
-  const unsigned grid = persistent_grid((n_units + kWarps - 1) / kWarps, d, occ);
-  if (narrow)
-    TAHQ_LAUNCH("quant_pack", st, launch_dependent(quant2_kernel<C, NQ, SR, true>, grid, kThreads, smem, st, a, tmap));
-  else
-    TAHQ_LAUNCH("quant_pack", st, launch_dependent(quant2_kernel<C, NQ, SR, false>, grid, kThreads, smem, st, a, tmap));
+  if constexpr (C::G >= 32) {
+    const uint64_t n_rounds = (a.n_tiles + LaneCfg<C>::TPR - 1) / LaneCfg<C>::TPR;
+    if (quant_lanes_pays<C>(n_rounds, d.sms)) {
+      const bool wide_ld = (reinterpret_cast<uintptr_t>(a.in) & 31u) == 0;   // 256-bit loads where the tensor is aligned to them
+      void (*const kernels[4])(Args) = {quant_lanes_kernel<C, SR, false, false>, quant_lanes_kernel<C, SR, false, true>,
+                                        quant_lanes_kernel<C, SR, true, false>, quant_lanes_kernel<C, SR, true, true>};
+      static std::atomic<int> occ[4][64];
+      const int k = 2 * narrow + wide_ld;
+      if (!prepare(kernels[k], QuantLanes<C>::NT, QuantLanes<C>::SMEM, d, occ[k])) return TAHQ_ERR_CUDA;
+      TAHQ_LAUNCH("quant_pack", st, launch_dependent(kernels[k], persistent_grid(n_rounds, d, 1), QuantLanes<C>::NT,
+                                                     QuantLanes<C>::SMEM, st, a));
+      return cudaGetLastError() == cudaSuccess ? TAHQ_OK : TAHQ_ERR_CUDA;
+    }
+  }
+  if constexpr (C::G < 32 || C::BF16) {
+    constexpr int NQ = 2;
+    const int smem = StreamCfg<C>::smem_bytes(NQ);
+    static std::atomic<int> occ_narrow[64], occ_wide[64];
+    const uint64_t n_units = (a.n_tiles * C::LPT + 31) / 32;
+    const int occ = narrow ? prepare(quant2_kernel<C, NQ, SR, true>, kThreads, smem, d, occ_narrow)
+                           : prepare(quant2_kernel<C, NQ, SR, false>, kThreads, smem, d, occ_wide);
+    if (!occ) return TAHQ_ERR_CUDA;
+    const unsigned grid = persistent_grid((n_units + kWarps - 1) / kWarps, d, occ);
+    if (narrow)
+      TAHQ_LAUNCH("quant_pack", st, launch_dependent(quant2_kernel<C, NQ, SR, true>, grid, kThreads, smem, st, a, tmap));
+    else
+      TAHQ_LAUNCH("quant_pack", st, launch_dependent(quant2_kernel<C, NQ, SR, false>, grid, kThreads, smem, st, a, tmap));
+  }
   return cudaGetLastError() == cudaSuccess ? TAHQ_OK : TAHQ_ERR_CUDA;
 }
 

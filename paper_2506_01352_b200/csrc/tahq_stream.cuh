@@ -259,14 +259,16 @@ __global__ void __launch_bounds__(kThreads, 2) score_kernel(const Args a, const 
   cp_async_wait<0>();
 }
 
+template <class C> using WidthOf = typename std::conditional<(C::G <= 32), WidthConst, WidthNone>::type;
+
 // Sec. 3.3-3.4 for a row that is not transformed, straight from its raw words: zero-point and scale
 // from the known range, codes (computed once), then the bit stream at the lane's own width.
 // Returns the stored {scale, zero}.
 template <class C, bool SR>
 __device__ __forceinline__ uint32_t encode_plain_words(const uint32_t (&w)[C::ROWB / 4], float mn, float mx,
-                                                       uint32_t bits, bool narrow, uint32_t *dst,
+                                                       uint32_t bits, bool hi, const WidthOf<C> &wc, bool narrow, uint32_t *dst,
                                                        unsigned long long seed, unsigned long long first) {
-  const Quantiser q = make_quantiser(mn, mx, bits);
+  const Quantiser q = make_quantiser(mn, mx, bits, hi, wc);
   if constexpr (SR) {
     float d[C::EPT];
 #pragma unroll
@@ -314,7 +316,7 @@ __device__ __forceinline__ uint32_t encode_plain_words(const uint32_t (&w)[C::RO
 // range, codes, bit stream, stores.
 template <class C, bool SR>
 __device__ __noinline__ void encode_queued_row(float tau, float eps_ratio, uint8_t *queue, int row, uint32_t bits,
-                                               bool narrow, uint32_t *dst, uint32_t *sz, uint8_t *pv,
+                                               bool hi, const WidthOf<C> wc, bool narrow, uint32_t *dst, uint32_t *sz, uint8_t *pv,
                                                unsigned long long seed, unsigned long long first) {
   float a1, a2;
   row_top2<C>(queue, row, a1, a2);
@@ -349,7 +351,7 @@ __device__ __noinline__ void encode_queued_row(float tau, float eps_ratio, uint8
   const float pre = (kFold && flag) ? hadamard_scale<C>() : 1.0f;
   mn *= pre;
   mx *= pre;
-  const Quantiser q = make_quantiser(mn, mx, bits);
+  const Quantiser q = make_quantiser(mn, mx, bits, hi, wc);
   if constexpr (SR) {
     float d[C::EPT];
 #pragma unroll
@@ -377,7 +379,7 @@ __device__ __noinline__ void encode_queued_row(float tau, float eps_ratio, uint8
 // (element 0 of the lower half with element d of either), the butterfly's last stage (stride 64), the range.
 template <class C, bool SR>
 __device__ __noinline__ void encode_queued_pair(float tau, float eps_ratio, uint8_t *queue, int row, bool live,
-                                                uint32_t bits, bool narrow, uint32_t *dst, uint32_t *sz, uint8_t *pv,
+                                                uint32_t bits, bool hi, const WidthOf<C> wc, bool narrow, uint32_t *dst, uint32_t *sz, uint8_t *pv,
                                                 unsigned long long seed, unsigned long long first) {
   const int half = row & 1;
   float a1, a2;
@@ -436,7 +438,7 @@ __device__ __noinline__ void encode_queued_pair(float tau, float eps_ratio, uint
   }
   mn = fminf(mn, __shfl_xor_sync(kFull, mn, 1));
   mx = fmaxf(mx, __shfl_xor_sync(kFull, mx, 1));
-  const Quantiser q = make_quantiser(mn, mx, bits);
+  const Quantiser q = make_quantiser(mn, mx, bits, hi, wc);
   if constexpr (SR) {
     float dd[C::EPT];
 #pragma unroll
@@ -562,6 +564,7 @@ __global__ void __launch_bounds__(kThreads, 2) quant2_kernel(const Args a, const
   const uint64_t row_bytes = (uint64_t)C::ROWB;
   const bool narrow = NARROW;
   const uint32_t lo = a.lo;
+  const WidthOf<C> wc(lo);
 
   // fetch the rows of the first n (<= 32) queued tiles again; lane j keeps the j-th tile's particulars
   auto gather = [&](uint32_t n) {
@@ -586,7 +589,7 @@ __global__ void __launch_bounds__(kThreads, 2) quant2_kernel(const Args a, const
       if ((uint32_t)lane < f_n) {
         const uint64_t tile = tile_cta + (f_tile >> 1);
         const uint64_t off = (uint64_t)kTB * ((uint64_t)lo * tile + f_hib);
-        encode_queued_row<C, SR>(a.tau, a.eps_ratio, fstage, lane, lo + (f_tile & 1u), narrow,
+        encode_queued_row<C, SR>(a.tau, a.eps_ratio, fstage, lane, lo + (f_tile & 1u), (f_tile & 1u) != 0u, wc, narrow,
                                  reinterpret_cast<uint32_t *>(payload + off), sz32 + tile, pivot + tile, a.seed,
                                  tile * (unsigned long long)C::G);
       }
@@ -595,7 +598,7 @@ __global__ void __launch_bounds__(kThreads, 2) quant2_kernel(const Args a, const
       const uint64_t tile = live ? tile_cta + (f_tile >> 2) : 0;
       const uint32_t bits = lo + (f_tile & 1u);
       const uint64_t off = live ? (uint64_t)kTB * ((uint64_t)lo * tile + f_hib) + (uint64_t)half * (C::EPT / 8) * bits : 0;
-      encode_queued_pair<C, SR>(a.tau, a.eps_ratio, fstage, lane, live, bits, narrow,
+      encode_queued_pair<C, SR>(a.tau, a.eps_ratio, fstage, lane, live, bits, (f_tile & 1u) != 0u, wc, narrow,
                                 reinterpret_cast<uint32_t *>(payload + off), sz32 + tile, pivot + tile, a.seed,
                                 tile * (unsigned long long)C::G + (unsigned)(half * C::EPT));
     }
@@ -655,7 +658,7 @@ __global__ void __launch_bounds__(kThreads, 2) quant2_kernel(const Args a, const
     if (live && !maybe) {
       const uint64_t tile = tile_cta + trel / R;
       const uint64_t off = (uint64_t)kTB * ((uint64_t)lo * tile + hib) + (uint64_t)half * (C::EPT / 8) * (lo + hi);
-      const uint32_t szw = encode_plain_words<C, SR>(w, mn, mx, lo + hi, narrow, reinterpret_cast<uint32_t *>(payload + off),
+      const uint32_t szw = encode_plain_words<C, SR>(w, mn, mx, lo + hi, hi != 0u, wc, narrow, reinterpret_cast<uint32_t *>(payload + off),
                                                      a.seed, tile * (unsigned long long)C::G + (unsigned)(half * C::EPT));
       if (R == 1 || half == 0) {
         sz32[tile] = szw;

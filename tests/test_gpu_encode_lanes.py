@@ -1,0 +1,49 @@
+"""The quantiser's reciprocal and division against the correctly rounded ones, over every scale and every width (one tile
+per scale whose range makes the scale); bf16 on both sides of the size where the tile kernel changes."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2506_01352_b200 import binding as T
+from tests.test_gpu_parity import check_decode, check_encode
+
+pytestmark = pytest.mark.gpu
+
+
+def check(x, **kw):
+    p = T.params_for(x, **kw)
+    packed, want, ws = check_encode(p, x)
+    check_decode(p, packed, want, ws)
+
+
+@pytest.mark.parametrize("bits", [2, 3, 4, 5, 6, 7, 8])
+def test_every_binary16_scale(bits):
+    """Tile j holds 32 values between 0 and scale j times 2^bits - 1 (as far as binary16 goes), some of them on and around
+    the midpoints between codes, where a reciprocal that is one unit off gives another code."""
+    s = np.arange(1, 0x7C00, dtype=np.uint16).view(np.float16).astype(np.float64)
+    q = 2 ** bits - 1
+    s = s[s * q < 60000]
+    x = (s[:, None] * (np.arange(32) % q + 0.5)[None, :]).astype(np.float32)
+    x[:, 0] = 0
+    x[:, 1] = (s * q).astype(np.float32)
+    x[:, 2::3] = np.nextafter(x[:, 2::3], np.float32(0))
+    x[:, 3::3] = np.nextafter(x[:, 3::3], np.float32(1e9))
+    n = len(x) // 8 * 8
+    check(torch.from_numpy(x[:n].reshape(n // 8, 256)).cuda(), tile=32, budget_millibits=bits * 1000, tau=float("inf"))
+
+
+@pytest.mark.parametrize("bits", [2, 3, 4, 5, 6, 7, 8])
+def test_ranges_that_round_both_ways(bits):
+    g = torch.Generator(device="cuda").manual_seed(bits)
+    x = torch.randn(3000, 256, generator=g, device="cuda") * torch.randn(3000, 1, generator=g, device="cuda").mul(9).exp()
+    check(x, tile=32, budget_millibits=bits * 1000)
+
+
+@pytest.mark.parametrize("G,tokens", [(32, 2959), (32, 2961), (64, 2959), (64, 2961), (128, 1479), (128, 1481)])
+@pytest.mark.parametrize("rounding", [0, 1])
+def test_bf16_around_two_rounds_per_warp(G, tokens, rounding):
+    """148 SMs x 20 warps x 2 rounds of 32, 16 or 8 tiles: 64, 32 or 32 tiles to a token put the line at 2960, 2960, 1480."""
+    g = torch.Generator(device="cuda").manual_seed(G)
+    x = torch.randn(tokens, G * (64 if G == 32 else 32), generator=g, device="cuda")
+    x[:, ::41] *= 30
+    check(x.bfloat16(), tile=G, budget_millibits=3600, rounding=rounding, seed=5)
