@@ -407,6 +407,99 @@ __global__ void __launch_bounds__(kLaneThreads, 1) decode_lanes_kernel(const Arg
   if (qn) decode_flagged_round<C, NARROW, WIDE_ST>(q_codes, q_info, rows, qhead, qn, out_cta);
 }
 
+// A lane's 64 bytes of the tensor, aligned to 16 or (WIDE) 32 bytes.
+template <bool WIDE>
+__device__ __forceinline__ void load_64_bytes(const uint8_t *src, uint32_t (&w)[16]) {
+  if constexpr (WIDE) {
+#pragma unroll
+    for (int i = 0; i < 16; i += 8)
+      asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                   : "=r"(w[i]), "=r"(w[i + 1]), "=r"(w[i + 2]), "=r"(w[i + 3]), "=r"(w[i + 4]), "=r"(w[i + 5]), "=r"(w[i + 6]),
+                     "=r"(w[i + 7])
+                   : "l"(src + 4 * i));
+  } else {
+#pragma unroll
+    for (int i = 0; i < 16; i += 4) {
+      const uint4 v = __ldg(reinterpret_cast<const uint4 *>(src + 4 * i));
+      w[i] = v.x; w[i + 1] = v.y; w[i + 2] = v.z; w[i + 3] = v.w;
+    }
+  }
+}
+
+// ------------------------------------------------------------------------------------------
+// Eq. 1-2, screening scores (see tile_score_screen for the formula and its error)
+// ------------------------------------------------------------------------------------------
+constexpr int kScoreThreads = 512;   // two CTAs on an SM
+
+// For bfloat16.  Bound by DRAM, with the logarithms (one MUFU instruction per element, 16 lanes a cycle and SM) close
+// behind: what counts is that both run at once.  With a lane per tile, rows in shared memory and 8 warps on an SM they took
+// turns: 8192 x 4096 15.4 -> 14.5 us, 65536 x 8192 201 -> 188 us, 4096 x 4096 in tiles of 128 8.4 -> 7.1 us, 16384 x 8192 in
+// tiles of 32 57.4 -> 49.1 us.  Two rounds ahead instead of one, or three CTAs of 384 threads, are no faster; binary32,
+// whose lanes lie 64 bytes apart at half the elements, is slower this way (33 MB 4.7 -> 7.4 us) and keeps score_kernel.
+template <class C, bool WIDE>
+__global__ void __launch_bounds__(kScoreThreads, 2) score_lanes_kernel(const Args a) {
+  using D = LaneCfg<C>;
+  static_assert(C::BF16, "binary32: score_kernel");
+  constexpr int P = D::P, TPR = D::TPR;
+  constexpr uint32_t WARPS = kScoreThreads / 32;
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, sub = lane % P;
+  TraceScope trace(a.trace, 1);
+  const uint32_t n_tiles = (uint32_t)a.n_tiles, n_rounds = (n_tiles + TPR - 1) / TPR;
+  const uint32_t r0 = (uint32_t)((uint64_t)n_rounds * blockIdx.x / gridDim.x);
+  // The CTA's rounds are read back to front: the rows read last are the ones the encoder, which walks the tensor front to
+  // back right afterwards, asks for first, while they are still in L2.
+  const uint32_t r1 = (uint32_t)((uint64_t)n_rounds * (blockIdx.x + 1u) / gridDim.x);
+  uint32_t raw[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) raw[i] = 0;
+  auto load = [&](uint32_t r) {
+    const uint32_t tile = r * TPR + lane / P;
+    if (tile < n_tiles) load_64_bytes<WIDE>(a.in + (uint64_t)tile * D::TB + sub * 64u, raw);
+  };
+  grid_dependency_wait();   // the tensor may be the work of the kernel in front
+  trace.started();
+  if (blockIdx.x == 0 && threadIdx.x == 0) *a.status = 0;   // nothing else of the workspace has to start at zero
+  uint32_t left = r1 - r0 > warp ? r1 - r0 - warp : 0u;     // the warp's next round is r0 + left - 1
+  if (left) load(r0 + left - 1u);
+  while (left) {
+    uint32_t w[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) w[i] = raw[i];
+    const uint32_t r = r0 + left - 1u;
+    left = left > WARPS ? left - WARPS : 0u;
+    if (left) load(r0 + left - 1u);
+    const float tiny = 1e-30f;
+    constexpr int NP = D::E / 2, NC = 4;   // pairs; chains that sum them
+    float2 L[NC], T[NC];
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+      float2 v;
+      bf2_add_f32(w[i] & 0x7fff7fffu, tiny, v.x, v.y);
+      const float2 l = f2(lg2_approx(v.x), lg2_approx(v.y));
+      const int c = i % NC;
+      if (i < NC) {
+        L[c] = v;
+        T[c] = f2(v.x * l.x, v.y * l.y);   // (scalar products: they feed the fused chain's addend)
+      } else {
+        L[c] = add2(L[c], v);
+        T[c] = fma2(v, l, T[c]);
+      }
+    }
+    const float2 L2 = add2(add2(L[0], L[1]), add2(L[2], L[3])), T2 = add2(add2(T[0], T[1]), add2(T[2], T[3]));
+    float Ls = L2.x + L2.y, Ts = T2.x + T2.y;
+#pragma unroll
+    for (int h = 1; h < P; h *= 2) {
+      Ls += __shfl_xor_sync(kFull, Ls, h);
+      Ts += __shfl_xor_sync(kFull, Ts, h);
+    }
+    const float Lp = Ls + a.eps_l1;
+    float rc;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rc) : "f"(Lp));
+    const uint32_t tile = r * TPR + lane / P;
+    if (sub == 0 && tile < n_tiles) a.scores[tile] = __fmaf_rn(lg2_approx(Lp), Ls, -Ts) * rc;
+  }
+}
+
 // ------------------------------------------------------------------------------------------
 // Quantise + pack (Eq. 3-4, Sec. 3.3-3.4)
 //
@@ -426,25 +519,6 @@ struct QuantLanes {
   static constexpr int WARP = 64 * (64 + 8);
   static constexpr int SMEM = WARPS * WARP;
 };
-
-// A lane's 64 bytes of the tensor, aligned to 16 or (WIDE) 32 bytes.
-template <bool WIDE>
-__device__ __forceinline__ void load_64_bytes(const uint8_t *src, uint32_t (&w)[16]) {
-  if constexpr (WIDE) {
-#pragma unroll
-    for (int i = 0; i < 16; i += 8)
-      asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                   : "=r"(w[i]), "=r"(w[i + 1]), "=r"(w[i + 2]), "=r"(w[i + 3]), "=r"(w[i + 4]), "=r"(w[i + 5]), "=r"(w[i + 6]),
-                     "=r"(w[i + 7])
-                   : "l"(src + 4 * i));
-  } else {
-#pragma unroll
-    for (int i = 0; i < 16; i += 4) {
-      const uint4 v = __ldg(reinterpret_cast<const uint4 *>(src + 4 * i));
-      w[i] = v.x; w[i + 1] = v.y; w[i + 2] = v.z; w[i + 3] = v.w;
-    }
-  }
-}
 
 // Codes of a lane -> the tile's bit stream.  t(k) = q_k + 1.5*2^23 for a compile-time k; `dst` = the tile's first word.
 // 16 codes of an odd width end in the middle of a word, which the lane shares with its neighbour: the even lane of the

@@ -17,21 +17,28 @@ static tahq_status encode_t(const Plan &pl, const Args &a_in, cudaStream_t st) {
   if (pl.mixed) {
     if (pl.alloc_m > 1) {   // Sec. 3.2 with A = m * G: one warp per allocation tile, exact scores
       if (launch_alloc_score(a, d, st) != TAHQ_OK) return TAHQ_ERR_CUDA;
+    } else if (C::G >= 32 && C::BF16 && !a.exact_scores) {
+      if constexpr (C::G >= 32 && C::BF16) {
+        const bool wide_ld = (reinterpret_cast<uintptr_t>(a.in) & 31u) == 0;   // 256-bit loads where the tensor is aligned to them
+        const uint64_t n_rounds = (a.n_tiles + LaneCfg<C>::TPR - 1) / LaneCfg<C>::TPR;
+        const unsigned grid = persistent_grid((n_rounds + 3) / 4, d, 2);
+        if (wide_ld) TAHQ_LAUNCH("stats", st, launch_dependent(score_lanes_kernel<C, true>, grid, kScoreThreads, 0, st, a));
+        else TAHQ_LAUNCH("stats", st, launch_dependent(score_lanes_kernel<C, false>, grid, kScoreThreads, 0, st, a));
+      }
     } else {
       constexpr int NS = C::ROWB <= 128 ? 3 : 2;
       const int smem = kWarps * NS * StreamCfg<C>::UNIT_BYTES + 256;   // ring slots, then the warps' mbarriers
       static std::atomic<int> occ_sc[64], occ_sc_exact[64];
-      const int occ = a.exact_scores ? prepare(score_kernel<C, NS, true>, kThreads, smem, d, occ_sc_exact)
-                                     : prepare(score_kernel<C, NS, false>, kThreads, smem, d, occ_sc);
-      if (!occ) return TAHQ_ERR_CUDA;
       const uint64_t n_units = (a.n_tiles * C::LPT + 31) / 32;
       // one CTA per SM: the kernel is bound by DRAM, and fewer, longer streams measured a little faster
-      // (15.8 against 16.4 us on the LLaMA-7B shape)
       const unsigned grid = persistent_grid((n_units + kWarps - 1) / kWarps, d, 1);
-      if (a.exact_scores)
+      if (a.exact_scores) {
+        if (!prepare(score_kernel<C, NS, true>, kThreads, smem, d, occ_sc_exact)) return TAHQ_ERR_CUDA;
         TAHQ_LAUNCH("stats", st, launch_dependent(score_kernel<C, NS, true>, grid, kThreads, smem, st, a, tmap));
-      else
+      } else if constexpr (C::G < 32 || !C::BF16) {
+        if (!prepare(score_kernel<C, NS, false>, kThreads, smem, d, occ_sc)) return TAHQ_ERR_CUDA;
         TAHQ_LAUNCH("stats", st, launch_dependent(score_kernel<C, NS, false>, grid, kThreads, smem, st, a, tmap));
+      }
     }
     if (launch_select(a, d, st) != TAHQ_OK) return TAHQ_ERR_CUDA;
   }

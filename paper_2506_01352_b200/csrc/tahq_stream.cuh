@@ -161,44 +161,9 @@ __device__ __forceinline__ void words_minmax(const uint32_t (&w)[C::ROWB / 4], f
 }
 
 // ------------------------------------------------------------------------------------------
-// Eq. 1-2: scores only, no group boundaries -- a warp streams units of 32 rows and stores their scores.
+// Eq. 1-2: scores only, no group boundaries -- a warp streams units of 32 rows and stores their scores.  (Screening
+// scores of bfloat16 tiles of 32 and more: score_lanes_kernel.)
 // ------------------------------------------------------------------------------------------
-
-// Screening score (see tile_score_screen for the formula and its error) of a row of bfloat16 held as raw
-// words, two elements per packed instruction where the arithmetic allows: per group of eight elements the
-// products a*log2(a) are summed in two chains of four, the magnitudes in a pairwise tree (the summation
-// order of this approximation is free; these are no longer than the ones its error bound was derived for).
-template <int NW, int LPT>
-__device__ __forceinline__ float screen_score_words_bf16(const uint32_t (&w)[NW], float eps_l1) {
-  constexpr int NO = NW / 4;   // groups of eight elements
-  const float tiny = 1e-30f;
-  float pl[NO], pt[NO];
-#pragma unroll
-  for (int o = 0; o < NO; ++o) {
-    float2 v[4], l[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      bf2_add_f32(w[4 * o + j] & 0x7fff7fffu, tiny, v[j].x, v[j].y);
-      l[j] = f2(lg2_approx(v[j].x), lg2_approx(v[j].y));
-    }
-    float2 t = f2(v[0].x * l[0].x, v[0].y * l[0].y);   // (scalar products: they feed the fused chain's addend)
-#pragma unroll
-    for (int j = 1; j < 4; ++j) t = fma2(v[j], l[j], t);
-    pt[o] = t.x + t.y;
-    const float2 s01 = add2(v[0], v[1]), s23 = add2(v[2], v[3]);
-    const float2 s = add2(s01, s23);
-    pl[o] = s.x + s.y;
-  }
-  float L = tree<NO>(pl), T = tree<NO>(pt);
-  if constexpr (LPT == 2) {   // the two halves of a 128-wide tile
-    L = L + __shfl_xor_sync(kFull, L, 1);
-    T = T + __shfl_xor_sync(kFull, T, 1);
-  }
-  const float Lp = L + eps_l1;
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(Lp));
-  return __fmaf_rn(lg2_approx(Lp), L, -T) * r;
-}
 
 template <class C, int NST, bool EXACT>
 __global__ void __launch_bounds__(kThreads, 2) score_kernel(const Args a, const __grid_constant__ CUtensorMap tmap) {
@@ -232,25 +197,12 @@ __global__ void __launch_bounds__(kThreads, 2) score_kernel(const Args a, const 
     const uint64_t u = unit_of(k);
     ring.wait(a, slot);
     const uint8_t *stage = ring.slot(slot);
-    float s;
-    if constexpr (!EXACT && C::BF16 && C::EPT >= 32) {
-      uint32_t w[S::WORDS];
-      row_load_words<C>(stage, lane, w);
-      __syncwarp();
-      {
-        const uint32_t kn = k + (uint32_t)NST * stride;
-        if (kn < nu) ring.issue(a, unit_of(kn), slot);
-        ring.commit();
-      }
-      s = screen_score_words_bf16<S::WORDS, C::LPT>(w, a.eps_l1);
-    } else {
-      s = EXACT ? tile_score<C>(stage, lane, a.eps_l1, a.eps_log) : tile_score_screen<C>(stage, lane, a.eps_l1);
-      __syncwarp();
-      {
-        const uint32_t kn = k + (uint32_t)NST * stride;
-        if (kn < nu) ring.issue(a, unit_of(kn), slot);
-        ring.commit();
-      }
+    const float s = EXACT ? tile_score<C>(stage, lane, a.eps_l1, a.eps_log) : tile_score_screen<C>(stage, lane, a.eps_l1);
+    __syncwarp();
+    {
+      const uint32_t kn = k + (uint32_t)NST * stride;
+      if (kn < nu) ring.issue(a, unit_of(kn), slot);
+      ring.commit();
     }
     slot = (slot + 1 == NST) ? 0 : slot + 1;
     const uint64_t tile = (u * 32 + lane) / C::LPT;
