@@ -208,8 +208,8 @@ tahq_status tahq_decode(const tahq_params *p, const void *d_packed, size_t packe
   fill_args(p, pl, static_cast<uint8_t *>(d_ws), &a);
   a.packed = const_cast<uint8_t *>(static_cast<const uint8_t *>(d_packed));
   a.out = static_cast<uint8_t *>(d_out);
-  // Up to 65536 bit-map words (256 KiB) the streaming kernel needs no look-back and nothing cleared: one launch.
-  a.own_prefix = (pl.L.n_tiles + 31) / 32 <= 65536;
+  // Up to 65536 bit-map words (256 KiB), and with one width, the kernels need no look-back and nothing cleared: one launch.
+  a.own_prefix = (p->tile >= 32 && !pl.mixed) || (pl.L.n_tiles + 31) / 32 <= 65536;
   if (!a.own_prefix && launch_clear(d_ws, pl.ws_zero_end, st) != TAHQ_OK) return TAHQ_ERR_CUDA;   // status + flags
   const bool bf = p->dtype == TAHQ_BF16;
   switch (p->tile) {

@@ -228,14 +228,16 @@ __device__ __forceinline__ void decode_flagged_round(const uint32_t *q_codes, co
   if (lane < n) store_64_bytes<WIDE_ST>(out_cta + (uint64_t)info.y * D::TB, o);
 }
 
-template <class C, bool NARROW, bool WIDE_ST>
+// MIXED: two widths in use.  With one, no offset depends on the bit map, and the codes are asked for along with the header
+// (256 x 1344 fp32 at 3 bits 4.2 -> 2.0 us, 8192 x 2048 bf16 at 4 bits 11.0 -> 10.0 us), and no call needs the look-back.
+template <class C, bool NARROW, bool WIDE_ST, bool MIXED>
 __global__ void __launch_bounds__(kLaneThreads, 1) decode_lanes_kernel(const Args a) {
   using D = LaneCfg<C>;
   using S = DecodeLanes<C, NARROW>;
   constexpr int NT = kLaneThreads, E = D::E, P = D::P, TPR = D::TPR, NWORD = S::NWORD;
   constexpr uint32_t kTB = C::G / 8;   // bytes of a tile's codes per bit of width
   extern __shared__ __align__(128) uint8_t smem_dl[];
-  __shared__ uint2 s_word[NT];         // the segment's bit-map words, higher-width tiles of the CTA in front of each
+  __shared__ uint2 s_word[MIXED ? NT : 1];         // the segment's bit-map words, higher-width tiles of the CTA in front of each
   __shared__ uint32_t s_sum[2][32];    // per warp: set bits of its words of the segment, of its share of the words in front
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t sub = (uint32_t)lane % P;   // this lane's part of its tile
@@ -259,13 +261,12 @@ __global__ void __launch_bounds__(kLaneThreads, 1) decode_lanes_kernel(const Arg
   const bool checks = blockIdx.x == 0 || a.own_prefix;
   const uint32_t hdr_w = (checks && threadIdx.x < 32) ? __ldg(reinterpret_cast<const uint32_t *>(a.packed) + threadIdx.x) : 0u;
   auto bm_word = [&](uint64_t i) -> uint32_t {   // bits beyond the last tile cleared
-    if (!a.mixed) return 0u;
     const uint64_t left = a.n_tiles - i * 32;
     return __ldg(bitmap + i) & (left >= 32u ? 0xffffffffu : ((1u << (uint32_t)left) - 1u));
   };
-  uint32_t word = u0 + threadIdx.x < u1 ? bm_word(u0 + threadIdx.x) : 0u;
+  uint32_t word = MIXED && u0 + threadIdx.x < u1 ? bm_word(u0 + threadIdx.x) : 0u;
   uint32_t front = 0;   // a.own_prefix: this thread's share of the higher-width tiles in front of the CTA's words
-  if (a.own_prefix && a.mixed) {   // 128-bit loads, four in flight per thread, then the last few words one by one
+  if (MIXED && a.own_prefix) {   // 128-bit loads, four in flight per thread, then the last few words one by one
     const uint4 *b4 = reinterpret_cast<const uint4 *>(bitmap);
     const uint32_t n4 = (uint32_t)(u0 / 4);
     for (uint32_t i = threadIdx.x; i < n4; i += 4u * NT) {
@@ -284,97 +285,110 @@ __global__ void __launch_bounds__(kLaneThreads, 1) decode_lanes_kernel(const Arg
   }
 
   const bool wrong = checks && threadIdx.x < 32 && hdr_w != a.header[threadIdx.x];
-  const uint8_t *pay = nullptr;   // the CTA's first code
   bool stop = false;
   uint32_t seg_hi = 0;   // higher-width tiles of this CTA's earlier segments
-  uint32_t pay_left = 0;   // bytes of the payload from the CTA's first code (a corrupt bit map must not lead outside)
   uint32_t qhead = 0, qn = 0;
   const uint32_t *const sz_cta = reinterpret_cast<const uint32_t *>(a.packed + a.off_sz) + tile_cta;
   const uint8_t *const pv_cta = a.packed + a.off_pivot + tile_cta;
   uint8_t *const out_cta = a.out + tile_cta * (uint64_t)D::TB + sub * 64u;
   const uint32_t n_rel = a.n_tiles - tile_cta < 0xffffffffull ? (uint32_t)(a.n_tiles - tile_cta) : 0xffffffffu;
 
-  for (uint64_t s0 = u0; s0 < u1; s0 += NT) {
-    const uint64_t s1 = s0 + NT < u1 ? s0 + NT : u1;
-    if (s0 != u0) {
-      word = s0 + threadIdx.x < u1 ? bm_word(s0 + threadIdx.x) : 0u;
-      __syncthreads();   // every warp is done with the previous segment's words
+  const uint8_t *pay = a.packed + a.off_payload + (uint64_t)kTB * a.lo * tile_cta;   // the CTA's first code (less the higher widths' bits)
+  uint32_t pay_left = 0;   // bytes of the payload from the CTA's first code (a corrupt bit map must not lead outside)
+  // a warp's rounds take the same bits of their words
+  uint32_t t = (uint32_t)((r0 + warp) % P) * TPR + (uint32_t)lane / P, bit = 1u << t, below = bit - 1u;
+  uint32_t w[NWORD], sz, wp;   // the next round: codes; scale and zero-point; width + 16 * pivot byte, 0: no tile
+  auto load = [&](uint32_t kk, uint32_t seg_tile) {   // round kk of the segment whose first word's tile `t` is seg_tile
+    const uint2 bw = MIXED ? s_word[kk / P] : make_uint2(0u, 0u);
+    const uint32_t tile = seg_tile + kk / P * 32u, W = a.lo + ((bw.x & bit) ? 1u : 0u);
+    const uint32_t off = kTB * (a.lo * tile + bw.y + (uint32_t)__popc(bw.x & below));
+    wp = 0;
+    if (tile < n_rel) {
+      load_codes<E, NWORD>(reinterpret_cast<const uint32_t *>(pay + off), sub, W, w);
+      sz = __ldg(sz_cta + tile);
+      wp = W | (uint32_t)__ldg(pv_cta + tile) << 4;
     }
-    // running count over the segment's words, one per thread; the words in front
-    uint32_t incl = (uint32_t)__popc(word);
-#pragma unroll
-    for (int o = 1; o < 32; o *= 2) {
-      const uint32_t v = __shfl_up_sync(kFull, incl, o);
-      if (lane >= o) incl += v;
-    }
-    front = __reduce_add_sync(kFull, front);
-    if (lane == 31) { s_sum[0][warp] = incl; s_sum[1][warp] = front; }
-    const bool refuse = __syncthreads_or(wrong) != 0;
-    const uint32_t sw = lane < kLaneWarps ? s_sum[0][lane] : 0u;
-    const uint32_t before = __reduce_add_sync(kFull, lane < warp ? sw : 0u), total = __reduce_add_sync(kFull, sw);
-    s_word[threadIdx.x] = make_uint2(word, seg_hi + before + incl - (uint32_t)__popc(word));
-    if (s0 == u0) {   // Sec. 3.4: higher-width tiles in front of the CTA's words; what was found in the header
-      // CTA 0 compares the received header with the one these parameters produce; what it finds travels with the
-      // offset prefix, so a refused buffer leaves the output untouched.  (a.own_prefix: every CTA does this itself
-      // and counts the bit map in front of its slice itself: nothing has to be cleared beforehand, and the last CTA,
-      // which sees the whole count, writes the status.)
-      const bool last = blockIdx.x == gridDim.x - 1 && threadIdx.x == 0;
-      uint64_t base_hi;
-      if (a.own_prefix) {
-        base_hi = __reduce_add_sync(kFull, lane < kLaneWarps ? s_sum[1][lane] : 0u);
-        stop = refuse;
-        if (last)   // (at most 65536 words: one segment)
-          *a.status = (refuse ? 1u /* TAHQ_DEV_BAD_HEADER */ : 0u) |
-                      ((a.mixed && !refuse && base_hi + total != a.n_groups * a.k_hi) ? 2u /* TAHQ_DEV_BAD_BITMAP */ : 0u);
-      } else {
-        // a CTA publishes the count of the words that start in its range (one shared by two CTAs counts in the first)
-        if (refuse && threadIdx.x == 0) atomicOr(a.status, 1u);
-        const uint64_t uc0 = (r0 + P - 1) / P;
-        uint32_t n = 0;
-        for (uint64_t i = uc0 + threadIdx.x; i < u1; i += NT) n += __popc(bm_word(i));
-        n = block_sum<NT>(n);
-        base_hi = cta_exclusive_prefix<NT>(a, n, refuse, stop);
-        if (last && a.mixed && !stop && base_hi + n != a.n_groups * a.k_hi) atomicOr(a.status, 2u);
-        if (uc0 != u0) base_hi -= (uint32_t)__popc(bm_word(u0));
-      }
-      const uint64_t pay0 = (uint64_t)kTB * ((uint64_t)a.lo * tile_cta + base_hi);
-      if (pay0 < a.payload_bytes) {
-        pay = a.packed + a.off_payload + pay0;
-        pay_left = a.payload_bytes - pay0 < 0xffffffffull ? (uint32_t)(a.payload_bytes - pay0) : 0xffffffffu;
-      }
-    }
-    __syncthreads();
-    if (stop) return;
+  };
+  if constexpr (!MIXED) {
+    const uint32_t k = (uint32_t)(r0 - u0 * P) + warp;
+    if (k < (uint32_t)(r1 - u0 * P)) load(k, t);
+    const bool refuse = __syncthreads_or(wrong) != 0;   // every CTA for itself (a.own_prefix)
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *a.status = refuse ? 1u /* TAHQ_DEV_BAD_HEADER */ : 0u;
+    if (refuse) return;
+  }
 
-    // the warp's rounds; their tiles take the same bits of their words
-    const uint64_t rs0 = s0 * P > r0 ? s0 * P : r0, rs1 = s1 * P < r1 ? s1 * P : r1;
-    const uint32_t k1 = (uint32_t)(rs1 - s0 * P);
-    uint32_t k = (uint32_t)(rs0 - s0 * P) + warp;
-    const uint32_t t = k % P * TPR + (uint32_t)lane / P, bit = 1u << t, below = bit - 1u;
-    const uint32_t seg_tile = (uint32_t)(s0 - u0) * 32u + t;   // from the CTA's first
-    {   // does the segment's last code lie inside the payload?  If not, the bit map is corrupt and the rest is left out.
+  for (uint64_t s0 = u0, s1; s0 < u1; s0 = s1) {
+    s1 = MIXED && s0 + NT < u1 ? s0 + NT : u1;
+    uint32_t total = 0;
+    if constexpr (MIXED) {
+      if (s0 != u0) {
+        word = s0 + threadIdx.x < u1 ? bm_word(s0 + threadIdx.x) : 0u;
+        __syncthreads();   // every warp is done with the previous segment's words
+      }
+      // running count over the segment's words, one per thread; the words in front
+      uint32_t incl = (uint32_t)__popc(word);
+#pragma unroll
+      for (int o = 1; o < 32; o *= 2) {
+        const uint32_t v = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += v;
+      }
+      front = __reduce_add_sync(kFull, front);
+      if (lane == 31) { s_sum[0][warp] = incl; s_sum[1][warp] = front; }
+      const bool refuse = __syncthreads_or(wrong) != 0;
+      const uint32_t sw = lane < kLaneWarps ? s_sum[0][lane] : 0u;
+      const uint32_t before = __reduce_add_sync(kFull, lane < warp ? sw : 0u);
+      total = __reduce_add_sync(kFull, sw);
+      s_word[threadIdx.x] = make_uint2(word, seg_hi + before + incl - (uint32_t)__popc(word));
+      if (s0 == u0) {   // Sec. 3.4: higher-width tiles in front of the CTA's words; what was found in the header
+        // CTA 0 compares the received header with the one these parameters produce; what it finds travels with the
+        // offset prefix, so a refused buffer leaves the output untouched.  (a.own_prefix: every CTA does this itself
+        // and counts the bit map in front of its slice itself: nothing has to be cleared beforehand, and the last CTA,
+        // which sees the whole count, writes the status.)
+        const bool last = blockIdx.x == gridDim.x - 1 && threadIdx.x == 0;
+        uint64_t base_hi;
+        if (a.own_prefix) {
+          base_hi = __reduce_add_sync(kFull, lane < kLaneWarps ? s_sum[1][lane] : 0u);
+          stop = refuse;
+          if (last)   // (at most 65536 words: one segment)
+            *a.status = (refuse ? 1u /* TAHQ_DEV_BAD_HEADER */ : 0u) |
+                        ((!refuse && base_hi + total != a.n_groups * a.k_hi) ? 2u /* TAHQ_DEV_BAD_BITMAP */ : 0u);
+        } else {
+          // a CTA publishes the count of the words that start in its range (one shared by two CTAs counts in the first)
+          if (refuse && threadIdx.x == 0) atomicOr(a.status, 1u);
+          const uint64_t uc0 = (r0 + P - 1) / P;
+          uint32_t n = 0;
+          for (uint64_t i = uc0 + threadIdx.x; i < u1; i += NT) n += __popc(bm_word(i));
+          n = block_sum<NT>(n);
+          base_hi = cta_exclusive_prefix<NT>(a, n, refuse, stop);
+          if (last && !stop && base_hi + n != a.n_groups * a.k_hi) atomicOr(a.status, 2u);
+          if (uc0 != u0) base_hi -= (uint32_t)__popc(bm_word(u0));
+        }
+        const uint64_t pay0 = (uint64_t)kTB * ((uint64_t)a.lo * tile_cta + base_hi);
+        if (pay0 < a.payload_bytes) {
+          pay += (uint64_t)kTB * base_hi;
+          pay_left = a.payload_bytes - pay0 < 0xffffffffull ? (uint32_t)(a.payload_bytes - pay0) : 0xffffffffu;
+        }
+      }
+      __syncthreads();
+      if (stop) return;
+      // does the segment's last code lie inside the payload?  If not, the bit map is corrupt and the rest is left out.
       const uint32_t tiles = (uint32_t)(s1 - u0) * 32u;
       if ((uint64_t)kTB * ((uint64_t)a.lo * (tiles < n_rel ? tiles : n_rel) + seg_hi + total) > pay_left) return;
     }
-    uint32_t w[NWORD], sz, wp;   // the next round: codes; scale and zero-point; width + 16 * pivot byte, 0: no tile
-    auto load = [&](uint32_t kk) {
-      const uint2 bw = s_word[kk / P];
-      const uint32_t tile = seg_tile + kk / P * 32u, W = a.lo + ((bw.x & bit) ? 1u : 0u);
-      const uint32_t off = kTB * (a.lo * tile + bw.y + (uint32_t)__popc(bw.x & below));
-      wp = 0;
-      if (tile < n_rel) {
-        load_codes<E, NWORD>(reinterpret_cast<const uint32_t *>(pay + off), sub, W, w);
-        sz = __ldg(sz_cta + tile);
-        wp = W | (uint32_t)__ldg(pv_cta + tile) << 4;
-      }
-    };
-    if (k < k1) load(k);
+
+    // the warp's rounds
+    const uint64_t rs0 = s0 * P > r0 ? s0 * P : r0, rs1 = s1 * P < r1 ? s1 * P : r1;
+    const uint32_t k1 = (uint32_t)(rs1 - s0 * P);
+    uint32_t k = (uint32_t)(rs0 - s0 * P) + warp;
+    if (MIXED) { t = k % P * TPR + (uint32_t)lane / P; bit = 1u << t; below = bit - 1u; }
+    const uint32_t seg_tile = (uint32_t)(s0 - u0) * 32u + t;   // from the CTA's first
+    if (MIXED && k < k1) load(k, seg_tile);
     for (; k < k1; k += kLaneWarps) {
       uint32_t cw[NWORD];
 #pragma unroll
       for (int j = 0; j < NWORD; ++j) cw[j] = w[j];
       const uint32_t csz = sz, cwp = wp, tile = seg_tile + k / P * 32u;
-      if (k + kLaneWarps < k1) load(k + kLaneWarps);
+      if (k + kLaneWarps < k1) load(k + kLaneWarps, seg_tile);
       const bool flagged = (cwp & 0x800u) != 0;
       const unsigned held = __ballot_sync(kFull, flagged);
       if (flagged) {   // put aside

@@ -82,10 +82,13 @@ static tahq_status decode_t(const Plan &pl, const Args &a, cudaStream_t st) {
   if constexpr (C::G >= 32) {
     // no width above 4 bits: the kernel compiled for just that; 256-bit stores where the tensor is aligned to them
     const bool narrow = a.lo + a.mixed <= 4u, wide_st = (reinterpret_cast<uintptr_t>(a.out) & 31u) == 0;
-    void (*const kernels[4])(Args) = {decode_lanes_kernel<C, false, false>, decode_lanes_kernel<C, false, true>,
-                                      decode_lanes_kernel<C, true, false>, decode_lanes_kernel<C, true, true>};
-    static std::atomic<int> occ[4][64];
-    const int k = 2 * narrow + wide_st, smem = narrow ? DecodeLanes<C, true>::SMEM : DecodeLanes<C, false>::SMEM;
+    void (*const kernels[8])(Args) = {
+        decode_lanes_kernel<C, false, false, false>, decode_lanes_kernel<C, false, true, false>,
+        decode_lanes_kernel<C, true, false, false>,  decode_lanes_kernel<C, true, true, false>,
+        decode_lanes_kernel<C, false, false, true>,  decode_lanes_kernel<C, false, true, true>,
+        decode_lanes_kernel<C, true, false, true>,   decode_lanes_kernel<C, true, true, true>};
+    static std::atomic<int> occ[8][64];
+    const int k = 4 * a.mixed + 2 * narrow + wide_st, smem = narrow ? DecodeLanes<C, true>::SMEM : DecodeLanes<C, false>::SMEM;
     if (!prepare(kernels[k], kLaneThreads, smem, d, occ[k])) return TAHQ_ERR_CUDA;
     const unsigned grid = persistent_grid((a.n_tiles + LaneCfg<C>::TPR - 1) / LaneCfg<C>::TPR, d, 1);
     TAHQ_LAUNCH("decode", st, launch_dependent(kernels[k], grid, kLaneThreads, smem, st, a));
