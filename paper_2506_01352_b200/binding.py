@@ -225,11 +225,10 @@ def trace_reset(buf: torch.Tensor) -> None:
     buf.copy_(v.reshape(-1).to(buf.device))
 
 
-def _stream_handle(stream) -> int:
-    if stream is not None:
-        return int(stream.cuda_stream)
-    # (torch.cuda.current_stream() builds an object around this number, in three microseconds)
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+# The current stream as a number (torch.cuda.current_stream() builds an object around it, in three microseconds).  The
+# tensors of a call exist, so CUDA is initialised.
+_device = getattr(torch._C, "_cuda_getDevice", None)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def tahq_encode(p: Params, d_in: int, d_packed: int, packed_cap: int, d_ws: int, ws_cap: int, stream: int) -> int:
@@ -283,8 +282,8 @@ def encode(p: Params, x: torch.Tensor, packed: torch.Tensor | None = None, ws: t
     if stream is not None and made:   # buffers made here belong to torch's current stream: tell the allocator who uses them
         packed.record_stream(stream)
         ws.record_stream(stream)
-    rc = tahq_encode(p, x.data_ptr(), packed.data_ptr(), packed.numel(), ws.data_ptr(), ws.numel(),
-                     _stream_handle(stream))
+    rc = (_call or call()).encode(p._bytes or p.raw(), x.data_ptr(), packed.data_ptr(), packed.numel(), ws.data_ptr(),
+                                  ws.numel(), _raw_stream(_device()) if stream is None else stream.cuda_stream)
     if rc != OK:
         raise TahqError(rc)
     return packed
@@ -301,8 +300,8 @@ def decode(p: Params, packed: torch.Tensor, out: torch.Tensor | None = None, ws:
         if made_ws:
             ws.record_stream(stream)
         out.record_stream(stream)
-    rc = tahq_decode(p, packed.data_ptr(), packed.numel(), out.data_ptr(), ws.data_ptr(), ws.numel(),
-                     _stream_handle(stream))
+    rc = (_call or call()).decode(p._bytes or p.raw(), packed.data_ptr(), packed.numel(), out.data_ptr(), ws.data_ptr(),
+                                  ws.numel(), _raw_stream(_device()) if stream is None else stream.cuda_stream)
     if rc != OK:
         raise TahqError(rc)
     return out
@@ -335,8 +334,8 @@ def qnaive_encode(p: QNaiveParams, x: torch.Tensor, packed: torch.Tensor | None 
         packed = torch.empty(qnaive_packed_bound(p), dtype=torch.uint8, device=x.device)
     if ws is None:
         ws = torch.empty(qnaive_workspace_bound(p), dtype=torch.uint8, device=x.device)
-    rc = tahq_qnaive_encode(p, x.data_ptr(), packed.data_ptr(), packed.numel(), ws.data_ptr(), ws.numel(),
-                            torch._C._cuda_getCurrentRawStream(x.device.index))
+    rc = (_call or call()).qnaive_encode(p._bytes or p.raw(), x.data_ptr(), packed.data_ptr(), packed.numel(), ws.data_ptr(),
+                                         ws.numel(), _raw_stream(x.get_device()))
     if rc:
         raise TahqError(rc)
     return packed, ws
@@ -348,8 +347,8 @@ def qnaive_decode(p: QNaiveParams, packed: torch.Tensor, out: torch.Tensor | Non
                           dtype=torch.float32 if p.dtype == F32 else torch.bfloat16)
     if ws is None:
         ws = torch.empty(qnaive_workspace_bound(p), dtype=torch.uint8, device=packed.device)
-    rc = tahq_qnaive_decode(p, packed.data_ptr(), packed.numel(), out.data_ptr(), ws.data_ptr(), ws.numel(),
-                            torch._C._cuda_getCurrentRawStream(packed.device.index))
+    rc = (_call or call()).qnaive_decode(p._bytes or p.raw(), packed.data_ptr(), packed.numel(), out.data_ptr(), ws.data_ptr(),
+                                         ws.numel(), _raw_stream(packed.get_device()))
     if rc:
         raise TahqError(rc)
     return out, ws
