@@ -58,7 +58,10 @@ static tahq_status encode_t(const Plan &pl, const Args &a_in, cudaStream_t st) {
     }
   }
   if constexpr (C::G < 32 || C::BF16) {
-    constexpr int NQ = 2;
+    // Rows of 128 bytes (a TMA copy per unit): one slot, refilled as soon as its row is in registers; the second one's 64 KB
+    // per SM serve better as L1 (65536 x 8192 bf16 358 -> 343 us, 16384 x 8192 in tiles of 128 123 -> 113 us).  Narrower rows
+    // come by cp.async and want two (16384 x 8192 in tiles of 32 82.2 us, with one slot 84.6 us).
+    constexpr int NQ = C::ROWB == 128 ? 1 : 2;
     const int smem = StreamCfg<C>::smem_bytes(NQ);
     static std::atomic<int> occ_narrow[64], occ_wide[64];
     const uint64_t n_units = (a.n_tiles * C::LPT + 31) / 32;
