@@ -5,9 +5,25 @@
 #include <vector>
 
 #include "tahq_host.cuh"
-#include "tahq_select.cuh"
+#include "tahq_select_launch.cuh"
 
 namespace tahq {
+
+// Zeroes 16-byte pieces; the call's first tile kernel is launched as its programmatic dependent.
+__global__ void __launch_bounds__(kThreads) clear_kernel(uint4 *p, uint64_t n16, unsigned long long *trace_buf) {
+  TraceScope trace(trace_buf, 0);
+  grid_dependency_wait();
+  for (uint64_t i = blockIdx.x * (uint64_t)kThreads + threadIdx.x; i < n16; i += (uint64_t)gridDim.x * kThreads)
+    p[i] = make_uint4(0, 0, 0, 0);
+}
+
+// Self-test of the bounded waits: CTA 1 waits for a count that CTA 0 never publishes.  The wait gives
+// up after kSpinLimit polls, the status word gets TAHQ_DEV_TIMEOUT, and the kernel returns.
+__global__ void __launch_bounds__(kThreads) wait_selftest_kernel(const Args a) {
+  if (blockIdx.x == 0) return;
+  bool unused;
+  cta_exclusive_prefix(a, 1, false, unused);
+}
 
 // ---- launch bookkeeping --------------------------------------------------------------------------------
 thread_local int g_launches = 0;
@@ -93,72 +109,7 @@ tahq_status launch_clear(void *p, uint64_t bytes, cudaStream_t st) {
   return cudaGetLastError() == cudaSuccess ? TAHQ_OK : TAHQ_ERR_CUDA;
 }
 
-// ---- selection on thread-block clusters ----------------------------------------------------------------
-constexpr size_t kSelSmem = (size_t)(kClKeys + kSelThreads) * 8 + (size_t)kBins * 4 + (size_t)kClKeys * 4 + (size_t)kWordsShared * 4;
-
-static bool select_ready(int dev) {
-  static std::atomic<int> ready[64];
-  if (ready[dev & 63].load(std::memory_order_acquire)) return true;
-  for (auto kernel : {select_kernel<true>, select_kernel<false>})
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSelSmem) != cudaSuccess ||
-        cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-      (void)cudaGetLastError();
-      return false;
-    }
-  ready[dev & 63].store(1, std::memory_order_release);
-  return true;
-}
-
-static void cluster_config(cudaLaunchConfig_t *cfg, cudaLaunchAttribute *attr, unsigned grid, uint32_t cs, cudaStream_t st) {
-  *cfg = {};
-  cfg->gridDim = dim3(grid);
-  cfg->blockDim = dim3(kSelThreads);
-  cfg->dynamicSmemBytes = kSelSmem;
-  cfg->stream = st;
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = cs;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg->attrs = attr;
-  cfg->numAttrs = 1;
-}
-
-// Clusters of 2^lg CTAs of the selection kernel that the device holds at the same time (asked once per device and size).
-// More ranking groups than that run in waves, each wave the whole chain of dependent steps.  0: cannot be asked.
-static uint32_t select_capacity(int dev, int lg) {
-  static std::atomic<int> cache[64][5];   // capacity + 1
-  std::atomic<int> &slot = cache[dev & 63][lg];
-  const int v = slot.load(std::memory_order_acquire);
-  if (v > 0) return (uint32_t)(v - 1);
-  cudaLaunchConfig_t cfg;
-  cudaLaunchAttribute attr[1];
-  cluster_config(&cfg, attr, 1u << lg, 1u << lg, nullptr);
-  int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, select_kernel<true>, &cfg) != cudaSuccess) { (void)cudaGetLastError(); return 0; }
-  slot.store(n + 1, std::memory_order_release);
-  return (uint32_t)n;
-}
-
-// One cluster per ranking group, launched as a programmatic dependent of the score kernel.
-tahq_status launch_select(const Args &a, const DevInfo &d, cudaStream_t st) {
-  if (!select_ready(d.dev)) return TAHQ_ERR_CUDA;
-  // The smallest cluster whose threads can hold their scores in registers (8192 x 768 in 8 groups of 12288: 5.9 us in
-  // clusters of 4, 8 us in clusters of 16), at most 16 CTAs, and one of which the device holds one per group at once.
-  int lg = 4;
-  constexpr uint64_t kSlice = (uint64_t)kHeld * kSelThreads;
-  while (lg > 0 && (a.rank_per_group <= kSlice << (lg - 1) || a.n_groups > select_capacity(d.dev, lg))) --lg;
-  const uint32_t cs = 1u << lg, per_cta = (uint32_t)(((a.rank_per_group + cs - 1) / cs + 31) / 32 * 32);
-  cudaLaunchConfig_t cfg;
-  cudaLaunchAttribute attr[2];
-  cluster_config(&cfg, attr, (unsigned)(a.n_groups * cs), cs, st);
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.numAttrs = 2;
-  cudaError_t e;
-  TAHQ_LAUNCH("select", st, e = cudaLaunchKernelEx(&cfg, per_cta <= (uint32_t)(kHeld * kSelThreads) ? select_kernel<true> : select_kernel<false>,
-                                                  a, per_cta));
-  return e == cudaSuccess ? TAHQ_OK : TAHQ_ERR_CUDA;
-}
+tahq_status launch_select(const Args &a, const DevInfo &d, cudaStream_t st) { return launch_select_with<void>(a, d, st); }
 
 tahq_status launch_alloc_score(const Args &a, const DevInfo &d, cudaStream_t st) {
   const uint64_t n_alloc = a.n_tiles / a.alloc_m;

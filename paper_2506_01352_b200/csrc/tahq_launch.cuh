@@ -4,6 +4,7 @@
 
 #include "tahq_host.cuh"
 #include "tahq_lanes.cuh"
+#include "tahq_select_launch.cuh"
 
 namespace tahq {
 
@@ -14,7 +15,14 @@ static tahq_status encode_t(const Plan &pl, const Args &a_in, cudaStream_t st) {
   Args a = a_in;
   CUtensorMap tmap;
   a.use_tma = (C::ROWB == 128 && make_row_map(a.in, a.n_tiles * C::LPT, C::BF16, &tmap)) ? 1u : 0u;   // rows of 128 bytes
-  if (pl.mixed) {
+  bool fused = false;
+  if constexpr (C::G >= 32) {
+    if (pl.mixed && fuse_scores<C>(a, d)) {
+      fused = true;
+      if (launch_select_with<C>(a, d, st) != TAHQ_OK) return TAHQ_ERR_CUDA;
+    }
+  }
+  if (pl.mixed && !fused) {
     if (pl.alloc_m > 1) {   // Sec. 3.2 with A = m * G: one warp per allocation tile, exact scores
       if (launch_alloc_score(a, d, st) != TAHQ_OK) return TAHQ_ERR_CUDA;
     } else if (C::G >= 32 && C::BF16 && !a.exact_scores) {

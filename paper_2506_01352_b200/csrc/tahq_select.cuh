@@ -1,11 +1,11 @@
 // Sec. 3.2 and 3.4 between scoring and quantise + pack (sm_100a): the exact top-k_hi selection of every ranking group,
 // the bit map and the running count of higher-width tiles; the scores of allocation tiles wider than the quantisation
-// tile; the workspace clear and the self-test of the bounded waits.  Compiled once (tahq_common.cu).
+// tile.
 #pragma once
 
 #include <cooperative_groups.h>
 
-#include "tahq_kernels.cuh"
+#include "tahq_lanes.cuh"
 
 namespace tahq {
 
@@ -16,23 +16,6 @@ constexpr int kClKeys = 4096;          // candidate keys that are ranked in shar
 constexpr int kClMaxCtas = 16;
 constexpr int kHeld = 8;               // scores a thread keeps in registers
 constexpr int kCoarse = 64, kFine = kBins / kCoarse;
-
-
-// Zeroes 16-byte pieces; the call's first tile kernel is launched as its programmatic dependent.
-__global__ void __launch_bounds__(kThreads) clear_kernel(uint4 *p, uint64_t n16, unsigned long long *trace_buf) {
-  TraceScope trace(trace_buf, 0);
-  grid_dependency_wait();
-  for (uint64_t i = blockIdx.x * (uint64_t)kThreads + threadIdx.x; i < n16; i += (uint64_t)gridDim.x * kThreads)
-    p[i] = make_uint4(0, 0, 0, 0);
-}
-
-// Self-test of the bounded waits: CTA 1 waits for a count that CTA 0 never publishes.  The wait gives
-// up after kSpinLimit polls, the status word gets TAHQ_DEV_TIMEOUT, and the kernel returns.
-__global__ void __launch_bounds__(kThreads) wait_selftest_kernel(const Args a) {
-  if (blockIdx.x == 0) return;
-  bool unused;
-  cta_exclusive_prefix(a, 1, false, unused);
-}
 
 // ------------------------------------------------------------------------------------------
 // Eq. 1-2 over allocation tiles wider than the quantisation tile (Sec. 3.2, A = m * G, up to 8192
@@ -242,8 +225,8 @@ __device__ __forceinline__ float exact_score_any(const uint8_t *tp, uint32_t noc
 // r-th largest of n distinct keys in shared memory (n <= kClKeys), the same value returned to every thread: they go
 // into kSelThreads buckets by score first and only the bucket that holds rank r is counted; thousands of equal scores
 // fall through to the radix selection.
-__device__ __noinline__ unsigned long long rank_keys_shared(unsigned long long *s_keys, uint32_t n, uint32_t r,
-                                                               unsigned long long *s_few /* kSelThreads */) {
+static __device__ __noinline__ unsigned long long rank_keys_shared(unsigned long long *s_keys, uint32_t n, uint32_t r,
+                                                                      unsigned long long *s_few /* kSelThreads */) {
   __shared__ unsigned long long s_ans;
   __shared__ uint32_t s_cnt[kSelThreads];
   __shared__ uint32_t s_sub[kSelThreads];
@@ -340,9 +323,9 @@ constexpr int kScreenBand = 6;
 // a radix selection over the finite scores of all slices, 8 bits a pass, gives the threshold key; every CTA sums the
 // cluster's digit counts for itself.  Sets the slice's words and returns the higher-width tiles of the slices before
 // it.  (Out of line: the usual path runs once per launch from a cold instruction cache and stays compact.)
-__device__ __noinline__ uint32_t selection_by_radix(const Args &a, float *sc, const uint8_t *tiles, uint32_t tile_bytes, uint32_t n_loc,
-                                                    uint32_t i0, int lo_v, int hi_v, uint32_t rr, uint32_t *words,
-                                                    uint32_t *s_digit, uint32_t *s_red, SelShared &sh) {
+static __device__ __noinline__ uint32_t selection_by_radix(const Args &a, float *sc, const uint8_t *tiles, uint32_t tile_bytes, uint32_t n_loc,
+                                                           uint32_t i0, int lo_v, int hi_v, uint32_t rr, uint32_t *words,
+                                                           uint32_t *s_digit, uint32_t *s_red, SelShared &sh) {
   cg::cluster_group cl = cg::this_cluster();
   const uint32_t CS = cl.num_blocks(), rank = cl.block_rank();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -446,9 +429,64 @@ __device__ __forceinline__ void find_bin(const uint32_t (&c)[PER], uint32_t k, u
   rank_in = __shfl_sync(kFull, r, src);
 }
 
+// Screening scores of n tiles from `first` on, by a CTA of the selection kernel, to shared and to global memory.
+template <class C>
+__device__ __forceinline__ void slice_scores(const Args &a, uint64_t first, uint32_t n, float *s_out, float *out) {
+  using D = LaneCfg<C>;
+  constexpr int P = D::P, TPR = D::TPR, NP = D::E / 2;
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, sub = lane % P;
+  const uint8_t *in = a.in + first * D::TB + sub * 64u;
+  const uint32_t n_rounds = (n + TPR - 1) / TPR;
+  uint32_t raw[16];
+  auto load = [&](uint32_t r) {
+    const uint32_t t = r * TPR + lane / P;
+    load_64_bytes<false>(in + (uint64_t)(t < n ? t : 0u) * D::TB, raw);
+  };
+  if (warp < n_rounds) load(warp);
+  for (uint32_t r = warp; r < n_rounds; r += kSelThreads / 32) {
+    uint32_t w[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) w[i] = raw[i];
+    if (r + kSelThreads / 32 < n_rounds) load(r + kSelThreads / 32);
+    float2 L[2], T[2];
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+      float2 v;
+      if constexpr (C::BF16) bf2_add_f32(w[i] & 0x7fff7fffu, 1e-30f, v.x, v.y);
+      else v = f2(fabsf(__uint_as_float(w[2 * i])) + 1e-30f, fabsf(__uint_as_float(w[2 * i + 1])) + 1e-30f);
+      const float2 l = f2(lg2_approx(v.x), lg2_approx(v.y));
+      if (i < 2) {
+        L[i] = v;
+        T[i] = f2(v.x * l.x, v.y * l.y);   // (scalar products: they feed the fused chain's addend)
+      } else {
+        L[i & 1] = add2(L[i & 1], v);
+        T[i & 1] = fma2(v, l, T[i & 1]);
+      }
+    }
+    const float2 L2 = add2(L[0], L[1]), T2 = add2(T[0], T[1]);
+    float Ls = L2.x + L2.y, Ts = T2.x + T2.y;
+#pragma unroll
+    for (int h = 1; h < P; h *= 2) {
+      Ls += __shfl_xor_sync(kFull, Ls, h);
+      Ts += __shfl_xor_sync(kFull, Ts, h);
+    }
+    const float Lp = Ls + a.eps_l1;
+    float rc;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rc) : "f"(Lp));
+    const uint32_t t = r * TPR + lane / P;
+    if (sub == 0 && t < n) {
+      const float s = __fmaf_rn(lg2_approx(Lp), Ls, -Ts) * rc;
+      s_out[t] = s;
+      out[t] = s;
+    }
+  }
+}
+
 // HELD: a thread's scores stay in registers between binning and deciding (slices of up to kHeld * kSelThreads);
 // longer slices are read again, from L2.
-template <bool HELD>
+// C: void, or the tile configuration of a call whose (screening) scores are formed here instead of in a kernel in front
+// (small tensors; groups of whole words): see fuse_scores.
+template <bool HELD, class C>
 __global__ void __launch_bounds__(kSelThreads, 2) select_kernel(const __grid_constant__ Args a, const uint32_t per_cta) {
   constexpr int NW = kSelThreads / 32;
   cg::cluster_group cl = cg::this_cluster();
@@ -482,14 +520,23 @@ __global__ void __launch_bounds__(kSelThreads, 2) select_kernel(const __grid_con
   for (uint32_t b = threadIdx.x; b < (uint32_t)kBins; b += kSelThreads) s_hist[b] = 0;
   if (threadIdx.x < 2 * kCoarse) s_sum[0][threadIdx.x] = 0;
   if (threadIdx.x == 0) { sh.n_keys = 0; sh.n_total = 0; s_ncand = 0; s_nabove = 0; s_made = 0; }
-  grid_dependency_wait();   // the scores are the score kernel's
+  grid_dependency_wait();   // the scores are the score kernel's (or the tensor a kernel's in front)
   trace.started();
   float *sc = a.scores + g * (uint64_t)ng + i0;
+  if constexpr (!std::is_void<C>::value) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *a.status = 0;   // nothing else of the workspace has to start at zero
+    // into this CTA's key list, which nobody writes before the first cluster barrier; and to memory, for the radix
+    slice_scores<C>(a, g * (uint64_t)ng + i0, n_loc, reinterpret_cast<float *>(s_keys), sc);
+    __syncthreads();
+  }
   // ---- 1: the slice's histogram.  In turn `it` warp w takes 128 tiles from 128 * (it * NW + w) on, a lane four of them.
   const bool vec = ((reinterpret_cast<uintptr_t>(sc)) & 15u) == 0;
+  const float *const s_own = reinterpret_cast<const float *>(s_keys);
   auto first_of = [&](uint32_t it) { return (it * NW + (uint32_t)warp) * 128u + (uint32_t)lane * 4u; };
   auto load4 = [&](uint32_t it) -> float4 {   // -2 behind the slice's end (a score is above -1e-4)
     const uint32_t i = first_of(it);
+    if constexpr (!std::is_void<C>::value)   // (slices of whole words)
+      return i < n_loc ? *reinterpret_cast<const float4 *>(s_own + i) : make_float4(-2.0f, -2.0f, -2.0f, -2.0f);
     if (vec && i + 4u <= n_loc) return __ldg(reinterpret_cast<const float4 *>(sc + i));
     return make_float4(i < n_loc ? __ldg(sc + i) : -2.0f, i + 1u < n_loc ? __ldg(sc + i + 1) : -2.0f,
                        i + 2u < n_loc ? __ldg(sc + i + 2) : -2.0f, i + 3u < n_loc ? __ldg(sc + i + 3) : -2.0f);

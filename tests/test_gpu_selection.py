@@ -49,3 +49,13 @@ def test_allocation_tiles_in_groups_that_share_words(S, G, A, equal):
 
 def test_one_group_of_thousands_of_equal_allocation_tiles():
     check(tensor(9001, 192, torch.bfloat16, 2, 0.95), tile=32, alloc_tile=96, group_tokens=9001, budget_millibits=3500)
+
+
+@pytest.mark.parametrize("groups,tiles,G,dtype", [
+    (1, 32, 32, torch.bfloat16), (74, 32, 64, torch.float32), (75, 32, 64, torch.float32),   # half the SMs' worth of CTAs
+    (3, 544, 32, torch.bfloat16), (2, 96, 128, torch.float32), (9, 288, 64, torch.bfloat16),
+    (2, 8192, 32, torch.float32), (2, 8224, 32, torch.float32),     # 16384 elements in each of 16 CTAs
+    (4, 4096, 64, torch.bfloat16), (4, 4128, 64, torch.bfloat16), (1, 2048, 128, torch.bfloat16), (1, 2080, 128, torch.bfloat16)])
+@pytest.mark.parametrize("equal", [0.0, 0.9])
+def test_scores_formed_in_the_selection(groups, tiles, G, dtype, equal):
+    check(tensor(groups * tiles, G, dtype, tiles, equal), tile=G, group_tokens=tiles, budget_millibits=3300)
