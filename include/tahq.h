@@ -112,7 +112,7 @@ tahq_status tahq_packed_layout(const tahq_params *p, tahq_layout *out);
 
 /*
  * Bytes of scratch that tahq_encode / tahq_decode need for these parameters
- * (tile scores, selection histograms and candidates, offset prefixes, status
+ * (tile scores, offset prefixes, the flags of a decode's offset look-back, status
  * word).  Returns 0 when the parameters are invalid.  Host-only.
  */
 size_t tahq_workspace_bound(const tahq_params *p);

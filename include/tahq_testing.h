@@ -13,7 +13,7 @@ extern "C" {
 
 /*
  * Self-test of the library's bounded device-side waits (the paper has no counterpart).  Launches a two-CTA
- * kernel in which one CTA waits, as the offset look-back of encode/decode does, for a count that is never
+ * kernel in which one CTA waits, as the offset look-back of decode does, for a count that is never
  * published.  The wait gives up after its fixed number of polls (about a second), the kernel returns, and
  * the device status word at d_ws[0..4) reads TAHQ_DEV_TIMEOUT; the CUDA context stays usable.  d_ws: at
  * least 32 KiB of device memory.
