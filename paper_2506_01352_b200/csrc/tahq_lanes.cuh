@@ -955,12 +955,15 @@ __global__ void __launch_bounds__(QuantLanes<C>::NT, 1) quant_lanes_kernel(const
   }
 }
 
-// Binary32 always; bfloat16 while a warp has at most two rounds, that is while the time is that of a warp's chain and not of
-// the instructions (both sides measured, 64-wide tiles, quant2_kernel against this: 1500 tiles 7.2 / 3.9 us, 59 thousand
-// 5.6 / 5.3, 95 thousand -- two rounds -- 6.8 / 6.3, 127 thousand 7.7 / 8.9, 524 thousand 22.5 / 27.8).
-template <class C>
-bool quant_lanes_pays(uint64_t n_rounds, int sms) {
-  return C::G >= 32 && (!C::BF16 || n_rounds <= 2ull * QuantLanes<C>::WARPS * (unsigned)sms);
+// Binary32 always; bfloat16 while the time is that of a warp's chain and not of the instructions: up to two rounds to a warp,
+// and one where quant2_kernel is at its best (tiles of 64, widths up to 4 bits, rounding to nearest).  Both sides measured,
+// encode with quant2_kernel against this one: tiles of 64 at 3.8 bits, 32 thousand 14.6 / 14.2 us, 51 thousand 15.7 / 15.8, 94
+// thousand 17.4 / 17.8, at 4 bits 6.7 / 7.5, at 6.8 bits 20.7 / 19.9; 51 thousand with stochastic rounding 21.8 / 21.3; tiles of
+// 128, 45 thousand -- two rounds -- 20.3 / 19.2.  Three rounds, 127 thousand tiles of 64: the kernels alone 7.7 / 8.9.
+template <class C, bool SR>
+bool quant_lanes_pays(uint64_t n_rounds, bool narrow, int sms) {
+  const uint64_t per_warp = C::G == 64 && narrow && !SR ? 1 : 2;
+  return C::G >= 32 && (!C::BF16 || n_rounds <= per_warp * QuantLanes<C>::WARPS * (unsigned)sms);
 }
 
 }  // namespace tahq

@@ -53,7 +53,7 @@ static tahq_status encode_t(const Plan &pl, const Args &a_in, cudaStream_t st) {
   const bool narrow = a.lo + a.mixed <= 4u;   // no width above 4 bits: the kernel compiled for just that
   if constexpr (C::G >= 32) {
     const uint64_t n_rounds = (a.n_tiles + LaneCfg<C>::TPR - 1) / LaneCfg<C>::TPR;
-    if (quant_lanes_pays<C>(n_rounds, d.sms)) {
+    if (quant_lanes_pays<C, SR>(n_rounds, narrow, d.sms)) {
       const bool wide_ld = (reinterpret_cast<uintptr_t>(a.in) & 31u) == 0;   // 256-bit loads where the tensor is aligned to them
       void (*const kernels[4])(Args) = {quant_lanes_kernel<C, SR, false, false>, quant_lanes_kernel<C, SR, false, true>,
                                         quant_lanes_kernel<C, SR, true, false>, quant_lanes_kernel<C, SR, true, true>};

@@ -47,3 +47,13 @@ def test_bf16_around_two_rounds_per_warp(G, tokens, rounding):
     x = torch.randn(tokens, G * (64 if G == 32 else 32), generator=g, device="cuda")
     x[:, ::41] *= 30
     check(x.bfloat16(), tile=G, budget_millibits=3600, rounding=rounding, seed=5)
+
+
+@pytest.mark.parametrize("tokens", [1479, 1480, 1481])
+@pytest.mark.parametrize("budget", [3600, 4000, 4600])
+def test_bf16_around_one_round_per_warp(tokens, budget):
+    """148 SMs x 20 warps x 16 tiles of 64, the line where no width is above 4 bits: 1480 tokens of 32 tiles."""
+    g = torch.Generator(device="cuda").manual_seed(tokens)
+    x = torch.randn(tokens, 2048, generator=g, device="cuda")
+    x[:, ::41] *= 30
+    check(x.bfloat16(), tile=64, budget_millibits=budget)
