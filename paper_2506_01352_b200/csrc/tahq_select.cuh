@@ -310,10 +310,12 @@ struct SelShared {
 // lie in [0, log2 A]; three quarters of the bins are given to the top two units, where most tiles and the threshold are:
 // with bins of one width a threshold in the dense part had 2.6 times as many candidates.
 struct StepMap { float lo, hi, off; };   // max(s * lo, s * hi - off)
-__device__ __forceinline__ float score_pos(float s, const StepMap &m) { return fmaxf(s * m.lo, __fmaf_rn(s, m.hi, -m.off)); }
-__device__ __forceinline__ int score_step(float s, const StepMap &m) {
-  return (int)fminf(fmaxf(score_pos(s, m), 0.0f), (float)(16 * kBins - 1));
+// A score below zero (p + varsigma above one: tiles with a single large element) stands at zero: it is in the first bin and
+// must not look as if it lay below it.
+__device__ __forceinline__ float score_pos(float s, const StepMap &m) {
+  return fmaxf(fmaxf(s * m.lo, __fmaf_rn(s, m.hi, -m.off)), 0.0f);
 }
+__device__ __forceinline__ int score_step(float s, const StepMap &m) { return (int)fminf(score_pos(s, m), (float)(16 * kBins - 1)); }
 // Screening scores differ from exact ones by less than 1e-4 (see tile_score_screen), 2.5 steps at most.  With k_hi-th largest
 // screening score in bin B, a tile whose screening score lies more than twice that outside bin B is certainly inside or
 // outside the top k_hi; six steps also cover the cut to whole steps.
