@@ -535,19 +535,21 @@ __global__ void __launch_bounds__(kSelThreads, 2) select_kernel(const __grid_con
   const bool vec = ((reinterpret_cast<uintptr_t>(sc)) & 15u) == 0;
   const float *const s_own = reinterpret_cast<const float *>(s_keys);
   auto first_of = [&](uint32_t it) { return (it * NW + (uint32_t)warp) * 128u + (uint32_t)lane * 4u; };
-  auto load4 = [&](uint32_t it) -> float4 {   // -2 behind the slice's end (a score is above -1e-4)
+  auto left_of = [&](uint32_t it) { return (int)n_loc - (int)first_of(it); };   // tiles of the slice from the lane's first on
+  auto load4 = [&](uint32_t it) -> float4 {   // (anything behind the slice's end: told by its place, not by its value)
     const uint32_t i = first_of(it);
     if constexpr (!std::is_void<C>::value)   // (slices of whole words)
-      return i < n_loc ? *reinterpret_cast<const float4 *>(s_own + i) : make_float4(-2.0f, -2.0f, -2.0f, -2.0f);
+      return i < n_loc ? *reinterpret_cast<const float4 *>(s_own + i) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if (vec && i + 4u <= n_loc) return __ldg(reinterpret_cast<const float4 *>(sc + i));
-    return make_float4(i < n_loc ? __ldg(sc + i) : -2.0f, i + 1u < n_loc ? __ldg(sc + i + 1) : -2.0f,
-                       i + 2u < n_loc ? __ldg(sc + i + 2) : -2.0f, i + 3u < n_loc ? __ldg(sc + i + 3) : -2.0f);
+    return make_float4(i < n_loc ? __ldg(sc + i) : 0.0f, i + 1u < n_loc ? __ldg(sc + i + 1) : 0.0f,
+                       i + 2u < n_loc ? __ldg(sc + i + 2) : 0.0f, i + 3u < n_loc ? __ldg(sc + i + 3) : 0.0f);
   };
-  auto bin4 = [&](const float4 &v) {
-    if (v.x > -1.0f) atomicAdd(&s_hist[score_step(v.x, map) >> 4], 1u);
-    if (v.y > -1.0f) atomicAdd(&s_hist[score_step(v.y, map) >> 4], 1u);
-    if (v.z > -1.0f) atomicAdd(&s_hist[score_step(v.z, map) >> 4], 1u);
-    if (v.w > -1.0f) atomicAdd(&s_hist[score_step(v.w, map) >> 4], 1u);
+  auto bin4 = [&](uint32_t it, const float4 &v) {
+    const int left = left_of(it);
+    if (left > 0) atomicAdd(&s_hist[score_step(v.x, map) >> 4], 1u);
+    if (left > 1) atomicAdd(&s_hist[score_step(v.y, map) >> 4], 1u);
+    if (left > 2) atomicAdd(&s_hist[score_step(v.z, map) >> 4], 1u);
+    if (left > 3) atomicAdd(&s_hist[score_step(v.w, map) >> 4], 1u);
   };
   float4 held[kHeld / 4];   // the scores, or (long slices) the first ones
 #pragma unroll
@@ -555,14 +557,14 @@ __global__ void __launch_bounds__(kSelThreads, 2) select_kernel(const __grid_con
   __syncthreads();
   if constexpr (HELD) {
 #pragma unroll
-    for (int it = 0; it < kHeld / 4; ++it) bin4(held[it]);
+    for (int it = 0; it < kHeld / 4; ++it) bin4(it, held[it]);
   } else {
     for (uint32_t it0 = 0; it0 < n_it; it0 += kHeld / 4) {
       float4 cur[kHeld / 4];
 #pragma unroll
       for (int j = 0; j < kHeld / 4; ++j) { cur[j] = held[j]; held[j] = load4(it0 + kHeld / 4 + j); }
 #pragma unroll
-      for (int j = 0; j < kHeld / 4; ++j) bin4(cur[j]);
+      for (int j = 0; j < kHeld / 4; ++j) bin4(it0 + j, cur[j]);
     }
   }
   __syncthreads();
@@ -606,12 +608,12 @@ __global__ void __launch_bounds__(kSelThreads, 2) select_kernel(const __grid_con
     uint32_t n_above = 0;
     auto decide = [&](uint32_t it, const float4 &v) {
       const float t[4] = {score_pos(v.x, map), score_pos(v.y, map), score_pos(v.z, map), score_pos(v.w, map)};
-      const float e[4] = {v.x, v.y, v.z, v.w};
+      const int left = left_of(it);
       uint32_t above = 0, cand = 0;   // of the lane's four tiles
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        above |= t[j] >= hi_f ? 1u << j : 0u;
-        cand |= (e[j] > -1.0f && !(t[j] >= hi_f) && !(t[j] < lo_f)) ? 1u << j : 0u;
+        above |= (j < left && t[j] >= hi_f) ? 1u << j : 0u;
+        cand |= (j < left && !(t[j] >= hi_f) && !(t[j] < lo_f)) ? 1u << j : 0u;
       }
       // eight lanes hold a word
       uint32_t word = above << (4 * (lane & 7));

@@ -38,3 +38,12 @@ FORMS = [dict(tile=64, group_tokens=64), dict(tile=64, group_tokens=37), dict(ti
 def test_scores_just_below_zero(eps_log, dense, form, dtype):
     tokens = form["group_tokens"] * 3
     check(one_hot(tokens, 512, dtype, 64, dense), budget_millibits=3500, eps_log=eps_log, **form)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("form", FORMS)
+@pytest.mark.parametrize("dense", [0.0, 1.0])
+@pytest.mark.parametrize("eps_log", [1.0, 4.0, 1e30])
+def test_scores_far_below_zero(eps_log, dense, form, dtype):
+    tokens = form["group_tokens"] * 3
+    check(one_hot(tokens, 512, dtype, 64, dense), budget_millibits=3500, eps_log=eps_log, **form)
