@@ -340,12 +340,23 @@ __device__ __forceinline__ float tile_score(const uint8_t *stage, int row, float
 // selects this function when that is at most 1.5e-5); the hardware log2 (2^-22) and the rounding of
 // the sums, each weighted by p or by |log2 a| <= 127 times a few units in the last place: under 1e-4
 // in all.  It is only used to decide which tiles are far enough from a group's threshold to be
-// classified without their exact score; see select_kernel.
+// classified without their exact score; see select_kernel.  All of this holds while L' is nowhere near the ends of binary32:
+// see screen_result.
 __device__ __forceinline__ float lg2_approx(float x) {
   float y;
   asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
+// The screening score s of a tile with L' = Lp; NaN where the screening does not hold: below 2^-60 the 1e-30 added to every
+// magnitude would count (a varepsilon near zero and a tile of next to nothing), above 2^60 the sums come near the largest
+// numbers.  The kernel that screens goes back to such tiles when it is through (exact_where_unscreened).
+__device__ __forceinline__ float screen_result(float s, float Lp) {
+  return Lp >= 0x1p-60f && Lp <= 0x1p60f ? s : __int_as_float(0x7fffffff);
+}
+// An exact score as it is stored and ranked: every one a number, of a size that the selection can calculate with.  (A tile of
+// zeroes without epsilon has p = 0/0; it ranks first, as its key without this would.)
+__device__ __forceinline__ float ranked_score(float s) { return s == s ? fminf(fmaxf(s, -1e30f), 1e30f) : 1e30f; }
+
 template <class C>
 __device__ __forceinline__ float tile_score_screen(const uint8_t *stage, int row, float eps_l1) {
   const float tiny = 1e-30f;
@@ -377,7 +388,7 @@ __device__ __forceinline__ float tile_score_screen(const uint8_t *stage, int row
   const float Lp = L + eps_l1;
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(Lp));
-  return __fmaf_rn(lg2_approx(Lp), L, -T) * r;
+  return screen_result(__fmaf_rn(lg2_approx(Lp), L, -T) * r, Lp);
 }
 
 // Exact score of one whole tile read straight from global memory by NOCT neighbouring lanes, lane o
@@ -415,6 +426,28 @@ __device__ __forceinline__ float exact_score_coop(const uint8_t *tile, int o, fl
 #pragma unroll
   for (int h = 1; h < NOCT; h *= 2) S = S + __shfl_xor_sync(kFull, S, h);
   return 0.0f - S;
+}
+
+// Exact scores for those of n <= 32 consecutive tiles whose score this warp has stored as NaN (screen_result); `also`: a second
+// copy of the scores, or null.  All lanes of the warp call this; out of line, since it is hardly ever run.
+template <int NOCT, bool BF16>
+static __device__ __noinline__ void exact_where_unscreened(const uint8_t *tiles, uint32_t n, float eps_l1, float eps_log, float *scores,
+                                                           float *also) {
+  const uint32_t lane = threadIdx.x & 31u, sub = lane % NOCT, grp = lane / NOCT;
+  __syncwarp();   // the scores were stored by other lanes
+  const float s = lane < n ? *(volatile float *)(scores + lane) : 0.0f;
+  unsigned m = __ballot_sync(kFull, s != s);
+  while (m) {
+    unsigned mine = m;   // the grp-th tile of those left
+    for (uint32_t i = 0; i < grp; ++i) mine &= mine - 1u;
+    const uint32_t t = mine ? (uint32_t)__ffs(mine) - 1u : 0u;
+    const float ex = ranked_score(exact_score_coop<NOCT, BF16>(tiles + t * (uint32_t)(NOCT * 8 * (BF16 ? 2 : 4)), sub, eps_l1, eps_log));
+    if (mine && sub == 0) {
+      scores[t] = ex;
+      if (also) also[t] = ex;
+    }
+    for (int i = 0; i < 32 / NOCT; ++i) m &= m - 1u;
+  }
 }
 
 // Order-preserving map binary32 -> uint32, and the 64-bit ranking key (score first, then the

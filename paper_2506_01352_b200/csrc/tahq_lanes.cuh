@@ -473,7 +473,9 @@ __global__ void __launch_bounds__(kScoreThreads, 2) score_lanes_kernel(const Arg
   grid_dependency_wait();   // the tensor may be the work of the kernel in front
   trace.started();
   if (blockIdx.x == 0 && threadIdx.x == 0) *a.status = 0;   // nothing else of the workspace has to start at zero
-  uint32_t left = r1 - r0 > warp ? r1 - r0 - warp : 0u;     // the warp's next round is r0 + left - 1
+  const uint32_t left0 = r1 - r0 > warp ? r1 - r0 - warp : 0u;
+  uint32_t left = left0;   // the warp's next round is r0 + left - 1
+  bool again = false;      // a tile that the screening does not hold for
   if (left) load(r0 + left - 1u);
   while (left) {
     uint32_t w[16];
@@ -510,8 +512,18 @@ __global__ void __launch_bounds__(kScoreThreads, 2) score_lanes_kernel(const Arg
     float rc;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rc) : "f"(Lp));
     const uint32_t tile = r * TPR + lane / P;
-    if (sub == 0 && tile < n_tiles) a.scores[tile] = __fmaf_rn(lg2_approx(Lp), Ls, -Ts) * rc;
+    if (sub == 0 && tile < n_tiles) {
+      const float s = screen_result(__fmaf_rn(lg2_approx(Lp), Ls, -Ts) * rc, Lp);
+      a.scores[tile] = s;
+      again |= s != s;
+    }
   }
+  if (__any_sync(kFull, again))
+    for (left = left0; left; left = left > WARPS ? left - WARPS : 0u) {
+      const uint32_t tile = (r0 + left - 1u) * TPR;
+      exact_where_unscreened<C::G / 8, C::BF16>(a.in + (uint64_t)tile * D::TB, n_tiles - tile < TPR ? n_tiles - tile : TPR, a.eps_l1,
+                                                a.eps_log, a.scores + tile, nullptr);
+    }
 }
 
 // ------------------------------------------------------------------------------------------

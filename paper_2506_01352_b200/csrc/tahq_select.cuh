@@ -112,9 +112,7 @@ __global__ void __launch_bounds__(kThreads) alloc_score_kernel(const Args a) {
       const float2 p = f2(m.x * inv, m.y * inv), l = lg2_fma2(add2(p, f2(a.eps_log)));
       return f2(p.x * l.x, p.y * l.y);
     });
-    if (lane == 0) {
-      a.scores[t] = 0.0f - S;
-    }
+    if (lane == 0) a.scores[t] = ranked_score(0.0f - S);
   }
 }
 
@@ -344,7 +342,7 @@ static __device__ __noinline__ uint32_t selection_by_radix(const Args &a, float 
     for (uint32_t q = 0; q < n; q += per) {
       const bool live = q + grp < n;
       const uint32_t b = __fns(m, 0, (int)(live ? q + grp : 0u) + 1);
-      const float ex = exact_score_any(tiles + (uint64_t)(c0 + b) * tile_bytes, noct, a.bf16 != 0, sub, a.eps_l1, a.eps_log);
+      const float ex = ranked_score(exact_score_any(tiles + (uint64_t)(c0 + b) * tile_bytes, noct, a.bf16 != 0, sub, a.eps_l1, a.eps_log));
       if (live && sub == 0) sc[c0 + b] = ex;
     }
   }
@@ -444,6 +442,7 @@ __device__ __forceinline__ void slice_scores(const Args &a, uint64_t first, uint
     const uint32_t t = r * TPR + lane / P;
     load_64_bytes<false>(in + (uint64_t)(t < n ? t : 0u) * D::TB, raw);
   };
+  bool again = false;   // a tile that the screening does not hold for
   if (warp < n_rounds) load(warp);
   for (uint32_t r = warp; r < n_rounds; r += kSelThreads / 32) {
     uint32_t w[16];
@@ -477,11 +476,16 @@ __device__ __forceinline__ void slice_scores(const Args &a, uint64_t first, uint
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rc) : "f"(Lp));
     const uint32_t t = r * TPR + lane / P;
     if (sub == 0 && t < n) {
-      const float s = __fmaf_rn(lg2_approx(Lp), Ls, -Ts) * rc;
+      const float s = screen_result(__fmaf_rn(lg2_approx(Lp), Ls, -Ts) * rc, Lp);
       s_out[t] = s;
       out[t] = s;
+      again |= s != s;
     }
   }
+  if (__any_sync(kFull, again))
+    for (uint32_t r = warp; r < n_rounds; r += kSelThreads / 32)
+      exact_where_unscreened<C::G / 8, C::BF16>(a.in + (first + r * TPR) * D::TB, n - r * TPR < TPR ? n - r * TPR : TPR, a.eps_l1, a.eps_log,
+                                                s_out + r * TPR, out + r * TPR);
 }
 
 // HELD: a thread's scores stay in registers between binning and deciding (slices of up to kHeld * kSelThreads);
@@ -673,7 +677,8 @@ __global__ void __launch_bounds__(kSelThreads, 2) select_kernel(const __grid_con
       const uint32_t j = j0 + threadIdx.x / noct;
       const bool live = j < n_listed;
       const uint32_t i = s_cand[live ? j : 0];
-      const float ex = a.exact_scores ? sc[i] : exact_score_any(tiles + (uint64_t)i * tile_bytes, noct, a.bf16 != 0, sub, a.eps_l1, a.eps_log);
+      const float ex = a.exact_scores ? sc[i] : ranked_score(exact_score_any(tiles + (uint64_t)i * tile_bytes, noct, a.bf16 != 0, sub,
+                                                                             a.eps_l1, a.eps_log));
       if (j0 == 0) __syncthreads();   // s_base
       // the keys go into every CTA's copy of the list: nobody has to fetch them from one CTA afterwards
       const uint32_t at = s_base + j;
