@@ -57,3 +57,15 @@ def test_bf16_around_one_round_per_warp(tokens, budget):
     x = torch.randn(tokens, 2048, generator=g, device="cuda")
     x[:, ::41] *= 30
     check(x.bfloat16(), tile=64, budget_millibits=budget)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("G", [8, 16, 32, 64, 128])
+@pytest.mark.parametrize("budget,rounding", [(3500, 0), (6500, 0), (8000, 1)])
+def test_transformed_tiles_whose_sums_overflow(budget, rounding, G, dtype):
+    """One or two magnitudes near the largest number in a tile: finite input whose transform (Eq. 4) is not."""
+    x = torch.zeros(60, 4 * G, device="cuda")
+    x[:, ::G] = 3e38
+    x[:, 3::G] = torch.linspace(0, 1.4e38, 60, device="cuda")[:, None]
+    x[1::2] *= -1
+    check(x.to(dtype), tile=G, budget_millibits=budget, rounding=rounding, seed=3)
