@@ -329,13 +329,21 @@ def tahq_qnaive_decode(p: QNaiveParams, d_packed: int, nbytes: int, d_out: int, 
     return (_call or call()).qnaive_decode(p.raw(), d_packed, nbytes, d_out, d_ws, ws_cap, stream)
 
 
+def _stream_of(t: torch.Tensor) -> int:
+    """The current stream of the tensor's device.  A tensor that is not on a GPU has none: the kernels could not reach it."""
+    device = t.get_device()
+    if device < 0:
+        raise ValueError(f"Expected a cuda device, but got: {t.device}")
+    return _raw_stream(device)
+
+
 def qnaive_encode(p: QNaiveParams, x: torch.Tensor, packed: torch.Tensor | None = None, ws: torch.Tensor | None = None):
     if packed is None:
         packed = torch.empty(qnaive_packed_bound(p), dtype=torch.uint8, device=x.device)
     if ws is None:
         ws = torch.empty(qnaive_workspace_bound(p), dtype=torch.uint8, device=x.device)
     rc = (_call or call()).qnaive_encode(p._bytes or p.raw(), x.data_ptr(), packed.data_ptr(), packed.numel(), ws.data_ptr(),
-                                         ws.numel(), _raw_stream(x.get_device()))
+                                         ws.numel(), _stream_of(x))
     if rc:
         raise TahqError(rc)
     return packed, ws
@@ -348,7 +356,7 @@ def qnaive_decode(p: QNaiveParams, packed: torch.Tensor, out: torch.Tensor | Non
     if ws is None:
         ws = torch.empty(qnaive_workspace_bound(p), dtype=torch.uint8, device=packed.device)
     rc = (_call or call()).qnaive_decode(p._bytes or p.raw(), packed.data_ptr(), packed.numel(), out.data_ptr(), ws.data_ptr(),
-                                         ws.numel(), _raw_stream(packed.get_device()))
+                                         ws.numel(), _stream_of(packed))
     if rc:
         raise TahqError(rc)
     return out, ws

@@ -2,6 +2,7 @@
 import copy
 
 import pytest
+import torch
 
 from paper_2506_01352_b200 import binding as T
 
@@ -26,3 +27,25 @@ def test_wrong_arguments_raise():
         with pytest.raises(TypeError):
             T.call().encode(*args)
     assert T.call().encode(p.raw(), None, 0, 0, None, 0, None) == 1
+
+
+def test_tensors_that_are_not_on_a_gpu_are_refused_before_the_call(monkeypatch):
+    """Their addresses mean nothing to the kernels; the four calls are replaced, so nothing is launched here either way."""
+    class Recorder:
+        def __getattr__(self, name):
+            return lambda *args: reached.append(name) or 0
+
+    reached = []
+    monkeypatch.setattr(T, "_call", Recorder())
+    monkeypatch.setattr(T, "_raw_stream", lambda device: 0)
+    monkeypatch.setattr(T, "_device", lambda: 0)
+    x, ws = torch.zeros(4, 64), torch.zeros(256, dtype=torch.uint8)
+    g = T.QNaiveParams(tokens=4, hidden=64)
+    packed = torch.zeros(T.qnaive_packed_bound(g), dtype=torch.uint8)
+    with pytest.raises(ValueError, match="cuda"):
+        T.qnaive_encode(g, x, packed=packed, ws=ws)
+    with pytest.raises(ValueError, match="cuda"):
+        T.qnaive_decode(g, packed, out=x, ws=ws)
+    with pytest.raises(ValueError, match="CUDA"):
+        T.encode(T.params_for(x), x, packed=packed, ws=ws)
+    assert reached == []
