@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(kQThreads, BF16 ? 3 : 2) qnaive_encode_kernel(
   constexpr int ESZ = BF16 ? 2 : 4;
   __shared__ uint32_t s_max[2][8];
   const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, C = a.hidden;
-  const uint32_t n_warps = blockDim.x >> 5, row_words = (uint32_t)(a.row_bytes / 4), lanes_all = (C + 31u) / 32u;
+  const uint32_t n_warps = blockDim.x >> 5, row_words = (uint32_t)(a.row_bytes / 4), lanes_all = C / 32u + (C % 32u != 0u);
   float *scales = reinterpret_cast<float *>(a.packed + a.off_scales);
   const bool wide = (reinterpret_cast<uintptr_t>(a.in) & 31u) == 0;
   grid_dependency_wait();   // launched as a programmatic dependent of the kernel in front
@@ -389,7 +389,7 @@ __global__ void __launch_bounds__(kQThreads, 4) qnaive_decode_kernel(const QArgs
         o[2 * k + 1] = __float_as_uint(x[k].y);
       }
     }
-    const uint32_t left = (C - p0 * (uint32_t)E) * ESZ;   // bytes of the row from this piece on: a multiple of 16
+    const uint32_t rest = C - p0 * (uint32_t)E, left = rest < (uint32_t)E ? rest * ESZ : 64u;   // bytes of the piece: a multiple of 16
     uint8_t *dst = a.out + ((uint64_t)r0 * C + p0 * (uint32_t)E) * ESZ;
 #pragma unroll
     for (int j = 0; j < 16; j += WIDE ? 8 : 4) {
@@ -409,7 +409,7 @@ __global__ void __launch_bounds__(kQThreads, 4) qnaive_decode_kernel(const QArgs
 template <bool BF16, int B>
 tahq_status qnaive_encode_b(QArgs a, const DevInfo &d, cudaStream_t st) {
   static std::atomic<int> occ[2][64];
-  const uint32_t parts = (a.hidden + 31) / 32, stretches = (parts + 31) / 32;
+  const uint32_t parts = a.hidden / 32 + (a.hidden % 32 != 0), stretches = (parts + 31) / 32;
   const bool lng = stretches > 8;
   void (*const kernel)(QArgs) = lng ? qnaive_encode_kernel<BF16, B, true> : qnaive_encode_kernel<BF16, B, false>;
   const int n = prepare(kernel, kQThreads, 0, d, occ[lng]);
@@ -431,7 +431,7 @@ tahq_status qnaive_decode_b(QArgs a, const DevInfo &d, cudaStream_t st) {
   void (*const kernel)(QArgs) = wide ? qnaive_decode_kernel<BF16, B, true> : qnaive_decode_kernel<BF16, B, false>;
   const int n = prepare(kernel, kQThreads, 0, d, occ[wide]);
   if (!n) return TAHQ_ERR_CUDA;
-  a.pieces = (a.hidden + E - 1) / E;
+  a.pieces = a.hidden / E + (a.hidden % E != 0);
   const uint64_t want = (a.tokens * a.pieces + kQThreads - 1) / kQThreads, cap = (uint64_t)d.sms * n;
   if (want > (1ull << 32) / kQThreads - cap) return TAHQ_ERR_UNSUPPORTED;   // (a tensor beyond 250 GB)
   TAHQ_LAUNCH("qnaive_decode", st, launch_dependent(kernel, (unsigned)(want < cap ? want : cap), kQThreads, 0, st, a));

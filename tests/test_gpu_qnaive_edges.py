@@ -53,3 +53,20 @@ def test_division_by_pre_scales_that_are_no_power_of_two(bits, c):
     x = rows(64, 2048, torch.float32, bits) * torch.logspace(-18, 18, 64, device="cuda")[:, None]
     x[5] = 0
     _check(x.contiguous(), bits, 0, c)
+
+
+@pytest.mark.parametrize("dtype,n", [(torch.float32, 1025), (torch.bfloat16, 2049)])
+def test_a_row_beyond_four_gibibytes(dtype, n):
+    """The tensor as a single row and as rows of 2^20 elements, with one scale: the same codes, the same values."""
+    dt = T.F32 if dtype == torch.float32 else T.BF16
+    x = torch.empty(n, 1 << 20, dtype=dtype, device="cuda")
+    for r in range(0, n, 205):
+        x[r:r + 205] = rows(min(205, n - r), 1 << 20, dtype, r)
+    short = T.QNaiveParams(tokens=n, hidden=1 << 20, dtype=dt, bits=2, per_tensor=1)
+    long = T.QNaiveParams(tokens=1, hidden=n << 20, dtype=dt, bits=2, per_tensor=1)
+    a, ws = T.qnaive_encode(short, x)
+    b, _ = T.qnaive_encode(long, x.view(1, -1), ws=ws)
+    assert T.device_status(ws) == 0 and torch.equal(a[128:], b[128:])
+    want, _ = T.qnaive_decode(short, a, ws=ws)
+    got, _ = T.qnaive_decode(long, b, out=x.view(1, -1).fill_(float("nan")), ws=ws)
+    assert T.device_status(ws) == 0 and torch.equal(got.view(n, -1), want)
