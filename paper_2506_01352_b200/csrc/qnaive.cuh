@@ -23,6 +23,7 @@
 namespace tahq {
 
 constexpr int kQThreads = 256;
+constexpr uint64_t kQPiecesPerLaunch = 1ull << 32;   // decode: less one step of the grid
 constexpr float kQMagic = 12582912.0f;     // 1.5 * 2^23
 constexpr uint32_t kQMagicBits = 0x4B400000u;
 
@@ -432,9 +433,18 @@ tahq_status qnaive_decode_b(QArgs a, const DevInfo &d, cudaStream_t st) {
   const int n = prepare(kernel, kQThreads, 0, d, occ[wide]);
   if (!n) return TAHQ_ERR_CUDA;
   a.pieces = a.hidden / E + (a.hidden % E != 0);
-  const uint64_t want = (a.tokens * a.pieces + kQThreads - 1) / kQThreads, cap = (uint64_t)d.sms * n;
-  if (want > (1ull << 32) / kQThreads - cap) return TAHQ_ERR_UNSUPPORTED;   // (a tensor beyond 250 GB)
-  TAHQ_LAUNCH("qnaive_decode", st, launch_dependent(kernel, (unsigned)(want < cap ? want : cap), kQThreads, 0, st, a));
+  const uint64_t cap = (uint64_t)d.sms * n, tokens = a.tokens;
+  // the kernel counts pieces in 32 bits: more of them (64 GiB, where a row is one piece of 16 bytes) go in several launches,
+  // of an even number of rows each, which keeps the alignment
+  const uint64_t rows = (kQPiecesPerLaunch - cap * kQThreads) / a.pieces / 2 * 2;
+  for (uint64_t r = 0; r < tokens; r += rows) {
+    a.tokens = tokens - r < rows ? tokens - r : rows;
+    const uint64_t want = (a.tokens * a.pieces + kQThreads - 1) / kQThreads;
+    TAHQ_LAUNCH("qnaive_decode", st, launch_dependent(kernel, (unsigned)(want < cap ? want : cap), kQThreads, 0, st, a));
+    a.off_scales += a.per_tensor ? 0 : 4 * rows;
+    a.off_payload += rows * a.row_bytes;
+    a.out += rows * a.hidden * (BF16 ? 2 : 4);
+  }
   return cudaGetLastError() == cudaSuccess ? TAHQ_OK : TAHQ_ERR_CUDA;
 }
 template <bool BF16, bool ENC, int B = 2>
