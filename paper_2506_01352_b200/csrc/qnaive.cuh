@@ -96,8 +96,8 @@ __device__ __forceinline__ float q_scale(float mg, float prescale, float &inv) {
 
 // 32 codes -> B words of the row's bit stream.  Four (b <= 8) or two codes are glued by a multiply-add chain on the
 // raw bits of fma(y, 1/s, 1.5 * 2^23); the constant part of those bits, less L per code, is taken off once per chain.
-// The clamp is left out: |y| <= m and s = m / L rounded give |y * (1/s)| < L + 1/2, so it never acts on finite
-// input.
+// The clamp is left out: |y| <= m and s = m / L rounded give |y * (1/s)| < L + 1/2, so it never acts on a finite c g.
+// (`prescale`: see the caller, where c g overflows.)
 template <bool BF16, int B>
 __device__ __forceinline__ void q_codes(const QRaw<BF16> &raw, float prescale, float inv, uint32_t (&w)[B]) {
   constexpr int GS = B <= 8 ? 4 : 2, GB = GS * B;   // codes and bits of a chain
@@ -202,9 +202,9 @@ __global__ void __launch_bounds__(kQThreads, BF16 ? 3 : 2) qnaive_encode_kernel(
     if (n == 32u) raw.load(src, wide);
     else if (n) raw.load_some(src, n);
   };
-  auto emit = [&](const QRaw<BF16> &raw, uint32_t *dst, uint32_t n, uint32_t room, float inv) {
+  auto emit = [&](const QRaw<BF16> &raw, uint32_t *dst, uint32_t n, uint32_t room, float c, float inv) {
     uint32_t w[B];
-    q_codes<BF16, B>(raw, a.prescale, inv, w);
+    q_codes<BF16, B>(raw, c, inv, w);
     if (n) q_store<B>(dst, n, room, w);
   };
   const uint64_t r_cta = (uint64_t)blockIdx.x * rows_at_once;
@@ -245,18 +245,21 @@ __global__ void __launch_bounds__(kQThreads, BF16 ? 3 : 2) qnaive_encode_kernel(
     }
     float inv;
     const float s = q_scale<B>(__uint_as_float(mg), a.prescale, inv);
+    // where c g overflows the scale is infinite, its reciprocal zero and, as with a scale of zero, every code that of zero; c g
+    // itself would put codes that are no number into the chains of q_codes, which their neighbours share
+    const float c = inv > 0.0f ? a.prescale : 0.0f;
     if (live) {
       if (part == 0) {
         if (!a.per_tensor || r == 0) scales[a.per_tensor ? 0 : r] = s;
         for (uint32_t o = lanes_all * (uint32_t)B; o < row_words; ++o) dst[o] = 0;   // the row's last words, behind its last lane's
       }
-      emit(cur, dst, n_mine, row_words - part * (uint32_t)B, inv);
+      emit(cur, dst, n_mine, row_words - part * (uint32_t)B, c, inv);
       if (LONG)
 #pragma unroll 1
         for (uint32_t p = part + parts_at_once; p < lanes_all; p += parts_at_once) {
           QRaw<BF16> more;
           load_at(more, a.in + (r * (uint64_t)C + 32u * p) * ESZ, elements(p));
-          emit(more, dst + (p - part) * (uint32_t)B, elements(p), row_words - p * (uint32_t)B, inv);
+          emit(more, dst + (p - part) * (uint32_t)B, elements(p), row_words - p * (uint32_t)B, c, inv);
         }
     }
     dst += d_dst;

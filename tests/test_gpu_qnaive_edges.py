@@ -70,3 +70,17 @@ def test_a_row_beyond_four_gibibytes(dtype, n):
     want, _ = T.qnaive_decode(short, a, ws=ws)
     got, _ = T.qnaive_decode(long, b, out=x.view(1, -1).fill_(float("nan")), ws=ws)
     assert T.device_status(ws) == 0 and torch.equal(got.view(n, -1), want)
+
+
+@pytest.mark.parametrize("bits", range(2, 17))
+@pytest.mark.parametrize("per_tensor", [0, 1])
+@pytest.mark.parametrize("dtype,shape", [(torch.float32, (9, 2056)), (torch.bfloat16, (9, 1024)), (torch.bfloat16, (3, 8392))])
+def test_rows_whose_scaled_gradients_overflow(dtype, shape, per_tensor, bits):
+    """Finite gradients, and c g beyond the largest number in every third element of every second row: the scale is infinite
+    and each code that of zero."""
+    x = rows(*shape, dtype, bits)
+    x[::2, ::3] = 3e37
+    dt = T.F32 if dtype == torch.float32 else T.BF16
+    kw = dict(tokens=shape[0], hidden=shape[1], dtype=dt, bits=bits, per_tensor=per_tensor, prescale=1024.0)
+    packed, _ = T.qnaive_encode(T.QNaiveParams(**kw), x)
+    assert np.array_equal(packed.cpu().numpy(), O.qnaive_encode(O.QNaiveParams(**kw), synth.to_host_array(x)))
