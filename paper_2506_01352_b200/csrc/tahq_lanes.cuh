@@ -593,6 +593,9 @@ __device__ __forceinline__ void pack_lane(F &&t, uint32_t W, uint32_t sub, uint3
       if (mine && (four || (three && !odd))) dst[1] = v1;
     }
   } else {
+    // The lanes that take the branch of the odd width below: the two widths of a call are neighbours, so it is one branch.
+    // (Asked for here, where the warp is together: in there a lane cannot know who else is.)
+    const unsigned odd_width = __ballot_sync(kFull, (W & 1u) != 0u);
     auto width = [&](auto wc) {
       constexpr int CW = decltype(wc)::value, NW = (E * CW + 31) / 32;
       uint32_t w[NW + 1];
@@ -613,7 +616,7 @@ __device__ __forceinline__ void pack_lane(F &&t, uint32_t W, uint32_t sub, uint3
       const uint32_t first = E == 32 ? sub * (uint32_t)CW : (sub * (uint32_t)CW + 1u) >> 1;
       uint32_t n = NW;
       if constexpr (E * CW % 32) {
-        const uint32_t o = __shfl_xor_sync(__activemask(), w[0], 1);   // (the neighbour has the same width)
+        const uint32_t o = __shfl_xor_sync(odd_width, w[0], 1);   // (the neighbour has the same width)
         if (sub & 1u) {
 #pragma unroll
           for (int j = 0; j < NW; ++j) w[j] = __funnelshift_r(w[j], w[j + 1], 16);

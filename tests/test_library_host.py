@@ -73,3 +73,12 @@ def test_invalid_and_unsupported_parameters():
     bad = p.c(); bad.struct_size = 8
     assert T.lib().tahq_packed_bound(C.byref(bad)) == 0
     assert T.status_string(0) == "ok" and "small" in T.status_string(3)
+
+
+def test_no_shuffle_takes_whoever_happens_to_be_there():
+    """__activemask() names the lanes that run together at that moment, which need not be all that take the branch: votes that
+    only choose between two ways to the same result may use it, an exchange between lanes may not."""
+    for f in sorted(os.listdir(os.path.join(ROOT, "paper_2506_01352_b200", "csrc"))):
+        if f.endswith((".cu", ".cuh")):
+            src = open(os.path.join(ROOT, "paper_2506_01352_b200", "csrc", f)).read()
+            assert not re.search(r"__(shfl|reduce|match)\w*_sync\(\s*__activemask", src), f
