@@ -39,19 +39,36 @@ class _Layout(C.Structure):
 
 
 class _Kept:
-    """Parameters whose C structure is laid out once, not on every call: any change of a field drops it."""
+    """Parameters whose C structure is laid out once, not on every call.
+
+    The bytes lie in a box; a change of a field puts an empty box in its place.  A thread that lays the structure out while
+    another one changes a field fills the box that it took before it read the fields, so what it read can be kept only as
+    long as it is current.  The box is no part of the object's state: not of ``vars()``, of copies or of pickles.
+    """
+
+    __slots__ = ("_box",)
 
     def __setattr__(self, name, value):
         object.__setattr__(self, name, value)
-        object.__setattr__(self, "_bytes", None)
+        _set_box(self, [None])
+
+    def __getstate__(self):
+        return self.__dict__
+
+    def __setstate__(self, state):
+        self.__dict__.update(state)
+        _set_box(self, [None])
 
     def raw(self) -> bytes:
         """The bytes of the C structure."""
-        b = self._bytes
+        box = self._box
+        b = box[0]
         if b is None:
-            b = bytes(self.c())
-            object.__setattr__(self, "_bytes", b)
+            b = box[0] = bytes(self.c())
         return b
+
+
+_set_box = _Kept._box.__set__
 
 
 @dataclass
@@ -282,7 +299,7 @@ def encode(p: Params, x: torch.Tensor, packed: torch.Tensor | None = None, ws: t
     if stream is not None and made:   # buffers made here belong to torch's current stream: tell the allocator who uses them
         packed.record_stream(stream)
         ws.record_stream(stream)
-    rc = (_call or call()).encode(p._bytes or p.raw(), x.data_ptr(), packed.data_ptr(), packed.numel(), ws.data_ptr(),
+    rc = (_call or call()).encode(p._box[0] or p.raw(), x.data_ptr(), packed.data_ptr(), packed.numel(), ws.data_ptr(),
                                   ws.numel(), _raw_stream(_device()) if stream is None else stream.cuda_stream)
     if rc != OK:
         raise TahqError(rc)
@@ -300,7 +317,7 @@ def decode(p: Params, packed: torch.Tensor, out: torch.Tensor | None = None, ws:
         if made_ws:
             ws.record_stream(stream)
         out.record_stream(stream)
-    rc = (_call or call()).decode(p._bytes or p.raw(), packed.data_ptr(), packed.numel(), out.data_ptr(), ws.data_ptr(),
+    rc = (_call or call()).decode(p._box[0] or p.raw(), packed.data_ptr(), packed.numel(), out.data_ptr(), ws.data_ptr(),
                                   ws.numel(), _raw_stream(_device()) if stream is None else stream.cuda_stream)
     if rc != OK:
         raise TahqError(rc)
@@ -342,7 +359,7 @@ def qnaive_encode(p: QNaiveParams, x: torch.Tensor, packed: torch.Tensor | None 
         packed = torch.empty(qnaive_packed_bound(p), dtype=torch.uint8, device=x.device)
     if ws is None:
         ws = torch.empty(qnaive_workspace_bound(p), dtype=torch.uint8, device=x.device)
-    rc = (_call or call()).qnaive_encode(p._bytes or p.raw(), x.data_ptr(), packed.data_ptr(), packed.numel(), ws.data_ptr(),
+    rc = (_call or call()).qnaive_encode(p._box[0] or p.raw(), x.data_ptr(), packed.data_ptr(), packed.numel(), ws.data_ptr(),
                                          ws.numel(), _stream_of(x))
     if rc:
         raise TahqError(rc)
@@ -355,7 +372,7 @@ def qnaive_decode(p: QNaiveParams, packed: torch.Tensor, out: torch.Tensor | Non
                           dtype=torch.float32 if p.dtype == F32 else torch.bfloat16)
     if ws is None:
         ws = torch.empty(qnaive_workspace_bound(p), dtype=torch.uint8, device=packed.device)
-    rc = (_call or call()).qnaive_decode(p._bytes or p.raw(), packed.data_ptr(), packed.numel(), out.data_ptr(), ws.data_ptr(),
+    rc = (_call or call()).qnaive_decode(p._box[0] or p.raw(), packed.data_ptr(), packed.numel(), out.data_ptr(), ws.data_ptr(),
                                          ws.numel(), _stream_of(packed))
     if rc:
         raise TahqError(rc)

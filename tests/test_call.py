@@ -1,5 +1,6 @@
 """The extension module behind the codec calls: a changed parameter is seen by the next call, wrong arguments raise."""
 import copy
+import pickle
 
 import pytest
 import torch
@@ -49,3 +50,31 @@ def test_tensors_that_are_not_on_a_gpu_are_refused_before_the_call(monkeypatch):
     with pytest.raises(ValueError, match="CUDA"):
         T.encode(T.params_for(x), x, packed=packed, ws=ws)
     assert reached == []
+
+
+def test_a_field_that_changes_while_the_structure_is_laid_out_is_not_missed(monkeypatch):
+    """Another thread's change, at the worst moment: between reading the fields and keeping the bytes."""
+    p = T.Params(tokens=128, hidden=256, group_tokens=64)
+    c = T.Params.c
+
+    def interrupted(self):
+        laid_out = c(self)
+        self.tile = 32
+        return laid_out
+
+    monkeypatch.setattr(T.Params, "c", interrupted)
+    p.raw()
+    monkeypatch.setattr(T.Params, "c", c)
+    assert p.raw() == bytes(p.c()) and p.c().tile == 32
+
+
+def test_parameters_travel_as_their_fields_alone():
+    p = T.Params(tokens=128, hidden=256, group_tokens=64)
+    g = T.QNaiveParams(tokens=4, hidden=64)
+    p.raw(), g.raw()
+    assert T.Params(**vars(p)) == p and T.QNaiveParams(**vars(g)) == g
+    for q in (pickle.loads(pickle.dumps(p)), copy.copy(p), copy.deepcopy(p)):
+        assert q == p and T.tahq_encode(q, 4096, 8192, 16, 12288, 1 << 30, 0) == 3
+        q.tile = 48
+        assert T.tahq_encode(q, 4096, 8192, 16, 12288, 1 << 30, 0) == 1 and T.tahq_encode(p, 4096, 8192, 16, 12288, 1 << 30, 0) == 3
+    assert p.__reduce_ex__(4)[2] == {k: getattr(p, k) for k in T.Params.__dataclass_fields__}   # what a file holds of it
