@@ -242,10 +242,11 @@ def trace_reset(buf: torch.Tensor) -> None:
     buf.copy_(v.reshape(-1).to(buf.device))
 
 
-# The current stream as a number (torch.cuda.current_stream() builds an object around it, in three microseconds).  The
-# tensors of a call exist, so CUDA is initialised.
-_device = getattr(torch._C, "_cuda_getDevice", None)
-_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+# The current stream as a number.  torch.cuda.current_stream() builds an object around it, in three microseconds; the two
+# functions that do without are private, so a torch that lacks one takes the public way.  The tensors of a call exist, so CUDA
+# is initialised.
+_device = getattr(torch._C, "_cuda_getDevice", torch.cuda.current_device)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", lambda device: torch.cuda.current_stream(device).cuda_stream)
 
 
 def tahq_encode(p: Params, d_in: int, d_packed: int, packed_cap: int, d_ws: int, ws_cap: int, stream: int) -> int:

@@ -1,6 +1,9 @@
 """The extension module behind the codec calls: a changed parameter is seen by the next call, wrong arguments raise."""
 import copy
+import importlib.util
 import pickle
+import sys
+import types
 
 import pytest
 import torch
@@ -78,3 +81,15 @@ def test_parameters_travel_as_their_fields_alone():
         q.tile = 48
         assert T.tahq_encode(q, 4096, 8192, 16, 12288, 1 << 30, 0) == 1 and T.tahq_encode(p, 4096, 8192, 16, 12288, 1 << 30, 0) == 3
     assert p.__reduce_ex__(4)[2] == {k: getattr(p, k) for k in T.Params.__dataclass_fields__}   # what a file holds of it
+
+
+def test_a_torch_without_the_private_stream_functions(monkeypatch):
+    for name in ("_cuda_getDevice", "_cuda_getCurrentRawStream"):
+        monkeypatch.delattr(torch._C, name, raising=False)
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 1)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda device: types.SimpleNamespace(cuda_stream=40 + device))
+    spec = importlib.util.spec_from_file_location("paper_2506_01352_b200._binding_again", T.__file__)
+    again = importlib.util.module_from_spec(spec)
+    monkeypatch.setitem(sys.modules, spec.name, again)   # (dataclasses look their module up)
+    spec.loader.exec_module(again)
+    assert again._raw_stream(again._device()) == 41
