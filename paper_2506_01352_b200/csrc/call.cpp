@@ -6,15 +6,41 @@
 
 #include <string.h>
 
+#include <initializer_list>
+
 #include "../../include/tahq.h"
 
 namespace {
 
-// an address or a size: a Python integer, or None for a null pointer
+// An address or a size: a Python integer (taken modulo 2^64), or None for a null pointer; else what ctypes would take, a
+// c_void_p or c_size_t by its value, and an object with an `_as_parameter_` (a torch stream has one).
 bool to_word(PyObject *o, unsigned long long *v) {
   if (o == Py_None) { *v = 0; return true; }
-  *v = PyLong_AsUnsignedLongLong(o);
-  return !(*v == (unsigned long long)-1 && PyErr_Occurred());
+  if (PyLong_Check(o)) {
+    *v = PyLong_AsUnsignedLongLongMask(o);
+    return !(*v == (unsigned long long)-1 && PyErr_Occurred());
+  }
+  for (const char *name : {"_as_parameter_", "value"}) {
+    PyObject *w = PyObject_GetAttrString(o, name);
+    if (!w) {
+      if (!PyErr_ExceptionMatches(PyExc_AttributeError)) return false;
+      PyErr_Clear();
+      continue;
+    }
+    bool ok = false;
+    if (w == Py_None || PyLong_Check(w)) {
+      ok = to_word(w, v);
+    } else {   // (a stream's parameter is a c_void_p)
+      PyObject *x = PyObject_GetAttrString(w, "value");
+      if (x && (x == Py_None || PyLong_Check(x))) ok = to_word(x, v);
+      else PyErr_Format(PyExc_TypeError, "expected an integer or None, got %.100s", Py_TYPE(w)->tp_name);
+      Py_XDECREF(x);
+    }
+    Py_DECREF(w);
+    return ok;
+  }
+  PyErr_Format(PyExc_TypeError, "expected an integer or None, got %.100s", Py_TYPE(o)->tp_name);
+  return false;
 }
 
 // (params: bytes, six words): pointer, pointer or size ... in the order of the C function

@@ -1,5 +1,6 @@
 """The extension module behind the codec calls: a changed parameter is seen by the next call, wrong arguments raise."""
 import copy
+import ctypes
 import importlib.util
 import pickle
 import sys
@@ -93,3 +94,19 @@ def test_a_torch_without_the_private_stream_functions(monkeypatch):
     monkeypatch.setitem(sys.modules, spec.name, again)   # (dataclasses look their module up)
     spec.loader.exec_module(again)
     assert again._raw_stream(again._device()) == 41
+
+
+@pytest.mark.parametrize("form", [int, ctypes.c_void_p, lambda v: types.SimpleNamespace(_as_parameter_=v),
+                                  lambda v: types.SimpleNamespace(_as_parameter_=ctypes.c_void_p(v)), lambda v: v - (1 << 64)])
+def test_the_forms_of_an_address(form):
+    """As ctypes takes them, addresses in the upper half as negative numbers among them: what is wrong with the call is its
+    alignment (4), not its arguments."""
+    p = T.Params(tokens=128, hidden=256, group_tokens=64)
+    odd, even = form(0x9000000000000008), form(0x9000000000000010)
+    assert T.tahq_encode(p, odd, even, 1 << 40, even, ctypes.c_size_t(1 << 40), even) == 4
+    assert T.tahq_decode(p, even, 1 << 40, odd, even, 1 << 40, form(0)) == 4
+    g = T.QNaiveParams(tokens=4, hidden=64)
+    assert T.tahq_qnaive_encode(g, even, odd, 1 << 40, even, 1 << 40, None) == 4
+    for wrong in ("x", b"x", 1.5, [1], types.SimpleNamespace(value="x")):
+        with pytest.raises(TypeError):
+            T.tahq_encode(p, wrong, 0, 0, 0, 0, 0)
