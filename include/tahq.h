@@ -148,8 +148,8 @@ tahq_status tahq_decode(const tahq_params *p, const void *d_packed, size_t packe
 /*
  * Encode without a caller-provided workspace (the paper has no counterpart; this is a convenience of
  * the library).  Same operation, same bytes in d_packed as tahq_encode, but the scratch memory lives
- * in a fixed TAHQ_NOALLOC_SCRATCH_BYTES (8 MiB) buffer that is part of the library image on every GPU
- * that loads it, so the call neither needs a workspace pointer nor allocates or frees anything.
+ * in a fixed buffer (TAHQ_NOALLOC_SCRATCH_BYTES and 8 MiB of prefixes) that is part of the library image
+ * on every GPU that loads it, so the call neither needs a workspace pointer nor allocates or frees anything.
  *
  * Who needs this: code that is handed device pointers but owns no allocator and may not call
  * cudaMalloc -- a communication plug-in working on buffers registered by its host framework, a
@@ -157,16 +157,16 @@ tahq_status tahq_decode(const tahq_params *p, const void *d_packed, size_t packe
  * where an allocation would force a device-wide synchronisation.
  *
  * Limits and rules
- *   - Accepts exactly the configurations with tahq_workspace_bound(p) <= TAHQ_NOALLOC_SCRATCH_BYTES
- *     (e.g. 8192 x 4096 elements at tile 64 needs 3.3 MB); anything larger returns
- *     TAHQ_ERR_TOO_LARGE and enqueues nothing.
+ *   - Accepts every configuration with tahq_workspace_bound(p) <= TAHQ_NOALLOC_SCRATCH_BYTES (8192 x 4096
+ *     elements at tile 64 need 2.3 MB).  Where ranking groups share words of the bit map, the offset
+ *     prefixes (4 bytes per 32 tiles) do not count towards that: the library has room for them.
+ *     Anything larger returns TAHQ_ERR_TOO_LARGE and enqueues nothing.
  *   - The first call on each device looks up the device address of the built-in buffer (a host-side
  *     set-up step, done once per device with that device current).  Make that first call before any
  *     stream capture begins.
- *   - All calls on one device share the one buffer.  It keeps the previous call's contents; each call
- *     clears the part that must start at zero on the given stream.  Two calls that may overlap on the
- *     GPU (different streams without an ordering between them) race on it: order them, or use
- *     tahq_encode with separate workspaces.
+ *   - All calls on one device share the one buffer.  It keeps the previous call's contents, of which no
+ *     call reads any.  Two calls that may overlap on the GPU (different streams without an ordering
+ *     between them) race on it: order them, or use tahq_encode with separate workspaces.
  *   - The device status word of the call cannot be read back by the caller; use tahq_encode when that
  *     is needed.
  * Errors: as tahq_encode, plus TAHQ_ERR_TOO_LARGE.

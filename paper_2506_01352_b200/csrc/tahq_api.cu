@@ -60,9 +60,6 @@ static tahq_status make_plan(const tahq_params *p, Plan *pl) {
   pl->ws_zero_end = o;                                      // [0, ws_zero_end) is cleared by a decode with a look-back
   pl->ws_scores = o; o = up(o + (pl->mixed ? 4 * (L.n_tiles / pl->alloc_m) : 0), 256);
   pl->ws_pre = o;    o = up(o + (pl->mixed ? 4 * ((L.n_tiles + 31) / 32) : 0), 256);
-  // words of the selection's slices, where a group's may not fit into shared memory
-  const bool long_groups = pl->mixed && pl->rank_per_group > 32ull * kWordsShared;
-  pl->ws_words = o;  o = up(o + (long_groups ? 8 * L.n_groups * ((pl->rank_per_group + 31) / 32 + 16) : 0), 256);
   pl->ws_total = o;
   return TAHQ_OK;
 }
@@ -117,7 +114,6 @@ static void fill_args(const tahq_params *p, const Plan &pl, uint8_t *ws, Args *a
   a->trace = g_trace;
   a->whole_words = pl.whole_words;
   a->pre = reinterpret_cast<uint32_t *>(ws + pl.ws_pre);
-  a->words = reinterpret_cast<uint32_t *>(ws + pl.ws_words);
   a->scores = reinterpret_cast<float *>(ws + pl.ws_scores);
   a->bf16 = p->dtype == TAHQ_BF16;
   a->tile = p->tile;
@@ -137,7 +133,10 @@ static bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 
 
 // Scratch for tahq_encode_noalloc: part of the library image, resident on every GPU that loads it.
 // In host code this name is only a handle; the device address is looked up once per device.
-static __device__ __align__(256) unsigned char g_noalloc_scratch[TAHQ_NOALLOC_SCRATCH_BYTES];
+// Room for TAHQ_NOALLOC_SCRATCH_BYTES, and behind that for the offset prefixes of calls whose ranking groups are no whole words
+// (4 bytes per 32 tiles, 2^26 tiles at most): the accepted calls are those that fit without them.
+constexpr uint64_t kNoallocPrefixes = 8ull << 20;
+static __device__ __align__(256) unsigned char g_noalloc_scratch[TAHQ_NOALLOC_SCRATCH_BYTES + kNoallocPrefixes + 256];
 static void *g_noalloc_addr[64];
 static std::atomic<int> g_noalloc_ready[64];
 
@@ -180,6 +179,9 @@ tahq_status tahq_encode(const tahq_params *p, const void *d_in, void *d_packed, 
   fill_args(p, pl, static_cast<uint8_t *>(d_ws), &a);
   a.in = static_cast<const uint8_t *>(d_in);
   a.packed = static_cast<uint8_t *>(d_packed);
+  // The selection of a group of more than 32 * kWordsShared tiles keeps the words of its slices, and their running counts,
+  // where quantise + pack puts the codes afterwards: 8 bytes per 32 ranked tiles (and 16 words more), whose codes are 64 and up.
+  a.words = reinterpret_cast<uint32_t *>(a.packed + a.off_payload);
   // groups that share words of the bit map: the selection puts those together on zeroes
   if (pl.mixed && !pl.whole_words && pl.alloc_m == 1 &&
       launch_clear(a.packed + a.off_bitmap, up((pl.L.n_tiles + 7) / 8, 128), st) != TAHQ_OK)
@@ -227,7 +229,7 @@ tahq_status tahq_encode_noalloc(const tahq_params *p, const void *d_in, void *d_
   Plan pl;
   const tahq_status s = make_plan(p, &pl);
   if (s != TAHQ_OK) return s;
-  if (pl.ws_total > (uint64_t)TAHQ_NOALLOC_SCRATCH_BYTES) return TAHQ_ERR_TOO_LARGE;
+  if ((pl.whole_words ? pl.ws_total : pl.ws_pre) > (uint64_t)TAHQ_NOALLOC_SCRATCH_BYTES) return TAHQ_ERR_TOO_LARGE;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return TAHQ_ERR_CUDA;
   if (!g_noalloc_ready[dev].load(std::memory_order_acquire)) {
@@ -237,7 +239,7 @@ tahq_status tahq_encode_noalloc(const tahq_params *p, const void *d_in, void *d_
     g_noalloc_addr[dev] = ptr;
     g_noalloc_ready[dev].store(1, std::memory_order_release);
   }
-  return tahq_encode(p, d_in, d_packed, packed_cap, g_noalloc_addr[dev], TAHQ_NOALLOC_SCRATCH_BYTES, stream);
+  return tahq_encode(p, d_in, d_packed, packed_cap, g_noalloc_addr[dev], sizeof(g_noalloc_scratch), stream);
 }
 
 // ---- fixed-point gradient compressor -------------------------------------------------------------------

@@ -24,7 +24,7 @@ struct Plan {
   uint32_t alloc_m;            // quantisation tiles per allocation tile (Sec. 3.2; 1 by default)
   uint64_t rank_per_group, rank_k;   // allocation tiles per ranking group, and how many of them get the higher width
   // workspace offsets
-  uint64_t ws_flags, ws_zero_end, ws_scores, ws_pre, ws_words, ws_total;
+  uint64_t ws_flags, ws_zero_end, ws_scores, ws_pre, ws_total;   // (ws_pre: the last section)
 };
 
 // ---- launch bookkeeping --------------------------------------------------------------------------------

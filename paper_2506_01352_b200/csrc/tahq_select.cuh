@@ -516,7 +516,8 @@ __global__ void __launch_bounds__(kSelThreads, 2) select_kernel(const __grid_con
   const uint32_t i0 = rank * per_cta;                                   // first tile of the slice, inside the group
   const uint32_t n_loc = i0 < ng ? (ng - i0 < per_cta ? ng - i0 : per_cta) : 0u;
   const uint32_t n_words = (n_loc + 31u) / 32u, n_it = (n_loc + 4 * kSelThreads - 1) / (4 * kSelThreads);
-  // the slice's words (and running counts): in shared memory, or in the workspace when the slice is very long
+  // the slice's words (and running counts): in shared memory, or in the payload section, where the codes come later, when the
+  // slice is very long
   const bool in_smem = per_cta <= 32u * kWordsShared;
   uint32_t *words = s_words, *wpre = s_hist;
   if (!in_smem) {
@@ -728,7 +729,7 @@ __global__ void __launch_bounds__(kSelThreads, 2) select_kernel(const __grid_con
   // ---- 5: running counts, words, and out.  512 words at a time.
   uint32_t *const bitmap = reinterpret_cast<uint32_t *>(a.packed + a.off_bitmap);
   const uint64_t t0 = (g * (uint64_t)ng + i0) * a.alloc_m;   // first quantisation tile of the slice
-  auto word_at = [&](uint32_t w) { return *(volatile const uint32_t *)(words + w); };   // (in the workspace: changed by atomics)
+  auto word_at = [&](uint32_t w) { return *(volatile const uint32_t *)(words + w); };   // (in global memory: changed by atomics)
   uint32_t carry = before;
   for (uint32_t w0 = 0; w0 < n_words; w0 += kSelThreads) {
     const uint32_t w = w0 + threadIdx.x, wv = w < n_words ? word_at(w) : 0u, c = (uint32_t)__popc(wv);

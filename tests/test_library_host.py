@@ -82,3 +82,13 @@ def test_no_shuffle_takes_whoever_happens_to_be_there():
         if f.endswith((".cu", ".cuh")):
             src = open(os.path.join(ROOT, "paper_2506_01352_b200", "csrc", f)).read()
             assert not re.search(r"__(shfl|reduce|match)\w*_sync\(\s*__activemask", src), f
+
+
+@pytest.mark.parametrize("tokens,M,G,m", [(9018, 214, 128, 1), (14572, 138, 64, 1), (16257, 244, 128, 2), (25921, 300, 128, 4),
+                                          (736428, 77, 64, 77), (669310, 3, 8, 1), (1023, 1024, 64, 1), (65535, 16, 64, 1)])
+def test_the_workspace_free_encode_takes_what_it_always_took(tokens, M, G, m):
+    """Scores (4 bytes a ranked tile) and look-back flags fit the built-in scratch; the offset prefixes have room of their own.
+    (Accepted is: refused for the packed buffer's size, or, without a GPU, for the lack of one.)"""
+    p = T.Params(tokens=tokens, hidden=M * G, group_tokens=4 if m == M else 0, tile=G, budget_millibits=3800, alloc_tile=m * G)
+    assert T.packed_bound(p) > 0 and 4 * tokens * M // m + 8 * 2048 + 512 <= T.NOALLOC_SCRATCH_BYTES
+    assert T.tahq_encode_noalloc(p, 4096, 8192, 16, 0) in (3, 5)
