@@ -349,9 +349,14 @@ __global__ void __launch_bounds__(kLaneThreads, 1) decode_lanes_kernel(const Arg
         if (a.own_prefix) {
           base_hi = __reduce_add_sync(kFull, lane < kLaneWarps ? s_sum[1][lane] : 0u);
           stop = refuse;
-          if (last)   // (at most 65536 words: one segment)
+          uint32_t rest = 0;   // (a device of fewer than 86 SMs: words of the CTA's later segments)
+          if (s1 < u1) {
+            for (uint64_t i = s1 + threadIdx.x; i < u1; i += NT) rest += __popc(bm_word(i));
+            rest = block_sum<NT>(rest);
+          }
+          if (last)
             *a.status = (refuse ? 1u /* TAHQ_DEV_BAD_HEADER */ : 0u) |
-                        ((!refuse && base_hi + total != a.n_groups * a.k_hi) ? 2u /* TAHQ_DEV_BAD_BITMAP */ : 0u);
+                        ((!refuse && base_hi + total + rest != a.n_groups * a.k_hi) ? 2u /* TAHQ_DEV_BAD_BITMAP */ : 0u);
         } else {
           // a CTA publishes the count of the words that start in its range (one shared by two CTAs counts in the first)
           if (refuse && threadIdx.x == 0) atomicOr(a.status, 1u);
