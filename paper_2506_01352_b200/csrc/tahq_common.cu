@@ -115,9 +115,13 @@ tahq_status launch_alloc_score(const Args &a, const DevInfo &d, cudaStream_t st)
   const uint64_t n_alloc = a.n_tiles / a.alloc_m;
   const uint64_t want = (n_alloc + kThreads / 32 - 1) / (kThreads / 32), cap = (uint64_t)d.sms * 8;
   const unsigned grid = (unsigned)(want < cap ? want : cap);
+  // a tile of up to 256 or 512 channels has one or two rounds: more at a time would be padding
+  const uint32_t A = a.alloc_m * a.tile;
+  void (*const kernels[6])(Args) = {alloc_score_kernel<false, 1>, alloc_score_kernel<false, 2>, alloc_score_kernel<false, 4>,
+                                    alloc_score_kernel<true, 1>,  alloc_score_kernel<true, 2>,  alloc_score_kernel<true, 4>};
   cudaError_t e;
-  if (a.bf16) TAHQ_LAUNCH("alloc_score", st, e = launch_dependent(alloc_score_kernel<true>, grid, kThreads, 0, st, a));
-  else TAHQ_LAUNCH("alloc_score", st, e = launch_dependent(alloc_score_kernel<false>, grid, kThreads, 0, st, a));
+  TAHQ_LAUNCH("alloc_score", st,
+              e = launch_dependent(kernels[3 * a.bf16 + (A <= 256 ? 0 : A <= 512 ? 1 : 2)], grid, kThreads, 0, st, a));
   return e == cudaSuccess ? TAHQ_OK : TAHQ_ERR_CUDA;
 }
 

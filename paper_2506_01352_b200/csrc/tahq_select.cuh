@@ -31,11 +31,10 @@ __device__ __forceinline__ float warp_tree(float x, uint32_t n, int lane) {   //
   }
   return __shfl_sync(kFull, x, 0);
 }
-// Four rounds of 256 elements go at a time: their loads and the steps of their trees are in flight together (one after the
+// U rounds of 256 elements go at a time: their loads and the steps of their trees are in flight together (one after the
 // other, the 16 rounds of a 2048-channel tile were a chain of load and shuffle latencies: 4096 x 2048 bf16 13.7 -> 10.8 us with two logarithms to an instruction).
-template <bool BF16, class F>
+template <bool BF16, int U, class F>
 __device__ __forceinline__ float alloc_tree(const uint8_t *base, uint32_t n_oct, int lane, F &&f) {
-  constexpr int U = 4;
   const uint32_t rounds = (n_oct + 31) / 32;
   float rs = 0.0f;   // lane r keeps the sum of round r
   for (uint32_t r = 0; r < rounds; r += U) {
@@ -93,7 +92,7 @@ __device__ __forceinline__ float alloc_tree(const uint8_t *base, uint32_t n_oct,
   }
   return warp_tree(rs, rounds, lane);
 }
-template <bool BF16>
+template <bool BF16, int U>
 __global__ void __launch_bounds__(kThreads) alloc_score_kernel(const Args a) {
   const int lane = threadIdx.x & 31;
   const uint64_t warp = ((uint64_t)blockIdx.x * kThreads + threadIdx.x) >> 5;
@@ -106,9 +105,9 @@ __global__ void __launch_bounds__(kThreads) alloc_score_kernel(const Args a) {
   clear_bitmap(a);
   for (uint64_t t = warp; t < n_alloc; t += n_warps) {
     const uint8_t *base = a.in + t * (uint64_t)A * (BF16 ? 2 : 4);
-    const float L1 = alloc_tree<BF16>(base, n_oct, lane, [](float2 m) { return m; });
+    const float L1 = alloc_tree<BF16, U>(base, n_oct, lane, [](float2 m) { return m; });
     const float inv = __fdiv_rn(1.0f, L1 + a.eps_l1);
-    const float S = alloc_tree<BF16>(base, n_oct, lane, [&](float2 m) {   // (scalar products: they are added to)
+    const float S = alloc_tree<BF16, U>(base, n_oct, lane, [&](float2 m) {   // (scalar products: they are added to)
       const float2 p = f2(m.x * inv, m.y * inv), l = lg2_fma2(add2(p, f2(a.eps_log)));
       return f2(p.x * l.x, p.y * l.y);
     });
