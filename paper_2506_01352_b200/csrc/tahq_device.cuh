@@ -341,24 +341,24 @@ __device__ __forceinline__ float tile_score(const uint8_t *stage, int row, float
 // the sums, each weighted by p or by |log2 a| <= 127 times a few units in the last place: under 1e-4
 // in all.  It is only used to decide which tiles are far enough from a group's threshold to be
 // classified without their exact score; see select_kernel.  All of this holds while L' is nowhere near the ends of binary32:
-// see screen_result.
+// see screen_range.
 __device__ __forceinline__ float lg2_approx(float x) {
   float y;
   asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-// The screening score s of a tile with L' = Lp; NaN where the screening does not hold: below 2^-60 the 1e-30 added to every
-// magnitude would count (a varepsilon near zero and a tile of next to nothing), above 2^60 the sums come near the largest
-// numbers.  The kernel that screens goes back to such tiles when it is through (exact_where_unscreened).
-__device__ __forceinline__ float screen_result(float s, float Lp) {
-  return Lp >= 0x1p-60f && Lp <= 0x1p60f ? s : __int_as_float(0x7fffffff);
-}
+// Does the screening hold for a tile with L' = Lp?  Not below 2^-60, where the 1e-30 added to every magnitude would count (a
+// varepsilon near zero and a tile of next to nothing), nor above 2^60, where the sums come near the largest numbers, nor where
+// it is no number.  A warp that screens keeps the largest of these; beyond kScreenRange it goes back over its tiles when it is
+// through (exact_scores_of).
+constexpr uint32_t kScreenRange = 120u << 23;   // from 2^-60 to 2^60, in the bits of binary32
+__device__ __forceinline__ uint32_t screen_range(float Lp) { return __float_as_uint(Lp) - 0x21800000u; }
 // An exact score as it is stored and ranked: every one a number, of a size that the selection can calculate with.  (A tile of
 // zeroes without epsilon has p = 0/0; it ranks first, as its key without this would.)
 __device__ __forceinline__ float ranked_score(float s) { return s == s ? fminf(fmaxf(s, -1e30f), 1e30f) : 1e30f; }
 
 template <class C>
-__device__ __forceinline__ float tile_score_screen(const uint8_t *stage, int row, float eps_l1) {
+__device__ __forceinline__ float tile_score_screen(const uint8_t *stage, int row, float eps_l1, uint32_t &range) {
   const float tiny = 1e-30f;
   float pl[C::NOCT], pt[C::NOCT];
 #pragma unroll
@@ -388,7 +388,8 @@ __device__ __forceinline__ float tile_score_screen(const uint8_t *stage, int row
   const float Lp = L + eps_l1;
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(Lp));
-  return screen_result(__fmaf_rn(lg2_approx(Lp), L, -T) * r, Lp);
+  range = max(range, screen_range(Lp));
+  return __fmaf_rn(lg2_approx(Lp), L, -T) * r;
 }
 
 // Exact score of one whole tile read straight from global memory by NOCT neighbouring lanes, lane o
@@ -428,25 +429,20 @@ __device__ __forceinline__ float exact_score_coop(const uint8_t *tile, int o, fl
   return 0.0f - S;
 }
 
-// Exact scores for those of n <= 32 consecutive tiles whose score this warp has stored as NaN (screen_result); `also`: a second
-// copy of the scores, or null.  All lanes of the warp call this; out of line, since it is hardly ever run.
+// Exact scores of n consecutive tiles by a warp; `also`: a second copy of the scores, or null.  (Hardly ever run; out of line it
+// costs every launch of its kernel 0.3 us all the same.)
 template <int NOCT, bool BF16>
-static __device__ __noinline__ void exact_where_unscreened(const uint8_t *tiles, uint32_t n, float eps_l1, float eps_log, float *scores,
-                                                           float *also) {
-  const uint32_t lane = threadIdx.x & 31u, sub = lane % NOCT, grp = lane / NOCT;
-  __syncwarp();   // the scores were stored by other lanes
-  const float s = lane < n ? *(volatile float *)(scores + lane) : 0.0f;
-  unsigned m = __ballot_sync(kFull, s != s);
-  while (m) {
-    unsigned mine = m;   // the grp-th tile of those left
-    for (uint32_t i = 0; i < grp; ++i) mine &= mine - 1u;
-    const uint32_t t = mine ? (uint32_t)__ffs(mine) - 1u : 0u;
-    const float ex = ranked_score(exact_score_coop<NOCT, BF16>(tiles + t * (uint32_t)(NOCT * 8 * (BF16 ? 2 : 4)), sub, eps_l1, eps_log));
-    if (mine && sub == 0) {
+__device__ __forceinline__ void exact_scores_of(const uint8_t *tiles, uint32_t n, float eps_l1, float eps_log, float *scores, float *also) {
+  const uint32_t lane = threadIdx.x & 31u, sub = lane % NOCT;
+  __syncwarp();   // (other lanes have stored the screening scores)
+  for (uint32_t t0 = 0; t0 < n; t0 += 32 / NOCT) {
+    const uint32_t t = t0 + lane / NOCT;
+    const bool live = t < n;
+    const float ex = ranked_score(exact_score_coop<NOCT, BF16>(tiles + (live ? t : t0) * (uint32_t)(NOCT * 8 * (BF16 ? 2 : 4)), sub, eps_l1, eps_log));
+    if (live && sub == 0) {
       scores[t] = ex;
       if (also) also[t] = ex;
     }
-    for (int i = 0; i < 32 / NOCT; ++i) m &= m - 1u;
   }
 }
 

@@ -480,7 +480,7 @@ __global__ void __launch_bounds__(kScoreThreads, 2) score_lanes_kernel(const Arg
   if (blockIdx.x == 0 && threadIdx.x == 0) *a.status = 0;   // nothing else of the workspace has to start at zero
   const uint32_t left0 = r1 - r0 > warp ? r1 - r0 - warp : 0u;
   uint32_t left = left0;   // the warp's next round is r0 + left - 1
-  bool again = false;      // a tile that the screening does not hold for
+  uint32_t range = 0;      // see screen_range
   if (left) load(r0 + left - 1u);
   while (left) {
     uint32_t w[16];
@@ -516,17 +516,14 @@ __global__ void __launch_bounds__(kScoreThreads, 2) score_lanes_kernel(const Arg
     const float Lp = Ls + a.eps_l1;
     float rc;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rc) : "f"(Lp));
+    range = max(range, screen_range(Lp));
     const uint32_t tile = r * TPR + lane / P;
-    if (sub == 0 && tile < n_tiles) {
-      const float s = screen_result(__fmaf_rn(lg2_approx(Lp), Ls, -Ts) * rc, Lp);
-      a.scores[tile] = s;
-      again |= s != s;
-    }
+    if (sub == 0 && tile < n_tiles) a.scores[tile] = __fmaf_rn(lg2_approx(Lp), Ls, -Ts) * rc;
   }
-  if (__any_sync(kFull, again))
+  if (__any_sync(kFull, range > kScreenRange))
     for (left = left0; left; left = left > WARPS ? left - WARPS : 0u) {
       const uint32_t tile = (r0 + left - 1u) * TPR;
-      exact_where_unscreened<C::G / 8, C::BF16>(a.in + (uint64_t)tile * D::TB, n_tiles - tile < TPR ? n_tiles - tile : TPR, a.eps_l1,
+      exact_scores_of<C::G / 8, C::BF16>(a.in + (uint64_t)tile * D::TB, n_tiles - tile < TPR ? n_tiles - tile : TPR, a.eps_l1,
                                                 a.eps_log, a.scores + tile, nullptr);
     }
 }

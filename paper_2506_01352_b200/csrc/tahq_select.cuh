@@ -441,7 +441,7 @@ __device__ __forceinline__ void slice_scores(const Args &a, uint64_t first, uint
     const uint32_t t = r * TPR + lane / P;
     load_64_bytes<false>(in + (uint64_t)(t < n ? t : 0u) * D::TB, raw);
   };
-  bool again = false;   // a tile that the screening does not hold for
+  uint32_t range = 0;   // see screen_range
   if (warp < n_rounds) load(warp);
   for (uint32_t r = warp; r < n_rounds; r += kSelThreads / 32) {
     uint32_t w[16];
@@ -473,17 +473,17 @@ __device__ __forceinline__ void slice_scores(const Args &a, uint64_t first, uint
     const float Lp = Ls + a.eps_l1;
     float rc;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rc) : "f"(Lp));
+    range = max(range, screen_range(Lp));
     const uint32_t t = r * TPR + lane / P;
     if (sub == 0 && t < n) {
-      const float s = screen_result(__fmaf_rn(lg2_approx(Lp), Ls, -Ts) * rc, Lp);
+      const float s = __fmaf_rn(lg2_approx(Lp), Ls, -Ts) * rc;
       s_out[t] = s;
       out[t] = s;
-      again |= s != s;
     }
   }
-  if (__any_sync(kFull, again))
+  if (__any_sync(kFull, range > kScreenRange))
     for (uint32_t r = warp; r < n_rounds; r += kSelThreads / 32)
-      exact_where_unscreened<C::G / 8, C::BF16>(a.in + (first + r * TPR) * D::TB, n - r * TPR < TPR ? n - r * TPR : TPR, a.eps_l1, a.eps_log,
+      exact_scores_of<C::G / 8, C::BF16>(a.in + (first + r * TPR) * D::TB, n - r * TPR < TPR ? n - r * TPR : TPR, a.eps_l1, a.eps_log,
                                                 s_out + r * TPR, out + r * TPR);
 }
 

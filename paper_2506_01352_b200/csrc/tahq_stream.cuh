@@ -193,12 +193,12 @@ __global__ void __launch_bounds__(kThreads, 2) score_kernel(const Args a, const 
     ring.commit();
   }
   int slot = 0;
-  bool again = false;   // (screening) a tile that it does not hold for
+  uint32_t range = 0;   // (screening) see screen_range
   for (uint32_t k = first; k < nu; k += stride) {
     const uint64_t u = unit_of(k);
     ring.wait(a, slot);
     const uint8_t *stage = ring.slot(slot);
-    const float s = EXACT ? ranked_score(tile_score<C>(stage, lane, a.eps_l1, a.eps_log)) : tile_score_screen<C>(stage, lane, a.eps_l1);
+    const float s = EXACT ? ranked_score(tile_score<C>(stage, lane, a.eps_l1, a.eps_log)) : tile_score_screen<C>(stage, lane, a.eps_l1, range);
     __syncwarp();
     {
       const uint32_t kn = k + (uint32_t)NST * stride;
@@ -207,18 +207,15 @@ __global__ void __launch_bounds__(kThreads, 2) score_kernel(const Args a, const 
     }
     slot = (slot + 1 == NST) ? 0 : slot + 1;
     const uint64_t tile = (u * 32 + lane) / C::LPT;
-    if (tile < a.n_tiles && (C::LPT == 1 || !(lane & 1))) {
-      a.scores[tile] = s;
-      if (!EXACT) again |= s != s;
-    }
+    if (tile < a.n_tiles && (C::LPT == 1 || !(lane & 1))) a.scores[tile] = s;
   }
   cp_async_wait<0>();
   if constexpr (!EXACT) {
     constexpr uint32_t TPU = 32 / C::LPT;   // tiles of a unit
-    if (__any_sync(kFull, again))
+    if (__any_sync(kFull, range > kScreenRange))   // (rows behind the last tile are zeroes and may say so too)
       for (uint32_t k = first; k < nu; k += stride) {
         const uint64_t tile = unit_of(k) * TPU, left = a.n_tiles - tile;
-        exact_where_unscreened<C::G / 8, C::BF16>(a.in + tile * (uint64_t)(C::G * C::ESZ), left < TPU ? (uint32_t)left : TPU, a.eps_l1,
+        exact_scores_of<C::G / 8, C::BF16>(a.in + tile * (uint64_t)(C::G * C::ESZ), left < TPU ? (uint32_t)left : TPU, a.eps_l1,
                                                   a.eps_log, a.scores + tile, nullptr);
       }
   }
