@@ -397,9 +397,8 @@ __device__ __forceinline__ float tile_score_screen(const uint8_t *stage, int row
 // arithmetic and summation tree as tile_score: the tree over the groups of eight runs as xor
 // shuffles (neighbours first; addition is commutative, so every lane ends with the same bits).
 // All 32 lanes of the warp must call it.
-template <int NOCT, bool BF16>
-__device__ __forceinline__ float exact_score_coop(const uint8_t *tile, int o, float eps_l1, float eps_log) {
-  float v[8];
+template <bool BF16>
+__device__ __forceinline__ void load_abs_oct_global(const uint8_t *tile, int o, float (&v)[8]) {
   if constexpr (BF16) {
     const uint4 w = __ldg(reinterpret_cast<const uint4 *>(tile) + o);
     const uint32_t u[4] = {w.x, w.y, w.z, w.w};
@@ -414,10 +413,15 @@ __device__ __forceinline__ float exact_score_coop(const uint8_t *tile, int o, fl
     v[0] = fabsf(a.x); v[1] = fabsf(a.y); v[2] = fabsf(a.z); v[3] = fabsf(a.w);
     v[4] = fabsf(b.x); v[5] = fabsf(b.y); v[6] = fabsf(b.z); v[7] = fabsf(b.w);
   }
+}
+// ZEROES: many of the tiles are expected to hold nothing (padding comes by the thousand of equal scores).
+template <int NOCT, bool ZEROES = false>
+__device__ __forceinline__ float exact_score_of_octs(float (&v)[8], float eps_l1, float eps_log) {
   float L1 = tree8(v);
 #pragma unroll
   for (int h = 1; h < NOCT; h *= 2) L1 = L1 + __shfl_xor_sync(kFull, L1, h);
   const float inv = __fdiv_rn(1.0f, L1 + eps_l1);
+  if (ZEROES && __all_sync(kFull, L1 == 0.0f && inv <= 3.402823466e38f)) return 0.0f;
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     const float p = v[k] * inv;
@@ -427,6 +431,12 @@ __device__ __forceinline__ float exact_score_coop(const uint8_t *tile, int o, fl
 #pragma unroll
   for (int h = 1; h < NOCT; h *= 2) S = S + __shfl_xor_sync(kFull, S, h);
   return 0.0f - S;
+}
+template <int NOCT, bool BF16>
+__device__ __forceinline__ float exact_score_coop(const uint8_t *tile, int o, float eps_l1, float eps_log) {
+  float v[8];
+  load_abs_oct_global<BF16>(tile, o, v);
+  return exact_score_of_octs<NOCT>(v, eps_l1, eps_log);
 }
 
 // Exact scores of n consecutive tiles by a warp; `also`: a second copy of the scores, or null.  (Hardly ever run; out of line it

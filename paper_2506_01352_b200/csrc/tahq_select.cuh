@@ -300,65 +300,202 @@ struct SelShared {
   uint32_t tot[kClMaxCtas];      // (radix) set bits in each CTA's words
   uint32_t n_keys;               // (first CTA) list slots handed out so far
   uint32_t n_total;              // candidates of the whole cluster (every CTA is told)
-  uint32_t digit_pick[2];        // radix selection: chosen digit, remaining rank
+  uint32_t overflow;             // a slice has so many that the list is not made
+  uint32_t digit_pick[3];        // radix selection: chosen digit, remaining rank, keys with that digit
+  uint32_t key_bits[4];          // (radix) bits that some key of this CTA has, bits that all have; low and high words
+  uint32_t red[32];              // sums of the warps
+  uint32_t n_cand, n_above;      // the slice's candidates, its tiles above the band
+};
+
+// The CTA's dynamic shared memory.
+struct SelMem {
+  unsigned long long *keys;      // [kClKeys + kSelThreads] the cluster's candidate keys
+  uint32_t *hist;                // [kBins]; later the words' running counts
+  uint32_t *cand;                // [kClKeys] band tiles of the slice
+  uint32_t *words;               // [kWordsShared]
+  __device__ __forceinline__ SelMem() {
+    extern __shared__ __align__(16) uint8_t smem_sel[];
+    keys = reinterpret_cast<unsigned long long *>(smem_sel);
+    hist = reinterpret_cast<uint32_t *>(keys + kClKeys + kSelThreads);
+    cand = hist + kBins;
+    words = cand + kClKeys;
+  }
 };
 
 // A score on the axis of the bins, in steps, 16 to a bin (non-decreasing in the score; not yet cut to whole steps).  Scores
 // lie in [0, log2 A]; three quarters of the bins are given to the top two units, where most tiles and the threshold are:
 // with bins of one width a threshold in the dense part had 2.6 times as many candidates.
 struct StepMap { float lo, hi, off; };   // max(s * lo, s * hi - off)
-// A score below zero (p + varsigma above one: tiles with a single large element) stands at zero: it is in the first bin and
-// must not look as if it lay below it.
-__device__ __forceinline__ float score_pos(float s, const StepMap &m) {
-  return fmaxf(fmaxf(s * m.lo, __fmaf_rn(s, m.hi, -m.off)), 0.0f);
+// Scores below zero (p + varsigma above one: tiles with a single large element) are in the first bin.
+__device__ __forceinline__ float score_pos(float s, const StepMap &m) { return fmaxf(s * m.lo, __fmaf_rn(s, m.hi, -m.off)); }
+__device__ __forceinline__ int score_step(float s, const StepMap &m) {
+  return (int)fminf(fmaxf(score_pos(s, m), 0.0f), (float)(16 * kBins - 1));
 }
-__device__ __forceinline__ int score_step(float s, const StepMap &m) { return (int)fminf(score_pos(s, m), (float)(16 * kBins - 1)); }
 // Screening scores differ from exact ones by less than 1e-4 (see tile_score_screen), 2.5 steps at most.  With k_hi-th largest
 // screening score in bin B, a tile whose screening score lies more than twice that outside bin B is certainly inside or
 // outside the top k_hi; six steps also cover the cut to whole steps.
 constexpr int kScreenBand = 6;
 
-// More candidates than the key list holds: the band's tiles get their exact score in place (decided ones +-infinity), and
-// a radix selection over the finite scores of all slices, 8 bits a pass, gives the threshold key; every CTA sums the
-// cluster's digit counts for itself.  Sets the slice's words and returns the higher-width tiles of the slices before
-// it.  (Out of line: the usual path runs once per launch from a cold instruction cache and stays compact.)
-static __device__ __noinline__ uint32_t selection_by_radix(const Args &a, float *sc, const uint8_t *tiles, uint32_t tile_bytes, uint32_t n_loc,
-                                                           uint32_t i0, int lo_v, int hi_v, uint32_t rr, uint32_t *words,
-                                                           uint32_t *s_digit, uint32_t *s_red, SelShared &sh) {
+// Exact scores of n listed tiles, `NOCT` lanes to a tile, by the warps of `threads` threads that call this together, as keys
+// (at the tile's place in the list; i0: the slice's first tile) or as scores (at the tile's place in the slice).  Two tiles of a
+// lane are on their way at a time, in a function of its own: one at a time, 131072 equal tiles took 152 us to select from
+// instead of 138; with four, or without the call, select_kernel no longer fits its registers, which every encode pays for.
+template <int NOCT, bool BF16>
+__device__ __forceinline__ void exact_listed(const uint8_t *tiles, const uint32_t *list, uint32_t n, uint32_t thread, uint32_t threads,
+                                             float eps_l1, float eps_log, uint32_t i0, unsigned long long *keys, float *scores) {
+  constexpr uint32_t TB = NOCT * 8 * (BF16 ? 2 : 4);
+  constexpr int U = 2;
+  const uint32_t sub = thread % NOCT, per = threads / NOCT;
+  for (uint32_t j0 = thread / NOCT; j0 - thread / NOCT < n; j0 += U * per) {
+    float v[U][8];
+#pragma unroll
+    for (int u = 0; u < U; ++u) load_abs_oct_global<BF16>(tiles + (uint64_t)list[j0 + u * per < n ? j0 + u * per : 0u] * TB, sub, v[u]);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const float ex = ranked_score(exact_score_of_octs<NOCT, true>(v[u], eps_l1, eps_log));
+      const uint32_t j = j0 + u * per;
+      if (j < n && sub == 0) {
+        if (keys) keys[j] = rank_key(ex, i0 + list[j]);
+        else scores[list[j]] = ex;
+      }
+    }
+  }
+}
+static __device__ __noinline__ void exact_listed_any(const Args &a, const uint8_t *tiles, const uint32_t *list, uint32_t n, uint32_t thread,
+                                                     uint32_t threads, uint32_t i0, unsigned long long *keys, float *scores) {
+  auto run = [&](auto noct) {
+    constexpr int N = decltype(noct)::value;
+    if (a.bf16) exact_listed<N, true>(tiles, list, n, thread, threads, a.eps_l1, a.eps_log, i0, keys, scores);
+    else exact_listed<N, false>(tiles, list, n, thread, threads, a.eps_l1, a.eps_log, i0, keys, scores);
+  };
+  switch (a.tile) {
+    case 8: run(std::integral_constant<int, 1>{}); break;
+    case 16: run(std::integral_constant<int, 2>{}); break;
+    case 32: run(std::integral_constant<int, 4>{}); break;
+    case 64: run(std::integral_constant<int, 8>{}); break;
+    default: run(std::integral_constant<int, 16>{}); break;
+  }
+}
+
+// More candidates than the key list holds, for thousands of equal scores or a very long group: a radix selection over the
+// candidates of all slices, 8 bits a pass, gives the threshold key; every CTA sums the cluster's digit counts for itself.  A
+// slice whose own candidates are all listed has their keys in shared memory; else every pass reads the slice, whose candidates
+// have their exact score and whose other tiles +-infinity, from there if it fits and in place if not.  A digit that all keys
+// share is skipped, and so is what lies behind a digit all of whose keys make it.  Sets the slice's words and returns the higher-width tiles of the slices before it.
+// (Out of line: the usual path runs once per launch from a cold instruction cache and stays compact.)
+static __device__ __noinline__ uint32_t selection_by_radix(const Args &a, uint32_t per_cta, int B, uint32_t rr, uint32_t *words, SelShared &sh) {
   cg::cluster_group cl = cg::this_cluster();
   const uint32_t CS = cl.num_blocks(), rank = cl.block_rank();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint32_t noct = a.tile / 8, per = 32u / noct, sub = (uint32_t)lane % noct, grp = (uint32_t)lane / noct;
-  for (uint32_t c0 = (uint32_t)warp * 32u; c0 < n_loc; c0 += kSelThreads) {
-    const uint32_t i = c0 + lane;
-    const float s = i < n_loc ? sc[i] : 0.0f;
-    const int v = score_step(s, {a.step_lo, a.step_hi, a.step_off});
-    const bool cand = i < n_loc && v >= lo_v && v < hi_v;
-    if (i < n_loc && !cand) sc[i] = __int_as_float(v >= hi_v ? 0x7f800000 : (int)0xff800000);
-    unsigned m = __ballot_sync(kFull, cand);
-    if (a.exact_scores) continue;
-    const uint32_t n = (uint32_t)__popc(m);
-    for (uint32_t q = 0; q < n; q += per) {
-      const bool live = q + grp < n;
-      const uint32_t b = __fns(m, 0, (int)(live ? q + grp : 0u) + 1);
-      const float ex = ranked_score(exact_score_any(tiles + (uint64_t)(c0 + b) * tile_bytes, noct, a.bf16 != 0, sub, a.eps_l1, a.eps_log));
-      if (live && sub == 0) sc[c0 + b] = ex;
+  const SelMem mem;
+  unsigned long long *const s_keys = mem.keys;
+  uint32_t *const s_cand = mem.cand, *const s_count = mem.hist /* [2][256] */, *const s_red = sh.red;
+  const uint32_t ng = (uint32_t)a.rank_per_group, i0 = rank * per_cta, n_loc = i0 < ng ? (ng - i0 < per_cta ? ng - i0 : per_cta) : 0u;
+  const uint64_t first = (uint64_t)(blockIdx.x / CS) * ng + i0;
+  float *const sc = a.scores + first;
+  const uint8_t *const tiles = a.in + first * (a.tile * (a.bf16 ? 2u : 4u));
+  const int band = a.exact_scores ? 0 : kScreenBand, lo_v = B * 16 - band, hi_v = (B + 1) * 16 + band;
+  const uint32_t nc = sh.n_cand;
+  const bool listed = nc <= (uint32_t)kClKeys;
+  float *const own = n_loc <= 2u * (kClKeys + kSelThreads) ? reinterpret_cast<float *>(s_keys) : sc;   // (not listed) the slice's scores
+  if (listed) {
+    if (a.exact_scores)
+      for (uint32_t j = threadIdx.x; j < nc; j += kSelThreads) s_keys[j] = rank_key(sc[s_cand[j]], i0 + s_cand[j]);
+    else
+      exact_listed_any(a, tiles, s_cand, nc, threadIdx.x, kSelThreads, i0, s_keys, nullptr);
+  } else {
+    __syncthreads();   // the list, which holds a part of the candidates only, makes room for one of 128 per warp
+    uint32_t *const mine = s_cand + warp * 128;
+    for (uint32_t c0 = (uint32_t)warp * 128u; c0 < n_loc; c0 += 4u * kSelThreads) {
+      uint32_t n = 0;
+#pragma unroll
+      for (uint32_t k = 0; k < 4; ++k) {
+        const uint32_t i = c0 + 32u * k + lane;
+        const float s = i < n_loc ? sc[i] : 0.0f;
+        const int v = score_step(s, {a.step_lo, a.step_hi, a.step_off});
+        const bool cand = i < n_loc && v >= lo_v && v < hi_v;
+        if (i < n_loc) own[i] = cand ? s : __int_as_float(v >= hi_v ? 0x7f800000 : (int)0xff800000);
+        const unsigned m = __ballot_sync(kFull, cand);
+        if (cand) mine[n + (uint32_t)__popc(m & ((1u << lane) - 1u))] = i;
+        n += (uint32_t)__popc(m);
+      }
+      if (a.exact_scores) continue;
+      __syncwarp();
+      exact_listed_any(a, tiles, mine, n, lane, 32u, i0, nullptr, own);
+      __syncwarp();
     }
   }
-  __threadfence_block();
-  unsigned long long prefix = 0, mask = 0;
-  uint32_t r = rr;
-  for (int shift = 56; shift >= 0; shift -= 8) {
-    if (threadIdx.x < 256) s_digit[threadIdx.x] = 0;
-    __syncthreads();
-    for (uint32_t i = threadIdx.x; i < n_loc; i += kSelThreads) {
-      const float s = __ldcg(sc + i);
-      if ((__float_as_uint(s) & 0x7f800000u) != 0x7f800000u) {
-        const unsigned long long key = rank_key(s, i0 + i);
-        if ((key & mask) == prefix) atomicAdd(&s_digit[(unsigned)(key >> shift) & 255u], 1u);
+  __syncthreads();
+  // f(takes part, key) for every candidate of the slice; whole warps at a time
+  auto each = [&](auto &&f) {
+    if (listed) {
+      for (uint32_t i = threadIdx.x; i - (uint32_t)lane < nc; i += kSelThreads) f(i < nc, i < nc ? s_keys[i] : 0ull);
+    } else {
+      for (uint32_t b = threadIdx.x; b - (uint32_t)lane < n_loc; b += 4 * kSelThreads) {
+        float s[4];   // (the loads together: they may come from memory)
+#pragma unroll
+        for (uint32_t u = 0; u < 4; ++u) s[u] = b + u * kSelThreads < n_loc ? own[b + u * kSelThreads] : __int_as_float(0x7f800000);
+#pragma unroll
+        for (uint32_t u = 0; u < 4; ++u)
+          f((__float_as_uint(s[u]) & 0x7f800000u) != 0x7f800000u, rank_key(s[u], i0 + b + u * kSelThreads));
       }
     }
+  };
+  // bits on which the cluster's keys differ
+  unsigned long long some = 0, all = ~0ull;
+  each([&](bool in, unsigned long long key) {
+    if (in) { some |= key; all &= key; }
+  });
+  auto reduce = [&]() {
+    some = (unsigned long long)__reduce_or_sync(kFull, (uint32_t)(some >> 32)) << 32 | __reduce_or_sync(kFull, (uint32_t)some);
+    all = (unsigned long long)__reduce_and_sync(kFull, (uint32_t)(all >> 32)) << 32 | __reduce_and_sync(kFull, (uint32_t)all);
+  };
+  if (threadIdx.x < 4) sh.key_bits[threadIdx.x] = threadIdx.x < 2 ? 0u : 0xffffffffu;
+  s_count[threadIdx.x] = 0;
+  static_assert(kSelThreads == 512, "a thread to each of the two times 256 counts");
+  reduce();
+  __syncthreads();
+  if (lane == 0) {
+    atomicOr(&sh.key_bits[0], (uint32_t)some);
+    atomicOr(&sh.key_bits[1], (uint32_t)(some >> 32));
+    atomicAnd(&sh.key_bits[2], (uint32_t)all);
+    atomicAnd(&sh.key_bits[3], (uint32_t)(all >> 32));
+  }
+  cl.sync();
+  some = 0;
+  all = ~0ull;
+  if (lane < (int)CS) {
+    const uint32_t *k = cl.map_shared_rank(&sh, lane)->key_bits;
+    some = (unsigned long long)k[1] << 32 | k[0];
+    all = (unsigned long long)k[3] << 32 | k[2];
+  }
+  reduce();
+  const unsigned long long varying = some ^ all;
+  unsigned long long prefix = 0, mask = 0;
+  uint32_t r = rr, buf = 0;
+  for (int shift = 56; shift >= 0; shift -= 8) {
+    if (((varying >> shift) & 0xffull) == 0) {
+      prefix |= some & (0xffull << shift);
+      mask |= 0xffull << shift;
+      continue;
+    }
+    uint32_t *const s_digit = s_count + 256 * buf;
+    each([&](bool in, unsigned long long key) {
+      in = in && (key & mask) == prefix;
+      const uint32_t d = (uint32_t)(key >> shift) & 255u;
+      const unsigned m = __ballot_sync(kFull, in);
+      if (m == 0u) return;
+      // the warp's keys often share the digit: one addition then
+      const uint32_t d0 = __shfl_sync(kFull, d, __ffs(m) - 1);
+      if (__ballot_sync(kFull, in && d == d0) == m) {
+        if (lane == 0) atomicAdd(&s_digit[d0], (uint32_t)__popc(m));
+      } else if (in) {
+        atomicAdd(&s_digit[d], 1u);
+      }
+    });
     cl.sync();
+    // (the other half of the counts was read by everybody before this barrier)
+    if (threadIdx.x < 256) s_count[256 * (buf ^ 1u) + threadIdx.x] = 0;
     uint32_t cnt = 0;   // thread d < 256: keys of the cluster with digit d
     if (threadIdx.x < 256)
       for (uint32_t q = 0; q < CS; ++q) cnt += cl.map_shared_rank(s_digit, q)[threadIdx.x];
@@ -373,20 +510,34 @@ static __device__ __noinline__ uint32_t selection_by_radix(const Args &a, float 
     if (threadIdx.x < 256) {
       uint32_t above = incl - cnt;
       for (int w = warp + 1; w < 8; ++w) above += s_red[w];
-      if (above < r && above + cnt >= r) { sh.digit_pick[0] = threadIdx.x; sh.digit_pick[1] = r - above; }
+      if (above < r && above + cnt >= r) { sh.digit_pick[0] = threadIdx.x; sh.digit_pick[1] = r - above; sh.digit_pick[2] = cnt; }
     }
-    cl.sync();   // everybody has read everybody's counts (they are cleared next pass) and made the pick
+    __syncthreads();
     prefix |= (unsigned long long)sh.digit_pick[0] << shift;
     mask |= 0xffull << shift;
     r = sh.digit_pick[1];
+    buf ^= 1u;
+    if (sh.digit_pick[2] == r) break;   // all keys that begin like this make it
+    __syncthreads();   // the pick is read, s_red is free
   }
-  // every tile against the threshold; the slices' counts have to be exchanged
+  // the candidates against the threshold; the slices' counts have to be exchanged
   uint32_t bits_here = 0;
-  for (uint32_t c0 = (uint32_t)warp * 32u; c0 < n_loc; c0 += kSelThreads) {
-    const uint32_t i = c0 + lane;
-    const unsigned m = __ballot_sync(kFull, i < n_loc && rank_key(__ldcg(sc + i), i0 + i) >= prefix);   // +inf is above every threshold
-    if (lane == 0) { words[c0 >> 5] = m; bits_here += (uint32_t)__popc(m); }
+  if (listed) {
+    for (uint32_t j = threadIdx.x; j < nc; j += kSelThreads)
+      if (s_keys[j] >= prefix) {
+        const uint32_t i = s_cand[j];
+        atomicOr(&words[i >> 5], 1u << (i & 31u));
+        ++bits_here;
+      }
+    if (threadIdx.x == 0) bits_here += sh.n_above;
+  } else {
+    for (uint32_t c0 = (uint32_t)warp * 32u; c0 < n_loc; c0 += kSelThreads) {
+      const uint32_t i = c0 + lane;
+      const unsigned m = __ballot_sync(kFull, i < n_loc && rank_key(own[i], i0 + i) >= prefix);   // +inf is above every threshold
+      if (lane == 0) { words[c0 >> 5] = m; bits_here += (uint32_t)__popc(m); }
+    }
   }
+  bits_here = __reduce_add_sync(kFull, bits_here);
   __syncthreads();
   if (lane == 0) s_red[warp] = bits_here;
   __syncthreads();
@@ -395,10 +546,9 @@ static __device__ __noinline__ uint32_t selection_by_radix(const Args &a, float 
     for (int w = 0; w < kSelThreads / 32; ++w) T += s_red[w];
     cl.map_shared_rank(&sh, threadIdx.x)->tot[rank] = T;
   }
-  cl.sync();
+  cl.sync();   // (the last time that a CTA touches another one's shared memory is before this)
   uint32_t before = 0;
   for (uint32_t q = 0; q < rank; ++q) before += sh.tot[q];
-  cl.sync();   // nobody leaves while its memory may still be written
   return before;
 }
 
@@ -500,16 +650,14 @@ __global__ void __launch_bounds__(kSelThreads, 2) select_kernel(const __grid_con
   const uint32_t ng = (uint32_t)a.rank_per_group, k = (uint32_t)a.rank_k;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const StepMap map = {a.step_lo, a.step_hi, a.step_off};
-  extern __shared__ __align__(16) uint8_t smem_sel[];
-  unsigned long long *s_keys = reinterpret_cast<unsigned long long *>(smem_sel);        // [kClKeys + kSelThreads]
-  uint32_t *s_hist = reinterpret_cast<uint32_t *>(s_keys + kClKeys + kSelThreads);      // [kBins]; later the words' running counts
-  uint32_t *s_cand = s_hist + kBins;                                                    // [kClKeys] band tiles of the slice
-  uint32_t *s_words = s_cand + kClKeys;                                                 // [kWordsShared]
+  const SelMem mem;
+  unsigned long long *const s_keys = mem.keys;
+  uint32_t *const s_hist = mem.hist, *const s_cand = mem.cand, *const s_words = mem.words;
   __shared__ SelShared sh;
-  __shared__ uint32_t s_coarse[256];          // the CTA's coarse counts [kCoarse]; (radix) digit counts
+  __shared__ uint32_t s_coarse[kCoarse];      // the CTA's coarse counts
   __shared__ __align__(8) uint32_t s_sum[2][kCoarse];   // the cluster's coarse counts; its fine counts in the chosen coarse bin
-  __shared__ uint32_t s_red[32];
-  __shared__ uint32_t s_ncand, s_nabove, s_base, s_made;
+  uint32_t *const s_red = sh.red;
+  __shared__ uint32_t s_base, s_made;
   TraceScope trace(a.trace, 2);
 
   const uint32_t i0 = rank * per_cta;                                   // first tile of the slice, inside the group
@@ -525,7 +673,7 @@ __global__ void __launch_bounds__(kSelThreads, 2) select_kernel(const __grid_con
   }
   for (uint32_t b = threadIdx.x; b < (uint32_t)kBins; b += kSelThreads) s_hist[b] = 0;
   if (threadIdx.x < 2 * kCoarse) s_sum[0][threadIdx.x] = 0;
-  if (threadIdx.x == 0) { sh.n_keys = 0; sh.n_total = 0; s_ncand = 0; s_nabove = 0; s_made = 0; }
+  if (threadIdx.x == 0) { sh.n_keys = 0; sh.n_total = 0; sh.overflow = 0; sh.n_cand = 0; sh.n_above = 0; s_made = 0; }
   grid_dependency_wait();   // the scores are the score kernel's (or the tensor a kernel's in front)
   trace.started();
   float *sc = a.scores + g * (uint64_t)ng + i0;
@@ -540,7 +688,7 @@ __global__ void __launch_bounds__(kSelThreads, 2) select_kernel(const __grid_con
   const float *const s_own = reinterpret_cast<const float *>(s_keys);
   auto first_of = [&](uint32_t it) { return (it * NW + (uint32_t)warp) * 128u + (uint32_t)lane * 4u; };
   auto left_of = [&](uint32_t it) { return (int)n_loc - (int)first_of(it); };   // tiles of the slice from the lane's first on
-  auto load4 = [&](uint32_t it) -> float4 {   // (anything behind the slice's end: told by its place, not by its value)
+  auto load4 = [&](uint32_t it) -> float4 {   // zeroes behind the slice's end (told by their place, not by their value)
     const uint32_t i = first_of(it);
     if constexpr (!std::is_void<C>::value)   // (slices of whole words)
       return i < n_loc ? *reinterpret_cast<const float4 *>(s_own + i) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
@@ -607,8 +755,8 @@ __global__ void __launch_bounds__(kSelThreads, 2) select_kernel(const __grid_con
   const int B = (int)(Bc * kFine + Bf), band = a.exact_scores ? 0 : kScreenBand;
   const int lo_v = B * 16 - band, hi_v = (B + 1) * 16 + band;
   {
-    // step(s) >= v for a whole v is score_pos(s) >= v; the last bin has nothing above it
-    const float lo_f = (float)lo_v, hi_f = hi_v > 16 * kBins - 1 ? __int_as_float(0x7f800000) : (float)hi_v;
+    // step(s) >= v for a whole v > 0 is score_pos(s) >= v; the first bin has nothing below it, the last one nothing above
+    const float lo_f = B > 0 ? (float)lo_v : __int_as_float(0xff800000), hi_f = hi_v > 16 * kBins - 1 ? __int_as_float(0x7f800000) : (float)hi_v;
     uint32_t n_above = 0;
     auto decide = [&](uint32_t it, const float4 &v) {
       const float t[4] = {score_pos(v.x, map), score_pos(v.y, map), score_pos(v.z, map), score_pos(v.w, map)};
@@ -616,7 +764,7 @@ __global__ void __launch_bounds__(kSelThreads, 2) select_kernel(const __grid_con
       uint32_t above = 0, cand = 0;   // of the lane's four tiles
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        above |= (j < left && t[j] >= hi_f) ? 1u << j : 0u;
+        above |= t[j] >= hi_f ? 1u << j : 0u;   // (a zero behind the slice's end is above nothing)
         cand |= (j < left && !(t[j] >= hi_f) && !(t[j] < lo_f)) ? 1u << j : 0u;
       }
       // eight lanes hold a word
@@ -635,7 +783,7 @@ __global__ void __launch_bounds__(kSelThreads, 2) select_kernel(const __grid_con
           if (lane >= o) incl += x;
         }
         uint32_t base = 0;
-        if (lane == 31) base = atomicAdd(&s_ncand, incl);
+        if (lane == 31) base = atomicAdd(&sh.n_cand, incl);
         uint32_t slot = __shfl_sync(kFull, base, 31) + incl - mine;
         const uint32_t i = first_of(it);
         for (uint32_t m = cand; m; m &= m - 1u, ++slot)
@@ -659,15 +807,18 @@ __global__ void __launch_bounds__(kSelThreads, 2) select_kernel(const __grid_con
       }
     }
     n_above = __reduce_add_sync(kFull, n_above);
-    if (lane == 0 && n_above) atomicAdd(&s_nabove, n_above);
+    if (lane == 0 && n_above) atomicAdd(&sh.n_above, n_above);
   }
   __syncthreads();
-  const uint32_t nc = s_ncand, n_listed = nc <= (uint32_t)kClKeys ? nc : 0u;   // (too many: the cluster's total says so to all)
+  // A slice with more than a quarter of what the list holds is nearly always one of many like it (equal scores): its keys are
+  // not made here, which would be for nothing, but in selection_by_radix.
+  const uint32_t nc = sh.n_cand, n_listed = nc <= (uint32_t)kClKeys / 4 ? nc : 0u;
   if (threadIdx.x == 0) s_base = nc ? atomicAdd(&cl.map_shared_rank(&sh, 0)->n_keys, nc) : 0u;
   if (threadIdx.x < CS) {
     SelShared *o = cl.map_shared_rank(&sh, threadIdx.x);
-    o->part[rank] = s_nabove;
+    o->part[rank] = sh.n_above;
     if (nc) atomicAdd(&o->n_total, nc);
+    if (nc != n_listed) o->overflow = 1;
   }
   const uint32_t tile_bytes = a.tile * (a.bf16 ? 2u : 4u);
   const uint8_t *tiles = a.in + (g * (uint64_t)ng + i0) * tile_bytes;   // (not used with wider allocation tiles: their scores are exact)
@@ -699,8 +850,8 @@ __global__ void __launch_bounds__(kSelThreads, 2) select_kernel(const __grid_con
     if (rank == 0 && threadIdx.x == 0) atomicOr(a.status, 8u /* TAHQ_DEV_INTERNAL */);
     rr = rr > n ? n : 1u;
   }
-  if (n > (uint32_t)kClKeys) {
-    before = selection_by_radix(a, sc, tiles, tile_bytes, n_loc, i0, lo_v, hi_v, rr, words, s_coarse, s_red, sh);
+  if (n > (uint32_t)kClKeys || sh.overflow) {
+    before = selection_by_radix(a, per_cta, B, rr, words, sh);
   } else {
     // band tiles that made it: those of the slices before this one are counted, those of this slice get their bit
     auto won = [&](unsigned long long key) {
@@ -729,9 +880,10 @@ __global__ void __launch_bounds__(kSelThreads, 2) select_kernel(const __grid_con
   uint32_t *const bitmap = reinterpret_cast<uint32_t *>(a.packed + a.off_bitmap);
   const uint64_t t0 = (g * (uint64_t)ng + i0) * a.alloc_m;   // first quantisation tile of the slice
   auto word_at = [&](uint32_t w) { return *(volatile const uint32_t *)(words + w); };   // (in global memory: changed by atomics)
-  uint32_t carry = before;
+  uint32_t carry = before, next = threadIdx.x < n_words ? word_at(threadIdx.x) : 0u;
   for (uint32_t w0 = 0; w0 < n_words; w0 += kSelThreads) {
-    const uint32_t w = w0 + threadIdx.x, wv = w < n_words ? word_at(w) : 0u, c = (uint32_t)__popc(wv);
+    const uint32_t w = w0 + threadIdx.x, wv = next, c = (uint32_t)__popc(wv);
+    next = w + kSelThreads < n_words ? word_at(w + kSelThreads) : 0u;   // (a round trip to L2 for a very long slice)
     uint32_t incl = c;
 #pragma unroll
     for (int o = 1; o < 32; o *= 2) {
