@@ -810,9 +810,9 @@ __global__ void __launch_bounds__(kSelThreads, 2) select_kernel(const __grid_con
     if (lane == 0 && n_above) atomicAdd(&sh.n_above, n_above);
   }
   __syncthreads();
-  // A slice with more than a quarter of what the list holds is nearly always one of many like it (equal scores): its keys are
-  // not made here, which would be for nothing, but in selection_by_radix.
-  const uint32_t nc = sh.n_cand, n_listed = nc <= (uint32_t)kClKeys / 4 ? nc : 0u;
+  // A slice with more than its part of what the list holds, or a quarter of that, is nearly always one of many like it (equal
+  // scores): its keys are not made here, which would be for nothing, but in selection_by_radix.
+  const uint32_t nc = sh.n_cand, n_listed = nc <= ((uint32_t)kClKeys >> (CS < 4u ? CS >> 1 : 2u)) ? nc : 0u;   // (CS: a power of two)
   if (threadIdx.x == 0) s_base = nc ? atomicAdd(&cl.map_shared_rank(&sh, 0)->n_keys, nc) : 0u;
   if (threadIdx.x < CS) {
     SelShared *o = cl.map_shared_rank(&sh, threadIdx.x);
