@@ -69,3 +69,18 @@ def test_transformed_tiles_whose_sums_overflow(budget, rounding, G, dtype):
     x[:, 3::G] = torch.linspace(0, 1.4e38, 60, device="cuda")[:, None]
     x[1::2] *= -1
     check(x.to(dtype), tile=G, budget_millibits=budget, rounding=rounding, seed=3)
+
+
+@pytest.mark.parametrize("bits", [2, 3, 4, 5, 6, 7, 8])
+def test_scales_up_to_the_largest_and_beyond(bits):
+    """As test_every_binary16_scale, for the scales that it leaves out, up to 65504, and ranges of up to 2^40 whose scale is that."""
+    s = np.arange(1, 0x7C00, dtype=np.uint16).view(np.float16).astype(np.float64)
+    q = 2 ** bits - 1
+    s = np.concatenate([s[s * q > 50000], 65504 * 2.0 ** (np.arange(1, 49) / 2)])
+    s = np.concatenate([s, s[-1:].repeat(-len(s) % 8)])
+    x = (s[:, None] * (np.arange(32) % q + 0.5)[None, :]).astype(np.float32)
+    x[:, 0] = 0
+    x[:, 1] = (s * q).astype(np.float32)
+    x[:, 2::3] = np.nextafter(x[:, 2::3], np.float32(0))
+    x[:, 3::3] = np.nextafter(x[:, 3::3], np.float32(1e30))
+    check(torch.from_numpy(x.reshape(-1, 256)).cuda(), tile=32, budget_millibits=bits * 1000, tau=float("inf"))
