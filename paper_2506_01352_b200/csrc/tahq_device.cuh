@@ -1,12 +1,10 @@
 // Device-side building blocks of the TAH-Quant boundary codec for sm_100a.
 //
-// Work decomposition: ONE THREAD OWNS ONE TILE (quantisation group, Sec. 3.1) -- or half of a
-// 128-wide tile -- and keeps its elements in registers, so that the Hadamard butterfly (Eq. 4),
-// the reductions of Eq. 1-3 and the bit packing need no cross-lane traffic.  Tiles reach the
-// thread through shared memory: rows are copied (16-byte cp.async, or tiled TMA with the 128-byte
-// swizzle) into an XOR-swizzled stage from which every thread reads its own row with conflict-free
-// 128-bit loads.  tahq_stream.cuh builds per-warp stages of 32 rows from these blocks,
-// 
+// Two decompositions of the work build on them.  In one a thread owns a whole tile (quantisation group, Sec. 3.1) -- or
+// half of a 128-wide tile -- in registers, so that the Hadamard butterfly (Eq. 4), the reductions of Eq. 1-3 and the bit
+// packing need no cross-lane traffic; tiles reach it through an XOR-swizzled stage of 32 rows per warp, filled by 16-byte
+// cp.async or tiled TMA with the 128-byte swizzle (tahq_stream.cuh).  In the other a lane owns 64 bytes of the tensor and
+// neighbouring lanes share a tile (tahq_lanes.cuh).
 #pragma once
 
 #include <cuda_bf16.h>
@@ -32,10 +30,7 @@ struct Cfg {
   static constexpr int ESZ = BF16 ? 2 : 4;
   static constexpr int ROWB = EPT * ESZ;           // bytes of one thread-row: 64 / 128 / 256
   static constexpr int CPR = ROWB / 16;            // 16-byte chunks per row: 4 / 8 / 16
-  static constexpr int TPC = kThreads / LPT;       // tiles per CTA chunk
-  static constexpr int STAGE_BYTES = kThreads * ROWB;
   static constexpr int NOCT = EPT / 8;             // groups of 8 elements per thread
-  static constexpr int MAX_PAY = kThreads * EPT;   // payload bytes of one chunk at 8 bits
 };
 
 // XOR swizzle of 16-byte chunks: the eight threads of a quarter-warp, whose rows are ROWB bytes
@@ -52,10 +47,6 @@ __device__ __forceinline__ int phys_chunk(int row, int q) {
 // ------------------------------------------------------------------------------------------
 // cp.async
 // ------------------------------------------------------------------------------------------
-__device__ __forceinline__ void cp_async4(void *smem, const void *gmem) {
-  unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(gmem) : "memory");
-}
 __device__ __forceinline__ void cp_async16(void *smem, const void *gmem, int src_bytes) {
   unsigned s = (unsigned)__cvta_generic_to_shared(smem);
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(s), "l"(gmem), "r"(src_bytes)
@@ -94,8 +85,7 @@ __device__ __forceinline__ void cp_async_wait() {
 }
 
 // ------------------------------------------------------------------------------------------
-// Bulk asynchronous copies (TMA, untiled) completing on an mbarrier: one thread moves a whole
-// contiguous slice; addresses and sizes are multiples of 16 bytes.  Every wait is bounded.
+// TMA copies completing on an mbarrier.  Every wait is bounded.
 // ------------------------------------------------------------------------------------------
 __device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void mbar_init(unsigned long long *bar, unsigned count) {
@@ -104,12 +94,6 @@ __device__ __forceinline__ void mbar_init(unsigned long long *bar, unsigned coun
 __device__ __forceinline__ void mbar_init_fence() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
 __device__ __forceinline__ void mbar_expect_tx(unsigned long long *bar, unsigned bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void bulk_copy_g2s(void *dst, const void *src, unsigned bytes, unsigned long long *bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   smem_u32(dst)),
-               "l"(src), "r"(bytes), "r"(smem_u32(bar))
-               : "memory");
 }
 __device__ __forceinline__ void fence_async_proxy() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 // true when the phase with the given parity has completed; gives up after a bounded number of polls
@@ -153,15 +137,6 @@ __device__ __forceinline__ void load_oct(const uint8_t *stage, int row, int o, f
     v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
     v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
   }
-}
-
-// One element of this thread's row (dynamic index), for the pivot.
-template <class C>
-__device__ __forceinline__ float load_elem(const uint8_t *stage, int row, int k) {
-  constexpr int EPC = 16 / C::ESZ;
-  const uint8_t *p = stage + (size_t)phys_chunk<C>(row, k / EPC) * 16 + (size_t)(k % EPC) * C::ESZ;
-  if constexpr (C::BF16) return __uint_as_float((uint32_t)(*reinterpret_cast<const uint16_t *>(p)) << 16);
-  else return *reinterpret_cast<const float *>(p);
 }
 
 // ------------------------------------------------------------------------------------------

@@ -113,7 +113,7 @@ struct UnitRing {
   }
 };
 
-// a row: shared memory <-> registers (raw words)
+// a row: shared memory -> registers (raw words)
 template <class C>
 __device__ __forceinline__ void row_load_words(const uint8_t *stage, int row, uint32_t (&w)[C::ROWB / 4]) {
 #pragma unroll
@@ -122,14 +122,6 @@ __device__ __forceinline__ void row_load_words(const uint8_t *stage, int row, ui
     w[4 * q] = v.x; w[4 * q + 1] = v.y; w[4 * q + 2] = v.z; w[4 * q + 3] = v.w;
   }
 }
-template <class C>
-__device__ __forceinline__ void row_store_words(uint8_t *stage, int row, const uint32_t (&w)[C::ROWB / 4]) {
-#pragma unroll
-  for (int q = 0; q < C::CPR; ++q)
-    *reinterpret_cast<uint4 *>(stage + (size_t)phys_chunk<C>(row, q) * 16) =
-        make_uint4(w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
-}
-
 // smallest and largest element of a row held as raw words
 template <class C>
 __device__ __forceinline__ void words_minmax(const uint32_t (&w)[C::ROWB / 4], float &mn, float &mx) {
