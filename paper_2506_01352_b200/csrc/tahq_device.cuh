@@ -26,10 +26,10 @@ struct Cfg {
   static constexpr int G = G_;
   static constexpr bool BF16 = BF16_;
   static constexpr int LPT = (G == 128) ? 2 : 1;   // lanes (threads) per tile
-  static constexpr int EPT = G / LPT;              // elements per thread: 32 or 64
+  static constexpr int EPT = G / LPT;              // elements per thread: 8 ... 64
   static constexpr int ESZ = BF16 ? 2 : 4;
-  static constexpr int ROWB = EPT * ESZ;           // bytes of one thread-row: 64 / 128 / 256
-  static constexpr int CPR = ROWB / 16;            // 16-byte chunks per row: 4 / 8 / 16
+  static constexpr int ROWB = EPT * ESZ;           // bytes of one thread-row: 16 ... 256
+  static constexpr int CPR = ROWB / 16;            // 16-byte chunks per row: 1 ... 16
   static constexpr int NOCT = EPT / 8;             // groups of 8 elements per thread
 };
 

@@ -973,10 +973,15 @@ __global__ void __launch_bounds__(QuantLanes<C>::NT, 1) quant_lanes_kernel(const
 }
 
 // Binary32 always; bfloat16 while the time is that of a warp's chain and not of the instructions: up to two rounds to a warp,
-// and one where quant2_kernel is at its best (tiles of 64, widths up to 4 bits, rounding to nearest).  Both sides measured,
-// encode with quant2_kernel against this one: tiles of 64 at 3.8 bits, 32 thousand 14.6 / 14.2 us, 51 thousand 15.7 / 15.8, 94
-// thousand 17.4 / 17.8, at 4 bits 6.7 / 7.5, at 6.8 bits 20.7 / 19.9; 51 thousand with stochastic rounding 21.8 / 21.3; tiles of
-// 128, 45 thousand -- two rounds -- 20.3 / 19.2.  Three rounds, 127 thousand tiles of 64: the kernels alone 7.7 / 8.9.
+// and one where quant2_kernel is at its best (tiles of 64, widths up to 4 bits, rounding to nearest).  Encode, us, with
+// quant2_kernel / with this one, at one, two and three rounds to a warp of 20 on 148 SMs:
+//   tiles of 64     3.8 bits 16.3/15.8 19.3/19.5 22.4/25.1   6.8 bits 18.5/17.0 22.3/20.8 25.2/27.2   stochastic 22.2/20.6 28.6/26.6 33.8/37.0
+//   tiles of 128    3.8 bits 16.5/15.6 21.2/20.9 25.3/24.8   6.8 bits 19.7/16.6 24.7/22.2 28.4/26.8   stochastic 23.5/20.7 34.2/30.7 40.4/37.0
+//   tiles of 32     3.8 bits 18.5/18.5 21.9/22.1 27.8/26.9   6.8 bits 20.2/19.8 24.4/24.1 30.2/29.6   stochastic 22.4/23.3 28.0/29.4 38.4/36.3
+// Tiles of 32 are even (within 5 % either way) and follow the rule of 128.  Binary32, 512 / 8192 x 4096: tiles of 64 at 3.5 bits
+// 18.0/16.4 71.0/68.7, at 6.5 bits 20.6/17.2 87.5/76.4, stochastic 25.1/19.9 145/103; of 128 18.0/15.7 79.3/72.9; of 32
+// 16.2/15.9 67.8/70.9, at 4 bits 5.0/5.1 30.7/32.4, stochastic 19.1/19.2 104.3/103.0 -- 4 % behind on large tensors of tiles of
+// 32, which do not get a kernel of their own for that.
 template <class C, bool SR>
 bool quant_lanes_pays(uint64_t n_rounds, bool narrow, int sms) {
   const uint64_t per_warp = C::G == 64 && narrow && !SR ? 1 : 2;

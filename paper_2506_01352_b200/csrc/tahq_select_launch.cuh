@@ -75,9 +75,11 @@ static int select_cluster_size(const Args &a, const DevInfo &d) {
 
 // Are the scores of this call formed in the selection kernel?  A launch less, and they are binned from shared memory; but a
 // group's tensor then goes through the few SMs of its cluster, and the scores of many clusters crowd each other where a grid
-// of score CTAs spreads evenly.  Encode (us), scores in front -> fused: 3 x 256 x 640 fp32 (48 CTAs of 10240 elements)
-// 13.5 -> 12.0, 16 x 128 x 512 bf16 (64 CTAs of 16384) 12.1 -> 11.8; 1 x 512 x 768 bf16 (16 of 24576) 12.0 -> 12.2,
-// 8 x 512 x 640 bf16 (128 of 20480) 14.8 -> 15.7.  Groups that share words of the bit map have its clear in front anyway.
+// of score CTAs spreads evenly.  Encode (us), scores in front -> fused.  Elements per CTA: 3 x 256 x 640 fp32 (48 CTAs of
+// 10240) 13.5 -> 12.0, 16 x 128 x 512 bf16 (64 CTAs of 16384) 12.1 -> 11.5; 1 x 512 x 768 bf16 (16 of 24576) 12.0 -> 12.2.
+// CTAs: groups of 16 x 1024 bf16, which have one each, gain at every number (74: 12.4 -> 11.5, 148: 13.9 -> 12.7, 296: 17.0 ->
+// 15.8), groups of two CTAs up to about half of the SMs (40 groups of 32 x 1024 12.7 -> 12.0, 80 groups 14.4 -> 15.0): the line is
+// where both gain.  Groups that share words of the bit map have its clear in front anyway.
 template <class C>
 static bool fuse_scores(const Args &a, const DevInfo &d) {
   if (!a.whole_words || a.exact_scores || !select_ready<C>(d.dev)) return false;
