@@ -43,13 +43,18 @@ class _Kept:
 
     The bytes lie in a box; a change of a field puts an empty box in its place.  A thread that lays the structure out while
     another one changes a field fills the box that it took before it read the fields, so what it read can be kept only as
-    long as it is current.  The box is no part of the object's state: not of ``vars()``, of copies or of pickles.
+    long as it is current.  The box is no part of the object's state: not of ``vars()``, of copies or of pickles.  (A value
+    that is put into ``vars()`` behind the object's back is seen after the next change of a field.)
     """
 
     __slots__ = ("_box",)
 
     def __setattr__(self, name, value):
         object.__setattr__(self, name, value)
+        _set_box(self, [None])
+
+    def __delattr__(self, name):   # (the field has its default again)
+        object.__delattr__(self, name)
         _set_box(self, [None])
 
     def __getstate__(self):

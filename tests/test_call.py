@@ -110,3 +110,10 @@ def test_the_forms_of_an_address(form):
     for wrong in ("x", b"x", 1.5, [1], types.SimpleNamespace(value="x")):
         with pytest.raises(TypeError):
             T.tahq_encode(p, wrong, 0, 0, 0, 0, 0)
+
+
+def test_a_field_that_is_deleted_has_its_default_again():
+    p = T.Params(tokens=128, hidden=256, group_tokens=64, tile=48)
+    assert T.tahq_encode(p, 4096, 8192, 16, 12288, 1 << 30, 0) == 1
+    del p.tile
+    assert p.raw() == bytes(p.c()) and T.tahq_encode(p, 4096, 8192, 16, 12288, 1 << 30, 0) == 3
